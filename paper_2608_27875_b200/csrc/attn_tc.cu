@@ -109,8 +109,9 @@ struct TcParams {
     const float* k_scales;
     const int32_t* vl_idx;
     const uint32_t* vl_bits;
-    uint32_t* redo;              // [0]: number of CTAs of the optimistic kernel that gave up, [1 + 3 i ...]: their block indices
-    int grid_x;                  // blockIdx.x range of the optimistic kernel (pairs of query tiles x slices)
+    uint32_t* redo;              // [0]: number of CTAs of the optimistic kernel that gave up, [1 + i]: their block indices
+    int grid_x;                  // work items per head (pairs of query tiles x slices)
+    int head_group;              // heads whose items are interleaved, longest first (a whole number of KV heads)
     const uint8_t* vl_tiles;     // FP8 / INT4 scores: the vertical-line operand tiles [B*Hq][mask_words/2][2048] (null: none)
     void* out;
     float* lse;
@@ -470,9 +471,13 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     const uint32_t n_items = EXACT ? p.redo[0] : 1u;
 #pragma unroll 1
     for (uint32_t item = EXACT ? blockIdx.x : 0u; item < n_items; item += (EXACT ? gridDim.x : 1u)) {
-    const int bx = EXACT ? (int)p.redo[1 + 3 * item] : (int)blockIdx.x;
-    const int h = EXACT ? (int)p.redo[2 + 3 * item] : (int)blockIdx.y, b = EXACT ? (int)p.redo[3 + 3 * item] : (int)blockIdx.z;
-    const int pt_lin = p.grid_x - 1 - bx;                    // pair of query tiles (and slice); longest rows first
+    // Block index -> (head, pair of query tiles and slice): the longest pairs of all heads of a group come first
+    // (launch_attn_tc says how large a group is)
+    const int bx = EXACT ? (int)p.redo[1 + item] : (int)blockIdx.x;
+    const int grp = bx / (p.head_group * p.grid_x), grp_r = bx - grp * (p.head_group * p.grid_x);
+    const int grp_n = min(p.head_group, p.B * p.Hq - grp * p.head_group);
+    const int qhead = grp * p.head_group + grp_r % grp_n;    // b * Hq + h
+    const int pt_lin = p.grid_x - 1 - grp_r / grp_n;
     const int pt = SPLIT ? pt_lin / p.splits : pt_lin;
     const int split = SPLIT ? pt_lin % p.splits : 0;
     const int L = p.Lq, W = p.window, g = p.Hq / p.Hkv;     // L: rows of the query block
@@ -484,7 +489,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     const int q_lim = (QUERY_BLOCK && p.fixed_tail) ? p.L - W - 1 : 0x7fffffff;
     const int q_sub = (QUERY_BLOCK && p.fixed_tail) ? 0 : W;
     auto qhi = [&](int x) -> int { return QUERY_BLOCK ? min(x, q_lim) - q_sub : x - W; };
-    const int qhead = b * p.Hq + h, kvhead = b * p.Hkv + h / g;
+    const int kvhead = qhead / g;                            // b * Hkv + h / g
     const int32_t* idx_row = p.vl_idx + (long)qhead * p.k;
 
     if (threadIdx.x == 0) {
@@ -587,9 +592,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
             const bool again = *restart_flag != 0 && *abort_flag == 0;
             if (again && warp == 4 && lane == 0) {
                 const uint32_t slot = atomicAdd(p.redo, 1u);
-                p.redo[1 + 3 * slot] = (uint32_t)bx;
-                p.redo[2 + 3 * slot] = (uint32_t)h;
-                p.redo[3 + 3 * slot] = (uint32_t)b;
+                p.redo[1 + slot] = (uint32_t)bx;
             }
             return again;
         };
@@ -1082,14 +1085,21 @@ int launch_attn_tc(const hyq_attn_args& a, float alpha, cudaStream_t st) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(kern_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_BYTES) != cudaSuccess)
         return HYQ_ERR_CUDA;
-    const dim3 grid((((int)Lq + QT * BM - 1) / (QT * BM)) * w.splits, a.Hq, a.B);
-    p.grid_x = (int)grid.x;
+    // Order of the CTAs: longest walk first over all heads whose K / V the L2 holds at once - with the order "head by
+    // head" the last heads' long CTAs ran beside idle SMs (L = 8192, 32 heads: the busiest SM 14 % above the mean).
+    // Whole KV heads, at most 48 MB of keys and values (half of L2), the heads shared out evenly over the groups.
+    p.grid_x = (((int)Lq + QT * BM - 1) / (QT * BM)) * w.splits;
+    const long kv_bytes = (long)a.L * (HYQ_D + 2 * HYQ_D + (p.vl_tiles ? 32 * (a.Hq / a.Hkv) : 0));   // codes, V^, vertical-line operands
+    const long kv_heads = (long)a.B * a.Hkv, cap = (48L << 20) / kv_bytes > 1 ? (48L << 20) / kv_bytes : 1;
+    const long groups = (kv_heads + cap - 1) / cap;
+    p.head_group = (int)((kv_heads + groups - 1) / groups) * (a.Hq / a.Hkv);
+    const long n_ctas = (long)p.grid_x * a.Hq * a.B;
+    if (n_ctas > 0x7fffffffL) return HYQ_ERR_UNSUPPORTED;
     p.redo = reinterpret_cast<uint32_t*>(base + w.redo);
     if (cudaMemsetAsync(p.redo, 0, sizeof(uint32_t), st) != cudaSuccess) return HYQ_ERR_CUDA;
     if (a.ev_kernel_start && cudaEventRecord(static_cast<cudaEvent_t>(a.ev_kernel_start), st) != cudaSuccess) return HYQ_ERR_CUDA;
-    kern<<<grid, TC_THREADS, TC_SMEM_BYTES, st>>>(maps, p);
+    kern<<<(unsigned)n_ctas, TC_THREADS, TC_SMEM_BYTES, st>>>(maps, p);
     if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-    const long n_ctas = (long)grid.x * grid.y * grid.z;
     {
         kern_exact<<<(unsigned)(n_ctas < 148 ? n_ctas : 148), TC_THREADS, TC_SMEM_BYTES, st>>>(maps, p);
         if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
