@@ -91,6 +91,7 @@ __device__ unsigned long long g_tc_restarts = 0ull;
 
 struct TcMaps {
     CUtensorMap q, k, qc, kc, v16, vh16, kvl, vvl;
+    CUtensorMap o;               // output (split keys: the partial accumulators), boxes of 32 rows x 128 bytes
 };
 
 struct TcParams {
@@ -137,14 +138,32 @@ __device__ __forceinline__ float ex2f(float x) {
     return y;
 }
 
-// number of entries of the ascending list idx[0..k) that are <= v
-__device__ __forceinline__ int count_le(const int32_t* __restrict__ idx, int k, int v) {
-    int lo = 0, hi = k;
+// number of entries of the ascending list idx[0..k) that are <= v; the whole warp takes part (32-way search: one
+// memory round trip per factor of 32 in k, where a binary search took one per factor of 2)
+__device__ __forceinline__ int count_le_warp(const int32_t* __restrict__ idx, int k, int v) {
+    int lo = 0, hi = k;                                          // the count lies in [lo, hi]
     while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(idx + mid) <= v) lo = mid + 1; else hi = mid;
+        const int step = (hi - lo + 31) >> 5, pos = lo + (int)(threadIdx.x & 31) * step;
+        const int f = __popc(__ballot_sync(0xffffffffu, pos < hi && __ldg(idx + pos) <= v));
+        const int top = (f < 32 && lo + f * step < hi) ? lo + f * step : hi;
+        lo = f ? lo + (f - 1) * step + 1 : lo;
+        hi = f ? top : lo;
     }
     return lo;
+}
+
+// vertical-line keys at positions (v, hi1], at most 127 of them apart: bits of up to five bitmask words
+__device__ __forceinline__ int vl_between(const uint32_t* __restrict__ bits, int v, int hi1) {
+    const int w0 = (v + 1) >> 5, w1 = hi1 >> 5;
+    int n = 0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        uint32_t m = (w0 + j <= w1) ? __ldg(bits + w0 + j) : 0u;
+        if (j == 0) m &= 0xFFFFFFFFu << ((v + 1) & 31);
+        if (w0 + j == w1) m &= 0xFFFFFFFFu >> (31 - (hi1 & 31));
+        n += __popc(m);
+    }
+    return n;
 }
 
 // the tile walk of one CTA: union of both query tiles' lists
@@ -300,28 +319,29 @@ __device__ __forceinline__ bool mma_issuer(int q, const QSched& sq, const Walk& 
     return true;
 }
 
-// TMA producer (one thread): the two query tiles once, then the K ring and the V ring along the CTA's walk
-template <int TBN>
-__device__ __forceinline__ bool tma_producer(const TcMaps& maps, const QSched& qs0, const QSched& qs1, const Walk& w, int qhead,
-                                             int kvhead, TcBarriers& bars, unsigned char* smem, volatile int* abort_flag,
-                                             long long limit, int drop_load, const uint8_t* vl_tiles, bool settle) {
-    using G = Geo<TBN>;
-    constexpr int BN = TBN, NST = G::NST;
-    prefetch_tmap(&maps.q);
-    prefetch_tmap(&maps.k);
-    prefetch_tmap(&maps.kc);
-    prefetch_tmap(&maps.vh16);
+// The two query tiles (one thread, before the CTA's first synchronisation: they need nothing but the barrier)
+__device__ __forceinline__ void load_queries(const TcMaps& maps, const QSched& qs0, const QSched& qs1, int qhead,
+                                             TcBarriers& bars, unsigned char* smem) {
     const int live[QT] = {qs0.live, qs1.live}, qi0[QT] = {qs0.i0, qs1.i0};
+    const bool codes = max(qs0.nA, qs1.nA) > 0;
     uint32_t qbytes = 0;
     for (int q = 0; q < QT; ++q)
-        if (live[q]) qbytes += Q_TILE_BYTES + (w.nA > 0 ? QC_TILE_BYTES : 0);
+        if (live[q]) qbytes += Q_TILE_BYTES + (codes ? QC_TILE_BYTES : 0);
     mbar_arrive_expect_tx(&bars.q_full, qbytes);
     for (int q = 0; q < QT; ++q) {
         if (!live[q]) continue;
+        if (codes) tma_load_3d(smem + SQC_OFF + q * QC_TILE_BYTES, &maps.qc, &bars.q_full, 0, qi0[q], qhead);
         tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES, &maps.q, &bars.q_full, 0, qi0[q], qhead);
         tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES + Q_TILE_BYTES / 2, &maps.q, &bars.q_full, 64, qi0[q], qhead);
-        if (w.nA > 0) tma_load_3d(smem + SQC_OFF + q * QC_TILE_BYTES, &maps.qc, &bars.q_full, 0, qi0[q], qhead);
     }
+}
+
+// TMA producer (one thread): the K ring and the V ring along the CTA's walk
+template <int TBN>
+__device__ __forceinline__ bool tma_producer(const TcMaps& maps, const Walk& w, int qhead, int kvhead, TcBarriers& bars, unsigned char* smem, volatile int* abort_flag,
+                                             long long limit, int drop_load, const uint8_t* vl_tiles, bool settle) {
+    using G = Geo<TBN>;
+    constexpr int BN = TBN, NST = G::NST;
     bool ok = true;
     int t = w.t0;
     for (; t < w.t1 && !*abort_flag; ++t) {
@@ -463,7 +483,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     __shared__ int abort_s, restart_s, cnt_b_s[QT];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0) {
+    if (EXACT && warp == 0) {
         tmem_alloc(&tmem_base_s, TM_COLS);
         tmem_relinquish();
     }
@@ -492,33 +512,6 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     const int kvhead = qhead / g;                            // b * Hkv + h / g
     const int32_t* idx_row = p.vl_idx + (long)qhead * p.k;
 
-    if (threadIdx.x == 0) {
-        mbar_init(&bars.q_full, 1);
-        for (int s = 0; s < NST; ++s) {
-            mbar_init(&bars.kv_full[s], 1);
-            mbar_init(&bars.kv_free[s], QT);
-        }
-        for (int q = 0; q < QT; ++q) {
-            for (int bf = 0; bf < 2; ++bf) {
-                mbar_init(&bars.s_full[q][bf], 1);
-                mbar_init(&bars.p_full[q][bf], 4);                  // one arrival per softmax warp of the query tile
-                mbar_init(&bars.o_done[q][bf], 1);
-            }
-            mbar_init(&bars.drain[q], 1);
-        }
-        fence_mbar_init();
-        restart_s = 0;
-        if (EXACT) atomicAdd(&g_tc_restarts, 1ull);
-    }
-    if (threadIdx.x < QT) {
-        const int a1 = off + min(pt * QT * BM + (int)threadIdx.x * BM + BM - 1, L - 1);
-        cnt_b_s[threadIdx.x] = (p.k > 0 && qhi(a1) >= 0) ? count_le(idx_row, p.k, qhi(a1)) : 0;
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tmem_base_s;
-
     auto make_sched = [&](int q) {
         QSched s;
         s.i0 = (pt * QT + q) * BM;
@@ -526,12 +519,65 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
         s.i1 = min(s.i0 + BM - 1, L - 1);
         const int a0 = s.i0 + off, a1 = s.i1 + off;             // positions of the tile's first and last row
         s.nA = (s.live && qhi(a1) >= 0) ? qhi(a1) / BN + 1 : 0;
-        s.nB = s.live ? (cnt_b_s[q] + BN - 1) / BN : 0;
+        s.nB = 0;                                               // (needs the count of vertical keys: below)
         s.tC0 = max(0, qhi(a0) + 1) / BN;
         s.tC1 = (s.live && W > 0) ? a1 / BN : -1;
         return s;
     };
-    const QSched qs0 = make_sched(0), qs1 = make_sched(1);
+    QSched qs0 = make_sched(0), qs1 = make_sched(1);
+    // vertical-line keys of the low-bit pass: with e4m3 scores an extra MMA step per tile adds -inf to their columns
+    const uint8_t* vl_tiles_head = (LOWBIT_FP8 && p.vl_tiles) ? p.vl_tiles + (long)qhead * (p.mask_words / 2) * VL_TILE_BYTES : nullptr;
+
+    // Everything up to the first synchronisation is independent work on different warps: barriers, query loads and
+    // tensor memory (warp 0), the counts of vertical keys (warps 1 and 2), the constant operand (all).
+    if (warp == 0) {
+        if (lane == 0) {
+            mbar_init(&bars.q_full, 1);
+            for (int s = 0; s < NST; ++s) {
+                mbar_init(&bars.kv_full[s], 1);
+                mbar_init(&bars.kv_free[s], QT);
+            }
+            for (int q = 0; q < QT; ++q) {
+                for (int bf = 0; bf < 2; ++bf) {
+                    mbar_init(&bars.s_full[q][bf], 1);
+                    mbar_init(&bars.p_full[q][bf], 4);              // one arrival per softmax warp of the query tile
+                    mbar_init(&bars.o_done[q][bf], 1);
+                }
+                mbar_init(&bars.drain[q], 1);
+            }
+            fence_mbar_init();
+            load_queries(maps, qs0, qs1, qhead, bars, smem);
+            restart_s = 0;
+            if (EXACT) atomicAdd(&g_tc_restarts, 1ull);
+        }
+        __syncwarp();
+        if (!EXACT) {
+            tmem_alloc(&tmem_base_s, TM_COLS);
+            tmem_relinquish();
+        }
+    } else if (warp == 1 || warp == 2) {
+        const QSched& s = warp == 1 ? qs0 : qs1;
+        const int v = qhi(s.i1 + off);
+        const int c = (s.live && p.k > 0 && v >= 0) ? count_le_warp(idx_row, p.k, v) : 0;
+        if (lane == 0) cnt_b_s[warp - 1] = c;
+    }
+    if (vl_tiles_head) {
+        // the constant operand of the -inf step, one copy per ring slot (the copy of a slot is overwritten by the slot's
+        // first full-precision tile, after which the slot holds no low-bit tile again)
+        const int n_slots = min(max(qs0.nA, qs1.nA), NST);
+        for (int c = threadIdx.x; c < n_slots * (int)(ONES_BYTES / 16); c += TC_THREADS) {
+            const int slot = c / (int)(ONES_BYTES / 16), chunk = c % (int)(ONES_BYTES / 16);   // chunks 0..127: element 0..15 of row `chunk`
+            *reinterpret_cast<uint4*>(smem + SK_OFF + slot * G::STAGE_BYTES + ONES_OFF + chunk * 16) =
+                make_uint4(chunk < BM ? 0x3Cu : 0u, 0u, 0u, 0u);                               // 0x3C = 1.0 in e5m2
+        }
+        fence_proxy_async();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base_s;
+    qs0.nB = (cnt_b_s[0] + BN - 1) / BN;
+    qs1.nB = (cnt_b_s[1] + BN - 1) / BN;
     Walk w;
     w.nA = max(qs0.nA, qs1.nA);
     w.nB = max(qs0.nB, qs1.nB);
@@ -540,21 +586,6 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     w.T = w.nA + w.nB + w.nC;
     w.t0 = SPLIT ? (int)((long)w.T * split / p.splits) : 0;
     w.t1 = SPLIT ? (int)((long)w.T * (split + 1) / p.splits) : w.T;
-
-    // vertical-line keys of the low-bit pass: with e4m3 scores an extra MMA step per tile adds -inf to their columns
-    const uint8_t* vl_tiles_head = (LOWBIT_FP8 && p.vl_tiles) ? p.vl_tiles + (long)qhead * (p.mask_words / 2) * VL_TILE_BYTES : nullptr;
-    if (vl_tiles_head) {
-        // the constant operand of that step, one copy per ring slot whose first tile is a low-bit tile (the copy of a
-        // slot is overwritten by the slot's first full-precision tile, after which the slot holds no low-bit tile again)
-        const int n_slots = min(min(w.nA, w.t1) - w.t0, NST);
-        for (int c = threadIdx.x; c < n_slots * (int)(ONES_BYTES / 16); c += TC_THREADS) {
-            const int slot = c / (int)(ONES_BYTES / 16), chunk = c % (int)(ONES_BYTES / 16);   // chunks 0..127: element 0..15 of row `chunk`
-            *reinterpret_cast<uint4*>(smem + SK_OFF + slot * G::STAGE_BYTES + ONES_OFF + chunk * 16) =
-                make_uint4(chunk < BM ? 0x3Cu : 0u, 0u, 0u, 0u);                               // 0x3C = 1.0 in e5m2
-        }
-        fence_proxy_async();
-    }
-    __syncthreads();
 
     volatile int* abort_flag = &abort_s;
     volatile int* restart_flag = &restart_s;
@@ -565,7 +596,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
 
     // the single-thread roles sit in the lowest warps (the softmax warps 4..19 keep warp % 4 = TMEM lane quarter)
     if (warp == 0) {
-        if (lane == 0 && !tma_producer<TBN>(maps, qs0, qs1, w, qhead, kvhead, bars, smem, abort_flag, limit, p.drop_load, vl_tiles_head, EXACT)) fail();
+        if (lane == 0 && !tma_producer<TBN>(maps, w, qhead, kvhead, bars, smem, abort_flag, limit, p.drop_load, vl_tiles_head, EXACT)) fail();
     } else if (warp == 1 || warp == 2) {
         if (lane == 0) {
             const int q = warp - 1;
@@ -858,7 +889,8 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
             }
             // ---- the remaining low-bit tiles, the vertical-line tiles and the window tiles
             // (number of vertical-line keys this row may use: only needed from here on)
-            const int cnt_r = (!aborted && sq.nB > 0 && row_live && qhi(ia) >= 0) ? count_le(idx_row, p.k, qhi(ia)) : 0;
+            const int cnt_r = (!aborted && sq.nB > 0 && row_live && qhi(ia) >= 0)
+                                  ? cnt_b_s[q] - vl_between(vl_ptr, qhi(ia), qhi(sq.i1 + off)) : 0;
             for (; n < n_total && !aborted; ++n) {
                 const int t = walk_pos(n);
                 const float ks = nks;
@@ -902,57 +934,61 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
             const bool again = agree(over);
             if (!aborted && !again) {                           // uniform over the query tile's softmax warps
                 tc_fence_after();
-                constexpr int NCH = 4;                          // 32-channel pieces of the row this thread writes
                 const float l_run = l_h;
-                const float inv = (l_run > 0.0f) ? 1.0f / l_run : 0.0f;
-                if (SPLIT) {
-                    // partial result of this slice: O as accumulated (relative to m_used), the pair (m_used, l)
-                    const long prow = ((long)split * p.Hq * p.B + qhead) * L + i;
-                    if (ok) {
+                // Rows leave through shared memory (this query tile's operands, which nothing reads any more) and TMA: a
+                // thread that stored its own 512-byte row made every store instruction touch 32 lines (10.3 k clocks of an
+                // average CTA's 141 k at L = 8192, fp32).  Per warp three 4 KB buffers of 32 rows x 128 bytes, pieces swizzled as the
+                // tensor map expects them.  Rows past the end are clipped by the map.
+                const float inv = SPLIT ? 1.0f : (l_run > 0.0f) ? 1.0f / l_run : 0.0f;   // (slices leave O as accumulated, relative to m_used)
+                if (ok) {
+                    unsigned char* buf0 = smem + SQ_OFF + q * Q_TILE_BYTES + (warp & 3) * 8192;
+                    unsigned char* buf2 = smem + SQC_OFF + q * QC_TILE_BYTES + (warp & 3) * 4096;
+                    const int row0 = sq.i0 + (warp & 3) * 32, z = SPLIT ? split * p.Hq * p.B + qhead : qhead;
+                    const bool f32 = SPLIT || p.out_fp32 != 0;
 #pragma unroll
-                        for (int c = 0; c < NCH; ++c) {
-                            uint32_t o[32];
-                            const int ch = c * 32;
-                            tmem_ld32(to + ch, o);
-                            tmem_wait_ld();
-                            if (row_live) {
-                                uint4* dst = reinterpret_cast<uint4*>(p.part_o + prow * HYQ_D + ch);
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) dst[e] = make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
-                            }
-                        }
-                        if (row_live) reinterpret_cast<float2*>(p.part_ml)[prow] = make_float2(m_used, l_run);
-                    }
-                } else if (ok) {
-#pragma unroll
-                    for (int c = 0; c < NCH; ++c) {
+                    for (int c = 0; c < 4; ++c) {
                         uint32_t o[32];
-                        const int ch = c * 32;
-                        tmem_ld32(to + ch, o);
+                        tmem_ld32(to + c * 32, o);
                         tmem_wait_ld();
-                        if (row_live) {
-                            if (p.out_fp32) {
-                                float4* dst = reinterpret_cast<float4*>(static_cast<float*>(p.out) + ((long)qhead * L + i) * HYQ_D + ch);
+                        unsigned char* buf = f32 ? (c == 2 ? buf2 : buf0 + (c & 1) * 4096) : buf0 + (c >> 1) * 4096;
+                        if (f32) {
+                            if (c == 3) {                           // buffer 1 again: its store was the second of three
+                                if (lane == 0) bulk_wait_read<1>();
+                                __syncwarp();
+                            }
 #pragma unroll
-                                for (int e = 0; e < 8; ++e)
-                                    dst[e] = make_float4(__uint_as_float(o[4 * e]) * inv, __uint_as_float(o[4 * e + 1]) * inv,
-                                                         __uint_as_float(o[4 * e + 2]) * inv, __uint_as_float(o[4 * e + 3]) * inv);
-                            } else {
-                                uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out) + ((long)qhead * L + i) * HYQ_D + ch);
+                            for (int e = 0; e < 8; ++e)
+                                *reinterpret_cast<float4*>(buf + lane * 128 + ((e ^ (lane & 7)) << 4)) =
+                                    make_float4(__uint_as_float(o[4 * e]) * inv, __uint_as_float(o[4 * e + 1]) * inv,
+                                                __uint_as_float(o[4 * e + 2]) * inv, __uint_as_float(o[4 * e + 3]) * inv);
+                        } else {
 #pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    uint32_t wd[4];
+                            for (int e = 0; e < 4; ++e) {
+                                uint32_t wd[4];
 #pragma unroll
-                                    for (int q2 = 0; q2 < 4; ++q2) {
-                                        const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(o[8 * e + 2 * q2]) * inv,
-                                                                                        __uint_as_float(o[8 * e + 2 * q2 + 1]) * inv);
-                                        wd[q2] = *reinterpret_cast<const uint32_t*>(&b2);
-                                    }
-                                    dst[e] = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+                                for (int q2 = 0; q2 < 4; ++q2) {
+                                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(o[8 * e + 2 * q2]) * inv,
+                                                                                    __uint_as_float(o[8 * e + 2 * q2 + 1]) * inv);
+                                    wd[q2] = *reinterpret_cast<const uint32_t*>(&b2);
                                 }
+                                *reinterpret_cast<uint4*>(buf + lane * 128 + (((e + 4 * (c & 1)) ^ (lane & 7)) << 4)) =
+                                    make_uint4(wd[0], wd[1], wd[2], wd[3]);
+                            }
+                        }
+                        if (f32 || (c & 1)) {
+                            fence_proxy_async();
+                            __syncwarp();
+                            if (lane == 0 && row0 < L) {
+                                tma_store_3d(&maps.o, buf, f32 ? c * 32 : (c >> 1) * 64, row0, z);
+                                bulk_commit();
                             }
                         }
                     }
+                    if (SPLIT && row_live)
+                        reinterpret_cast<float2*>(p.part_ml)[((long)split * p.Hq * p.B + qhead) * L + i] = make_float2(m_used, l_run);
+                    if (lane == 0) bulk_wait_read<0>();             // the buffers outlive the copies
+                }
+                if (!SPLIT && ok) {
                     if (p.lse && row_live) p.lse[(long)qhead * L + i] = (m_used + log2f(l_run)) * 0.6931471805599453f;
                 }
             }
@@ -1040,6 +1076,12 @@ int launch_attn_tc(const hyq_attn_args& a, float alpha, cudaStream_t st) {
     ok &= make_tmap_3d(&maps.vh16, base + w.vh16, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, HYQ_D, L, kvh, 64, TBN);
     ok &= make_tmap_3d(&maps.kvl, base + w.kvl, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, kk, qh, 64, TBN);
     ok &= make_tmap_3d(&maps.vvl, base + w.vvl, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, HYQ_D, kk, qh, 64, TBN);
+    if (w.splits > 1)
+        ok &= make_tmap_3d(&maps.o, base + w.part_o, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, HYQ_D, Lq, qh * w.splits, 32, 32);
+    else if (a.out_dtype == 1)
+        ok &= make_tmap_3d(&maps.o, a.out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, HYQ_D, Lq, qh, 32, 32);
+    else
+        ok &= make_tmap_3d(&maps.o, a.out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, Lq, qh, 64, 32);
     if (!ok) return HYQ_ERR_CUDA;
 
     TcParams p{};

@@ -36,7 +36,7 @@ def _close(tc, lse_tc, simt, lse_simt):
     diff = (tc - simt).abs()
     assert torch.isfinite(tc).all() and float(diff.max()) <= MAX_ABS_TOL
     assert float(diff.sum() / simt.abs().sum()) <= MEAN_REL_TOL
-    assert float((lse_tc - lse_simt).abs().max()) <= 5e-3       # the bound of the suite's other LSE comparisons
+    assert float((lse_tc - lse_simt).abs().max()) <= 2e-3       # the bound of the suite's other LSE comparisons
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,L,Lq", [
