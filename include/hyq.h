@@ -177,8 +177,8 @@ int hyq_quantize_blocks(const void* x, int B, int H, int L, int D, int block_tok
  *   q_scales ceil(Lq/64) entries per head (quantization blocks counted from the first row of the block, as
  *   hyq_quantize_blocks writes them for a [B,Hq,Lq,D] tensor) and lse Lq entries; K, V and vl_idx are those
  *   of the whole context.  Lq = 0 or Lq = L is the whole prefill.  Lq > L -> HYQ_ERR_INVALID_ARG.
- *   (For short blocks the tensor-core path splits the keys over several CTAs per query tile and merges the
- *   partial results; the workspace query accounts for their buffers.  Results do not depend on the split up to
+ *   (Where 256-row units of query rows are too few or too unequal to fill the GPU, the tensor-core path shares their
+ *   keys out over several CTAs and merges the partial results; the workspace query accounts for their buffers.  Results do not depend on the split up to
  *   fp32 rounding.)
  *
  *   Window form: HYQ_WINDOW_SLIDING - key j is a window key of the row at position i iff i - j < window (every
@@ -248,9 +248,10 @@ int hyq_hybrid_attention_prefill(const hyq_attn_args* args, void* stream);
  *   a HOST array of n_seq vertical counts (0 <= k_s <= max(0, L_s - window)); the packed index buffer holds
  *   [Hq, k_s] per sequence, sequence s starting at Hq * (sum of k_r over r < s).
  *
- *   The sequences are processed one after the other on `stream` (longest first); one workspace of the size the
- *   plain query returns for the LONGEST sequence (B = 1) serves them all.  Host arrays are read during the call
- *   and may be freed afterwards.  Errors: as the plain calls, checked for every sequence before anything is
+ *   hyq_select_vertical_varlen and hyq_hybrid_attention_prefill_varlen run with one workspace of the size the plain
+ *   query returns for the LONGEST sequence (B = 1); the attention call puts as many consecutive sequences into a
+ *   launch as the workspace holds, all of them with hyq_hybrid_attention_prefill_varlen_workspace bytes.  Host arrays
+ *   are read during the call and may be freed afterwards.  Errors: as the plain calls, checked for every sequence before anything is
  *   launched; n_seq <= 0 or a non-ascending cu_seqlens -> INVALID_ARG.
  *
  *   hyq_hybrid_attention_prefill_varlen takes a hyq_attn_args whose tensor pointers are the PACKED buffers and
@@ -264,6 +265,8 @@ int hyq_quantize_blocks_varlen(const void* x, int n_seq, const int32_t* cu_seqle
                                int block_tokens, int format, void* codes_out, float* scales_out, void* stream);
 int hyq_hybrid_attention_prefill_varlen(const hyq_attn_args* args, int n_seq, const int32_t* cu_seqlens /* host */,
                                         const int32_t* k_per_seq /* host */, void* stream);
+int hyq_hybrid_attention_prefill_varlen_workspace(const hyq_attn_args* args, int n_seq, const int32_t* cu_seqlens /* host */,
+                                                  const int32_t* k_per_seq /* host */, size_t* bytes /* host, out */);
 
 /* ---------------------------------------------------------------------------------------------
  * hyq_test_set_attention_hooks - test hook (the paper has no counterpart): exercises the tensor-core

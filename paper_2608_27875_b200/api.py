@@ -21,7 +21,7 @@ EXPORTS = ("hyq_status_string", "hyq_version", "hyq_paper_k", "hyq_select_vertic
            "hyq_select_vertical", "hyq_select_vertical_static", "hyq_select_vertical_mass_workspace",
            "hyq_select_vertical_mass", "hyq_quantize_blocks", "hyq_hybrid_attention_prefill_workspace",
            "hyq_hybrid_attention_prefill", "hyq_test_set_attention_hooks", "hyq_test_read_attention_restarts", "hyq_select_vertical_varlen",
-           "hyq_quantize_blocks_varlen", "hyq_hybrid_attention_prefill_varlen")
+           "hyq_quantize_blocks_varlen", "hyq_hybrid_attention_prefill_varlen", "hyq_hybrid_attention_prefill_varlen_workspace")
 
 
 class HyqError(RuntimeError):
@@ -78,6 +78,8 @@ def lib() -> ctypes.CDLL:
         L.hyq_quantize_blocks_varlen.argtypes = ([ctypes.c_void_p, ctypes.c_int, i32p] + [ctypes.c_int] * 4 +
                                                  [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p])
         L.hyq_hybrid_attention_prefill_varlen.argtypes = [ctypes.POINTER(AttnArgs), ctypes.c_int, i32p, i32p, ctypes.c_void_p]
+        L.hyq_hybrid_attention_prefill_varlen_workspace.argtypes = [ctypes.POINTER(AttnArgs), ctypes.c_int, i32p, i32p,
+                                                                    ctypes.POINTER(ctypes.c_size_t)]
         _lib = L
     return _lib
 
@@ -334,7 +336,10 @@ def hybrid_prefill_varlen(qs, ks, vs, window: int, k_per_seq, fmts=(FMT_INT8, FM
     a.q_scales, a.k_scales, a.v_scales = (s_.data_ptr() for s_ in scales)
     a.vl_idx, a.out, a.status_word = idx.data_ptr(), out.data_ptr(), status.data_ptr()
     a.k = k_per_seq[lens.index(max(lens))]
-    wsa = torch.empty(max(16, hyq_hybrid_attention_prefill_workspace(a)), dtype=torch.uint8, device=dev)   # the longest sequence's need
+    need_a = ctypes.c_size_t(0)
+    _check(lib().hyq_hybrid_attention_prefill_varlen_workspace(ctypes.byref(a), n, cu_c, k_c, ctypes.byref(need_a)),
+           "hyq_hybrid_attention_prefill_varlen_workspace")
+    wsa = torch.empty(max(16, need_a.value), dtype=torch.uint8, device=dev)
     a.workspace, a.workspace_bytes = wsa.data_ptr(), wsa.numel()
     _check(lib().hyq_hybrid_attention_prefill_varlen(ctypes.byref(a), n, cu_c, k_c, _stream()), "hyq_hybrid_attention_prefill_varlen")
     res, ko, no = [], 0, 0

@@ -6,11 +6,10 @@
 namespace hyq {
 size_t attn_simt_workspace_bytes(const hyq_attn_args& a);
 int launch_attn_simt(const hyq_attn_args& a, float alpha, cudaStream_t st);
-size_t attn_tc_workspace_bytes(const hyq_attn_args& a);
-int launch_attn_tc(const hyq_attn_args& a, float alpha, cudaStream_t st);
+int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, float alpha, cudaStream_t st);
 int tc_restarts(unsigned long long* count, bool reset);
 namespace tcbt {
-int launch_attn_tc(const hyq_attn_args& a, float alpha, cudaStream_t st);     // 32- and 128-token quantization blocks
+int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, float alpha, cudaStream_t st);     // 32- and 128-token quantization blocks
 int tc_restarts(unsigned long long* count, bool reset);
 }
 }  // namespace hyq
@@ -182,23 +181,39 @@ static int check_attn(const hyq_attn_args* a, bool need_pointers) {
 
 static bool use_simt(const hyq_attn_args* a) { return a->impl == HYQ_IMPL_SIMT; }
 
+// the tensor-core path of a planned call (arguments checked)
+static int launch_planned(const hyq_attn_args& a, const TcPlan& plan, float alpha, cudaStream_t st) {
+    if (!a.workspace || a.workspace_bytes < plan.w.total) return HYQ_ERR_WORKSPACE;
+    return a.block_tokens == HYQ_BLOCK_TOKENS ? launch_attn_tc(a, plan, alpha, st) : tcbt::launch_attn_tc(a, plan, alpha, st);
+}
+
 int hyq_hybrid_attention_prefill_workspace(const hyq_attn_args* args, size_t* bytes) {
     if (!bytes) return HYQ_ERR_INVALID_ARG;
     const int rc = check_attn(args, false);
     if (rc != HYQ_OK) return rc;
-    *bytes = use_simt(args) ? attn_simt_workspace_bytes(*args) : attn_tc_workspace_bytes(*args);
+    if (use_simt(args)) {
+        *bytes = attn_simt_workspace_bytes(*args);
+        return HYQ_OK;
+    }
+    TcPlan plan;
+    if (!tc_plain_plan(*args, plan)) return HYQ_ERR_UNSUPPORTED;
+    *bytes = plan.w.total;
     return HYQ_OK;
 }
 
 int hyq_hybrid_attention_prefill(const hyq_attn_args* args, void* stream) {
     const int rc = check_attn(args, true);
     if (rc != HYQ_OK) return rc;
-    const size_t need = use_simt(args) ? attn_simt_workspace_bytes(*args) : attn_tc_workspace_bytes(*args);
-    if (need > 0 && (!args->workspace || args->workspace_bytes < need)) return HYQ_ERR_WORKSPACE;
     const float alpha = args->softmax_scale != 0.0f ? args->softmax_scale : 1.0f / sqrtf((float)args->D);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (use_simt(args)) return launch_attn_simt(*args, alpha, st);
-    return args->block_tokens == HYQ_BLOCK_TOKENS ? launch_attn_tc(*args, alpha, st) : tcbt::launch_attn_tc(*args, alpha, st);
+    if (use_simt(args)) {
+        const size_t need = attn_simt_workspace_bytes(*args);
+        if (need > 0 && (!args->workspace || args->workspace_bytes < need)) return HYQ_ERR_WORKSPACE;
+        return launch_attn_simt(*args, alpha, st);
+    }
+    TcPlan plan;
+    if (!tc_plain_plan(*args, plan)) return HYQ_ERR_UNSUPPORTED;
+    return launch_planned(*args, plan, alpha, st);
 }
 
 // ---- ragged batches: the plain calls, sequence by sequence, on packed buffers ---------------------------------
@@ -276,6 +291,76 @@ int hyq_quantize_blocks_varlen(const void* x, int n_seq, const int32_t* cu, int 
     return rc;
 }
 
+// Plan of the consecutive sequences [s0, s0 + n) of a ragged call as one launch; their packed buffers' first bytes in `a`.
+// False when one launch cannot hold them.
+static bool plan_group(const hyq_attn_args& args, int s0, int n, const int32_t* cu, const int32_t* k_per_seq, TcPlan& plan) {
+    if (n > TC_MAX_SEQ) return false;
+    TcSeq seq[TC_MAX_SEQ];
+    size_t k_before = 0, nb_before = 0;
+    for (int i = 0; i < n; ++i) {
+        const int L = cu[s0 + i + 1] - cu[s0 + i];
+        seq[i] = tc_ragged_seq(args, L, k_per_seq[s0 + i], (size_t)(cu[s0 + i] - cu[s0]), k_before, nb_before);
+        k_before += (size_t)k_per_seq[s0 + i];
+        nb_before += (size_t)((L + args.block_tokens - 1) / args.block_tokens);
+    }
+    return tc_make_plan(args, seq, n, args.Hq, args.Hq / args.Hkv, plan);
+}
+// the largest group of sequences from s0 on that one launch within `bytes` of workspace can hold (halved until it fits)
+static int next_group(const hyq_attn_args& args, int s0, int n_seq, const int32_t* cu, const int32_t* k_per_seq, size_t bytes, TcPlan& plan) {
+    int n = n_seq - s0 < TC_MAX_SEQ ? n_seq - s0 : TC_MAX_SEQ;
+    while (!(plan_group(args, s0, n, cu, k_per_seq, plan) && plan.w.total <= bytes)) {
+        if (n == 1) return 0;
+        n = (n + 1) / 2;
+    }
+    return n;
+}
+
+// the arguments of the sequences from s on: packed pointers advanced to sequence s
+static hyq_attn_args at_sequence(const hyq_attn_args& args, int L, int k, size_t t0, size_t k_before, size_t nb_before) {
+    const size_t q_row = args.q_format == HYQ_FMT_INT4 ? HYQ_D / 2 : HYQ_D, k_row = args.k_format == HYQ_FMT_INT4 ? HYQ_D / 2 : HYQ_D;
+    const size_t v_row = args.v_format == HYQ_FMT_INT4 ? HYQ_D / 2 : HYQ_D;
+    hyq_attn_args a = args;
+    a.B = 1; a.L = L; a.Lq = 0; a.k = k;
+    auto at = [](const void* base, size_t bytes) -> const void* { return base ? static_cast<const char*>(base) + bytes : nullptr; };
+    a.q = at(args.q, (size_t)args.Hq * HYQ_D * t0 * 2);
+    a.k_ = at(args.k_, (size_t)args.Hkv * HYQ_D * t0 * 2);
+    a.v = at(args.v, (size_t)args.Hkv * HYQ_D * t0 * 2);
+    a.q_codes = at(args.q_codes, (size_t)args.Hq * q_row * t0);
+    a.k_codes = at(args.k_codes, (size_t)args.Hkv * k_row * t0);
+    a.v_codes = at(args.v_codes, (size_t)args.Hkv * v_row * t0);
+    a.q_scales = args.q_scales ? args.q_scales + (size_t)args.Hq * nb_before : nullptr;
+    a.k_scales = args.k_scales ? args.k_scales + (size_t)args.Hkv * nb_before : nullptr;
+    a.v_scales = args.v_scales ? args.v_scales + (size_t)args.Hkv * nb_before : nullptr;
+    a.vl_idx = args.vl_idx ? args.vl_idx + (size_t)args.Hq * k_before : nullptr;
+    a.out = const_cast<void*>(at(args.out, (size_t)args.Hq * HYQ_D * t0 * (args.out_dtype == 1 ? 4 : 2)));
+    a.lse = args.lse ? args.lse + (size_t)args.Hq * t0 : nullptr;
+    return a;
+}
+
+int hyq_hybrid_attention_prefill_varlen_workspace(const hyq_attn_args* args, int n_seq, const int32_t* cu, const int32_t* k_per_seq,
+                                                  size_t* bytes) {
+    int rc = check_cu(n_seq, cu);
+    if (rc != HYQ_OK) return rc;
+    if (!bytes || !k_per_seq || !args || args->struct_size != sizeof(hyq_attn_args)) return HYQ_ERR_INVALID_ARG;
+    size_t most = 0;
+    TcPlan plan;
+    for (int s = 0; s < n_seq && rc == HYQ_OK; ++s) {
+        const int L = cu[s + 1] - cu[s];
+        hyq_attn_args a = at_sequence(*args, L, k_per_seq[s], 0, 0, 0);
+        if (a.k < 0 || a.k > (L - a.window > 0 ? L - a.window : 0)) return HYQ_ERR_INVALID_ARG;
+        rc = check_attn(&a, false);
+        if (rc == HYQ_OK && use_simt(&a) && attn_simt_workspace_bytes(a) > most) most = attn_simt_workspace_bytes(a);
+    }
+    if (rc != HYQ_OK || use_simt(args)) { *bytes = most; return rc; }
+    for (int s = 0, n; s < n_seq; s += n) {
+        n = next_group(*args, s, n_seq, cu, k_per_seq, (size_t)-1, plan);
+        if (n == 0) return HYQ_ERR_UNSUPPORTED;
+        if (plan.w.total > most) most = plan.w.total;
+    }
+    *bytes = most;
+    return HYQ_OK;
+}
+
 int hyq_hybrid_attention_prefill_varlen(const hyq_attn_args* args, int n_seq, const int32_t* cu, const int32_t* k_per_seq,
                                         void* stream) {
     int rc = check_cu(n_seq, cu);
@@ -283,46 +368,38 @@ int hyq_hybrid_attention_prefill_varlen(const hyq_attn_args* args, int n_seq, co
     if (!args || args->struct_size != sizeof(hyq_attn_args) || !k_per_seq) return HYQ_ERR_INVALID_ARG;
     const int bt = args->block_tokens;
     if (!block_tokens_ok(bt)) return HYQ_ERR_UNSUPPORTED;
-    const size_t q_row = args->q_format == HYQ_FMT_INT4 ? HYQ_D / 2 : HYQ_D, k_row = args->k_format == HYQ_FMT_INT4 ? HYQ_D / 2 : HYQ_D;
-    const size_t v_row = args->v_format == HYQ_FMT_INT4 ? HYQ_D / 2 : HYQ_D;
-    // one argument block per sequence, all checked before the first launch
-    hyq_attn_args* per = new hyq_attn_args[n_seq];
-    int* order = new int[n_seq];
+    // every sequence is checked, alone, before the first launch: any of them fits the workspace by itself
+    TcPlan plan;
     size_t nb_before = 0, k_before = 0;
     for (int s = 0; s < n_seq && rc == HYQ_OK; ++s) {
         const int L = cu[s + 1] - cu[s];
-        hyq_attn_args a = *args;
-        a.B = 1; a.L = L; a.Lq = 0; a.k = k_per_seq[s];
-        const size_t t0 = (size_t)cu[s];
-        auto at = [](const void* base, size_t bytes) -> const void* { return base ? static_cast<const char*>(base) + bytes : nullptr; };
-        a.q = at(args->q, (size_t)args->Hq * HYQ_D * t0 * 2);
-        a.k_ = at(args->k_, (size_t)args->Hkv * HYQ_D * t0 * 2);
-        a.v = at(args->v, (size_t)args->Hkv * HYQ_D * t0 * 2);
-        a.q_codes = at(args->q_codes, (size_t)args->Hq * q_row * t0);
-        a.k_codes = at(args->k_codes, (size_t)args->Hkv * k_row * t0);
-        a.v_codes = at(args->v_codes, (size_t)args->Hkv * v_row * t0);
-        a.q_scales = args->q_scales ? args->q_scales + (size_t)args->Hq * nb_before : nullptr;
-        a.k_scales = args->k_scales ? args->k_scales + (size_t)args->Hkv * nb_before : nullptr;
-        a.v_scales = args->v_scales ? args->v_scales + (size_t)args->Hkv * nb_before : nullptr;
-        a.vl_idx = (args->vl_idx && a.k > 0) ? args->vl_idx + (size_t)args->Hq * k_before : nullptr;
-        a.out = const_cast<void*>(at(args->out, (size_t)args->Hq * HYQ_D * t0 * (args->out_dtype == 1 ? 4 : 2)));
-        a.lse = args->lse ? args->lse + (size_t)args->Hq * t0 : nullptr;
+        const hyq_attn_args a = at_sequence(*args, L, k_per_seq[s], (size_t)cu[s], k_before, nb_before);
         if (a.k < 0 || a.k > (L - a.window > 0 ? L - a.window : 0)) rc = HYQ_ERR_INVALID_ARG;
         if (rc == HYQ_OK) rc = check_attn(&a, true);
         if (rc == HYQ_OK) {
-            const size_t need = use_simt(&a) ? attn_simt_workspace_bytes(a) : attn_tc_workspace_bytes(a);
-            if (need > 0 && (!a.workspace || a.workspace_bytes < need)) rc = HYQ_ERR_WORKSPACE;
+            if (!use_simt(&a) && !plan_group(*args, s, 1, cu, k_per_seq, plan)) rc = HYQ_ERR_UNSUPPORTED;
+            const size_t need = use_simt(&a) ? attn_simt_workspace_bytes(a) : plan.w.total;
+            if (rc == HYQ_OK && need > 0 && (!a.workspace || a.workspace_bytes < need)) rc = HYQ_ERR_WORKSPACE;
         }
-        per[s] = a;
         nb_before += (size_t)(L + bt - 1) / bt;
         k_before += (size_t)k_per_seq[s];
     }
-    if (rc == HYQ_OK) {
-        longest_first(n_seq, cu, order);
-        for (int n = 0; n < n_seq && rc == HYQ_OK; ++n) rc = hyq_hybrid_attention_prefill(&per[order[n]], stream);
+    const float alpha = args->softmax_scale != 0.0f ? args->softmax_scale : 1.0f / sqrtf((float)args->D);
+    nb_before = k_before = 0;
+    for (int s = 0, n; s < n_seq && rc == HYQ_OK; s += n) {
+        const hyq_attn_args a = at_sequence(*args, cu[s + 1] - cu[s], k_per_seq[s], (size_t)cu[s], k_before, nb_before);
+        if (use_simt(&a)) {
+            n = 1;
+            rc = launch_attn_simt(a, alpha, static_cast<cudaStream_t>(stream));
+        } else {
+            n = next_group(*args, s, n_seq, cu, k_per_seq, args->workspace_bytes, plan);
+            rc = n > 0 ? launch_planned(a, plan, alpha, static_cast<cudaStream_t>(stream)) : HYQ_ERR_WORKSPACE;
+        }
+        for (int i = s; i < s + n; ++i) {
+            nb_before += (size_t)(cu[i + 1] - cu[i] + bt - 1) / bt;
+            k_before += (size_t)k_per_seq[i];
+        }
     }
-    delete[] per;
-    delete[] order;
     return rc;
 }
 

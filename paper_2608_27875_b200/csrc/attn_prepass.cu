@@ -1,6 +1,7 @@
 // Pre-pass of the fused attention: lays out in the caller's workspace what the tensor-core kernel
-// streams with TMA.  All kernels are simple, coalesced and bound by memory traffic.
-//   - vertical-line bitmask per (b, h) over key positions
+// streams with TMA.  One launch; its blocks take one of five independent pieces of work each, all coalesced and bound by
+// memory traffic (separate launches cost a short prompt 5 launches and 2 memsets of 2-4 us each).
+//   - vertical-line bitmask per (b, h) over key positions and, with e4m3 scores, the operand tiles made from it
 //   - gathered vertical-line K rows (bf16) and V rows (fp16) per query head, in ascending position
 //     order (the physical "reorder" of Algorithm 2 Stage 1, done per query head because under
 //     GQA the heads that share a KV head select different keys)
@@ -31,44 +32,48 @@ __global__ void vl_bitmask_kernel(const int32_t* __restrict__ idx, long n_heads,
     if (j >= 0 && j < L) atomicOr(&bits[head * mask_words + (j >> 5)], 1u << (j & 31));
 }
 
-// one warp per gathered row: lane copies 4 channels
-__global__ void gather_vl_kernel(const __nv_bfloat16* __restrict__ kmat, const __nv_bfloat16* __restrict__ vmat,
-                                 const int32_t* __restrict__ idx, int Hq, int Hkv, int L, int k, long n_rows,
-                                 __nv_bfloat16* __restrict__ kvl, __half* __restrict__ vvl) {
-    const long row = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (row >= n_rows) return;
-    const long head = row / k;                       // b * Hq + h
-    const int b = (int)(head / Hq), h = (int)(head % Hq), g = Hq / Hkv;
-    int j = idx[row];
-    j = min(max(j, 0), L - 1);
-    const long src = (((long)b * Hkv + h / g) * L + j) * HYQ_D + lane * 4;
-    const uint2 kw = *reinterpret_cast<const uint2*>(kmat + src);
-    const uint2 vw = *reinterpret_cast<const uint2*>(vmat + src);
-    *reinterpret_cast<uint2*>(kvl + row * HYQ_D + lane * 4) = kw;
-    uint2 o;
-    o.x = f16x2_sat(bf16_lo(vw.x), bf16_hi(vw.x));
-    o.y = f16x2_sat(bf16_lo(vw.y), bf16_hi(vw.y));
-    *reinterpret_cast<uint2*>(vvl + row * HYQ_D + lane * 4) = o;
-}
+// ---- the pieces --------------------------------------------------------------------------------------------------
+constexpr int PRE_THREADS = 256;
+constexpr int PRE_MASK_WORDS = 32;           // bitmask words (16 tiles of 64 keys) a block builds
+
+struct PreParams {
+    unsigned v_end, gather_end, mask_end, k_end, q_end;      // block ranges of the pieces
+    int mask_blocks[TC_MAX_SEQ];                             // mask blocks before each sequence
+    int bt_shift;                                      // log2(tokens per quantization block)
+    const uint4 *k, *v;                                      // bf16 rows of 16 x 16 bytes
+    const uint2* v_codes;
+    const float* v_scales;
+    const int32_t* vl_idx;
+    const uint2 *q_codes, *k_codes;                          // packed INT4
+    uint4 *v16, *vh16, *kvl, *vvl, *q8, *k8;
+    uint32_t* bits;
+    uint8_t* tiles;
+    uint32_t* redo;
+    long q_vecs, k_vecs;
+};
+
+// sequence that a row of a flattened view belongs to (member `row0`: its first row; LEN: its number of rows)
+#define HYQ_SEQ_OF(tab, row0, LEN, row)                                                                     \
+    ([&]() {                                                                                                \
+        int s_ = 0;                                                                                         \
+        while (s_ + 1 < (tab).n_seq && !((row) >= (tab).seq[s_].row0 && (row) < (tab).seq[s_].row0 + (LEN))) ++s_; \
+        return s_;                                                                                          \
+    }())
 
 // V (bf16) -> fp16 and V^ = code * scale -> fp16; one thread per 8 channels
 template <int V_FMT>
-__global__ void v_to_fp16_kernel(const uint4* __restrict__ v, const uint2* __restrict__ v_codes,
-                                 const float* __restrict__ v_scales, int L, int nb, int block_tokens, long n_vec,
-                                 uint4* __restrict__ v16, uint4* __restrict__ vh16) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n_vec) return;
-    const long row = e / (HYQ_D / 8);                // global token row over all (b, kv head)
-    const long head = row / L;
-    const int tok = (int)(row - head * L);
-    const float sc = v_scales[head * nb + tok / block_tokens];
-    const uint4 w = __ldg(v + e);
+__device__ __forceinline__ void pre_values(const TcSeqTable& tab, const PreParams& p, long e) {
+    const long row = e >> 4;
+    if (row >= tab.kv_rows) return;
+    const TcSeq& sq = tab.seq[HYQ_SEQ_OF(tab, kv_row0, tab.heads / tab.g * tab.seq[s_].L, row)];
+    const int local = (int)row - sq.kv_row0, head = local / sq.L, tok = local - head * sq.L;
+    const float sc = __ldg(p.v_scales + sq.ks0 + (long)head * sq.nb + (tok >> p.bt_shift));
+    const uint4 w = __ldg(p.v + e);
     const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
     uint32_t o[4], oh[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) o[c] = f16x2_sat(bf16_lo(ws[c]), bf16_hi(ws[c]));
-    const uint2 cw = __ldg(v_codes + e);
+    const uint2 cw = __ldg(p.v_codes + e);
     const uint32_t cs[2] = {cw.x, cw.y};
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -85,38 +90,91 @@ __global__ void v_to_fp16_kernel(const uint4* __restrict__ v, const uint2* __res
         }
         oh[c] = f16x2_sat(f0 * sc, f1 * sc);
     }
-    v16[e] = make_uint4(o[0], o[1], o[2], o[3]);
-    vh16[e] = make_uint4(oh[0], oh[1], oh[2], oh[3]);
+    p.v16[e] = make_uint4(o[0], o[1], o[2], o[3]);
+    p.vh16[e] = make_uint4(oh[0], oh[1], oh[2], oh[3]);
 }
 
-// packed INT4 codes -> one e4m3 byte per code; one thread per 8 codes
-__global__ void int4_to_e4m3_kernel(const uint32_t* __restrict__ packed, long n_words, uint2* __restrict__ out) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n_words) return;
-    // e4m3 encodings of 0..8 (1 = 0x38, 2 = 0x40, 3 = 0x44, ...); sign goes to bit 7
-    const uint32_t w = __ldg(packed + e);
-    uint32_t o[2] = {0u, 0u};
-#pragma unroll
-    for (int n = 0; n < 8; ++n) {
-        const int v = ((int)(w << (28 - 4 * n))) >> 28;
-        const int a = abs(v);
-        // magnitudes 0..8 -> 0x00,0x38,0x40,0x44,0x48,0x4A,0x4C,0x4E,0x50
-        const uint64_t lut = 0x4E4C4A4844403800ull;
-        uint32_t code = (a == 8) ? 0x50u : (uint32_t)((lut >> (8 * a)) & 0xFF);
-        code |= (v < 0) ? 0x80u : 0u;
-        o[n >> 2] |= code << ((n & 3) * 8);
+// gathered vertical-line rows: K as it is, V as fp16; one thread per 16 bytes of a row
+__device__ __forceinline__ void pre_gather(const TcSeqTable& tab, const PreParams& p, long e) {
+    const long row = e >> 4;
+    if (row >= tab.vl_rows) return;
+    const TcSeq& sq = tab.seq[HYQ_SEQ_OF(tab, vl_row0, tab.heads * tab.seq[s_].k, row)];
+    const int head = ((int)row - sq.vl_row0) / sq.k;
+    const int j = min(max(__ldg(p.vl_idx + row), 0), sq.L - 1);
+    const long src = ((long)sq.kv_row0 + (long)(head / tab.g) * sq.L + j) * 16 + (e & 15);
+    const uint4 kw = __ldg(p.k + src), vw = __ldg(p.v + src);
+    p.kvl[e] = kw;
+    p.vvl[e] = make_uint4(f16x2_sat(bf16_lo(vw.x), bf16_hi(vw.x)), f16x2_sat(bf16_lo(vw.y), bf16_hi(vw.y)),
+                          f16x2_sat(bf16_lo(vw.z), bf16_hi(vw.z)), f16x2_sat(bf16_lo(vw.w), bf16_hi(vw.w)));
+}
+
+// 32 bitmask words (1024 keys) of one head, and with e4m3 scores their 16 operand tiles: the byte 0xFC (-inf in e5m2) in
+// element 0 of a vertical key's row, zero elsewhere
+__device__ __forceinline__ void pre_masks(const TcSeqTable& tab, const PreParams& p, int block) {
+    __shared__ uint32_t words[PRE_MASK_WORDS];
+    int s = 0;
+    for (int n = 1; n < tab.n_seq; ++n) s += p.mask_blocks[n] <= block;
+    const TcSeq& sq = tab.seq[s];
+    const int local = block - p.mask_blocks[s], per_head = (sq.mask_words + PRE_MASK_WORDS - 1) / PRE_MASK_WORDS;
+    const int head = local / per_head, w0 = (local - head * per_head) * PRE_MASK_WORDS;
+    const int n_words = min(PRE_MASK_WORDS, sq.mask_words - w0);
+    if (threadIdx.x < PRE_MASK_WORDS) words[threadIdx.x] = 0u;
+    __syncthreads();
+    if (sq.k > 0) {
+        const int32_t* idx = p.vl_idx + sq.vl_row0 + (long)head * sq.k;
+        const int lo = w0 * 32, hi = min(lo + PRE_MASK_WORDS * 32, sq.L);
+        int a = 0, b = sq.k;                                 // first index >= lo (every thread the same loads)
+        while (a < b) {
+            const int mid = (a + b) >> 1;
+            if (__ldg(idx + mid) < lo) a = mid + 1; else b = mid;
+        }
+        for (int i = a + threadIdx.x; i < sq.k; i += PRE_THREADS) {
+            const int j = __ldg(idx + i);
+            if (j >= hi) break;
+            if (j >= lo) atomicOr(&words[(j - lo) >> 5], 1u << (j & 31));
+        }
     }
-    out[e] = make_uint2(o[0], o[1]);
+    __syncthreads();
+    const long word0 = sq.mask0 + (long)head * sq.mask_words + w0;
+    if ((int)threadIdx.x < n_words) p.bits[word0 + threadIdx.x] = words[threadIdx.x];
+    if (p.tiles) {
+        uint4* dst = reinterpret_cast<uint4*>(p.tiles + (word0 >> 1) * VL_TILE_BYTES);
+        for (int c = threadIdx.x; c < (n_words >> 1) * (VL_TILE_BYTES / 16); c += PRE_THREADS) {
+            const int tile = c >> 7, chunk = c & 127;        // chunks 0..63: elements 0..15 of key `chunk`; 64..127: zeros
+            const bool on = chunk < 64 && ((words[2 * tile + (chunk >> 5)] >> (chunk & 31)) & 1u);
+            dst[c] = make_uint4(on ? 0xFCu : 0u, 0u, 0u, 0u);
+        }
+    }
 }
 
-// one thread per vertical-line index: the byte 0xFC (-inf in e5m2) into element 0 of the key's row of its tile's operand
-__global__ void vl_mask_tiles_kernel(const int32_t* __restrict__ idx, long n_heads, int k, int L, int tiles_per_head,
-                                     uint8_t* __restrict__ tiles) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n_heads * k) return;
-    const long head = e / k;
-    const int j = __ldg(idx + e);
-    if (j >= 0 && j < L) tiles[(head * tiles_per_head + (j >> 6)) * VL_TILE_BYTES + (j & 63) * 16] = 0xFC;
+// four two's-complement nibbles -> four e4m3 bytes (-8 .. 7 are exact): byte permutes look the magnitudes of the
+// non-negative and of the negative codes up by the low three bits, a third spreads the sign bits (32 x 32768 rows of Q and 8 x 32768 of K: the
+// look-up by shifts took 102 us in launches of its own, the whole pre-pass now 88 us, 149 before)
+__device__ __forceinline__ uint32_t nibbles_to_e4m3(uint32_t w) {
+    const uint32_t sel = w & 0x7777u;
+    const uint32_t pos = __byte_perm(0x44403800u, 0x4E4C4A48u, sel), neg = __byte_perm(0x4A4C4E50u, 0x38404448u, sel);
+    uint32_t m;                                               // selector bit 3: the byte's sign, spread over the byte
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(m) : "r"(0x80u), "r"(w & 0x8888u));
+    m &= 0x7F7F7F7Fu;                                         // 0x7F where the code is negative
+    return ((pos & ~m) | (neg & m)) | ((m << 1) & 0x80808080u);
+}
+__device__ __forceinline__ void pre_widen(const uint2* __restrict__ in, uint4* __restrict__ out, long n, long e) {
+    if (e >= n) return;
+    const uint2 w = __ldg(in + e);
+    out[e] = make_uint4(nibbles_to_e4m3(w.x), nibbles_to_e4m3(w.x >> 16), nibbles_to_e4m3(w.y), nibbles_to_e4m3(w.y >> 16));
+}
+
+template <int V_FMT>
+__global__ void __launch_bounds__(PRE_THREADS)
+tc_prepass_kernel(const __grid_constant__ TcSeqTable tab, const __grid_constant__ PreParams p) {
+    pdl_wait();
+    const unsigned b = blockIdx.x;
+    if (b == 0 && threadIdx.x == 0) *p.redo = 0u;            // (the attention kernel's list of pieces to redo starts empty)
+    if (b < p.v_end) pre_values<V_FMT>(tab, p, (long)b * PRE_THREADS + threadIdx.x);
+    else if (b < p.gather_end) pre_gather(tab, p, (long)(b - p.v_end) * PRE_THREADS + threadIdx.x);
+    else if (b < p.mask_end) pre_masks(tab, p, (int)(b - p.gather_end));
+    else if (b < p.k_end) pre_widen(p.k_codes, p.k8, p.k_vecs, (long)(b - p.mask_end) * PRE_THREADS + threadIdx.x);
+    else pre_widen(p.q_codes, p.q8, p.q_vecs, (long)(b - p.k_end) * PRE_THREADS + threadIdx.x);
 }
 
 int launch_vl_bitmask(const int32_t* idx, long n_heads, int k, int L, int mask_words, uint32_t* bits, cudaStream_t st) {
@@ -127,82 +185,164 @@ int launch_vl_bitmask(const int32_t* idx, long n_heads, int k, int L, int mask_w
     return launch_status();
 }
 
+
 // ---------------------------------------------------------------------------------------------
-int tc_key_splits(const hyq_attn_args& a) {
-    const int Lq = query_rows(a);
-    if (Lq >= a.L) return 1;                                     // the whole prefill fills the GPU by itself
-    const long ctas = (long)((Lq + 255) / 256) * a.Hq * a.B;
-    const long target = 2 * 148;                                 // about two CTAs per SM
-    if (ctas >= target / 2) return 1;
-    const int key_tiles = (a.L + 63) / 64;                       // upper bound of a CTA's walk
-    long s = (target + ctas - 1) / ctas;
-    s = s < 8 ? s : 8;
-    while (s > 1 && key_tiles / s < 16) --s;                     // at least 16 key tiles per slice
-    return (int)s;
+// Whether a sequence's units are shared out over CTAs tile by tile (each CTA a contiguous share of the sequence's key
+// tiles, units longest first), and over how many CTAs.  In units of a key tile (about 0.75 us): a CTA costs about 10 tiles
+// beside its keys, a split about as much again for partial results and their merge.  One CTA per unit takes at least the
+// mean load of an SM, and for every w at least w times the shortest of the longest 148 (w - 1) + 1 units.  Measured (attention launches, INT8, 2 heads x
+// 2048 tokens): one CTA per unit 54.6 us, shared 34.8; the last 1024 rows of 32 heads x 32768 keys (INT4): three equal
+// slices per unit 499 us, shared 435.
+static int split_ctas(const hyq_attn_args& a, const TcSeq& q, int heads, long& total) {
+    constexpr long CTA_COST = 10, MERGE_COST = 8, MIN_TILES = 4;
+    const bool ft = a.window_mode == HYQ_WINDOW_FIXED_TAIL;
+    const long units = (long)q.levels * heads;
+    total = 0;
+    if (units > 4 * TC_SMS) return 0;                           // enough units for the longest-first order to balance
+    long bound = 0, seen = 0;
+    for (int l = 0; l < q.levels; ++l) {
+        const long t = tc_unit_tiles(q.L, q.Lq, q.k, a.window, ft, q.levels - 1 - l);
+        const long waves = (seen + heads + TC_SMS - 1) / TC_SMS;         // some SM runs as many of the units seen so far
+        if (waves * (t + CTA_COST) > bound) bound = waves * (t + CTA_COST);
+        total += heads * t;
+        seen += heads;
+    }
+    const long mean = (total + units * CTA_COST) / TC_SMS;
+    if (mean > bound) bound = mean;
+    long ctas = total / MIN_TILES < TC_SMS ? total / MIN_TILES : TC_SMS;
+    if (ctas < 2) return 0;
+    const long split = (total + ctas - 1) / ctas + 2 * CTA_COST + MERGE_COST;
+    return split * 100 < bound * 93 ? (int)ctas : 0;
 }
 
-TcWorkspace tc_workspace_layout(const hyq_attn_args& a) {
-    TcWorkspace w{};
+bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads, int g, TcPlan& plan) {
+    if (n_seq < 1 || n_seq > TC_MAX_SEQ) return false;
+    TcSeqTable& t = plan.t.tab;
+    t.n_seq = n_seq; t.heads = heads; t.g = g;
+    t.n_unsplit = t.unsplit_ctas = 0;
+    const int bt = a.block_tokens;
+    TcSeq all[TC_MAX_SEQ];
+    long kv_rows = 0, vl_rows = 0, q_rows = 0, words = 0, units = 0;
+    for (int s = 0; s < n_seq; ++s) {
+        TcSeq& q = all[s] = seq[s];
+        long total;
+        q.levels = (q.Lq + TC_ROWS - 1) / TC_ROWS;
+        q.nb = (q.L + bt - 1) / bt; q.nbq = (q.Lq + bt - 1) / bt;
+        q.mask_words = (q.L + 127) / 128 * 4;
+        q.split = split_ctas(a, q, heads, total);
+        q.tiles = (int)total;
+        if (q.split == 0 && n_seq > 1 && q.levels > TC_MAX_LEVELS) return false;
+        kv_rows += (long)(heads / g) * q.L; vl_rows += (long)heads * q.k; q_rows += (long)heads * q.Lq; words += (long)heads * q.mask_words;
+        units += (long)heads * q.levels;
+    }
+    if (q_rows > 0x7fffffffL || kv_rows > 0x7fffffffL || words > 0x7fffffffL || units > 0x3fffffffL) return false;
+    t.kv_rows = (int)kv_rows; t.vl_rows = (int)vl_rows; t.q_rows = (int)q_rows;
+    // unsplit sequences first, most units per head first; the others behind them as they come
+    bool used[TC_MAX_SEQ] = {};
+    int n = 0;
+    for (;;) {
+        int best = -1;
+        for (int s = 0; s < n_seq; ++s)
+            if (!used[s] && all[s].split == 0 && (best < 0 || all[s].levels > all[best].levels)) best = s;
+        if (best < 0) break;
+        used[best] = true;
+        t.seq[n++] = all[best];
+    }
+    t.n_unsplit = n;
+    for (int s = 0; s < n_seq; ++s)
+        if (!used[s]) t.seq[n++] = all[s];
+    if (t.n_unsplit > 1) {
+        int acc = 0, with = 0;
+        for (int l = 0; l < t.seq[0].levels; ++l) {              // level l: the units at position levels - 1 - l of their head
+            const int pt = t.seq[0].levels - 1 - l;
+            while (with < t.n_unsplit && t.seq[with].levels > pt) ++with;
+            plan.t.lev.cum[l] = acc;
+            acc += with * heads;
+        }
+    }
+    for (int s = 0; s < t.n_unsplit; ++s) t.unsplit_ctas += heads * t.seq[s].levels;
+    t.ctas = t.unsplit_ctas;
+    int slots = 0, pieces = t.unsplit_ctas, mask0 = 0;
+    for (int s = 0; s < n_seq; ++s) {
+        TcSeq& q = t.seq[s];
+        q.mask0 = mask0; mask0 += heads * q.mask_words;
+        q.cta0 = t.ctas; q.slot0 = slots;
+        t.ctas += q.split; slots += 2 * q.split;
+        if (q.split) pieces += heads * q.levels + 2 * q.split;
+    }
+
+    TcWorkspace& w = plan.w;
+    w = TcWorkspace{};
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += align_up(bytes, 1024); return o; };
-    const size_t kv_elems = (size_t)a.B * a.Hkv * a.L * HYQ_D, q_elems = (size_t)a.B * a.Hq * query_rows(a) * HYQ_D;
-    w.mask_words = (a.L + 127) / 128 * 4;
-    w.vl_bits = take((size_t)a.B * a.Hq * w.mask_words * 4);
+    const size_t kv_elems = (size_t)kv_rows * HYQ_D, q_elems = (size_t)q_rows * HYQ_D, vl_elems = (size_t)(vl_rows > 0 ? vl_rows : 1) * HYQ_D;
+    w.mask_words = (int)words;
+    w.slots = slots;
+    w.pieces = pieces;
+    w.vl_bits = take((size_t)words * 4);
     w.v16 = take(kv_elems * 2);
     w.vh16 = take(kv_elems * 2);
-    w.kvl = take((size_t)a.B * a.Hq * (a.k > 0 ? a.k : 1) * HYQ_D * 2);
-    w.vvl = take((size_t)a.B * a.Hq * (a.k > 0 ? a.k : 1) * HYQ_D * 2);
+    w.kvl = take(vl_elems * 2);
+    w.vvl = take(vl_elems * 2);
     const bool int4 = a.q_format == HYQ_FMT_INT4;
     w.q8 = int4 ? take(q_elems) : 0;
     w.k8 = int4 ? take(kv_elems) : 0;
-    w.vl_tiles = (a.q_format != HYQ_FMT_INT8 && a.k > 0) ? take((size_t)a.B * a.Hq * (w.mask_words / 2) * VL_TILE_BYTES) : 0;
-    w.splits = tc_key_splits(a);
-    w.redo = take((1 + (size_t)((query_rows(a) + 255) / 256) * w.splits * a.Hq * a.B) * 4);
-    const size_t rows = (size_t)a.B * a.Hq * query_rows(a);
-    w.part_o = w.splits > 1 ? take((size_t)w.splits * rows * HYQ_D * 4) : 0;
-    w.part_ml = w.splits > 1 ? take((size_t)w.splits * rows * 2 * 4) : 0;
+    w.vl_tiles = (a.q_format != HYQ_FMT_INT8 && vl_rows > 0) ? take((size_t)(words / 2) * VL_TILE_BYTES) : 0;
+    w.redo = take((size_t)(1 + pieces) * 16);
+    w.part_o = slots ? take((size_t)slots * TC_ROWS * HYQ_D * 4) : 0;
+    w.part_ml = slots ? take((size_t)slots * TC_ROWS * 2 * 4) : 0;
     w.total = off;
-    return w;
+    return true;
 }
 
-int launch_tc_prepass(const hyq_attn_args& a, const TcWorkspace& w, cudaStream_t st) {
+bool tc_plain_plan(const hyq_attn_args& a, TcPlan& plan) {
+    TcSeq q{};
+    q.L = a.L; q.Lq = query_rows(a); q.k = a.k;
+    return tc_make_plan(a, &q, 1, a.B * a.Hq, a.Hq / a.Hkv, plan);
+}
+
+TcSeq tc_ragged_seq(const hyq_attn_args& a, int L, int k, size_t tokens_before, size_t k_before, size_t nb_before) {
+    TcSeq q{};
+    q.L = q.Lq = L; q.k = k;
+    q.q_row0 = (int)(a.Hq * tokens_before); q.kv_row0 = (int)(a.Hkv * tokens_before); q.vl_row0 = (int)(a.Hq * k_before);
+    q.qs0 = (int)(a.Hq * nb_before); q.ks0 = (int)(a.Hkv * nb_before);
+    return q;
+}
+
+int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, cudaStream_t st) {
     char* base = static_cast<char*>(a.workspace);
-    const long n_heads = (long)a.B * a.Hq;
-    uint32_t* bits = reinterpret_cast<uint32_t*>(base + w.vl_bits);
-    if (launch_vl_bitmask(a.vl_idx, n_heads, a.k, a.L, w.mask_words, bits, st) != HYQ_OK) return HYQ_ERR_CUDA;
-    if (a.k > 0) {
-        const long n = n_heads * a.k;
-        gather_vl_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(
-            static_cast<const __nv_bfloat16*>(a.k_), static_cast<const __nv_bfloat16*>(a.v), a.vl_idx, a.Hq, a.Hkv, a.L,
-            a.k, n, reinterpret_cast<__nv_bfloat16*>(base + w.kvl), reinterpret_cast<__half*>(base + w.vvl));
-        if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
+    const TcSeqTable& t = plan.t.tab;
+    const TcWorkspace& w = plan.w;
+    PreParams p{};
+    auto blocks = [](long threads) { return (threads + PRE_THREADS - 1) / PRE_THREADS; };
+    long n = blocks((long)t.kv_rows * 16);
+    p.v_end = (unsigned)n;
+    p.gather_end = (unsigned)(n += blocks((long)t.vl_rows * 16));
+    long mb = 0;
+    for (int s = 0; s < t.n_seq; ++s) {
+        p.mask_blocks[s] = (int)mb;
+        mb += (long)t.heads * ((t.seq[s].mask_words + PRE_MASK_WORDS - 1) / PRE_MASK_WORDS);
     }
-    if (a.q_format != HYQ_FMT_INT8 && a.k > 0) {
-        uint8_t* tiles = reinterpret_cast<uint8_t*>(base + w.vl_tiles);
-        if (cudaMemsetAsync(tiles, 0, (size_t)n_heads * (w.mask_words / 2) * VL_TILE_BYTES, st) != cudaSuccess) return HYQ_ERR_CUDA;
-        const long n = n_heads * a.k;
-        vl_mask_tiles_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a.vl_idx, n_heads, a.k, a.L, w.mask_words / 2, tiles);
-        if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-    }
-    const int nb = (a.L + a.block_tokens - 1) / a.block_tokens;
-    const long n_vec = (long)a.B * a.Hkv * a.L * (HYQ_D / 8);
-    const unsigned vgrid = (unsigned)((n_vec + 255) / 256);
-    if (a.v_format == HYQ_FMT_INT8)
-        v_to_fp16_kernel<HYQ_FMT_INT8><<<vgrid, 256, 0, st>>>(static_cast<const uint4*>(a.v), static_cast<const uint2*>(a.v_codes),
-            a.v_scales, a.L, nb, a.block_tokens, n_vec, reinterpret_cast<uint4*>(base + w.v16), reinterpret_cast<uint4*>(base + w.vh16));
-    else
-        v_to_fp16_kernel<HYQ_FMT_FP8_E4M3><<<vgrid, 256, 0, st>>>(static_cast<const uint4*>(a.v), static_cast<const uint2*>(a.v_codes),
-            a.v_scales, a.L, nb, a.block_tokens, n_vec, reinterpret_cast<uint4*>(base + w.v16), reinterpret_cast<uint4*>(base + w.vh16));
-    if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-    if (a.q_format == HYQ_FMT_INT4) {
-        const long qw = (long)a.B * a.Hq * query_rows(a) * (HYQ_D / 8), kw = (long)a.B * a.Hkv * a.L * (HYQ_D / 8);
-        int4_to_e4m3_kernel<<<(unsigned)((qw + 255) / 256), 256, 0, st>>>(static_cast<const uint32_t*>(a.q_codes), qw,
-                                                                        reinterpret_cast<uint2*>(base + w.q8));
-        int4_to_e4m3_kernel<<<(unsigned)((kw + 255) / 256), 256, 0, st>>>(static_cast<const uint32_t*>(a.k_codes), kw,
-                                                                        reinterpret_cast<uint2*>(base + w.k8));
-        if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-    }
-    return HYQ_OK;
+    p.mask_end = (unsigned)(n += mb);
+    const bool int4 = a.q_format == HYQ_FMT_INT4;
+    p.k_vecs = int4 ? (long)t.kv_rows * 8 : 0;
+    p.q_vecs = int4 ? (long)t.q_rows * 8 : 0;
+    p.k_end = (unsigned)(n += blocks(p.k_vecs));
+    p.q_end = (unsigned)(n += blocks(p.q_vecs));
+    if (n > 0x7fffffffL) return HYQ_ERR_UNSUPPORTED;
+    p.bt_shift = a.block_tokens == 32 ? 5 : a.block_tokens == 64 ? 6 : 7;
+    p.k = static_cast<const uint4*>(a.k_); p.v = static_cast<const uint4*>(a.v);
+    p.v_codes = static_cast<const uint2*>(a.v_codes); p.v_scales = a.v_scales;
+    p.vl_idx = a.vl_idx;
+    p.q_codes = static_cast<const uint2*>(a.q_codes); p.k_codes = static_cast<const uint2*>(a.k_codes);
+    p.v16 = reinterpret_cast<uint4*>(base + w.v16); p.vh16 = reinterpret_cast<uint4*>(base + w.vh16);
+    p.kvl = reinterpret_cast<uint4*>(base + w.kvl); p.vvl = reinterpret_cast<uint4*>(base + w.vvl);
+    p.q8 = reinterpret_cast<uint4*>(base + w.q8); p.k8 = reinterpret_cast<uint4*>(base + w.k8);
+    p.bits = reinterpret_cast<uint32_t*>(base + w.vl_bits);
+    p.tiles = (a.q_format != HYQ_FMT_INT8 && t.vl_rows > 0) ? reinterpret_cast<uint8_t*>(base + w.vl_tiles) : nullptr;
+    p.redo = reinterpret_cast<uint32_t*>(base + w.redo);
+    auto kern = a.v_format == HYQ_FMT_INT8 ? tc_prepass_kernel<HYQ_FMT_INT8> : tc_prepass_kernel<HYQ_FMT_FP8_E4M3>;
+    return launch_pdl(kern, dim3((unsigned)n), dim3(PRE_THREADS), 0, st, t, p);
 }
 
 }  // namespace hyq

@@ -91,7 +91,7 @@ __device__ unsigned long long g_tc_restarts = 0ull;
 
 struct TcMaps {
     CUtensorMap q, k, qc, kc, v16, vh16, kvl, vvl;
-    CUtensorMap o;               // output (split keys: the partial accumulators), boxes of 32 rows x 128 bytes
+    CUtensorMap o, po;           // output, partial accumulators of split sequences: boxes of 32 rows x 128 bytes
 };
 
 struct TcParams {
@@ -101,17 +101,15 @@ struct TcParams {
 #endif
     int Lq, nbq;                 // query rows (end-aligned with the L keys: row i sits at position L - Lq + i), their blocks
     int fixed_tail;              // window form: the last `window` keys for every row instead of each row's own
-    int splits;                  // CTAs per pair of query tiles, each on a slice of the walk (short query blocks)
-    float* part_o;               // splits > 1: unnormalised partial outputs [splits][B*Hq][Lq][D] ...
-    float* part_ml;              // ... and (reference maximum in log2 units, row sum) [splits][B*Hq][Lq][2]
+    float* part_ml;              // split sequences: (reference maximum in log2 units, row sum) per partial row [slots][256][2]
     int out_fp32;
     float scale_log2;            // softmax_scale * log2(e)
     const float* q_scales;
     const float* k_scales;
     const int32_t* vl_idx;
     const uint32_t* vl_bits;
-    uint32_t* redo;              // [0]: number of CTAs of the optimistic kernel that gave up, [1 + i]: their block indices
-    int grid_x;                  // work items per head (pairs of query tiles x slices)
+    int4* redo;                  // [0].x: pieces of work of the optimistic kernel that it gave up, [1 + i]: what they are (Piece)
+    int grid_x;                  // plain whole prefill: units per head
     int head_group;              // heads whose items are interleaved, longest first (a whole number of KV heads)
     const uint8_t* vl_tiles;     // FP8 / INT4 scores: the vertical-line operand tiles [B*Hq][mask_words/2][2048] (null: none)
     void* out;
@@ -125,6 +123,83 @@ struct TcBarriers {
     uint64_t q_full, kv_full[MAX_STAGES], kv_free[MAX_STAGES];   // ring stage = K tile and V tile of one walk position
     uint64_t s_full[QT][2], p_full[QT][2], o_done[QT][2], drain[QT];
 };
+
+// A piece of work: the tiles [t0, t1) of a unit's walk (256 query rows of one head), and where its result goes.
+struct Piece {
+    int seq, unit;               // sequence, unit in the sequence: level * heads + head, level 0 the last rows (plain: the block index)
+    int t0, t1;
+    int slot;                    // -1: the output; otherwise the slot for partial results
+};
+template <bool GENERAL> struct Tables : TcTables {};
+template <> struct Tables<false> {};         // a plain whole prefill finds its work from the block index alone
+
+// The unit that tile `pos` of a split sequence falls into, its first tile and its number of tiles (warp-collective; the
+// tiles of the sequence are counted unit by unit, longest units first)
+struct UnitAt {
+    int unit, first, tiles;
+};
+__device__ __forceinline__ UnitAt unit_at(const TcSeq& q, int heads, int window, int fixed_tail, int pos) {
+    UnitAt u = {0, 0, 1};
+    int base = 0;
+    for (int l0 = 0; l0 < q.levels; l0 += 32) {
+        const int l = l0 + (int)(threadIdx.x & 31);
+        const int t = l < q.levels ? tc_unit_tiles(q.L, q.Lq, q.k, window, fixed_tail, q.levels - 1 - l) : 0;
+        int incl = t * heads;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if ((int)(threadIdx.x & 31) >= o) incl += v;
+        }
+        const unsigned hit = __ballot_sync(0xffffffffu, base + incl > pos);
+        if (hit) {
+            const int f = __ffs(hit) - 1, tf = __shfl_sync(0xffffffffu, t, f);
+            const int excl = base + __shfl_sync(0xffffffffu, incl, f) - tf * heads, r = (pos - excl) / tf;
+            u.unit = (l0 + f) * heads + r; u.first = excl + r * tf; u.tiles = tf;
+            break;
+        }
+        base += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    return u;
+}
+// first tile of CTA c of a sequence whose tiles are shared by `split` CTAs, and the CTA that works on tile x
+__host__ __device__ inline int split_begin(int tiles, int split, int c) { return (int)((long)tiles * c / split); }
+__host__ __device__ inline int split_of(int tiles, int split, int x) { return (int)((((long)x + 1) * split - 1) / tiles); }
+
+// Work of a CTA of a general launch, from tile `pos` of its share on (-1: from the start).  Returns in `next` the tile to
+// go on from, -1 when nothing is left.
+__device__ __forceinline__ Piece find_piece(const TcTables& t, int window, int fixed_tail, int pos, int& next) {
+    const TcSeqTable& tab = t.tab;
+    Piece pc = {0, 0, 0, 0x7fffffff, -1};
+    next = -1;
+    const int cta = blockIdx.x;
+    if (cta < tab.unsplit_ctas) {
+        pc.unit = cta;
+        if (tab.n_unsplit > 1) {                 // level by level over all sequences that are long enough
+            int lo = 0, hi = tab.seq[0].levels - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (t.lev.cum[mid] <= cta) lo = mid; else hi = mid - 1;
+            }
+            const int r = cta - t.lev.cum[lo];
+            pc.seq = r / tab.heads;
+            pc.unit = (lo - (tab.seq[0].levels - tab.seq[pc.seq].levels)) * tab.heads + r % tab.heads;
+        }
+        return pc;
+    }
+    int s = tab.n_unsplit;
+    while (s + 1 < tab.n_seq && tab.seq[s + 1].cta0 <= cta) ++s;
+    const TcSeq& q = tab.seq[s];
+    const int c = cta - q.cta0, begin = split_begin(q.tiles, q.split, c), end = split_begin(q.tiles, q.split, c + 1);
+    if (pos < 0) pos = begin;
+    const UnitAt u = unit_at(q, tab.heads, window, fixed_tail, pos);
+    pc.seq = s; pc.unit = u.unit;
+    pc.t0 = pos - u.first;
+    pc.t1 = min(u.tiles, end - u.first);
+    if (pc.t0 == 0 && pc.t1 == u.tiles) pc.t1 = 0x7fffffff;
+    else pc.slot = q.slot0 + 2 * c + (pos == begin ? 0 : 1);
+    if (u.first + u.tiles < end) next = u.first + u.tiles;
+    return pc;
+}
 
 // which key tiles a 128-row query tile visits in each pass (i0, i1: first and last row of the tile in the query
 // block; the tile lists follow from their positions among the keys)
@@ -320,7 +395,7 @@ __device__ __forceinline__ bool mma_issuer(int q, const QSched& sq, const Walk& 
 }
 
 // The two query tiles (one thread, before the CTA's first synchronisation: they need nothing but the barrier)
-__device__ __forceinline__ void load_queries(const TcMaps& maps, const QSched& qs0, const QSched& qs1, int qhead,
+__device__ __forceinline__ void load_queries(const TcMaps& maps, const QSched& qs0, const QSched& qs1, int q_y, int q_z,
                                              TcBarriers& bars, unsigned char* smem) {
     const int live[QT] = {qs0.live, qs1.live}, qi0[QT] = {qs0.i0, qs1.i0};
     const bool codes = max(qs0.nA, qs1.nA) > 0;
@@ -330,15 +405,15 @@ __device__ __forceinline__ void load_queries(const TcMaps& maps, const QSched& q
     mbar_arrive_expect_tx(&bars.q_full, qbytes);
     for (int q = 0; q < QT; ++q) {
         if (!live[q]) continue;
-        if (codes) tma_load_3d(smem + SQC_OFF + q * QC_TILE_BYTES, &maps.qc, &bars.q_full, 0, qi0[q], qhead);
-        tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES, &maps.q, &bars.q_full, 0, qi0[q], qhead);
-        tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES + Q_TILE_BYTES / 2, &maps.q, &bars.q_full, 64, qi0[q], qhead);
+        if (codes) tma_load_3d(smem + SQC_OFF + q * QC_TILE_BYTES, &maps.qc, &bars.q_full, 0, q_y + qi0[q], q_z);
+        tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES, &maps.q, &bars.q_full, 0, q_y + qi0[q], q_z);
+        tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES + Q_TILE_BYTES / 2, &maps.q, &bars.q_full, 64, q_y + qi0[q], q_z);
     }
 }
 
 // TMA producer (one thread): the K ring and the V ring along the CTA's walk
 template <int TBN>
-__device__ __forceinline__ bool tma_producer(const TcMaps& maps, const Walk& w, int qhead, int kvhead, TcBarriers& bars, unsigned char* smem, volatile int* abort_flag,
+__device__ __forceinline__ bool tma_producer(const TcMaps& maps, const Walk& w, int kv_y, int kv_z, int vl_y, int vl_z, TcBarriers& bars, unsigned char* smem, volatile int* abort_flag,
                                              long long limit, int drop_load, const uint8_t* vl_tiles, bool settle) {
     using G = Geo<TBN>;
     constexpr int BN = TBN, NST = G::NST;
@@ -349,8 +424,8 @@ __device__ __forceinline__ bool tma_producer(const TcMaps& maps, const Walk& w, 
         unsigned char* sk = smem + SK_OFF + st * G::STAGE_BYTES;
         unsigned char* sv = smem + SV_OFF + st * G::STAGE_BYTES;
         const bool lowbit = t < w.nA, vl = !lowbit && t < w.nA + w.nB;
-        const int row = lowbit ? t * BN : (vl ? (t - w.nA) * BN : (w.tC0 + t - w.nA - w.nB) * BN);
-        const int hd = vl ? qhead : kvhead;
+        const int row = (vl ? vl_y : kv_y) + (lowbit ? t : (vl ? t - w.nA : w.tC0 + t - w.nA - w.nB)) * BN;
+        const int hd = vl ? vl_z : kv_z;
         if (use > 0 && !mbar_wait_sleepy(&bars.kv_free[st], (use - 1) & 1, limit)) { ok = false; break; }
         if (lowbit) {
             mbar_arrive_expect_tx(&bars.kv_full[st], G::KC_TILE_BYTES + G::STAGE_BYTES + (vl_tiles ? VL_TILE_BYTES : 0));
@@ -389,6 +464,10 @@ constexpr int TC_THREADS = 384;                     // TMA producer, 2 MMA issue
 constexpr float P_SUM_LIMIT = 65504.0f;             // a tile's row sum below the largest fp16 number: none of its P overflowed
 constexpr int WARM_TILES = 8;                       // tiles at the start of a walk whose maximum is always looked at, and ...
 constexpr float WARM_SPREAD = 6.0f;                 // ... how far apart (log2 units) their maxima may lie for the rest to go without
+// the same for short pieces of a shared unit (four tiles and more): two maxima say less than eight, so they have to lie
+// closer (rows with heavy tails, sigma of 7 to 10 log2 units, practically never pass: they differ by 5 on average)
+constexpr int WARM_TILES_SHORT = 2;
+constexpr float WARM_SPREAD_SHORT = 3.0f;
 constexpr float RAISE_THRESHOLD = 14.0f;            // log2 units by which a tile must exceed the reference to raise it (P stays below 2^14, inside fp16)
 
 // row maximum of 32 float scores held in registers
@@ -458,29 +537,30 @@ __device__ __forceinline__ void mask_cols32(uint32_t (&raw)[32], int c0, int lo_
     for (int e = 0; e < 32; ++e) raw[e] = ((unsigned)(c0 + e - lo_eff) <= span) ? raw[e] : knock;
 }
 
-// LOWBIT_FP8: the low-bit codes are e4m3 bytes (kind::f8f6f4), else int8 (kind::i8).  QUERY_BLOCK: the query rows
-// are the last Lq < L positions (a compile-time zero offset keeps one register out of the whole-prefill loop:
-// 2.6 % on the benchmark workload).
-// SPLIT (short query blocks only): several CTAs share a pair of query tiles, each on a contiguous slice of the
-// walk; they leave unnormalised partial results that attn_merge_kernel combines by their reference maxima.
-// EXACT = false is the kernel of the first launch: one CTA per block index.  After the first tiles of a row's low-bit pass
+// LOWBIT_FP8: the low-bit codes are e4m3 bytes (kind::f8f6f4), else int8 (kind::i8).  GENERAL: everything but a plain
+// whole prefill - a query block of the last Lq < L positions, the fixed window, several sequences in one launch, units
+// shared by several CTAs (which leave unnormalised partial results that attn_merge_kernel combines by their reference
+// maxima).  A CTA then finds its pieces of work in `tabs`, and rows are addressed in the flattened views of the buffers;
+// the plain kernel keeps a position offset and these look-ups out of its registers (2.6 % on the benchmark workload).
+// EXACT = false is the kernel of the first launch.  After the first tiles of a row's low-bit pass
 // (and if their maxima lie close together) it takes the exponentials against the row's reference as it stands, without
 // looking for the tile's maximum, and every tile's row sum tells afterwards whether that was safe (no P beyond fp16).  If it was not for any row of the
-// CTA - a score more than 2^16 above everything the row had seen - the CTA writes no output and puts its block
-// index on a list.  EXACT = true is the kernel of the second launch, a small grid that goes through that list
+// piece - a score more than 2^16 above everything the row had seen - the CTA writes no output for it and puts the piece
+// on a list.  EXACT = true is the kernel of the second launch, a small grid that goes through that list
 // (normally empty) with the maximum looked at in every tile.
-template <bool LOWBIT_FP8, bool QUERY_BLOCK, bool SPLIT = false, bool EXACT = false>
+template <bool LOWBIT_FP8, bool GENERAL, bool EXACT = false>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
+attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcParams p, const __grid_constant__ Tables<GENERAL> tabs) {
     constexpr int TBN = 64, BN = 64;
-    if (EXACT && p.redo[0] == 0u) return;
+    pdl_wait();
+    if (EXACT && p.redo[0].x == 0) return;
     using G = Geo<TBN>;
     constexpr int NST = G::NST;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ TcBarriers bars;
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s, restart_s, cnt_b_s[QT];
+    __shared__ int abort_s, restart_s, cnt_b_s[QT], next_s;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (EXACT && warp == 0) {
@@ -488,29 +568,59 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
         tmem_relinquish();
     }
     if (threadIdx.x == 0) abort_s = 0;
-    const uint32_t n_items = EXACT ? p.redo[0] : 1u;
+    if (GENERAL && !EXACT && threadIdx.x == 0) next_s = -1;
+    if (GENERAL && !EXACT) __syncthreads();
+    int item = blockIdx.x;                                   // second launch: place on the list
 #pragma unroll 1
-    for (uint32_t item = EXACT ? blockIdx.x : 0u; item < n_items; item += (EXACT ? gridDim.x : 1u)) {
-    // Block index -> (head, pair of query tiles and slice): the longest pairs of all heads of a group come first
-    // (launch_attn_tc says how large a group is)
-    const int bx = EXACT ? (int)p.redo[1 + item] : (int)blockIdx.x;
-    const int grp = bx / (p.head_group * p.grid_x), grp_r = bx - grp * (p.head_group * p.grid_x);
-    const int grp_n = min(p.head_group, p.B * p.Hq - grp * p.head_group);
-    const int qhead = grp * p.head_group + grp_r % grp_n;    // b * Hq + h
-    const int pt_lin = p.grid_x - 1 - grp_r / grp_n;
-    const int pt = SPLIT ? pt_lin / p.splits : pt_lin;
-    const int split = SPLIT ? pt_lin % p.splits : 0;
-    const int L = p.Lq, W = p.window, g = p.Hq / p.Hkv;     // L: rows of the query block
-    const int off = QUERY_BLOCK ? p.L - p.Lq : 0;           // position of query row 0 among the keys
+    for (;;) {
+    if (EXACT && item >= p.redo[0].x) break;
+    Piece pc = {0, (int)blockIdx.x, 0, 0x7fffffff, -1};
+    int next = -1;                                           // first launch: where this CTA's next piece begins
+    if (EXACT) {
+        const int4 r = p.redo[1 + item];
+        pc.seq = r.x & 0xff; pc.slot = (r.x >> 8) - 1; pc.unit = r.y; pc.t0 = r.z; pc.t1 = r.w;
+    } else if constexpr (GENERAL) {
+        pc = find_piece(tabs, p.window, p.fixed_tail, next_s, next);
+    }
+    const bool settle = EXACT || next >= 0 || (GENERAL && pc.slot >= 0);      // the barriers may be initialised again
+    int qhead, kvhead, pt, L, off, lim0, k_vl, q_y, q_z, kv_y, kv_z, vl_y, vl_z;
+    long qs_at, ks_at, mask_at, lse_at;
+    const int W = p.window, g = p.Hq / p.Hkv;
+    if constexpr (GENERAL) {
+        const TcSeq& sq_ = tabs.tab.seq[pc.seq];
+        const int level = pc.unit / tabs.tab.heads;
+        qhead = pc.unit - level * tabs.tab.heads;
+        kvhead = qhead / g;
+        pt = sq_.levels - 1 - level;
+        L = sq_.Lq; off = sq_.L - sq_.Lq; lim0 = sq_.L; k_vl = sq_.k;
+        q_y = sq_.q_row0 + qhead * sq_.Lq; kv_y = sq_.kv_row0 + kvhead * sq_.L; vl_y = sq_.vl_row0 + qhead * sq_.k;
+        q_z = kv_z = vl_z = 0;
+        qs_at = sq_.qs0 + (long)qhead * sq_.nbq; ks_at = sq_.ks0 + (long)kvhead * sq_.nb;
+        mask_at = sq_.mask0 + (long)qhead * sq_.mask_words;
+        lse_at = q_y;
+    } else {
+        // Block index -> (head, pair of query tiles): the longest pairs of all heads of a group come first
+        // (launch_attn_tc says how large a group is)
+        const int grp = pc.unit / (p.head_group * p.grid_x), grp_r = pc.unit - grp * (p.head_group * p.grid_x);
+        const int grp_n = min(p.head_group, p.B * p.Hq - grp * p.head_group);
+        qhead = grp * p.head_group + grp_r % grp_n;          // b * Hq + h
+        kvhead = qhead / g;                                  // b * Hkv + h / g
+        pt = p.grid_x - 1 - grp_r / grp_n;
+        L = p.Lq; off = 0; lim0 = p.L; k_vl = p.k;
+        q_y = kv_y = vl_y = 0;
+        q_z = vl_z = qhead; kv_z = kvhead;
+        qs_at = (long)qhead * p.nbq; ks_at = (long)kvhead * p.nb;
+        mask_at = (long)qhead * p.mask_words;
+        lse_at = (long)qhead * L;
+    }
     const long long limit = p.wait_limit;
     // Last low-bit-eligible key position of the row at position x: x - W with the per-row sliding window,
     // min(x, L_K - W - 1) with the fixed tail window (both as min(x, lim) - wsub).  Its window keys start right
     // after it, and the vertical keys it may use are those at or below it.
-    const int q_lim = (QUERY_BLOCK && p.fixed_tail) ? p.L - W - 1 : 0x7fffffff;
-    const int q_sub = (QUERY_BLOCK && p.fixed_tail) ? 0 : W;
-    auto qhi = [&](int x) -> int { return QUERY_BLOCK ? min(x, q_lim) - q_sub : x - W; };
-    const int kvhead = qhead / g;                            // b * Hkv + h / g
-    const int32_t* idx_row = p.vl_idx + (long)qhead * p.k;
+    const int q_lim = (GENERAL && p.fixed_tail) ? lim0 - W - 1 : 0x7fffffff;
+    const int q_sub = (GENERAL && p.fixed_tail) ? 0 : W;
+    auto qhi = [&](int x) -> int { return GENERAL ? min(x, q_lim) - q_sub : x - W; };
+    const int32_t* idx_row = p.vl_idx + (GENERAL ? (long)vl_y : (long)qhead * p.k);
 
     auto make_sched = [&](int q) {
         QSched s;
@@ -526,7 +636,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     };
     QSched qs0 = make_sched(0), qs1 = make_sched(1);
     // vertical-line keys of the low-bit pass: with e4m3 scores an extra MMA step per tile adds -inf to their columns
-    const uint8_t* vl_tiles_head = (LOWBIT_FP8 && p.vl_tiles) ? p.vl_tiles + (long)qhead * (p.mask_words / 2) * VL_TILE_BYTES : nullptr;
+    const uint8_t* vl_tiles_head = (LOWBIT_FP8 && p.vl_tiles) ? p.vl_tiles + (mask_at >> 1) * VL_TILE_BYTES : nullptr;
 
     // Everything up to the first synchronisation is independent work on different warps: barriers, query loads and
     // tensor memory (warp 0), the counts of vertical keys (warps 1 and 2), the constant operand (all).
@@ -546,19 +656,19 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
                 mbar_init(&bars.drain[q], 1);
             }
             fence_mbar_init();
-            load_queries(maps, qs0, qs1, qhead, bars, smem);
+            load_queries(maps, qs0, qs1, q_y, q_z, bars, smem);
             restart_s = 0;
             if (EXACT) atomicAdd(&g_tc_restarts, 1ull);
         }
         __syncwarp();
-        if (!EXACT) {
+        if (!EXACT && (!GENERAL || next_s < 0)) {            // (once: the first piece)
             tmem_alloc(&tmem_base_s, TM_COLS);
             tmem_relinquish();
         }
     } else if (warp == 1 || warp == 2) {
         const QSched& s = warp == 1 ? qs0 : qs1;
         const int v = qhi(s.i1 + off);
-        const int c = (s.live && p.k > 0 && v >= 0) ? count_le_warp(idx_row, p.k, v) : 0;
+        const int c = (s.live && k_vl > 0 && v >= 0) ? count_le_warp(idx_row, k_vl, v) : 0;
         if (lane == 0) cnt_b_s[warp - 1] = c;
     }
     if (vl_tiles_head) {
@@ -576,6 +686,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
+    if (GENERAL && !EXACT && threadIdx.x == 0) next_s = next;    // (read again behind the synchronisation that ends this piece)
     qs0.nB = (cnt_b_s[0] + BN - 1) / BN;
     qs1.nB = (cnt_b_s[1] + BN - 1) / BN;
     Walk w;
@@ -584,8 +695,8 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     w.tC0 = qs0.tC0;
     w.nC = (W > 0) ? max(qs0.tC1, qs1.tC1) - w.tC0 + 1 : 0;
     w.T = w.nA + w.nB + w.nC;
-    w.t0 = SPLIT ? (int)((long)w.T * split / p.splits) : 0;
-    w.t1 = SPLIT ? (int)((long)w.T * (split + 1) / p.splits) : w.T;
+    w.t0 = GENERAL ? pc.t0 : 0;
+    w.t1 = GENERAL ? max(pc.t0, min(pc.t1, w.T)) : w.T;
 
     volatile int* abort_flag = &abort_s;
     volatile int* restart_flag = &restart_s;
@@ -596,12 +707,12 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
 
     // the single-thread roles sit in the lowest warps (the softmax warps 4..19 keep warp % 4 = TMEM lane quarter)
     if (warp == 0) {
-        if (lane == 0 && !tma_producer<TBN>(maps, w, qhead, kvhead, bars, smem, abort_flag, limit, p.drop_load, vl_tiles_head, EXACT)) fail();
+        if (lane == 0 && !tma_producer<TBN>(maps, w, kv_y, kv_z, vl_y, vl_z, bars, smem, abort_flag, limit, p.drop_load, vl_tiles_head, settle)) fail();
     } else if (warp == 1 || warp == 2) {
         if (lane == 0) {
             const int q = warp - 1;
             const bool ok = mma_issuer<LOWBIT_FP8, TBN>(q, q ? qs1 : qs0, w, bars, smem, tmem, abort_flag, limit, vl_tiles_head != nullptr);
-            if (EXACT || !ok || *abort_flag) {
+            if (settle || !ok || *abort_flag) {
                 // leaving early, or going on to another piece of work: none of this thread's MMAs, and none of their
                 // arrivals at barriers, may be on its way when the CTA gives up its tensor memory or initialises its barriers again
                 umma_commit(&bars.drain[q]);
@@ -622,20 +733,16 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
             bar_sync_named(1, 8 * 32);
             const bool again = *restart_flag != 0 && *abort_flag == 0;
             if (again && warp == 4 && lane == 0) {
-                const uint32_t slot = atomicAdd(p.redo, 1u);
-                p.redo[1 + slot] = (uint32_t)bx;
+                const int at = atomicAdd(&p.redo[0].x, 1);
+                p.redo[1 + at] = make_int4(pc.seq | ((pc.slot + 1) << 8), pc.unit, pc.t0, pc.t1);
             }
             return again;
         };
         // own tiles of this CTA: numbers [n0, n_total) in the query tile's own list (all of it unless the keys are split)
-        const int n0 = SPLIT ? own_before(own, w.t0) : 0;
-        const int n_total = SPLIT ? own_before(own, w.t1) : own.a_end + (own.b_end - own.b_beg) + (own.c_end - own.c_beg);
-        if (SPLIT && sq.live && n_total <= n0) {
-            // nothing of this query tile lies in the slice: an empty partial result
-            const int i = sq.i0 + (warp & 3) * 32 + lane;
-            if (i < L)
-                reinterpret_cast<float2*>(p.part_ml)[((long)split * p.Hq * p.B + qhead) * L + i] = make_float2(-INFINITY, 0.0f);
-        }
+        const int n0 = GENERAL ? own_before(own, w.t0) : 0;
+        const int n_total = GENERAL ? own_before(own, w.t1) : own.a_end + (own.b_end - own.b_beg) + (own.c_end - own.c_beg);
+        if (GENERAL && pc.slot >= 0 && sq.live && n_total <= n0)   // nothing of this query tile lies in the piece: an empty partial result
+            reinterpret_cast<float2*>(p.part_ml)[(long)pc.slot * TC_ROWS + q * BM + (warp & 3) * 32 + lane] = make_float2(-INFINITY, 0.0f);
         if (sq.live && n_total > n0) {
             const int r = (warp & 3) * 32 + lane;               // query row inside the tile = TMEM lane
             const int i = sq.i0 + r;                           // row of the query block ...
@@ -646,9 +753,9 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
             const uint32_t to = tmem + tm_o(q) + lane_addr, ts0 = tmem + tm_s(q) + lane_addr;
 #if HYQ_TC_VARIANT_BT
             const int bsh = p.bt_shift;
-            const float q_scale = row_live ? __ldg(p.q_scales + (long)qhead * p.nbq + (i >> bsh)) : 0.0f;
+            const float q_scale = row_live ? __ldg(p.q_scales + qs_at + (i >> bsh)) : 0.0f;
 #else
-            const float q_scale = row_live ? __ldg(p.q_scales + (long)qhead * p.nbq + i / HYQ_BLOCK_TOKENS) : 0.0f;
+            const float q_scale = row_live ? __ldg(p.q_scales + qs_at + i / HYQ_BLOCK_TOKENS) : 0.0f;
 #endif
             constexpr uint32_t knock_lq = LOWBIT_FP8 ? KNOCKOUT_F32 : KNOCKOUT_S32;
             float m_used = -INFINITY, l_h = 0.0f;               // reference maximum of the row; row sum
@@ -664,13 +771,9 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
             };
             // K scale and this half's vertical-line bitmask word of a low-bit tile, fetched one tile ahead of their use
             // (tile n of the low-bit pass sits at walk position n; its block and mask words exist for n < a_end)
-#if HYQ_TC_VARIANT_BT
-            // a 64-key tile n lies in block n / 2 (128-token blocks) or in blocks 2n and 2n + 1, one per column half (32)
-            const float* ks_ptr = p.k_scales + (long)kvhead * p.nb;
-#else
-            const float* ks_ptr = p.k_scales + (long)kvhead * p.nb;
-#endif
-            const uint32_t* vl_ptr = p.vl_bits + (long)qhead * p.mask_words;
+            // (other block sizes: a 64-key tile n lies in block n / 2 or in blocks 2n and 2n + 1, one per column half)
+            const float* ks_ptr = p.k_scales + ks_at;
+            const uint32_t* vl_ptr = p.vl_bits + mask_at;
             float nks = 0.0f;
 #if HYQ_TC_VARIANT_BT
             float nks_b = 0.0f, cs_hi = 0.0f;                   // K scale and score factor of columns 32-63 (32-token blocks: their own block)
@@ -806,14 +909,16 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
                 prefetch_tile(n + 1);
                 return do_tile(std::false_type{}, n, cs, vl, !LOWBIT_FP8, 0, 0u);
             };
-            if (!EXACT && n_plain_end - n0 > WARM_TILES) {
+            const bool brief = GENERAL && pc.slot >= 0 && n_plain_end - n0 <= 2 * WARM_TILES;
+            const int n_warm = n0 + (brief ? WARM_TILES_SHORT : WARM_TILES);
+            if (!EXACT && n_plain_end > n_warm) {
                 float mt_lo = INFINITY, mt_hi = -INFINITY;
-                for (; n < n0 + WARM_TILES; ++n) {
+                for (; n < n_warm; ++n) {
                     if (!plain_tile()) { aborted = true; break; }
                     mt_lo = fminf(mt_lo, tile_max);
                     mt_hi = fmaxf(mt_hi, tile_max);
                 }
-                warm = !aborted && __all_sync(0xffffffffu, m_used > -INFINITY && mt_hi - mt_lo < WARM_SPREAD);
+                warm = !aborted && __all_sync(0xffffffffu, m_used > -INFINITY && mt_hi - mt_lo < (brief ? WARM_SPREAD_SHORT : WARM_SPREAD));
             }
             if (!warm) {
                 for (; n < n_plain_end && !aborted; ++n)
@@ -937,14 +1042,19 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
                 const float l_run = l_h;
                 // Rows leave through shared memory (this query tile's operands, which nothing reads any more) and TMA: a
                 // thread that stored its own 512-byte row made every store instruction touch 32 lines (10.3 k clocks of an
-                // average CTA's 141 k at L = 8192, fp32).  Per warp three 4 KB buffers of 32 rows x 128 bytes, pieces swizzled as the
-                // tensor map expects them.  Rows past the end are clipped by the map.
-                const float inv = SPLIT ? 1.0f : (l_run > 0.0f) ? 1.0f / l_run : 0.0f;   // (slices leave O as accumulated, relative to m_used)
+                // average CTA's 141 k at L = 8192, fp32; now 5.0 k).  Per warp three 4 KB buffers of 32 rows x 128 bytes, pieces swizzled as the
+                // tensor map expects them.  Rows past the end are clipped by the plain kernel's map; in the flattened view they would be
+                // the next head's, so a warp with such rows copies its own ones instead.
+                const bool part = GENERAL && pc.slot >= 0;      // (a partial result leaves O as accumulated, relative to m_used)
+                const float inv = part ? 1.0f : (l_run > 0.0f) ? 1.0f / l_run : 0.0f;
                 if (ok) {
                     unsigned char* buf0 = smem + SQ_OFF + q * Q_TILE_BYTES + (warp & 3) * 8192;
                     unsigned char* buf2 = smem + SQC_OFF + q * QC_TILE_BYTES + (warp & 3) * 4096;
-                    const int row0 = sq.i0 + (warp & 3) * 32, z = SPLIT ? split * p.Hq * p.B + qhead : qhead;
-                    const bool f32 = SPLIT || p.out_fp32 != 0;
+                    const int row0 = sq.i0 + (warp & 3) * 32, rows = min(32, L - row0);
+                    const bool f32 = part || p.out_fp32 != 0;
+                    const CUtensorMap* map = part ? &maps.po : &maps.o;
+                    const int o_y = part ? pc.slot * TC_ROWS + q * BM + (warp & 3) * 32 : q_y + row0, o_z = part ? 0 : q_z;
+                    const bool by_tma = !GENERAL || part || rows == 32;
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         uint32_t o[32];
@@ -976,20 +1086,26 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
                             }
                         }
                         if (f32 || (c & 1)) {
-                            fence_proxy_async();
-                            __syncwarp();
-                            if (lane == 0 && row0 < L) {
-                                tma_store_3d(&maps.o, buf, f32 ? c * 32 : (c >> 1) * 64, row0, z);
-                                bulk_commit();
+                            if (by_tma) {
+                                fence_proxy_async();
+                                __syncwarp();
+                                if (lane == 0 && rows > 0) {
+                                    tma_store_3d(map, buf, f32 ? c * 32 : (c >> 1) * 64, o_y, o_z);
+                                    bulk_commit();
+                                }
+                            } else {
+                                __syncwarp();
+                                const int row_bytes = f32 ? HYQ_D * 4 : HYQ_D * 2, col = (f32 ? c : c >> 1) * 128 + (lane & 7) * 16;
+                                for (int rr = lane >> 3; rr < rows; rr += 4)
+                                    *reinterpret_cast<uint4*>(static_cast<char*>(p.out) + (long)(o_y + rr) * row_bytes + col) =
+                                        *reinterpret_cast<const uint4*>(buf + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
+                                __syncwarp();
                             }
                         }
                     }
-                    if (SPLIT && row_live)
-                        reinterpret_cast<float2*>(p.part_ml)[((long)split * p.Hq * p.B + qhead) * L + i] = make_float2(m_used, l_run);
+                    if (part) reinterpret_cast<float2*>(p.part_ml)[(long)pc.slot * TC_ROWS + q * BM + r] = make_float2(m_used, l_run);
+                    else if (p.lse && row_live) p.lse[lse_at + i] = (m_used + log2f(l_run)) * 0.6931471805599453f;
                     if (lane == 0) bulk_wait_read<0>();             // the buffers outlive the copies
-                }
-                if (!SPLIT && ok) {
-                    if (p.lse && row_live) p.lse[(long)qhead * L + i] = (m_used + log2f(l_run)) * 0.6931471805599453f;
                 }
             }
             if (!ok) fail();
@@ -1001,7 +1117,9 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (EXACT && abort_s) break;
+    if (!EXACT && !GENERAL) break;
+    if (abort_s || (!EXACT && next_s < 0)) break;
+    item += gridDim.x;
     }
     tc_fence_before();
     __syncthreads();
@@ -1011,43 +1129,60 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     }
 }
 
-// Combines the partial results of the key slices of a short query block: every slice s left, per row, its
-// accumulator O_s relative to its own reference maximum m_s (log2 units) and its row sum l_s; the row's result is
-// sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s with M = max_s m_s.  One thread per row and four channels.
+// Combines the partial results of a split sequence's units: every piece s of a unit left, per row, its accumulator O_s
+// relative to its own reference maximum m_s (log2 units) and its row sum l_s; the row's result is
+// sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s with M = max_s m_s.  One warp per row; units that one CTA did alone are
+// complete already.
 __global__ void __launch_bounds__(256)
-attn_merge_kernel(const float* __restrict__ part_o, const float* __restrict__ part_ml, int splits, long n_rows, void* out,
-                  int out_fp32, float* lse) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long row = e / (HYQ_D / 4);
-    const int c4 = (int)(e % (HYQ_D / 4));
-    if (row >= n_rows) return;
+attn_merge_kernel(const __grid_constant__ TcSeq q, int heads, int window, int fixed_tail, const float* __restrict__ part_o,
+                  const float* __restrict__ part_ml, void* out, int out_fp32, float* lse) {
+    pdl_wait();
+    const int unit = blockIdx.x >> 5, level = unit / heads, lane = threadIdx.x & 31;
+    // first tile of the unit: the units before it, level by level
+    int first = 0, tiles = 0;
+    for (int l0 = 0; l0 <= level; l0 += 32) {
+        const int l = l0 + lane;
+        const int t = l <= level ? tc_unit_tiles(q.L, q.Lq, q.k, window, fixed_tail, q.levels - 1 - l) : 0;
+        int sum = l < level ? t * heads : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        first += sum;
+        if (level - l0 < 32) tiles = __shfl_sync(0xffffffffu, t, level - l0);
+    }
+    first += (unit - level * heads) * tiles;
+    const int c0 = split_of(q.tiles, q.split, first), c1 = split_of(q.tiles, q.split, first + tiles - 1);
+    if (c0 == c1) return;
+    const int row = (blockIdx.x & 31) * 8 + (threadIdx.x >> 5), i = (q.levels - 1 - level) * TC_ROWS + row;
+    if (i >= q.Lq) return;
+    // the unit's first piece is its CTA's first or a later one, all others are their CTAs' first
+    const int s0 = q.slot0 + 2 * c0 + (split_begin(q.tiles, q.split, c0) == first ? 0 : 1);
+    auto slot = [&](int c) -> long { return (long)(c == c0 ? s0 : q.slot0 + 2 * c) * TC_ROWS + row; };
     float m = -INFINITY;
-    for (int s = 0; s < splits; ++s) m = fmaxf(m, __ldg(part_ml + ((long)s * n_rows + row) * 2));
+    for (int c = c0; c <= c1; ++c) m = fmaxf(m, __ldg(part_ml + slot(c) * 2));
     float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     float l = 0.0f;
-    for (int s = 0; s < splits; ++s) {
-        const float2 ml = __ldg(reinterpret_cast<const float2*>(part_ml) + (long)s * n_rows + row);
-        if (!(ml.y > 0.0f)) continue;                           // empty slice: its accumulator was not written
+    for (int c = c0; c <= c1; ++c) {
+        const float2 ml = __ldg(reinterpret_cast<const float2*>(part_ml) + slot(c));
+        if (!(ml.y > 0.0f)) continue;                           // empty piece: its accumulator was not written
         const float wgt = exp2f(ml.x - m);
-        const float4 o = __ldg(reinterpret_cast<const float4*>(part_o + ((long)s * n_rows + row) * HYQ_D) + c4);
+        const float4 o = __ldg(reinterpret_cast<const float4*>(part_o + slot(c) * HYQ_D) + lane);
         acc.x = fmaf(wgt, o.x, acc.x); acc.y = fmaf(wgt, o.y, acc.y); acc.z = fmaf(wgt, o.z, acc.z); acc.w = fmaf(wgt, o.w, acc.w);
         l = fmaf(wgt, ml.y, l);
     }
     const float inv = (l > 0.0f) ? 1.0f / l : 0.0f;
     acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+    const long orow = q.q_row0 + (long)(unit - level * heads) * q.Lq + i;
     if (out_fp32) {
-        reinterpret_cast<float4*>(static_cast<float*>(out) + row * HYQ_D)[c4] = acc;
+        reinterpret_cast<float4*>(static_cast<float*>(out) + orow * HYQ_D)[lane] = acc;
     } else {
         const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
-        reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + row * HYQ_D)[c4] =
+        reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + orow * HYQ_D)[lane] =
             make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
     }
-    if (lse && c4 == 0) lse[row] = (m + log2f(l)) * 0.6931471805599453f;
+    if (lse && lane == 0) lse[orow] = (m + log2f(l)) * 0.6931471805599453f;
 }
 
 // ---------------------------------------------------------------------------------------------
-size_t attn_tc_workspace_bytes(const hyq_attn_args& a) { return tc_workspace_layout(a).total; }
-
 // CTAs of this translation unit's kernels whose work was done a second time (synchronises the device)
 int tc_restarts(unsigned long long* count, bool reset) {
     if (cudaMemcpyFromSymbol(count, g_tc_restarts, sizeof(*count)) != cudaSuccess) return HYQ_ERR_CUDA;
@@ -1056,101 +1191,94 @@ int tc_restarts(unsigned long long* count, bool reset) {
     return HYQ_OK;
 }
 
-int launch_attn_tc(const hyq_attn_args& a, float alpha, cudaStream_t st) {
+template <bool GENERAL>
+static int launch_attn_tc_kernels(const hyq_attn_args& a, const TcPlan& plan, const TcMaps& maps, const TcParams& p, int n_ctas,
+                                  int pieces, cudaStream_t st) {
+    Tables<GENERAL> tabs;
+    if constexpr (GENERAL) static_cast<TcTables&>(tabs) = plan.t;
+    // e4m3 bytes on the low-bit side: FP8 codes as they are, or INT4 codes widened by the pre-pass
+    const bool lowbit_fp8 = a.q_format != HYQ_FMT_INT8;
+    auto kern = lowbit_fp8 ? attn_tc_kernel<true, GENERAL> : attn_tc_kernel<false, GENERAL>;
+    // the same instantiation for the second launch (every maximum looked at; works through the first launch's list)
+    auto kern_exact = lowbit_fp8 ? attn_tc_kernel<true, GENERAL, true> : attn_tc_kernel<false, GENERAL, true>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(kern_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_BYTES) != cudaSuccess)
+        return HYQ_ERR_CUDA;
+    int rc = launch_pdl(kern, dim3((unsigned)n_ctas), dim3(TC_THREADS), TC_SMEM_BYTES, st, maps, p, tabs);
+    if (rc != HYQ_OK) return rc;
+    return launch_pdl(kern_exact, dim3((unsigned)(pieces < TC_SMS ? pieces : TC_SMS)), dim3(TC_THREADS), TC_SMEM_BYTES, st, maps, p, tabs);
+}
+
+int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, float alpha, cudaStream_t st) {
     constexpr int TBN = 64;                                             // keys per tile
-    const TcWorkspace w = tc_workspace_layout(a);
-    const int rc = launch_tc_prepass(a, w, st);
+    const TcWorkspace& w = plan.w;
+    const TcSeqTable& tab = plan.t.tab;
+    int rc = launch_tc_prepass(a, plan, st);
     if (rc != HYQ_OK) return rc;
     char* base = static_cast<char*>(a.workspace);
-    const bool int4 = a.q_format == HYQ_FMT_INT4;
-    const uint64_t qh = (uint64_t)a.B * a.Hq, kvh = (uint64_t)a.B * a.Hkv, L = a.L, Lq = query_rows(a);
-    const uint64_t kk = a.k > 0 ? a.k : 1;
+    const bool packed = a.q_format == HYQ_FMT_INT4;
+    // the general kernel addresses the flattened views (everything but a plain whole prefill, see there)
+    const TcSeq& s0 = tab.seq[0];
+    const bool general = tab.n_seq > 1 || s0.split > 0 || s0.Lq < s0.L || a.window_mode == HYQ_WINDOW_FIXED_TAIL;
+    const uint64_t qh = general ? 1 : tab.heads, kvh = general ? 1 : tab.heads / tab.g;
+    const uint64_t L = tab.kv_rows / kvh, Lq = tab.q_rows / qh, kk = tab.vl_rows > 0 ? tab.vl_rows / qh : 1;
 
     TcMaps maps;
     bool ok = true;
     ok &= make_tmap_3d(&maps.q, a.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, Lq, qh, 64, BM);
     ok &= make_tmap_3d(&maps.k, a.k_, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, L, kvh, 64, TBN);
-    ok &= make_tmap_3d(&maps.qc, int4 ? (const void*)(base + w.q8) : a.q_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, HYQ_D, Lq, qh, 128, BM);
-    ok &= make_tmap_3d(&maps.kc, int4 ? (const void*)(base + w.k8) : a.k_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, HYQ_D, L, kvh, 128, TBN);
+    ok &= make_tmap_3d(&maps.qc, packed ? (const void*)(base + w.q8) : a.q_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, HYQ_D, Lq, qh, 128, BM);
+    ok &= make_tmap_3d(&maps.kc, packed ? (const void*)(base + w.k8) : a.k_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, HYQ_D, L, kvh, 128, TBN);
     ok &= make_tmap_3d(&maps.v16, base + w.v16, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, HYQ_D, L, kvh, 64, TBN);
     ok &= make_tmap_3d(&maps.vh16, base + w.vh16, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, HYQ_D, L, kvh, 64, TBN);
     ok &= make_tmap_3d(&maps.kvl, base + w.kvl, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, kk, qh, 64, TBN);
     ok &= make_tmap_3d(&maps.vvl, base + w.vvl, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, HYQ_D, kk, qh, 64, TBN);
-    if (w.splits > 1)
-        ok &= make_tmap_3d(&maps.o, base + w.part_o, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, HYQ_D, Lq, qh * w.splits, 32, 32);
-    else if (a.out_dtype == 1)
+    if (a.out_dtype == 1)
         ok &= make_tmap_3d(&maps.o, a.out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, HYQ_D, Lq, qh, 32, 32);
     else
         ok &= make_tmap_3d(&maps.o, a.out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, Lq, qh, 64, 32);
+    maps.po = maps.o;
+    if (w.slots)
+        ok &= make_tmap_3d(&maps.po, base + w.part_o, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, HYQ_D, (uint64_t)w.slots * TC_ROWS, 1, 32, 32);
     if (!ok) return HYQ_ERR_CUDA;
 
     TcParams p{};
-    p.B = a.B; p.Hq = a.Hq; p.Hkv = a.Hkv; p.L = a.L; p.window = a.window; p.k = a.k;
+    p.B = tab.heads / a.Hq; p.Hq = a.Hq; p.Hkv = a.Hkv; p.L = s0.L; p.window = a.window; p.k = s0.k;
+    p.nb = s0.nb; p.nbq = s0.nbq;
 #if HYQ_TC_VARIANT_BT
-    p.nb = (a.L + a.block_tokens - 1) / a.block_tokens;
     p.bt_shift = a.block_tokens == 32 ? 5 : 7;
-#else
-    p.nb = (a.L + HYQ_BLOCK_TOKENS - 1) / HYQ_BLOCK_TOKENS;
 #endif
-    p.Lq = (int)Lq;
+    p.Lq = s0.Lq;
     p.fixed_tail = a.window_mode == HYQ_WINDOW_FIXED_TAIL;
-    p.splits = w.splits;
-    p.part_o = reinterpret_cast<float*>(base + w.part_o);
     p.part_ml = reinterpret_cast<float*>(base + w.part_ml);
-#if HYQ_TC_VARIANT_BT
-    p.nbq = ((int)Lq + a.block_tokens - 1) / a.block_tokens;
-#else
-    p.nbq = ((int)Lq + HYQ_BLOCK_TOKENS - 1) / HYQ_BLOCK_TOKENS;
-#endif
-    p.mask_words = w.mask_words;
+    p.mask_words = s0.mask_words;
     p.out_fp32 = a.out_dtype == 1;
     p.scale_log2 = alpha * 1.4426950408889634f;
     p.q_scales = a.q_scales; p.k_scales = a.k_scales; p.vl_idx = a.vl_idx;
     p.vl_bits = reinterpret_cast<const uint32_t*>(base + w.vl_bits);
-    p.vl_tiles = (a.q_format != HYQ_FMT_INT8 && a.k > 0) ? reinterpret_cast<const uint8_t*>(base + w.vl_tiles) : nullptr;
+    p.vl_tiles = (a.q_format != HYQ_FMT_INT8 && tab.vl_rows > 0) ? reinterpret_cast<const uint8_t*>(base + w.vl_tiles) : nullptr;
     p.out = a.out; p.lse = a.lse; p.status = a.status_word;
     const TcTestHooks hooks = tc_test_hooks();
     p.wait_limit = hooks.wait_limit > 0 ? hooks.wait_limit : WAIT_LIMIT_DEFAULT;
     p.drop_load = hooks.drop_load;
 
-    const bool blk = Lq < L || p.fixed_tail;      // the general instantiation (the other one is the whole prefill)
-    // e4m3 bytes on the low-bit side: FP8 codes as they are, or INT4 codes widened by the pre-pass
-    const bool lowbit_fp8 = a.q_format != HYQ_FMT_INT8;
-    const bool split = w.splits > 1;               // (only ever chosen for short query blocks)
-    auto kern = split ? (lowbit_fp8 ? attn_tc_kernel<true, true, true> : attn_tc_kernel<false, true, true>)
-              : lowbit_fp8 ? (blk ? attn_tc_kernel<true, true> : attn_tc_kernel<true, false>)
-                           : (blk ? attn_tc_kernel<false, true> : attn_tc_kernel<false, false>);
-    // the same instantiation for the second launch (every maximum looked at; works through the first launch's list)
-    auto kern_exact = split ? (lowbit_fp8 ? attn_tc_kernel<true, true, true, true> : attn_tc_kernel<false, true, true, true>)
-                    : lowbit_fp8 ? (blk ? attn_tc_kernel<true, true, false, true> : attn_tc_kernel<true, false, false, true>)
-                                 : (blk ? attn_tc_kernel<false, true, false, true> : attn_tc_kernel<false, false, false, true>);
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(kern_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_BYTES) != cudaSuccess)
-        return HYQ_ERR_CUDA;
     // Order of the CTAs: longest walk first over all heads whose K / V the L2 holds at once - with the order "head by
     // head" the last heads' long CTAs ran beside idle SMs (L = 8192, 32 heads: the busiest SM 14 % above the mean).
     // Whole KV heads, at most 48 MB of keys and values (half of L2), the heads shared out evenly over the groups.
-    p.grid_x = (((int)Lq + QT * BM - 1) / (QT * BM)) * w.splits;
-    const long kv_bytes = (long)a.L * (HYQ_D + 2 * HYQ_D + (p.vl_tiles ? 32 * (a.Hq / a.Hkv) : 0));   // codes, V^, vertical-line operands
-    const long kv_heads = (long)a.B * a.Hkv, cap = (48L << 20) / kv_bytes > 1 ? (48L << 20) / kv_bytes : 1;
+    p.grid_x = s0.levels;
+    const long kv_bytes = (long)s0.L * (HYQ_D + 2 * HYQ_D + (p.vl_tiles ? 32 * (a.Hq / a.Hkv) : 0));   // codes, V^, vertical-line operands
+    const long kv_heads = tab.heads / tab.g, cap = (48L << 20) / kv_bytes > 1 ? (48L << 20) / kv_bytes : 1;
     const long groups = (kv_heads + cap - 1) / cap;
     p.head_group = (int)((kv_heads + groups - 1) / groups) * (a.Hq / a.Hkv);
-    const long n_ctas = (long)p.grid_x * a.Hq * a.B;
-    if (n_ctas > 0x7fffffffL) return HYQ_ERR_UNSUPPORTED;
-    p.redo = reinterpret_cast<uint32_t*>(base + w.redo);
-    if (cudaMemsetAsync(p.redo, 0, sizeof(uint32_t), st) != cudaSuccess) return HYQ_ERR_CUDA;
+    p.redo = reinterpret_cast<int4*>(base + w.redo);           // (its count starts at zero: the pre-pass)
     if (a.ev_kernel_start && cudaEventRecord(static_cast<cudaEvent_t>(a.ev_kernel_start), st) != cudaSuccess) return HYQ_ERR_CUDA;
-    kern<<<(unsigned)n_ctas, TC_THREADS, TC_SMEM_BYTES, st>>>(maps, p);
-    if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-    {
-        kern_exact<<<(unsigned)(n_ctas < 148 ? n_ctas : 148), TC_THREADS, TC_SMEM_BYTES, st>>>(maps, p);
-        if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-    }
-    if (split) {
-        const long n_rows = (long)a.B * a.Hq * (long)Lq, n_thr = n_rows * (HYQ_D / 4);
-        attn_merge_kernel<<<(unsigned)((n_thr + 255) / 256), 256, 0, st>>>(p.part_o, p.part_ml, w.splits, n_rows, a.out, p.out_fp32, a.lse);
-        if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-    }
+    rc = general ? launch_attn_tc_kernels<true>(a, plan, maps, p, tab.ctas, w.pieces, st)
+                 : launch_attn_tc_kernels<false>(a, plan, maps, p, tab.ctas, w.pieces, st);
+    for (int s = tab.n_unsplit; rc == HYQ_OK && s < tab.n_seq; ++s)
+        rc = launch_pdl(attn_merge_kernel, dim3((unsigned)(tab.seq[s].levels * tab.heads * 32)), dim3(256), 0, st, tab.seq[s], tab.heads,
+                        a.window, p.fixed_tail, reinterpret_cast<const float*>(base + w.part_o), static_cast<const float*>(p.part_ml),
+                        a.out, p.out_fp32, a.lse);
+    if (rc != HYQ_OK) return rc;
     if (a.ev_kernel_stop && cudaEventRecord(static_cast<cudaEvent_t>(a.ev_kernel_stop), st) != cudaSuccess) return HYQ_ERR_CUDA;
     return HYQ_OK;
 }

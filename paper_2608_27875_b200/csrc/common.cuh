@@ -22,6 +22,22 @@ __host__ __device__ constexpr size_t align_up(size_t x, size_t a) { return (x + 
 
 static inline int launch_status() { return cudaGetLastError() == cudaSuccess ? HYQ_OK : HYQ_ERR_CUDA; }
 
+// Launch whose grid may be set up while the kernel before it on the stream still runs (programmatic dependent launch):
+// the kernel calls pdl_wait() before it touches memory, which returns when the one before has completed.  Every kernel of
+// this library that is launched this way calls it, so that completion is passed on along the stream.
+template <typename... P, typename... A>
+static inline int launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...) == cudaSuccess ? HYQ_OK : HYQ_ERR_CUDA;
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 // internal launchers (defined in the kernel files)
 int launch_quantize(const void* x, long n_heads, int L, int block_tokens, int format, void* codes, float* scales, cudaStream_t st);
 static inline bool block_tokens_ok(int bt) { return bt == 32 || bt == 64 || bt == 128; }

@@ -48,3 +48,47 @@ def test_heads_interleaved_in_groups(B, Hq, Hkv, L, Lq):
     ensure_built()
     Q, K, V = _normal((B, Hq, Lq, 128), L), _normal((B, Hkv, L, 128), L + 1), _normal((B, Hkv, L, 128), L + 2)
     _close(*_both_kernels(Q, K, V, INT8, 256, 100))
+
+
+@pytest.mark.parametrize("fmts", [INT8, FP8ALL, INT4FP8])
+@pytest.mark.parametrize("Hq,Hkv,L,Lq,W,k,mode,out", [
+    (2, 2, 2048, 2048, 128, 32, 0, torch.float32),      # a whole prefill of few units
+    (1, 1, 3333, 3333, 100, 70, 0, torch.bfloat16),     # ragged last tile, bf16 rows from the merge and from whole pieces
+    (4, 2, 9000, 777, 256, 200, 0, torch.float32),      # a query block, last unit of 9 rows
+    (4, 1, 6000, 1500, 512, 100, 1, torch.bfloat16),    # fixed window: equal units
+    (1, 1, 20000, 1, 64, 300, 0, torch.float32),        # one row: most pieces have one live query tile
+])
+def test_units_shared_by_several_ctas(fmts, Hq, Hkv, L, Lq, W, k, mode, out):
+    ensure_built()
+    Q, K, V = _normal((1, Hq, Lq, 128), L), _normal((1, Hkv, L, 128), L + 1), _normal((1, Hkv, L, 128), L + 2)
+    _close(*_both_kernels(Q, K, V, fmts, W, k, out, window_mode=mode))
+
+
+@pytest.mark.parametrize("fmts", [INT8, INT4FP8])
+def test_ragged_batches_of_any_launch_grouping_give_the_same_bits(fmts, monkeypatch):
+    """40 prompts (more than one launch holds) with all the workspace, and with the longest prompt's alone (the smallest
+    the call accepts: launches of a few prompts each); among them prompts whose units are shared by several CTAs."""
+    ensure_built()
+    rng = np.random.default_rng(5)
+    lens = [int(x) for x in np.exp(rng.uniform(np.log(1), np.log(3000), 39))] + [3000]
+    qs, ks, vs = ([_normal((h, L, 128), 100 * h + n) for n, L in enumerate(lens)] for h in (6, 2, 2))
+    k_per = [max(0, L - 128) // 40 for L in lens]
+    one = api.hybrid_prefill_varlen(qs, ks, vs, 128, k_per, fmts)
+    lib = api.lib()
+
+    class Small:                              # the same library, but the ragged query answers with the longest prompt's need
+        def __getattr__(self, name):
+            if name != "hyq_hybrid_attention_prefill_varlen_workspace":
+                return getattr(lib, name)
+
+            def longest(a, n, cu, kk, out):
+                return lib.hyq_hybrid_attention_prefill_workspace(a, out)
+            return longest
+    monkeypatch.setattr(api, "lib", lambda: Small())
+    few = api.hybrid_prefill_varlen(qs, ks, vs, 128, k_per, fmts)
+    monkeypatch.undo()
+    for a, b in zip(one, few):
+        assert torch.equal(a["out"], b["out"])
+    for n in (0, 17, 39):                     # and the plain call's
+        alone = api.hybrid_prefill(qs[n][None], ks[n][None], vs[n][None], 128, k_per[n], fmts)
+        assert torch.equal(alone["out"][0], one[n]["out"])
