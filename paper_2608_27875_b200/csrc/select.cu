@@ -1,113 +1,201 @@
 // Vertical token identification (Algorithm 1): tail-query mean -> GQA-native dot-product
 // scores over the non-window prefix -> exact top-k per query head.
 //
-// Three kernels, all bound by memory traffic:
-//   tail_mean_kernel   qbar[b,h,:] = (1/t) sum of the last t query rows, fp64, added in row order
-//   vscore_kernel      S[b,h,p] = qbar[b,h,:] . K[b,h/g,p,:], an fp64 fma chain in channel
+// Three kernels, each over all sequences of a call (one plain batch, or the prompts of a ragged one):
+//   tail_mean_kernel   qbar[h,:] = (1/t) sum of the last t query rows, fp64, as if added in row order
+//   vscore_kernel      S[h,p] = qbar[h,:] . K[h/g,p,:], an fp64 fma chain in channel
 //                      order; each K row is read once per KV head and scored for its g query heads
-//   topk_kernel        per (b,h): MSB-first radix select of the k-th largest score on an
-//                      order-preserving 64-bit key, then an ordered compaction that emits the
-//                      selected positions ascending; equal scores go to the lower position.
+//   topk_kernel        per head: radix select of the k-th largest score on an order-preserving 64-bit
+//                      key, then an ordered compaction that emits the selected positions ascending;
+//                      equal scores go to the lower position.
 // The fp64 chain is what makes the selected set reproducible bit for bit: ranking in lower
 // precision flips pairs whose scores differ by less than its rounding error.
+#include <cooperative_groups.h>
+
 #include <mutex>
 
-#include "common.cuh"
+#include "select_common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace hyq {
 
-constexpr int SCORE_KEYS = 128;      // keys per CTA in vscore_kernel
-constexpr int SCORE_GC = 4;          // query heads scored per pass over the staged K tile
-constexpr int TOPK_THREADS = 1024;
-constexpr int SCAN_DEPTH = 8;         // loads of the score row a thread of the radix select keeps in flight
-constexpr int TOPK_CAND = 1536;      // candidate keys that the radix select keeps in shared memory
+// A bf16 number (its bits the upper half of `f`) as a double scaled by 2^-896: the float's exponent field becomes the double's
+// as it stands, so this is a shift and a mask where the conversion instruction runs at a quarter of the fp64 rate.  Exact for
+// every finite input (bf16 subnormals become double subnormals of the same value); the factor is taken out with K_UNIT.
+__device__ __forceinline__ double bf16_small(uint32_t f) { return __hiloint2double(((int)f >> 3) & 0x8FFFE000, 0); }
+constexpr double K_UNIT = 0x1p896;
 
 // -------------------------------------------------------------------------------------------
-// The t tail rows are added in ascending row order in fp64, one running sum per (b, h, channel) - the order of
-// Algorithm 1's mean as it is written down, so the result is the same double for every finite input, whatever the
-// spread of the exponents (a split into partial sums would only agree while every partial sum is exact).  A CTA owns
-// 32 channels of one (b, h): all its threads stage 512 rows at a time in shared memory (the loads are what takes
-// time), then one thread per channel runs the addition chain over the staged rows.
-constexpr int MEAN_CH = 32, MEAN_ROWS = 512, MEAN_THREADS = 256;
+// The mean is defined by the t tail rows added in ascending row order in fp64.  Whenever every partial sum of every order is
+// exact - the largest and the smallest non-zero exponent of the rows lie so close that all bits of any sum fit the 53 of a
+// double - the order does not matter, and the rows are shared out over the threads; the kernel checks that on the rows it
+// reads and goes through them in order otherwise (wide exponent spreads).  A CTA owns 32 channels of one head, 64 rows at a
+// time, 8 channels per thread.  The chain alone took 38 clocks per row (1024 rows of 32 heads: 19.6 us, now 10.4).
+constexpr int MEAN_THREADS = 256, MEAN_CH = 32, MEAN_GROUPS = MEAN_THREADS / (MEAN_CH / 8);
 
 __global__ void __launch_bounds__(MEAN_THREADS)
-tail_mean_kernel(const __nv_bfloat16* __restrict__ q, int Lq, int t, double* __restrict__ qbar) {
-    __shared__ __nv_bfloat16 tile[MEAN_ROWS][MEAN_CH + 2];         // +2: the chain's column reads stay conflict-free enough
-    const long bh = blockIdx.x;
-    const int c0 = blockIdx.y * MEAN_CH;
-    const __nv_bfloat16* base = q + (bh * Lq + (Lq - t)) * (long)HYQ_D + c0;
-    double s = 0.0;
-    for (int r0 = 0; r0 < t; r0 += MEAN_ROWS) {
-        const int rows = min(MEAN_ROWS, t - r0);
-        __syncthreads();
-        // 16 threads per row, 4 bytes each
-        for (int e = threadIdx.x; e < rows * (MEAN_CH / 2); e += MEAN_THREADS) {
-            const int r = e / (MEAN_CH / 2), c2 = (e % (MEAN_CH / 2)) * 2;
-            *reinterpret_cast<uint32_t*>(&tile[r][c2]) = __ldg(reinterpret_cast<const uint32_t*>(base + (long)(r0 + r) * HYQ_D + c2));
+tail_mean_kernel(const __grid_constant__ SelTable tab, double* __restrict__ qbar) {
+    pdl_wait();
+    __shared__ double part[MEAN_GROUPS][MEAN_CH];
+    __shared__ uint32_t red_max[MEAN_THREADS / 32], red_min[MEAN_THREADS / 32];
+    const SelSeq& sq = tab.seq[blockIdx.y];
+    const int t = sq.t, c8 = threadIdx.x & (MEAN_CH / 8 - 1), grp = threadIdx.x / (MEAN_CH / 8), lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (sq.P == 0 || sq.k_sel == 0) return;
+    const uint4* rows = reinterpret_cast<const uint4*>(sq.q + ((long)blockIdx.x * sq.Lq + (sq.Lq - t)) * HYQ_D) + blockIdx.z * (MEAN_CH / 8);
+    double s[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] = 0.0;
+    uint32_t mx = 0u, mn = 0xFFFFFFFFu;                          // packed halves: largest magnitude; smallest non-zero one minus one
+    for (int r0 = grp; r0 < t; r0 += 4 * MEAN_GROUPS) {
+        uint4 w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int r = r0 + u * MEAN_GROUPS;
+            w[u] = r < t ? __ldg(rows + (long)r * 16 + c8) : make_uint4(0u, 0u, 0u, 0u);
         }
-        __syncthreads();
-        if (threadIdx.x < MEAN_CH) {
-            int r = 0;
-            for (; r + 8 <= rows; r += 8) {
-                float v[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = __bfloat162float(tile[r + j][threadIdx.x]);
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t x[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
 #pragma unroll
-                for (int j = 0; j < 8; ++j) s += (double)v[j];
+            for (int j = 0; j < 4; ++j) {
+                s[2 * j] += bf16_small(x[j] << 16);
+                s[2 * j + 1] += bf16_small(x[j] & 0xFFFF0000u);
+                const uint32_t a = x[j] & 0x7FFF7FFFu;
+                mx = __vmaxu2(mx, a);
+                mn = __vminu2(mn, __vsub2(a, 0x00010001u));
             }
-            for (; r < rows; ++r) s += (double)__bfloat162float(tile[r][threadIdx.x]);
         }
     }
-    if (threadIdx.x < MEAN_CH) qbar[bh * HYQ_D + c0 + threadIdx.x] = s / (double)t;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) part[grp][c8 * 8 + j] = s[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        mx = __vmaxu2(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        mn = __vminu2(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    }
+    if (lane == 0) { red_max[wid] = mx; red_min[wid] = mn; }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < MEAN_THREADS / 32; ++w) { mx = __vmaxu2(mx, red_max[w]); mn = __vminu2(mn, red_min[w]); }
+    // exponents; 0xFFFF in `mn` means that no value was non-zero.  A sum of t values is below 2^(emax + 1 + ceil(log2 t)) and a
+    // multiple of 2^(emin - 7).
+    const int hi = (int)max(mx & 0xFFFFu, mx >> 16) >> 7, lo_v = (int)min(mn & 0xFFFFu, mn >> 16) + 1, lo = lo_v > 0xFFFF ? hi : lo_v >> 7;
+    const int emax = max(hi, 1), emin = max(lo, 1);              // (subnormals share the exponent of the smallest normals)
+    const int bits = emax - emin + 8 + (t > 1 ? 32 - __clz(t - 1) : 0);
+    if (threadIdx.x < MEAN_CH) {
+        double sum = 0.0;
+        if (bits <= 53) {
+            double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+            for (int gidx = 0; gidx < MEAN_GROUPS; ++gidx) a[gidx & 3] += part[gidx][threadIdx.x];
+            sum = ((a[0] + a[1]) + (a[2] + a[3])) * K_UNIT;
+        } else {
+            const __nv_bfloat16* col = reinterpret_cast<const __nv_bfloat16*>(rows) + threadIdx.x;
+            int r = 0;
+            for (; r + 8 <= t; r += 8) {
+                float v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = __bfloat162float(col[(long)(r + j) * HYQ_D]);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) sum += (double)v[j];
+            }
+            for (; r < t; ++r) sum += (double)__bfloat162float(col[(long)r * HYQ_D]);
+        }
+        qbar[((long)blockIdx.y * tab.heads + blockIdx.x) * HYQ_D + blockIdx.z * MEAN_CH + threadIdx.x] = sum / (double)t;
+    }
 }
 
 // -------------------------------------------------------------------------------------------
-constexpr int KROW_WORDS = HYQ_D / 2 + 1;    // 65 words per staged key row: conflict-free column reads
+// A CTA owns 64 * KPT consecutive keys of one KV head, each thread KPT of them for up to GC query heads: KPT * GC
+// independent fma chains per thread, and per pair of channels GC broadcast loads of q for 2 * KPT * GC fma.  Bound by the
+// fp64 pipe (64 fma per clock and SM) beside the K stream; with one key per thread and converted operands the broadcasts and
+// conversions cost as much again (32768 keys, 32 heads of 8 KV heads: 33.5 us, now 27; five heads per KV head, 4 x 16384
+// keys: 98 us in two rounds of four, now 54).  KPT = 1 where the grid of KPT = 2 would leave SMs idle.  K rows are staged at
+// a pitch of 17 16-byte pieces (conflict-free for row-wise writes and one-row-per-thread reads), a quarter of the channels
+// at a time, so that the sums of one quarter run while the next is on its way; small CTAs keep the last wave short.  q as
+// doubles scaled by 2^896 against the keys' 2^-896 (the products are the same numbers).
+constexpr int SCORE_THREADS = 64;
+constexpr int SCORE_PARTS = 4;
+constexpr int SCORE_PITCH = HYQ_D / 8 + 1;
 
-__global__ void __launch_bounds__(SCORE_KEYS)
-vscore_kernel(const __nv_bfloat16* __restrict__ kmat, const double* __restrict__ qbar, int Hq, int Hkv, int Lk,
-              int P, double* __restrict__ scores) {
+template <int GC, int KPT>
+__global__ void __launch_bounds__(SCORE_THREADS)
+vscore_kernel(const __grid_constant__ SelTable tab, const double* __restrict__ qbar, double* __restrict__ scores) {
+    constexpr int KEYS = SCORE_THREADS * KPT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int g = Hq / Hkv;
-    uint32_t* ktile = reinterpret_cast<uint32_t*>(smem_raw);                          // [SCORE_KEYS][KROW_WORDS]
-    double* qs = reinterpret_cast<double*>(smem_raw + align_up(SCORE_KEYS * KROW_WORDS * 4, 16));  // [g][D]
+    uint4* ktile = reinterpret_cast<uint4*>(smem_raw);                              // [KEYS][SCORE_PITCH]
+    double* qs = reinterpret_cast<double*>(smem_raw + KEYS * SCORE_PITCH * 16);     // [GC][D]
+    pdl_wait();
+    int n_s = 0;
+    while (n_s + 1 < tab.n_seq && tab.seq[n_s + 1].block0 <= (int)blockIdx.x) ++n_s;
+    const SelSeq& sq = tab.seq[n_s];
+    const int per_head = (sq.P + KEYS - 1) / KEYS, local = blockIdx.x - sq.block0;
+    const int kvh = local / per_head, p0 = (local - kvh * per_head) * KEYS;
+    const int n_keys = min(KEYS, sq.P - p0);
 
-    const int p0 = blockIdx.x * SCORE_KEYS;
-    const int kvh = blockIdx.y, b = blockIdx.z;
-    const int n_keys = min(SCORE_KEYS, P - p0);
-
-    // stage the K rows (coalesced 16-byte reads, 4-byte shared stores)
-    const uint4* src = reinterpret_cast<const uint4*>(kmat + (((long)b * Hkv + kvh) * Lk + p0) * HYQ_D);
-    for (int v = threadIdx.x; v < n_keys * (HYQ_D / 8); v += SCORE_KEYS) {
-        const uint4 w = __ldg(src + v);
-        const int row = v / (HYQ_D / 8), c4 = (v % (HYQ_D / 8)) * 4;
-        uint32_t* dst = ktile + row * KROW_WORDS + c4;
-        dst[0] = w.x; dst[1] = w.y; dst[2] = w.z; dst[3] = w.w;
+    const uint4* src = reinterpret_cast<const uint4*>(sq.k + ((long)kvh * sq.Lk + p0) * HYQ_D);
+    const uint32_t dst0 = (uint32_t)__cvta_generic_to_shared(ktile);
+#pragma unroll
+    for (int part = 0; part < SCORE_PARTS; ++part) {
+        for (int v = threadIdx.x; v < n_keys * 4; v += SCORE_THREADS) {
+            const int at = (v >> 2) * 16 + part * 4 + (v & 3);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst0 + ((v >> 2) * SCORE_PITCH + part * 4 + (v & 3)) * 16), "l"(src + at) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    for (int e = threadIdx.x; e < g * HYQ_D; e += SCORE_KEYS)
-        qs[e] = qbar[((long)b * Hq + (long)kvh * g) * HYQ_D + e];
-    __syncthreads();
-    if ((int)threadIdx.x >= n_keys) return;
 
-    const uint32_t* krow = ktile + threadIdx.x * KROW_WORDS;
-    for (int r0 = 0; r0 < g; r0 += SCORE_GC) {
-        double s[SCORE_GC];
-        const double* qr[SCORE_GC];
+    for (int r0 = 0; r0 < tab.g; r0 += GC) {
+        const long h0 = (long)n_s * tab.heads + (long)kvh * tab.g + r0;
+        const int n_heads = min(GC, tab.g - r0);
+        if (r0 > 0) __syncthreads();
+        for (int e = threadIdx.x; e < GC * HYQ_D; e += SCORE_THREADS)
+            qs[e] = e < n_heads * HYQ_D ? qbar[h0 * HYQ_D + e] * K_UNIT : 0.0;
+        double s[KPT][GC];
 #pragma unroll
-        for (int c = 0; c < SCORE_GC; ++c) { s[c] = 0.0; qr[c] = qs + min(r0 + c, g - 1) * HYQ_D; }
-#pragma unroll 4
-        for (int w = 0; w < HYQ_D / 2; ++w) {
-            const uint32_t kw = krow[w];
-            const double k0 = (double)bf16_lo(kw), k1 = (double)bf16_hi(kw);
+        for (int u = 0; u < KPT; ++u)
 #pragma unroll
-            for (int c = 0; c < SCORE_GC; ++c) {
-                s[c] = fma(qr[c][2 * w], k0, s[c]);
-                s[c] = fma(qr[c][2 * w + 1], k1, s[c]);
+            for (int c = 0; c < GC; ++c) s[u][c] = 0.0;
+        const uint4* krow = ktile + threadIdx.x * SCORE_PITCH;
+#pragma unroll 1
+        for (int v = 0; v < HYQ_D / 8; ++v) {
+            if ((v & 3) == 0 && (r0 == 0 || v == 0)) {               // the next quarter has landed (and q, the first time)
+                if (v == 0) asm volatile("cp.async.wait_group 3;" ::: "memory");
+                else if (v == 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
+                else if (v == 8) asm volatile("cp.async.wait_group 1;" ::: "memory");
+                else asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncthreads();
+            }
+            uint4 kw[KPT];
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) kw[u] = krow[u * SCORE_THREADS * SCORE_PITCH + v];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                double k0[KPT], k1[KPT];
+#pragma unroll
+                for (int u = 0; u < KPT; ++u) {
+                    const uint32_t x = w == 0 ? kw[u].x : w == 1 ? kw[u].y : w == 2 ? kw[u].z : kw[u].w;
+                    k0[u] = bf16_small(x << 16);
+                    k1[u] = bf16_small(x & 0xFFFF0000u);
+                }
+#pragma unroll
+                for (int c = 0; c < GC; ++c) {
+                    const double2 qv = *reinterpret_cast<const double2*>(qs + c * HYQ_D + 8 * v + 2 * w);
+#pragma unroll
+                    for (int u = 0; u < KPT; ++u) {
+                        s[u][c] = fma(qv.x, k0[u], s[u][c]);
+                        s[u][c] = fma(qv.y, k1[u], s[u][c]);
+                    }
+                }
             }
         }
 #pragma unroll
-        for (int c = 0; c < SCORE_GC; ++c)
-            if (r0 + c < g) scores[(((long)b * Hq + (long)kvh * g + r0 + c)) * P + p0 + threadIdx.x] = s[c];
+        for (int u = 0; u < KPT; ++u) {
+            const int p = threadIdx.x + u * SCORE_THREADS;
+#pragma unroll
+            for (int c = 0; c < GC; ++c)
+                if (p < n_keys && c < n_heads) scores[sq.score0 + (long)(kvh * tab.g + r0 + c) * sq.P + p0 + p] = s[u][c];
+        }
     }
 }
 
@@ -118,147 +206,179 @@ __device__ __forceinline__ unsigned long long order_key(double s) {
     return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
-// One CTA per (b, query head); every warp owns a contiguous segment of the row (coalesced reads, no CTA-wide
-// synchronisation inside a scan of the row).
+// A cluster of CTAs per score row, each with a contiguous segment of it, kept as keys in shared memory (RESIDENT; rows of more
+// than 8 segments of TOPK_SEG keys are read again in every sweep).  The k-th largest key is searched by its distance below the
+// row's maximum, 11 bits at a time from bit 45 on - 128 bins per octave, 16 octaves below the maximum, where the threshold of
+// a top-few-percent lies - so that one sweep usually leaves a handful of keys, which are then ranked directly; distances beyond
+// those 16 octaves start over from bit 53, which covers every key.  The histograms of a cluster's CTAs are added up through
+// distributed shared memory.  Bound by latency: one CTA per row and eight 8-bit sweeps took 18.7 us for 1920 keys, 41 us for
+// 31744 and 122 us for 130048; now 7.9, 24 and 82 us.
+constexpr int TOPK_THREADS = 512;
+constexpr int TOPK_SEG = 24 * 1024;   // keys that a CTA can hold
+constexpr int TOPK_BINS = 2048;
+constexpr int TOPK_CAND = 256;        // keys left in the race that are ranked directly
+
+template <bool RESIDENT>
 __global__ void __launch_bounds__(TOPK_THREADS)
-topk_kernel(const double* __restrict__ scores, int P, int k, int32_t* __restrict__ idx_out) {
-    constexpr int NW = TOPK_THREADS / 32;
-    __shared__ int whist[NW][256];                     // one digit histogram per warp (no contention across warps)
-    __shared__ int hist[256];
-    __shared__ int warp_gt[NW], warp_eq[NW];
-    __shared__ unsigned long long sh_prefix;
-    __shared__ int sh_krem, sh_bin, n_cand;
-    __shared__ unsigned long long cand[TOPK_CAND];     // the keys still in the race once few are left
-    const double* row = scores + (long)blockIdx.x * P;
-    int32_t* out = idx_out + (long)blockIdx.x * k;
+topk_kernel(const __grid_constant__ SelTable tab, const double* __restrict__ scores, int32_t* __restrict__ idx_out) {
+    typedef unsigned long long u64;
+    constexpr int NW = TOPK_THREADS / 32, PER = TOPK_BINS / TOPK_THREADS;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    u64* keys = reinterpret_cast<u64*>(smem_raw);
+    __shared__ __align__(16) int hist[TOPK_BINS];
+    __shared__ u64 cand[TOPK_CAND], mine_cand[TOPK_CAND];
+    __shared__ u64 red[NW], sh_max, sh_thr;
+    __shared__ int wsum[NW], warp_gt[NW], warp_eq[NW], tot_gt, tot_eq, n_cand, sh_bin, sh_above, sh_cnt, sh_krem;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    pdl_wait();
+    const int row_no = blockIdx.x / C, s_no = row_no / tab.heads, head = row_no - s_no * tab.heads;
+    const SelSeq& sq = tab.seq[s_no];
+    const int P = sq.P, k = sq.k_sel;
+    if (P == 0 || k == 0) return;                       // (the whole cluster)
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int per = (P + NW - 1) / NW;
-    const int seg0 = min(P, wid * per), seg1 = min(P, seg0 + per);
+    const int per = (P + C - 1) / C, seg0 = min(P, rank * per), n = min(P, seg0 + per) - seg0;
+    const double* row = scores + sq.score0 + (long)head * P + seg0;
+    int32_t* out = idx_out + sq.idx0 + (long)head * k;
+    auto sync_cluster = [&]() { if (C > 1) cl.sync(); else __syncthreads(); };
+    auto key_at = [&](int i) -> u64 { return RESIDENT ? keys[i] : order_key(__ldg(row + i)); };
 
-    // radix select: after the loop `prefix` is the key of the k-th largest score and k_rem how
-    // many positions holding exactly that key are still to be taken
-    // Once a pass leaves no more than TOPK_CAND keys sharing the digits fixed so far, those keys are gathered into
-    // shared memory (one more sweep over the row) and the remaining passes run over that short list.
-    unsigned long long prefix = 0ull;
-    int k_rem = k;
-    bool gathered = false;
-    for (int pass = 0; pass < 8; ++pass) {
-        const int shift = 56 - 8 * pass;
+    u64 mx = 0ull;
+    for (int i0 = threadIdx.x; i0 < n; i0 += 4 * TOPK_THREADS) {
+        double v[4];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) whist[wid][lane + 32 * e] = 0;
-        __syncwarp();
-        if (gathered) {
-            const int nc = n_cand;
-            for (int c = threadIdx.x; c < nc; c += TOPK_THREADS) {
-                const unsigned long long key = cand[c];
-                if ((key >> (shift + 8)) == (prefix >> (shift + 8))) atomicAdd(&whist[wid][(int)((key >> shift) & 0xFF)], 1);
-            }
+        for (int u = 0; u < 4; ++u) v[u] = i0 + u * TOPK_THREADS < n ? __ldg(row + i0 + u * TOPK_THREADS) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (i0 + u * TOPK_THREADS >= n) break;
+            const u64 key = order_key(v[u]);
+            if (RESIDENT) keys[i0 + u * TOPK_THREADS] = key;
+            mx = key > mx ? key : mx;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) { const u64 v = __shfl_xor_sync(0xffffffffu, mx, o); mx = v > mx ? v : mx; }
+    if (lane == 0) red[wid] = mx;
+    if (threadIdx.x == 0) n_cand = 0;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NW; ++w) mx = red[w] > mx ? red[w] : mx;
+    if (threadIdx.x == 0) sh_max = mx;
+    sync_cluster();
+    for (int c = 0; c < C; ++c) { const u64 v = *cl.map_shared_rank(&sh_max, c); mx = v > mx ? v : mx; }
+
+    // distances d = maximum - key: the k-th smallest lies in [base, base + 2^width), `above` distances lie below base
+    u64 base = 0ull;
+    int shift = 45, width = 64, above = 0, count = P;
+    while (count > TOPK_CAND && width > 0) {
+#pragma unroll
+        for (int b = 0; b < PER; ++b) hist[threadIdx.x + b * TOPK_THREADS] = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += TOPK_THREADS) {
+            const u64 d = mx - key_at(i) - base;                 // (wraps to a large number below base)
+            if (width < 64 && (d >> width)) continue;
+            const u64 b = d >> shift;
+            if (b < TOPK_BINS) atomicAdd(&hist[(int)b], 1);      // (beyond them: only with width 64, found again from bit 53 on)
+        }
+        sync_cluster();
+        int4 sum = make_int4(0, 0, 0, 0);
+        static_assert(PER == 4, "one int4 of bins per thread");
+        for (int c = 0; c < C; ++c) {
+            const int4 v = *(reinterpret_cast<const int4*>(cl.map_shared_rank(hist, c)) + threadIdx.x);
+            sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+        }
+        int incl = sum.x + sum.y + sum.z + sum.w;
+        const int mine = incl;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+        if (lane == 31) wsum[wid] = incl;
+        if (threadIdx.x == 0) sh_bin = -1;
+        __syncthreads();
+        int before = above + incl - mine;
+        for (int w = 0; w < wid; ++w) before += wsum[w];
+        if (before < k && k <= before + mine) {                  // at most one thread
+            const int v[4] = {sum.x, sum.y, sum.z, sum.w};
+            int b = 0;
+            while (before + v[b] < k) before += v[b++];
+            sh_bin = threadIdx.x * PER + b; sh_above = before; sh_cnt = v[b];
+        }
+        __syncthreads();
+        if (sh_bin < 0) {                                        // more than 16 octaves below the maximum
+            shift = 53;
         } else {
-            // (eight loads in flight per thread: a scan of the row is bound by their latency)
-            for (int p0 = seg0 + lane; p0 < seg1; p0 += 32 * SCAN_DEPTH) {
-                double v[SCAN_DEPTH];
-#pragma unroll
-                for (int j = 0; j < SCAN_DEPTH; ++j) v[j] = (p0 + 32 * j < seg1) ? __ldg(row + p0 + 32 * j) : 0.0;
-#pragma unroll
-                for (int j = 0; j < SCAN_DEPTH; ++j) {
-                    const unsigned long long key = order_key(v[j]);
-                    if (p0 + 32 * j < seg1 && (pass == 0 || (key >> (shift + 8)) == (prefix >> (shift + 8))))
-                        atomicAdd(&whist[wid][(int)((key >> shift) & 0xFF)], 1);
-                }
-            }
+            base += (u64)sh_bin << shift;
+            above = sh_above; count = sh_cnt;
+            width = shift;
+            shift = shift > 11 ? shift - 11 : 0;
+        }
+        if (count > TOPK_CAND && width > 0) sync_cluster();      // every CTA has read the histograms before they are cleared
+    }
+    // threshold key: directly the one left (width 0: all `count` keys are equal), or ranked among the candidates
+    u64 thr = mx - base;
+    int k_rem = k - above;
+    if (width > 0) {
+        // every CTA lists its own candidates, reads all lists and ranks the keys itself
+        for (int i = threadIdx.x; i < n; i += TOPK_THREADS) {
+            const u64 key = key_at(i), d = mx - key - base;
+            if (width == 64 || !(d >> width)) mine_cand[atomicAdd(&n_cand, 1)] = key;
+        }
+        sync_cluster();
+        int got = 0;
+        for (int c = 0; c < C; ++c) {
+            const int nc = *cl.map_shared_rank(&n_cand, c);
+            const u64* list = cl.map_shared_rank(mine_cand, c);
+            for (int i = threadIdx.x; i < nc; i += TOPK_THREADS) cand[got + i] = list[i];
+            got += nc;
         }
         __syncthreads();
-        if (threadIdx.x < 256) {
-            int tot = 0;
-#pragma unroll 8
-            for (int w = 0; w < NW; ++w) tot += whist[w][threadIdx.x];
-            hist[threadIdx.x] = tot;
+        if ((int)threadIdx.x < count) {
+            const u64 me = cand[threadIdx.x];
+            int gt = 0, ge = 0;
+#pragma unroll 4
+            for (int o = 0; o < count; ++o) { const u64 v = cand[o]; gt += v > me; ge += v >= me; }
+            if (gt < k_rem && k_rem <= ge) { sh_thr = me; sh_krem = k_rem - gt; }         // (equal keys write the same)
         }
         __syncthreads();
-        // the digit d whose bin holds the k_rem-th largest candidate: the largest d with
-        // count(bins above d) < k_rem <= count(bins d and above); lane l of warp 0 looks at bins 255-8l .. 248-8l
-        if (wid == 0) {
-            const int hi = 255 - 8 * lane;
-            int mine = 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) mine += hist[hi - j];
-            int incl = mine;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
-            }
-            int above = incl - mine;                   // candidates in bins above this lane's eight
-            if (above < k_rem && k_rem <= incl) {      // exactly one lane (the candidates number at least k_rem)
-                int d = hi;
-                for (; d > hi - 7; --d) {
-                    if (above + hist[d] >= k_rem) break;
-                    above += hist[d];
-                }
-                sh_prefix = prefix | ((unsigned long long)d << shift);
-                sh_krem = k_rem - above;
-                sh_bin = hist[d];                      // keys that share all digits fixed so far
-                if (!gathered) n_cand = 0;
-            }
-        }
-        __syncthreads();
-        prefix = sh_prefix;
+        thr = sh_thr;
         k_rem = sh_krem;
-        if (!gathered && pass < 6 && sh_bin <= TOPK_CAND) {
-            for (int p0 = seg0 + lane; p0 < seg1; p0 += 32 * SCAN_DEPTH) {
-                double v[SCAN_DEPTH];
-#pragma unroll
-                for (int j = 0; j < SCAN_DEPTH; ++j) v[j] = (p0 + 32 * j < seg1) ? __ldg(row + p0 + 32 * j) : 0.0;
-#pragma unroll
-                for (int j = 0; j < SCAN_DEPTH; ++j) {
-                    const unsigned long long key = order_key(v[j]);
-                    if (p0 + 32 * j < seg1 && (key >> shift) == (prefix >> shift)) cand[atomicAdd(&n_cand, 1)] = key;
-                }
-            }
-            gathered = true;                           // (uniform over the CTA: sh_bin is)
-            __syncthreads();
-        }
     }
 
-    // ordered compaction: positions ascending; among keys equal to the threshold the first k_rem.
-    // Scan 1 counts, per warp segment, the keys above and equal to the threshold; scan 2 writes: the output
-    // slot of a selected position = (keys above the threshold before it) + min(keys equal before it, k_rem).
+    // ordered compaction: positions ascending; among keys equal to the threshold the first k_rem.  Sweep 1 counts, per warp
+    // segment, the keys above and equal to the threshold; sweep 2 writes: the slot of a selected position = (keys above
+    // the threshold before it) + min(keys equal before it, k_rem).
+    const int wper = (n + NW - 1) / NW, w0 = min(n, wid * wper), w1 = min(n, w0 + wper);
     int n_gt = 0, n_eq = 0;
-    for (int base = seg0; base < seg1; base += 32 * SCAN_DEPTH) {
-        double v[SCAN_DEPTH];
-#pragma unroll
-        for (int j = 0; j < SCAN_DEPTH; ++j) v[j] = (base + 32 * j + lane < seg1) ? __ldg(row + base + 32 * j + lane) : 0.0;
-#pragma unroll
-        for (int j = 0; j < SCAN_DEPTH; ++j) {
-            const bool live = base + 32 * j + lane < seg1;
-            const unsigned long long key = order_key(v[j]);
-            n_gt += __popc(__ballot_sync(0xffffffffu, live && key > prefix));
-            n_eq += __popc(__ballot_sync(0xffffffffu, live && key == prefix));
-        }
+    for (int i = w0 + lane; i < w1; i += 32) {
+        const u64 key = key_at(i);
+        n_gt += key > thr;
+        n_eq += key == thr;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) { n_gt += __shfl_xor_sync(0xffffffffu, n_gt, o); n_eq += __shfl_xor_sync(0xffffffffu, n_eq, o); }
     if (lane == 0) { warp_gt[wid] = n_gt; warp_eq[wid] = n_eq; }
     __syncthreads();
-    int gt_run = 0, eq_run = 0;
-    for (int w = 0; w < wid; ++w) { gt_run += warp_gt[w]; eq_run += warp_eq[w]; }
-    const unsigned lt_mask = (1u << lane) - 1u;
-    for (int base = seg0; base < seg1; base += 32 * SCAN_DEPTH) {
-        double v[SCAN_DEPTH];
+    int gt_run = 0, eq_run = 0, gt_all = 0, eq_all = 0;
 #pragma unroll
-        for (int j = 0; j < SCAN_DEPTH; ++j) v[j] = (base + 32 * j + lane < seg1) ? __ldg(row + base + 32 * j + lane) : 0.0;
-#pragma unroll
-        for (int j = 0; j < SCAN_DEPTH; ++j) {
-            const int p = base + 32 * j + lane;
-            const bool live = p < seg1;
-            const unsigned long long key = order_key(v[j]);
-            const bool gt = live && key > prefix, eq = live && key == prefix;
-            const unsigned b_gt = __ballot_sync(0xffffffffu, gt), b_eq = __ballot_sync(0xffffffffu, eq);
-            const int eq_rank = eq_run + __popc(b_eq & lt_mask);
-            const int pos = gt_run + __popc(b_gt & lt_mask) + min(eq_rank, k_rem);
-            if ((gt || (eq && eq_rank < k_rem)) && pos < k) out[pos] = p;
-            gt_run += __popc(b_gt);
-            eq_run += __popc(b_eq);
-        }
+    for (int w = 0; w < NW; ++w) {
+        if (w == wid) { gt_run = gt_all; eq_run = eq_all; }
+        gt_all += warp_gt[w]; eq_all += warp_eq[w];
     }
+    if (threadIdx.x == 0) { tot_gt = gt_all; tot_eq = eq_all; }
+    sync_cluster();
+    for (int c = 0; c < rank; ++c) { gt_run += *cl.map_shared_rank(&tot_gt, c); eq_run += *cl.map_shared_rank(&tot_eq, c); }
+    const unsigned lt_mask = (1u << lane) - 1u;
+    for (int i0 = w0; i0 < w1; i0 += 32) {
+        const int i = i0 + lane;
+        const u64 key = i < w1 ? key_at(i) : 0ull;
+        const bool gt = i < w1 && key > thr, eq = i < w1 && key == thr;
+        const unsigned b_gt = __ballot_sync(0xffffffffu, gt), b_eq = __ballot_sync(0xffffffffu, eq);
+        const int eq_rank = eq_run + __popc(b_eq & lt_mask);
+        const int pos = gt_run + __popc(b_gt & lt_mask) + min(eq_rank, k_rem);
+        if ((gt || (eq && eq_rank < k_rem)) && pos < k) out[pos] = seg0 + i;
+        gt_run += __popc(b_gt);
+        eq_run += __popc(b_eq);
+    }
+    if (C > 1) cl.sync();                                        // (no CTA leaves while another reads its counts)
 }
 
 // -------------------------------------------------------------------------------------------
@@ -266,35 +386,81 @@ size_t select_workspace_bytes(int B, int Hq, int Lk, int window) {
     const long P = (Lk - window > 0) ? Lk - window : 0;
     return align_up((size_t)B * Hq * HYQ_D * sizeof(double), 256) + align_up((size_t)B * Hq * P * sizeof(double), 256);
 }
+static size_t qbar_bytes(const SelTable& tab) { return align_up((size_t)tab.n_seq * tab.heads * HYQ_D * sizeof(double), 256); }
+size_t select_scratch_bytes(const SelTable& tab) {
+    size_t scores = 0;
+    for (int s = 0; s < tab.n_seq; ++s) scores += (size_t)tab.heads * tab.seq[s].P;
+    return qbar_bytes(tab) + align_up(scores * sizeof(double), 256);
+}
+
+int launch_topk_table(const SelTable& tab, const double* scores, int32_t* idx_out, cudaStream_t st) {
+    int max_p = 0;
+    for (int s = 0; s < tab.n_seq; ++s)
+        if (tab.seq[s].k_sel > 0 && tab.seq[s].P > max_p) max_p = tab.seq[s].P;
+    if (max_p == 0) return HYQ_OK;
+    // CTAs per row: about 4096 keys each, fewer where the rows alone fill the GPU
+    const long rows = (long)tab.n_seq * tab.heads;
+    int C = max_p <= 4096 ? 1 : max_p <= 8192 ? 2 : max_p <= 16384 ? 4 : 8;
+    while (C > 1 && rows * C > 4 * 148 && (max_p + C / 2 - 1) / (C / 2) <= TOPK_SEG / 2) C /= 2;
+    const int per = (max_p + C - 1) / C;
+    const bool resident = per <= TOPK_SEG;
+    auto kern = resident ? topk_kernel<true> : topk_kernel<false>;
+    const size_t smem = resident ? (size_t)per * 8 : 0;
+    if (smem > 32 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TOPK_SEG * 8) != cudaSuccess) return HYQ_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(rows * C)); cfg.blockDim = dim3(TOPK_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)C; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, tab, scores, idx_out) == cudaSuccess ? HYQ_OK : HYQ_ERR_CUDA;
+}
+
+template <int GC, int KPT>
+static int launch_vscore(const SelTable& tab, long blocks, const double* qbar, double* scores, cudaStream_t st) {
+    constexpr int smem = SCORE_THREADS * KPT * SCORE_PITCH * 16 + GC * HYQ_D * 8;
+    static_assert(smem <= 48 * 1024, "needs no opt-in");
+    return launch_pdl(vscore_kernel<GC, KPT>, dim3((unsigned)blocks), dim3(SCORE_THREADS), smem, st, tab, qbar, scores);
+}
+
+int launch_select_table(SelTable& tab, int32_t* idx_out, void* ws, cudaStream_t st) {
+    double* qbar = static_cast<double*>(ws);
+    double* scores = reinterpret_cast<double*>(static_cast<char*>(ws) + qbar_bytes(tab));
+    long score0 = 0, blocks = 0;
+    auto count_blocks = [&](int keys) {
+        blocks = 0;
+        for (int s = 0; s < tab.n_seq; ++s) {
+            tab.seq[s].block0 = (int)blocks;
+            if (tab.seq[s].k_sel > 0) blocks += (long)((tab.seq[s].P + keys - 1) / keys) * (tab.heads / tab.g);
+        }
+    };
+    for (int s = 0; s < tab.n_seq; ++s) { tab.seq[s].score0 = score0; score0 += (long)tab.heads * tab.seq[s].P; }
+    count_blocks(2 * SCORE_THREADS);
+    const bool two = blocks >= 4 * 148;                          // two keys per thread where that still gives every SM four CTAs
+    if (!two) count_blocks(SCORE_THREADS);
+    if (blocks == 0) return HYQ_OK;
+    if (blocks > 0x7fffffffL) return HYQ_ERR_UNSUPPORTED;
+    int rc = launch_pdl(tail_mean_kernel, dim3((unsigned)tab.heads, (unsigned)tab.n_seq, HYQ_D / MEAN_CH), dim3(MEAN_THREADS), 0, st, tab, qbar);
+    if (rc != HYQ_OK) return rc;
+    const int g = tab.g;
+#define HYQ_VSCORE(GC_) (two ? launch_vscore<GC_, 2>(tab, blocks, qbar, scores, st) : launch_vscore<GC_, 1>(tab, blocks, qbar, scores, st))
+    rc = g == 1 ? HYQ_VSCORE(1) : g == 2 ? HYQ_VSCORE(2) : g <= 4 ? HYQ_VSCORE(4) : g == 5 ? HYQ_VSCORE(5) : HYQ_VSCORE(8);
+#undef HYQ_VSCORE
+    if (rc != HYQ_OK) return rc;
+    return launch_topk_table(tab, scores, idx_out, st);
+}
 
 int launch_select(const void* q, const void* k, int B, int Hq, int Hkv, int Lq, int Lk, int window, int n_tail,
                   int k_sel, int32_t* idx_out, void* ws, cudaStream_t st) {
-    const int P = (Lk - window > 0) ? Lk - window : 0;
-    const int t = n_tail ? n_tail : (window < Lq ? window : Lq);
-    const int g = Hq / Hkv;
-    double* qbar = static_cast<double*>(ws);
-    double* scores = reinterpret_cast<double*>(static_cast<char*>(ws) + align_up((size_t)B * Hq * HYQ_D * sizeof(double), 256));
-
-    tail_mean_kernel<<<dim3(B * Hq, HYQ_D / MEAN_CH), MEAN_THREADS, 0, st>>>(static_cast<const __nv_bfloat16*>(q), Lq, t, qbar);
-    if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-
-    const size_t smem = align_up(SCORE_KEYS * KROW_WORDS * 4, 16) + (size_t)g * HYQ_D * sizeof(double);
-    if (smem > 200 * 1024) return HYQ_ERR_UNSUPPORTED;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(vscore_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return HYQ_ERR_CUDA;
-    const dim3 grid((P + SCORE_KEYS - 1) / SCORE_KEYS, Hkv, B);
-    vscore_kernel<<<grid, SCORE_KEYS, smem, st>>>(static_cast<const __nv_bfloat16*>(k), qbar, Hq, Hkv, Lk, P, scores);
-    if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-
-    topk_kernel<<<B * Hq, TOPK_THREADS, 0, st>>>(scores, P, k_sel, idx_out);
-    return launch_status();
-}
-
-// top-k of `rows` score rows of length P (shared with the column-mass selector)
-int launch_topk(const double* scores, long rows, int P, int k_sel, int32_t* idx_out, cudaStream_t st) {
-    topk_kernel<<<(unsigned)rows, TOPK_THREADS, 0, st>>>(scores, P, k_sel, idx_out);
-    return launch_status();
+    SelTable tab{};
+    tab.n_seq = 1; tab.heads = B * Hq; tab.g = Hq / Hkv;
+    SelSeq& s = tab.seq[0];
+    s.q = static_cast<const __nv_bfloat16*>(q); s.k = static_cast<const __nv_bfloat16*>(k);
+    s.Lq = Lq; s.Lk = Lk; s.t = n_tail ? n_tail : (window < Lq ? window : Lq);
+    s.P = (Lk - window > 0) ? Lk - window : 0; s.k_sel = k_sel;
+    return launch_select_table(tab, idx_out, ws, st);
 }
 
 // -------------------------------------------------------------------------------------------

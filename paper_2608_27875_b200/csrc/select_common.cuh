@@ -1,0 +1,28 @@
+// Declarations of the vertical-line selectors.
+#pragma once
+#include "common.cuh"
+
+namespace hyq {
+
+constexpr int SEL_MAX_SEQ = 32;      // sequences of one launch (the table travels as a kernel parameter)
+
+// One sequence: a plain call is one with B * Hq heads, a ragged call has one per prompt.
+struct SelSeq {
+    const __nv_bfloat16 *q, *k;      // [heads][Lq][D], [heads / g][Lk][D]
+    int Lq, Lk, t;                   // t: tail rows of the mean
+    int P, k_sel;                    // candidate keys, keys to select
+    int block0;                      // first block of the score kernel
+    long score0, idx0;               // first score / first index of the sequence
+};
+struct SelTable {
+    int n_seq, heads, g;
+    SelSeq seq[SEL_MAX_SEQ];
+};
+
+// top-k of the score rows of every sequence (shared by the selectors)
+int launch_topk_table(const SelTable& tab, const double* scores, int32_t* idx_out, cudaStream_t st);
+// tail means, scores, top-k; scratch of select_scratch_bytes
+size_t select_scratch_bytes(const SelTable& tab);
+int launch_select_table(SelTable& tab, int32_t* idx_out, void* ws, cudaStream_t st);
+
+}  // namespace hyq

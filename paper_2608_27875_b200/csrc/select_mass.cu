@@ -16,7 +16,7 @@
 // Both passes use the same tile: a CTA of 256 threads owns 256 consecutive keys (four chunks) of one (b, kv head), each thread
 // keeps its key row in registers as bf16 pairs and scores it against MASS_TQ queries at a time, whose rows sit
 // in shared memory as doubles (broadcast reads).
-#include "common.cuh"
+#include "select_common.cuh"
 
 namespace hyq {
 
@@ -246,7 +246,10 @@ int launch_select_mass(const void* q, const void* k, int B, int Hq, int Hkv, int
     mass_column_kernel<<<dim3((P + MASS_THREADS - 1) / MASS_THREADS, Hkv, B), MASS_THREADS, smem, st>>>(qb, kb, Hq, Hkv, Lq, Lk, P, nT, alpha,
                                                                                                 row_mz, scores);
     if (launch_status() != HYQ_OK) return HYQ_ERR_CUDA;
-    return launch_topk(scores, (long)B * Hq, P, k_sel, idx_out, st);
+    SelTable tab{};
+    tab.n_seq = 1; tab.heads = B * Hq; tab.g = Hq / Hkv;
+    tab.seq[0].P = P; tab.seq[0].k_sel = k_sel;
+    return launch_topk_table(tab, scores, idx_out, st);
 }
 
 }  // namespace hyq

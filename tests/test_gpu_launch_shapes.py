@@ -92,3 +92,60 @@ def test_ragged_batches_of_any_launch_grouping_give_the_same_bits(fmts, monkeypa
     for n in (0, 17, 39):                     # and the plain call's
         alone = api.hybrid_prefill(qs[n][None], ks[n][None], vs[n][None], 128, k_per[n], fmts)
         assert torch.equal(alone["out"][0], one[n]["out"])
+
+
+# ---- selection: the oracle's index sets bit for bit ---------------------------------------------------------------
+def _select_is_the_oracles(Q, K, W, k, n_tail=0):
+    import oracle
+    got = api.hyq_select_vertical(Q.cuda(), K.cuda(), W, k, n_tail=n_tail).cpu().numpy()
+    np.testing.assert_array_equal(got, oracle.select_vertical(wl.bits(Q), wl.bits(K), W, k, n_tail=n_tail))
+
+
+@pytest.mark.parametrize("P,k", [(1, 1), (255, 255), (257, 3), (4096, 80), (4097, 4097), (8193, 160), (16385, 5), (40001, 900)])
+def test_topk_over_one_to_eight_ctas(P, k):
+    ensure_built()
+    W = 64
+    Q, K = _normal((1, 2, W, 128), P).cpu(), _normal((1, 1, P + W, 128), P + 1).cpu()
+    _select_is_the_oracles(Q, K, W, k)
+
+
+@pytest.mark.parametrize("kind", ["ties", "all_equal", "far_below_the_maximum", "narrow", "most_negative"])
+def test_topk_where_one_sweep_does_not_settle_it(kind):
+    """Scores are K's channel 0 times the tail mean's (the other channels are zero): equal keys, a threshold more than 16
+    octaves below the maximum, scores that agree in all leading bits, a threshold among negative scores."""
+    ensure_built()
+    W, P = 32, 6000
+    g = torch.Generator().manual_seed(11)
+    c = {"ties": torch.randint(0, 4, (P,), generator=g).float(),
+         "all_equal": torch.full((P,), 3.0),
+         "far_below_the_maximum": torch.cat([torch.full((5,), 2.0**60), torch.rand(P - 5, generator=g)]),
+         "narrow": 128.0 + torch.randint(0, 3, (P,), generator=g).float(),
+         "most_negative": torch.randn(P, generator=g) - 3.0}[kind]
+    K = torch.zeros(1, 1, P + W, 128)
+    K[0, 0, :P, 0] = c
+    Q = torch.zeros(1, 2, W, 128)
+    Q[:, :, :, 0] = 1.0
+    _select_is_the_oracles(Q.bfloat16(), K.bfloat16(), W, 700)
+
+
+@pytest.mark.parametrize("Hq,Hkv,P", [(1, 1, 129), (2, 1, 300), (3, 1, 257), (5, 1, 700), (8, 1, 128), (9, 1, 513), (16, 8, 9000), (40, 8, 9001)])
+def test_scores_for_every_group_size_and_both_key_counts_per_thread(Hq, Hkv, P):
+    ensure_built()
+    W = 48
+    Q, K = _normal((1, Hq, W, 128), P).cpu(), _normal((1, Hkv, P + W, 128), P + 1).cpu()
+    K[0, 0, 5] = 2.0**-130                     # bf16 subnormals, an all-zero row, one large row
+    K[0, 0, 6] = 0.0
+    K[0, 0, 7] = 2.0**100
+    _select_is_the_oracles(Q, K, W, max(1, P // 10))
+
+
+@pytest.mark.parametrize("t", [1, 2, 15, 16, 65, 300])
+@pytest.mark.parametrize("spread", [0, 20, 34, 60])
+def test_tail_mean_in_any_order_and_in_row_order(t, spread):
+    """Exponent spreads on either side of what keeps every partial sum exact (53 - 8 - log2 t bits)."""
+    ensure_built()
+    Q, K = _normal((1, 2, 300, 128), t).cpu().float(), _normal((1, 1, 400, 128), t + 1).cpu()
+    e = torch.randint(-spread // 2, spread // 2 + 1, Q.shape, generator=torch.Generator().manual_seed(t + spread))
+    Q = (Q * torch.exp2(e.float())).bfloat16()
+    Q[0, 0, -1, :7] = 0.0
+    _select_is_the_oracles(Q, K, 100, 150, n_tail=t)
