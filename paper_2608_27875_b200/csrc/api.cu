@@ -2,6 +2,8 @@
 #include <cmath>
 
 #include "attn_common.cuh"
+#include "quantize.cuh"
+#include "select_common.cuh"
 
 namespace hyq {
 size_t attn_simt_workspace_bytes(const hyq_attn_args& a);
@@ -224,18 +226,7 @@ static int check_cu(int n_seq, const int32_t* cu) {
     return HYQ_OK;
 }
 
-// sequence numbers, longest first (ties by position)
-static void longest_first(int n_seq, const int32_t* cu, int* order) {
-    for (int s = 0; s < n_seq; ++s) order[s] = s;
-    for (int a = 1; a < n_seq; ++a) {                       // insertion sort: batches are small
-        const int v = order[a], lv = cu[v + 1] - cu[v];
-        int b = a - 1;
-        while (b >= 0 && cu[order[b] + 1] - cu[order[b]] < lv) { order[b + 1] = order[b]; --b; }
-        order[b + 1] = v;
-    }
-}
-
-int hyq_select_vertical_varlen(const void* q, const void* k_, int n_seq, const int32_t* cu, int Hq, int Hkv, int D,
+int hyq_select_vertical_varlen(const void* q_, const void* k_, int n_seq, const int32_t* cu, int Hq, int Hkv, int D,
                                int window, int n_tail, const int32_t* k_per_seq, int32_t* idx_out, void* workspace,
                                size_t workspace_bytes, void* stream) {
     int rc = check_cu(n_seq, cu);
@@ -244,30 +235,34 @@ int hyq_select_vertical_varlen(const void* q, const void* k_, int n_seq, const i
     size_t need = 0;
     for (int s = 0; s < n_seq; ++s) {
         const int L = cu[s + 1] - cu[s];
-        rc = check_select(q, k_, 1, Hq, Hkv, L, L, D, window, n_tail, k_per_seq[s]);
+        rc = check_select(q_, k_, 1, Hq, Hkv, L, L, D, window, n_tail, k_per_seq[s]);
         if (rc != HYQ_OK) return rc;
         const long P = L - window > 0 ? (long)L - window : 0;
         if (P > 0 && k_per_seq[s] > 0) need = need > select_workspace_bytes(1, Hq, L, window) ? need : select_workspace_bytes(1, Hq, L, window);
     }
     if (need == 0) return HYQ_OK;
-    if (!q || !k_ || !idx_out || !workspace) return HYQ_ERR_INVALID_ARG;
-    if (!aligned16(q) || !aligned16(k_) || !aligned16(workspace) || (reinterpret_cast<uintptr_t>(idx_out) & 3u)) return HYQ_ERR_ALIGNMENT;
+    if (!q_ || !k_ || !idx_out || !workspace) return HYQ_ERR_INVALID_ARG;
+    if (!aligned16(q_) || !aligned16(k_) || !aligned16(workspace) || (reinterpret_cast<uintptr_t>(idx_out) & 3u)) return HYQ_ERR_ALIGNMENT;
     if (workspace_bytes < need) return HYQ_ERR_WORKSPACE;
-    int* order = new int[n_seq];
-    long* koff = new long[n_seq];
-    long acc = 0;
-    for (int s = 0; s < n_seq; ++s) { koff[s] = acc; acc += k_per_seq[s]; }
-    longest_first(n_seq, cu, order);
-    for (int n = 0; n < n_seq && rc == HYQ_OK; ++n) {
-        const int s = order[n], L = cu[s + 1] - cu[s], ks = k_per_seq[s];
-        if (ks == 0 || L - window <= 0) continue;
-        const char* qs = static_cast<const char*>(q) + (size_t)Hq * D * cu[s] * 2;
-        const char* kk = static_cast<const char*>(k_) + (size_t)Hkv * D * cu[s] * 2;
-        rc = launch_select(qs, kk, 1, Hq, Hkv, L, L, window, n_tail, ks, idx_out + (size_t)Hq * koff[s], workspace,
-                           static_cast<cudaStream_t>(stream));
+    // as many consecutive prompts per launch as the table and the workspace hold (each fits alone)
+    size_t k_before = 0;
+    for (int s = 0; s < n_seq && rc == HYQ_OK;) {
+        SelTable tab;
+        tab.n_seq = 0; tab.heads = Hq; tab.g = Hq / Hkv;
+        for (; s < n_seq && tab.n_seq < SEL_MAX_SEQ; ++s) {
+            const int L = cu[s + 1] - cu[s];
+            SelSeq& q = tab.seq[tab.n_seq++] = SelSeq{};
+            q.q = static_cast<const __nv_bfloat16*>(q_) + (size_t)Hq * D * cu[s];
+            q.k = static_cast<const __nv_bfloat16*>(k_) + (size_t)Hkv * D * cu[s];
+            q.Lq = q.Lk = L; q.t = n_tail ? n_tail : (window < L ? window : L);
+            q.k_sel = L > window ? k_per_seq[s] : 0;
+            q.P = q.k_sel > 0 ? L - window : 0;
+            q.idx0 = (long)Hq * (long)k_before;
+            if (tab.n_seq > 1 && select_scratch_bytes(tab) > workspace_bytes) { --tab.n_seq; break; }
+            k_before += (size_t)k_per_seq[s];
+        }
+        rc = launch_select_table(tab, idx_out, workspace, static_cast<cudaStream_t>(stream));
     }
-    delete[] order;
-    delete[] koff;
     return rc;
 }
 
@@ -281,12 +276,18 @@ int hyq_quantize_blocks_varlen(const void* x, int n_seq, const int32_t* cu, int 
     if (!aligned16(x) || !aligned16(codes_out) || (reinterpret_cast<uintptr_t>(scales_out) & 3u)) return HYQ_ERR_ALIGNMENT;
     const size_t row_bytes = format == HYQ_FMT_INT4 ? D / 2 : D;
     size_t nb_before = 0;
-    for (int s = 0; s < n_seq && rc == HYQ_OK; ++s) {
-        const int L = cu[s + 1] - cu[s];
-        rc = launch_quantize(static_cast<const char*>(x) + (size_t)H * D * cu[s] * 2, H, L, block_tokens, format,
-                             static_cast<char*>(codes_out) + (size_t)H * row_bytes * cu[s], scales_out + (size_t)H * nb_before,
-                             static_cast<cudaStream_t>(stream));
-        nb_before += (size_t)(L + block_tokens - 1) / block_tokens;
+    for (int s = 0; s < n_seq && rc == HYQ_OK;) {
+        QuantJobs jobs;
+        for (jobs.n = 0; s < n_seq && jobs.n < QUANT_MAX_JOBS; ++s) {
+            const int L = cu[s + 1] - cu[s];
+            QuantJob& j = jobs.job[jobs.n++] = QuantJob{};
+            j.x = reinterpret_cast<const uint4*>(static_cast<const char*>(x) + (size_t)H * D * cu[s] * 2);
+            j.codes = static_cast<uint8_t*>(codes_out) + (size_t)H * row_bytes * cu[s];
+            j.scales = scales_out + (size_t)H * nb_before;
+            j.L = L; j.heads = H; j.format = format;
+            nb_before += (size_t)(L + block_tokens - 1) / block_tokens;
+        }
+        rc = launch_quantize_jobs(jobs, block_tokens, static_cast<cudaStream_t>(stream));
     }
     return rc;
 }

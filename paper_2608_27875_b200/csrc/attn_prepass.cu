@@ -13,15 +13,9 @@
 #include <cuda_fp8.h>
 
 #include "attn_common.cuh"
+#include "quantize.cuh"
 
 namespace hyq {
-
-// two floats -> fp16 pair, saturated to the largest finite fp16: a value row beyond the documented range
-// (|V| < 65504) then degrades the result instead of putting an infinity, and with it NaNs, into the output
-__device__ __forceinline__ uint32_t f16x2_sat(float a, float b) {
-    const __half2 h2 = __floats2half2_rn(fminf(fmaxf(a, -65504.0f), 65504.0f), fminf(fmaxf(b, -65504.0f), 65504.0f));
-    return *reinterpret_cast<const uint32_t*>(&h2);
-}
 
 __global__ void vl_bitmask_kernel(const int32_t* __restrict__ idx, long n_heads, int k, int L, int mask_words,
                                   uint32_t* __restrict__ bits) {
@@ -147,17 +141,6 @@ __device__ __forceinline__ void pre_masks(const TcSeqTable& tab, const PreParams
     }
 }
 
-// four two's-complement nibbles -> four e4m3 bytes (-8 .. 7 are exact): byte permutes look the magnitudes of the
-// non-negative and of the negative codes up by the low three bits, a third spreads the sign bits (32 x 32768 rows of Q and 8 x 32768 of K: the
-// look-up by shifts took 102 us in launches of its own, the whole pre-pass now 88 us, 149 before)
-__device__ __forceinline__ uint32_t nibbles_to_e4m3(uint32_t w) {
-    const uint32_t sel = w & 0x7777u;
-    const uint32_t pos = __byte_perm(0x44403800u, 0x4E4C4A48u, sel), neg = __byte_perm(0x4A4C4E50u, 0x38404448u, sel);
-    uint32_t m;                                               // selector bit 3: the byte's sign, spread over the byte
-    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(m) : "r"(0x80u), "r"(w & 0x8888u));
-    m &= 0x7F7F7F7Fu;                                         // 0x7F where the code is negative
-    return ((pos & ~m) | (neg & m)) | ((m << 1) & 0x80808080u);
-}
 __device__ __forceinline__ void pre_widen(const uint2* __restrict__ in, uint4* __restrict__ out, long n, long e) {
     if (e >= n) return;
     const uint2 w = __ldg(in + e);

@@ -6,29 +6,30 @@
 // shared-memory step across the 4 warps, and the codes leave as 16-byte (8-bit formats) or
 // 8-byte (INT4) vector stores.  The tile is read once and written once: HBM-bound.
 //
+// One launch covers any number of tensors (QuantJob: the Q, K and V of a call, of every prompt of a ragged batch), whose
+// tiles are numbered through; a tile looks its tensor up.  Inside the whole-path call a job may also write what the
+// attention kernel streams - V and V^ = code * scale as fp16, INT4 codes widened to e4m3 bytes - while the tile is in registers.
+//
 // Arithmetic is fp32 with one IEEE rounding per operation (no FMA contraction, no fast-math):
 //   scale = absmax / c ; inv = c / absmax ; code = rint(x * inv) clamped, or e4m3(x * inv).
 #include <cuda_fp8.h>
 
-#include "common.cuh"
+#include "quantize.cuh"
 
 namespace hyq {
 
 constexpr int QUANT_GROUPS = 4;                       // groups of 16 elements per thread
 
-template <int FMT, int BT>
-__global__ void __launch_bounds__(2 * BT)
-quantize_tiles_kernel(const uint4* __restrict__ x, int L, int nb, uint8_t* __restrict__ codes,
-                      float* __restrict__ scales) {
+template <int FMT, int BT, bool EXTRAS>
+__device__ __forceinline__ void quantize_tile(const QuantJob& job, int tile) {     // tile: head * nb + n
     constexpr int QUANT_THREADS = 2 * BT;
-    const long tile = blockIdx.x;                     // (b*H + h) * nb + n
+    const int nb = (job.L + BT - 1) / BT;
     const long head = tile / nb;
-    const int n = (int)(tile - head * nb);
-    const int t0 = n * BT;
-    const int tokens = min(BT, L - t0);
+    const int t0 = (tile - (int)head * nb) * BT;
+    const int tokens = min(BT, job.L - t0);
     const int n_elems = tokens * HYQ_D;
-    const long elem0 = (head * L + t0) * (long)HYQ_D;
-    const uint4* src = x + elem0 / 8;
+    const long elem0 = (head * job.L + t0) * (long)HYQ_D;
+    const uint4* src = job.x + elem0 / 8;
 
     uint4 r[QUANT_GROUPS][2];
     float amax = 0.0f;
@@ -60,16 +61,17 @@ quantize_tiles_kernel(const uint4* __restrict__ x, int L, int nb, uint8_t* __res
 
     constexpr float c = (FMT == HYQ_FMT_INT8) ? 127.0f : (FMT == HYQ_FMT_FP8_E4M3) ? 448.0f : 7.0f;
     const bool dead = !(amax >= 0x1p-100f);
-    const float inv = dead ? 0.0f : __fdiv_rn(c, amax);
-    if (threadIdx.x == 0) scales[tile] = dead ? 0.0f : __fdiv_rn(amax, c);
+    const float inv = dead ? 0.0f : __fdiv_rn(c, amax), scale = dead ? 0.0f : __fdiv_rn(amax, c);
+    if (threadIdx.x == 0) job.scales[tile] = scale;
 
     constexpr int ROW_BYTES = (FMT == HYQ_FMT_INT4) ? HYQ_D / 2 : HYQ_D;
-    uint8_t* dst = codes + (head * L + t0) * (long)ROW_BYTES;
+    uint8_t* dst = job.codes + (head * job.L + t0) * (long)ROW_BYTES;
 #pragma unroll
     for (int gi = 0; gi < QUANT_GROUPS; ++gi) {
         const int e = (threadIdx.x + gi * QUANT_THREADS) * 16;
         if (e >= n_elems) continue;
         const uint32_t* w = reinterpret_cast<const uint32_t*>(&r[gi][0]);
+        uint32_t vh[8];                                  // V^ as fp16 pairs
         if (FMT == HYQ_FMT_FP8_E4M3) {
             uint32_t o[4];
 #pragma unroll
@@ -79,6 +81,14 @@ quantize_tiles_kernel(const uint4* __restrict__ x, int L, int nb, uint8_t* __res
                 const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(y0, y1), __NV_SATFINITE, __NV_E4M3);
                 const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(y2, y3), __NV_SATFINITE, __NV_E4M3);
                 o[c4] = dead ? 0u : (lo | (hi << 16));      // an all-zero tile has all-zero codes (no -0)
+                if (EXTRAS && job.vh16) {
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((o[c4] >> (16 * half)) & 0xFFFFu), __NV_E4M3);
+                        const float2 ff = __half22float2(__half2(hr));
+                        vh[2 * c4 + half] = f16x2_sat(ff.x * scale, ff.y * scale);
+                    }
+                }
             }
             *reinterpret_cast<uint4*>(dst + e) = make_uint4(o[0], o[1], o[2], o[3]);
         } else {
@@ -95,41 +105,95 @@ quantize_tiles_kernel(const uint4* __restrict__ x, int L, int nb, uint8_t* __res
                     o[c4] = (uint32_t)(q[4 * c4] & 0xFF) | ((uint32_t)(q[4 * c4 + 1] & 0xFF) << 8) |
                             ((uint32_t)(q[4 * c4 + 2] & 0xFF) << 16) | ((uint32_t)(q[4 * c4 + 3] & 0xFF) << 24);
                 *reinterpret_cast<uint4*>(dst + e) = make_uint4(o[0], o[1], o[2], o[3]);
+                if (EXTRAS && job.vh16) {
+#pragma unroll
+                    for (int c2 = 0; c2 < 8; ++c2) vh[c2] = f16x2_sat((float)q[2 * c2] * scale, (float)q[2 * c2 + 1] * scale);
+                }
             } else {
                 uint32_t o[2] = {0u, 0u};
 #pragma unroll
                 for (int c16 = 0; c16 < 16; ++c16) o[c16 >> 3] |= (uint32_t)(q[c16] & 0xF) << ((c16 & 7) * 4);
                 *reinterpret_cast<uint2*>(dst + e / 2) = make_uint2(o[0], o[1]);
+                if (EXTRAS && job.wide)
+                    *reinterpret_cast<uint4*>(job.wide + elem0 + e) = make_uint4(nibbles_to_e4m3(o[0]), nibbles_to_e4m3(o[0] >> 16),
+                                                                                 nibbles_to_e4m3(o[1]), nibbles_to_e4m3(o[1] >> 16));
+            }
+        }
+        if (EXTRAS && FMT != HYQ_FMT_INT4 && job.vh16) {
+            uint4* dh = job.vh16 + (elem0 + e) / 8;
+            dh[0] = make_uint4(vh[0], vh[1], vh[2], vh[3]);
+            dh[1] = make_uint4(vh[4], vh[5], vh[6], vh[7]);
+            uint4* dv = job.v16 + (elem0 + e) / 8;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const uint32_t* x = w + 4 * half;
+                dv[half] = make_uint4(f16x2_sat(bf16_lo(x[0]), bf16_hi(x[0])), f16x2_sat(bf16_lo(x[1]), bf16_hi(x[1])),
+                                      f16x2_sat(bf16_lo(x[2]), bf16_hi(x[2])), f16x2_sat(bf16_lo(x[3]), bf16_hi(x[3])));
             }
         }
     }
 }
 
-template <int BT>
-static int launch_quantize_bt(const uint4* xs, long tiles, int L, int nb, int format, uint8_t* cs, float* scales, cudaStream_t st) {
-    const dim3 grid((unsigned)tiles), block(2 * BT);
-    switch (format) {
-        case HYQ_FMT_INT8: quantize_tiles_kernel<HYQ_FMT_INT8, BT><<<grid, block, 0, st>>>(xs, L, nb, cs, scales); break;
-        case HYQ_FMT_FP8_E4M3: quantize_tiles_kernel<HYQ_FMT_FP8_E4M3, BT><<<grid, block, 0, st>>>(xs, L, nb, cs, scales); break;
-        case HYQ_FMT_INT4: quantize_tiles_kernel<HYQ_FMT_INT4, BT><<<grid, block, 0, st>>>(xs, L, nb, cs, scales); break;
-        default: return HYQ_ERR_UNSUPPORTED;
+// (format and extras are compile-time: with all of them in one kernel the registers of the largest cost every tile a
+// fifth; a call with two formats takes two launches)
+template <int FMT, int BT, bool EXTRAS, int MAX>
+__global__ void __launch_bounds__(2 * BT)
+quantize_kernel(const __grid_constant__ QuantList<MAX> jobs) {
+    pdl_wait();
+    int lo = 0, hi = jobs.n - 1;                          // the job whose tiles this one is among
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (jobs.job[mid].tile0 <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
     }
-    return launch_status();
+    quantize_tile<FMT, BT, EXTRAS>(jobs.job[lo], blockIdx.x - jobs.job[lo].tile0);
+}
+
+template <int FMT, int BT, bool EXTRAS>
+static int launch_quantize_bt(const QuantJobs& jobs, long tiles, cudaStream_t st) {
+    if (jobs.n > QUANT_FEW_JOBS)
+        return launch_pdl(quantize_kernel<FMT, BT, EXTRAS, QUANT_MAX_JOBS>, dim3((unsigned)tiles), dim3(2 * BT), 0, st, jobs);
+    QuantList<QUANT_FEW_JOBS> few;
+    few.n = jobs.n;
+    for (int j = 0; j < jobs.n; ++j) few.job[j] = jobs.job[j];
+    return launch_pdl(quantize_kernel<FMT, BT, EXTRAS, QUANT_FEW_JOBS>, dim3((unsigned)tiles), dim3(2 * BT), 0, st, few);
+}
+
+// the jobs of one format
+template <int FMT>
+static int launch_quantize_fmt(const QuantJobs& all, int block_tokens, cudaStream_t st) {
+    QuantJobs jobs;
+    jobs.n = 0;
+    long tiles = 0;
+    bool extras = false;
+    for (int j = 0; j < all.n; ++j) {
+        if (all.job[j].format != FMT) continue;
+        QuantJob& q = jobs.job[jobs.n++] = all.job[j];
+        q.tile0 = (int)tiles;
+        tiles += (long)q.heads * ((q.L + block_tokens - 1) / block_tokens);
+        if (tiles > 0x7fffffffL) return HYQ_ERR_INVALID_ARG;
+        extras |= q.vh16 != nullptr || q.wide != nullptr;
+    }
+    if (tiles == 0) return HYQ_OK;
+#define HYQ_QUANT(BT_) (extras ? launch_quantize_bt<FMT, BT_, true>(jobs, tiles, st) : launch_quantize_bt<FMT, BT_, false>(jobs, tiles, st))
+    return block_tokens == 32 ? HYQ_QUANT(32) : block_tokens == 64 ? HYQ_QUANT(64) : block_tokens == 128 ? HYQ_QUANT(128) : HYQ_ERR_UNSUPPORTED;
+#undef HYQ_QUANT
+}
+
+int launch_quantize_jobs(const QuantJobs& jobs, int block_tokens, cudaStream_t st) {
+    int rc = launch_quantize_fmt<HYQ_FMT_INT8>(jobs, block_tokens, st);
+    if (rc == HYQ_OK) rc = launch_quantize_fmt<HYQ_FMT_INT4>(jobs, block_tokens, st);
+    if (rc == HYQ_OK) rc = launch_quantize_fmt<HYQ_FMT_FP8_E4M3>(jobs, block_tokens, st);
+    return rc;
 }
 
 int launch_quantize(const void* x, long n_heads, int L, int block_tokens, int format, void* codes, float* scales, cudaStream_t st) {
-    const int nb = (L + block_tokens - 1) / block_tokens;
-    const long tiles = n_heads * nb;
-    if (tiles <= 0) return HYQ_OK;
-    if (tiles > 0x7fffffffL) return HYQ_ERR_INVALID_ARG;
-    const uint4* xs = static_cast<const uint4*>(x);
-    uint8_t* cs = static_cast<uint8_t*>(codes);
-    switch (block_tokens) {
-        case 32: return launch_quantize_bt<32>(xs, tiles, L, nb, format, cs, scales, st);
-        case 64: return launch_quantize_bt<64>(xs, tiles, L, nb, format, cs, scales, st);
-        case 128: return launch_quantize_bt<128>(xs, tiles, L, nb, format, cs, scales, st);
-        default: return HYQ_ERR_UNSUPPORTED;
-    }
+    if (n_heads > 0x7fffffffL) return HYQ_ERR_INVALID_ARG;
+    QuantJobs jobs;
+    jobs.n = 1;
+    QuantJob& j = jobs.job[0] = QuantJob{};
+    j.x = static_cast<const uint4*>(x); j.codes = static_cast<uint8_t*>(codes); j.scales = scales;
+    j.L = L; j.heads = (int)n_heads; j.format = format;
+    return launch_quantize_jobs(jobs, block_tokens, st);
 }
 
 }  // namespace hyq
