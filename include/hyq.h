@@ -269,6 +269,46 @@ int hyq_hybrid_attention_prefill_varlen_workspace(const hyq_attn_args* args, int
                                                   const int32_t* k_per_seq /* host */, size_t* bytes /* host, out */);
 
 /* ---------------------------------------------------------------------------------------------
+ * hyq_hybrid_prefill - Algorithm 2 in one call: hyq_select_vertical, hyq_quantize_blocks of Q, K and V and
+ * hyq_hybrid_attention_prefill over n_seq whole prompts, with the results those calls (the *_varlen calls for n_seq > 1)
+ * write, bit for bit.  The stages hand their intermediate layouts to one another, so the call reads V and the codes once
+ * less and takes fewer launches than the stages one by one; the prompts' Q, K and V are read where they lie.
+ *
+ *   lengths, k_per_seq, q, k_, v: HOST arrays of n_seq entries (q, k_, v: device pointers to contiguous
+ *   [B,Hq,L_s,D] / [B,Hkv,L_s,D] bf16, 16-byte aligned).  B > 1 only with n_seq == 1.
+ *   idx, codes, scales, out, lse: packed as the *_varlen calls pack them ([B,H,...] for n_seq == 1).
+ *   Everything else, and the errors, as in the single calls; workspace: hyq_hybrid_prefill_workspace bytes.
+ * ------------------------------------------------------------------------------------------- */
+typedef struct {
+  uint32_t struct_size;
+  int32_t n_seq, B, Hq, Hkv, D;
+  int32_t window, n_tail, block_tokens;
+  int32_t q_format, k_format, v_format;
+  int32_t out_dtype;                 /* 0 = bf16, 1 = fp32 */
+  float softmax_scale;               /* 0 => 1/sqrt(D) */
+  const int32_t* lengths;
+  const int32_t* k_per_seq;
+  const void* const* q;
+  const void* const* k_;
+  const void* const* v;
+  int32_t* idx;
+  void* q_codes;
+  void* k_codes;
+  void* v_codes;
+  float* q_scales;
+  float* k_scales;
+  float* v_scales;
+  void* out;
+  float* lse;                        /* optional */
+  int32_t* status_word;              /* optional */
+  void* workspace;
+  size_t workspace_bytes;
+} hyq_prefill_args;
+
+int hyq_hybrid_prefill_workspace(const hyq_prefill_args* args, size_t* bytes /* host, out */);
+int hyq_hybrid_prefill(const hyq_prefill_args* args, void* stream);
+
+/* ---------------------------------------------------------------------------------------------
  * hyq_test_set_attention_hooks - test hook (the paper has no counterpart): exercises the tensor-core
  * kernel's bounded-wait unwind without faulting anything.  Process-wide, not thread-safe, meant for tests only.
  *   wait_limit_clocks    SM clocks a single device-side barrier wait may take before the kernel gives up

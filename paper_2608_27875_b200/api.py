@@ -21,7 +21,8 @@ EXPORTS = ("hyq_status_string", "hyq_version", "hyq_paper_k", "hyq_select_vertic
            "hyq_select_vertical", "hyq_select_vertical_static", "hyq_select_vertical_mass_workspace",
            "hyq_select_vertical_mass", "hyq_quantize_blocks", "hyq_hybrid_attention_prefill_workspace",
            "hyq_hybrid_attention_prefill", "hyq_test_set_attention_hooks", "hyq_test_read_attention_restarts", "hyq_select_vertical_varlen",
-           "hyq_quantize_blocks_varlen", "hyq_hybrid_attention_prefill_varlen", "hyq_hybrid_attention_prefill_varlen_workspace")
+           "hyq_quantize_blocks_varlen", "hyq_hybrid_attention_prefill_varlen", "hyq_hybrid_attention_prefill_varlen_workspace",
+           "hyq_hybrid_prefill_workspace", "hyq_hybrid_prefill")
 
 
 class HyqError(RuntimeError):
@@ -41,6 +42,17 @@ class AttnArgs(ctypes.Structure):
                                                 "workspace")] +
                 [("workspace_bytes", ctypes.c_size_t), ("ev_kernel_start", ctypes.c_void_p),
                  ("ev_kernel_stop", ctypes.c_void_p), ("Lq", ctypes.c_int32), ("window_mode", ctypes.c_int32)])
+
+
+class PrefillArgs(ctypes.Structure):
+    """Mirror of ``hyq_prefill_args``."""
+    _fields_ = ([("struct_size", ctypes.c_uint32)] +
+                [(n, ctypes.c_int32) for n in ("n_seq", "B", "Hq", "Hkv", "D", "window", "n_tail", "block_tokens", "q_format",
+                                               "k_format", "v_format", "out_dtype")] +
+                [("softmax_scale", ctypes.c_float)] +
+                [(n, ctypes.c_void_p) for n in ("lengths", "k_per_seq", "q", "k_", "v", "idx", "q_codes", "k_codes", "v_codes",
+                                                "q_scales", "k_scales", "v_scales", "out", "lse", "status_word", "workspace")] +
+                [("workspace_bytes", ctypes.c_size_t)])
 
 
 _lib = None
@@ -80,6 +92,8 @@ def lib() -> ctypes.CDLL:
         L.hyq_hybrid_attention_prefill_varlen.argtypes = [ctypes.POINTER(AttnArgs), ctypes.c_int, i32p, i32p, ctypes.c_void_p]
         L.hyq_hybrid_attention_prefill_varlen_workspace.argtypes = [ctypes.POINTER(AttnArgs), ctypes.c_int, i32p, i32p,
                                                                     ctypes.POINTER(ctypes.c_size_t)]
+        L.hyq_hybrid_prefill_workspace.argtypes = [ctypes.POINTER(PrefillArgs), ctypes.POINTER(ctypes.c_size_t)]
+        L.hyq_hybrid_prefill.argtypes = [ctypes.POINTER(PrefillArgs), ctypes.c_void_p]
         _lib = L
     return _lib
 
@@ -94,7 +108,8 @@ def _check(code: int, where: str):
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # the current stream's handle (torch.cuda.current_stream() builds a Stream object for it: 2-3 us a call)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
@@ -268,16 +283,54 @@ def hyq_hybrid_attention_prefill(q, k, v, q_codes, k_codes, v_codes, q_scales, k
     return out
 
 
+def _prefill(qs, ks, vs, B, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens, out_dtype, dev, status=None):
+    """hyq_hybrid_prefill on prompts where they lie; returns the packed results: idx, codes, scales (three each), out."""
+    n, D, total = len(lens), 128, sum(lens)
+    nb = sum([-(-L_ // block_tokens) for L_ in lens])
+    empty = torch.empty
+    idx = empty(B * Hq * sum(k_per_seq), dtype=torch.int32, device=dev)
+    codes = [empty(B * H * total * code_row_bytes(f, D), dtype=torch.uint8, device=dev) for H, f in zip((Hq, Hkv, Hkv), fmts)]
+    scales = [empty(B * H * nb, dtype=torch.float32, device=dev) for H in (Hq, Hkv, Hkv)]
+    out = empty(B * Hq * total * D, dtype=out_dtype, device=dev)
+    a = PrefillArgs(ctypes.sizeof(PrefillArgs), n, B, Hq, Hkv, D, window, 0, block_tokens, *fmts,
+                    1 if out_dtype == torch.float32 else 0, 0.0)
+    host = [_i32(lens), _i32(k_per_seq)] + [(ctypes.c_void_p * n)(*[t.data_ptr() for t in ts]) for ts in (qs, ks, vs)]   # (outlives the call)
+    a.lengths, a.k_per_seq, a.q, a.k_, a.v = (ctypes.addressof(h) for h in host)
+    a.idx, a.out = idx.data_ptr() or None, out.data_ptr()
+    a.q_codes, a.k_codes, a.v_codes = (c.data_ptr() for c in codes)
+    a.q_scales, a.k_scales, a.v_scales = (c.data_ptr() for c in scales)
+    a.status_word = None if status is None else status.data_ptr()
+    need = ctypes.c_size_t(0)
+    _check(lib().hyq_hybrid_prefill_workspace(ctypes.byref(a), ctypes.byref(need)), "hyq_hybrid_prefill_workspace")
+    ws = empty(max(need.value, 16), dtype=torch.uint8, device=dev)
+    a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+    _check(lib().hyq_hybrid_prefill(ctypes.byref(a), _stream()), "hyq_hybrid_prefill")
+    return idx, codes, scales, out
+
+
 def hybrid_prefill(q, k, v, window: int, k_sel: int, fmts=(FMT_INT8, FMT_INT8, FMT_INT8), impl: int = IMPL_AUTO,
                    out_dtype=torch.float32):
     """The whole path on device tensors: select -> quantize Q, K, V -> fused attention."""
-    idx = hyq_select_vertical(q, k, window, k_sel)
-    qc, qs = hyq_quantize_blocks(q, fmts[0])
-    kc, ks = hyq_quantize_blocks(k, fmts[1])
-    vc, vs = hyq_quantize_blocks(v, fmts[2])
-    out = hyq_hybrid_attention_prefill(q, k, v, qc, kc, vc, qs, ks, vs, fmts, idx, window, impl=impl,
-                                       out_dtype=out_dtype)
-    return dict(idx=idx, q_codes=qc, k_codes=kc, v_codes=vc, q_scales=qs, k_scales=ks, v_scales=vs, out=out)
+    if impl == IMPL_SIMT or q.shape[2] != k.shape[2]:        # stage by stage
+        idx = hyq_select_vertical(q, k, window, k_sel)
+        qc, qs = hyq_quantize_blocks(q, fmts[0])
+        kc, ks = hyq_quantize_blocks(k, fmts[1])
+        vc, vs = hyq_quantize_blocks(v, fmts[2])
+        out = hyq_hybrid_attention_prefill(q, k, v, qc, kc, vc, qs, ks, vs, fmts, idx, window, impl=impl,
+                                           out_dtype=out_dtype)
+        return dict(idx=idx, q_codes=qc, k_codes=kc, v_codes=vc, q_scales=qs, k_scales=ks, v_scales=vs, out=out)
+    for t, n in ((q, "q"), (k, "k"), (v, "v")):
+        _dev(t, torch.bfloat16, n)
+    B, Hq, L, D = q.shape
+    Hkv = k.shape[1]
+    if D != 128:
+        raise HyqError(2, "hybrid_prefill")
+    k_eff = k_sel if L - window > 0 else 0
+    idx, c, s, out = _prefill((q,), (k,), (v,), B, Hq, Hkv, (L,), window, (k_eff,), fmts, 64, out_dtype, q.device)
+    nb = -(-L // 64)
+    return dict(idx=idx.view(B, Hq, k_eff), q_codes=c[0].view(B, Hq, L, -1), k_codes=c[1].view(B, Hkv, L, -1),
+                v_codes=c[2].view(B, Hkv, L, -1), q_scales=s[0].view(B, Hq, nb), k_scales=s[1].view(B, Hkv, nb),
+                v_scales=s[2].view(B, Hkv, nb), out=out.view(B, Hq, L, D))
 
 
 # ---- ragged batches --------------------------------------------------------------------------------------------
@@ -297,51 +350,28 @@ def pack_sequences(seqs) -> tuple[torch.Tensor, list[int]]:
 def hybrid_prefill_varlen(qs, ks, vs, window: int, k_per_seq, fmts=(FMT_INT8, FMT_INT8, FMT_INT8), block_tokens: int = 64,
                           out_dtype=torch.float32):
     """The whole path over a ragged batch: ``qs[s]`` is [Hq, L_s, D], ``ks[s]`` / ``vs[s]`` are [Hkv, L_s, D] (bf16,
-    CUDA).  Packs the prompts, runs the three *_varlen calls and returns per-sequence views of the results:
+    CUDA).  Runs hyq_hybrid_prefill on the prompts where they lie and returns per-sequence views of the packed results:
     a list of dicts with idx [Hq, k_s], codes, scales and out [Hq, L_s, D]."""
     n = len(qs)
+    # (a prompt that is a view of the caller's buffer may be strided or lie off a 16-byte boundary: copied then)
+    qs, ks, vs = ([t if t.is_contiguous() and t.data_ptr() % 16 == 0 else t.clone(memory_format=torch.contiguous_format) for t in ts]
+                  for ts in (qs, ks, vs))
+    for ts in (qs, ks, vs):
+        for t in ts:
+            _dev(t, torch.bfloat16, "q, k, v")
     Hq, _, D = qs[0].shape
     Hkv = ks[0].shape[0]
+    if D != 128:
+        raise HyqError(2, "hybrid_prefill_varlen")
     dev = qs[0].device
-    qp, cu = pack_sequences(qs)
-    kp, _ = pack_sequences(ks)
-    vp, _ = pack_sequences(vs)
-    lens = [cu[s + 1] - cu[s] for s in range(n)]
-    k_per_seq = [int(k) if lens[s] - window > 0 else 0 for s, k in enumerate(k_per_seq)]
-    cu_c, k_c = _i32(cu), _i32(k_per_seq)
-    total, nbs = cu[-1], [-(-L_ // block_tokens) for L_ in lens]
-    idx = torch.empty(max(1, Hq * sum(k_per_seq)), dtype=torch.int32, device=dev)
-    need = max([hyq_select_vertical_workspace(1, Hq, Hkv, L_, L_, D, window, k_) for L_, k_ in zip(lens, k_per_seq)] + [16])
-    ws = torch.empty(need, dtype=torch.uint8, device=dev)
-    _check(lib().hyq_select_vertical_varlen(qp.data_ptr(), kp.data_ptr(), n, cu_c, Hq, Hkv, D, window, 0, k_c, idx.data_ptr(),
-                                            ws.data_ptr(), ws.numel(), _stream()), "hyq_select_vertical_varlen")
-    codes, scales = [], []
-    for x, H, f in ((qp, Hq, fmts[0]), (kp, Hkv, fmts[1]), (vp, Hkv, fmts[2])):
-        c = torch.empty(H * total * code_row_bytes(f, D), dtype=torch.uint8, device=dev)
-        sc = torch.empty(H * sum(nbs), dtype=torch.float32, device=dev)
-        _check(lib().hyq_quantize_blocks_varlen(x.data_ptr(), n, cu_c, H, D, block_tokens, f, c.data_ptr(), sc.data_ptr(), _stream()),
-               "hyq_quantize_blocks_varlen")
-        codes.append(c)
-        scales.append(sc)
-    out = torch.empty(Hq * total * D, dtype=out_dtype, device=dev)
+    lens = [t.shape[1] for t in qs]
+    cu = [0]
+    for L_ in lens:
+        cu.append(cu[-1] + L_)
+    k_per_seq = [int(k) if L_ - window > 0 else 0 for L_, k in zip(lens, k_per_seq)]
+    nbs = [-(-L_ // block_tokens) for L_ in lens]
     status = torch.zeros(1, dtype=torch.int32, device=dev)
-    a = AttnArgs()
-    a.struct_size = ctypes.sizeof(AttnArgs)
-    a.B, a.Hq, a.Hkv, a.L, a.D, a.Lq = 1, Hq, Hkv, max(lens), D, 0
-    a.window, a.k, a.block_tokens = window, max(k_per_seq), block_tokens
-    a.q_format, a.k_format, a.v_format = fmts
-    a.out_dtype, a.impl, a.softmax_scale, a.window_mode = (1 if out_dtype == torch.float32 else 0), IMPL_AUTO, 0.0, WINDOW_SLIDING
-    a.q, a.k_, a.v = qp.data_ptr(), kp.data_ptr(), vp.data_ptr()
-    a.q_codes, a.k_codes, a.v_codes = (c.data_ptr() for c in codes)
-    a.q_scales, a.k_scales, a.v_scales = (s_.data_ptr() for s_ in scales)
-    a.vl_idx, a.out, a.status_word = idx.data_ptr(), out.data_ptr(), status.data_ptr()
-    a.k = k_per_seq[lens.index(max(lens))]
-    need_a = ctypes.c_size_t(0)
-    _check(lib().hyq_hybrid_attention_prefill_varlen_workspace(ctypes.byref(a), n, cu_c, k_c, ctypes.byref(need_a)),
-           "hyq_hybrid_attention_prefill_varlen_workspace")
-    wsa = torch.empty(max(16, need_a.value), dtype=torch.uint8, device=dev)
-    a.workspace, a.workspace_bytes = wsa.data_ptr(), wsa.numel()
-    _check(lib().hyq_hybrid_attention_prefill_varlen(ctypes.byref(a), n, cu_c, k_c, _stream()), "hyq_hybrid_attention_prefill_varlen")
+    idx, codes, scales, out = _prefill(qs, ks, vs, 1, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens, out_dtype, dev, status)
     res, ko, no = [], 0, 0
     for s in range(n):
         L_, k_, nb = lens[s], k_per_seq[s], nbs[s]
@@ -354,7 +384,7 @@ def hybrid_prefill_varlen(qs, ks, vs, window: int, k_per_seq, fmts=(FMT_INT8, FM
             v_scales=scales[2][Hkv * no:Hkv * (no + nb)].view(Hkv, nb), out=view(out, Hq, D)))
         ko += k_
         no += nb
-    torch.cuda.synchronize()
-    if int(status.item()) != 0:
-        raise HyqError(int(status.item()), "hyq_hybrid_attention_prefill_varlen (device)")
+    code = int(status.item())                                # (waits for the results)
+    if code != 0:
+        raise HyqError(code, "hybrid_prefill_varlen (device)")
     return res

@@ -8,10 +8,8 @@
 namespace hyq {
 size_t attn_simt_workspace_bytes(const hyq_attn_args& a);
 int launch_attn_simt(const hyq_attn_args& a, float alpha, cudaStream_t st);
-int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, float alpha, cudaStream_t st);
 int tc_restarts(unsigned long long* count, bool reset);
 namespace tcbt {
-int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, float alpha, cudaStream_t st);     // 32- and 128-token quantization blocks
 int tc_restarts(unsigned long long* count, bool reset);
 }
 }  // namespace hyq
@@ -184,9 +182,9 @@ static int check_attn(const hyq_attn_args* a, bool need_pointers) {
 static bool use_simt(const hyq_attn_args* a) { return a->impl == HYQ_IMPL_SIMT; }
 
 // the tensor-core path of a planned call (arguments checked)
-static int launch_planned(const hyq_attn_args& a, const TcPlan& plan, float alpha, cudaStream_t st) {
+static int launch_planned(const hyq_attn_args& a, const TcPlan& plan, const TcSources* src, float alpha, cudaStream_t st) {
     if (!a.workspace || a.workspace_bytes < plan.w.total) return HYQ_ERR_WORKSPACE;
-    return a.block_tokens == HYQ_BLOCK_TOKENS ? launch_attn_tc(a, plan, alpha, st) : tcbt::launch_attn_tc(a, plan, alpha, st);
+    return a.block_tokens == HYQ_BLOCK_TOKENS ? launch_attn_tc(a, plan, src, alpha, st) : tcbt::launch_attn_tc(a, plan, src, alpha, st);
 }
 
 int hyq_hybrid_attention_prefill_workspace(const hyq_attn_args* args, size_t* bytes) {
@@ -215,7 +213,7 @@ int hyq_hybrid_attention_prefill(const hyq_attn_args* args, void* stream) {
     }
     TcPlan plan;
     if (!tc_plain_plan(*args, plan)) return HYQ_ERR_UNSUPPORTED;
-    return launch_planned(*args, plan, alpha, st);
+    return launch_planned(*args, plan, nullptr, alpha, st);
 }
 
 // ---- ragged batches: the plain calls, sequence by sequence, on packed buffers ---------------------------------
@@ -394,7 +392,7 @@ int hyq_hybrid_attention_prefill_varlen(const hyq_attn_args* args, int n_seq, co
             rc = launch_attn_simt(a, alpha, static_cast<cudaStream_t>(stream));
         } else {
             n = next_group(*args, s, n_seq, cu, k_per_seq, args->workspace_bytes, plan);
-            rc = n > 0 ? launch_planned(a, plan, alpha, static_cast<cudaStream_t>(stream)) : HYQ_ERR_WORKSPACE;
+            rc = n > 0 ? launch_planned(a, plan, nullptr, alpha, static_cast<cudaStream_t>(stream)) : HYQ_ERR_WORKSPACE;
         }
         for (int i = s; i < s + n; ++i) {
             nb_before += (size_t)(cu[i + 1] - cu[i] + bt - 1) / bt;
@@ -402,6 +400,159 @@ int hyq_hybrid_attention_prefill_varlen(const hyq_attn_args* args, int n_seq, co
         }
     }
     return rc;
+}
+
+// ---- the whole path in one call ---------------------------------------------------------------------------------
+// the attention arguments of the sequences from s on (offsets in tokens / indices / blocks of the packed results)
+static hyq_attn_args attn_args_of(const hyq_prefill_args& a, int s, size_t t0, size_t k_before, size_t nb_before) {
+    hyq_attn_args x{};
+    x.struct_size = sizeof(x);
+    x.B = a.B; x.Hq = a.Hq; x.Hkv = a.Hkv; x.L = a.lengths[s]; x.D = a.D;
+    x.window = a.window; x.k = a.k_per_seq[s]; x.block_tokens = a.block_tokens;
+    x.q_format = a.q_format; x.k_format = a.k_format; x.v_format = a.v_format;
+    x.out_dtype = a.out_dtype; x.softmax_scale = a.softmax_scale;
+    x.q = a.q ? a.q[s] : nullptr; x.k_ = a.k_ ? a.k_[s] : nullptr; x.v = a.v ? a.v[s] : nullptr;
+    auto row = [](int fmt) -> size_t { return fmt == HYQ_FMT_INT4 ? HYQ_D / 2 : HYQ_D; };
+    auto at = [](const void* base, size_t bytes) -> const void* { return base ? static_cast<const char*>(base) + bytes : nullptr; };
+    x.q_codes = at(a.q_codes, a.Hq * row(a.q_format) * t0);
+    x.k_codes = at(a.k_codes, a.Hkv * row(a.k_format) * t0);
+    x.v_codes = at(a.v_codes, a.Hkv * row(a.v_format) * t0);
+    x.q_scales = a.q_scales ? a.q_scales + a.Hq * nb_before : nullptr;
+    x.k_scales = a.k_scales ? a.k_scales + a.Hkv * nb_before : nullptr;
+    x.v_scales = a.v_scales ? a.v_scales + a.Hkv * nb_before : nullptr;
+    x.vl_idx = a.idx ? a.idx + a.Hq * k_before : nullptr;
+    x.out = const_cast<void*>(at(a.out, (size_t)a.Hq * HYQ_D * t0 * (a.out_dtype == 1 ? 4 : 2)));
+    x.lse = a.lse ? a.lse + a.Hq * t0 : nullptr;
+    x.status_word = a.status_word;
+    x.workspace = a.workspace; x.workspace_bytes = a.workspace_bytes;
+    return x;
+}
+
+static int check_prefill(const hyq_prefill_args* a, bool need_pointers) {
+    if (!a || a->struct_size != sizeof(hyq_prefill_args) || a->n_seq <= 0 || !a->lengths || !a->k_per_seq) return HYQ_ERR_INVALID_ARG;
+    if (a->B <= 0 || (a->B > 1 && a->n_seq > 1)) return HYQ_ERR_INVALID_ARG;
+    if (need_pointers && (!a->q || !a->k_ || !a->v)) return HYQ_ERR_INVALID_ARG;
+    if (!block_tokens_ok(a->block_tokens)) return HYQ_ERR_UNSUPPORTED;
+    if (need_pointers && ((reinterpret_cast<uintptr_t>(a->idx) | reinterpret_cast<uintptr_t>(a->q_scales) |
+                           reinterpret_cast<uintptr_t>(a->k_scales) | reinterpret_cast<uintptr_t>(a->v_scales)) & 3u))
+        return HYQ_ERR_ALIGNMENT;
+    size_t t0 = 0, k0 = 0, nb0 = 0;
+    for (int s = 0; s < a->n_seq; ++s) {
+        const int L = a->lengths[s];
+        int rc = check_select(nullptr, nullptr, a->B, a->Hq, a->Hkv, L, L, a->D, a->window, a->n_tail, a->k_per_seq[s]);
+        if (rc != HYQ_OK) return rc;
+        if (a->k_per_seq[s] > (L - a->window > 0 ? L - a->window : 0)) return HYQ_ERR_INVALID_ARG;
+        const hyq_attn_args x = attn_args_of(*a, s, t0, k0, nb0);
+        rc = check_attn(&x, need_pointers);
+        if (rc != HYQ_OK) return rc;
+        t0 += (size_t)L; k0 += (size_t)a->k_per_seq[s]; nb0 += (size_t)((L + a->block_tokens - 1) / a->block_tokens);
+    }
+    return HYQ_OK;
+}
+
+// what one round of launches needs: sequences [s, s + n) of a call
+struct PrefillGroup {
+    TcPlan plan;
+    SelTable sel;
+    size_t sel_at, total;
+};
+static bool plan_prefill(const hyq_prefill_args& a, int s, int n, PrefillGroup& g) {
+    const hyq_attn_args x = attn_args_of(a, s, 0, 0, 0);
+    TcSeq seq[TC_MAX_SEQ];
+    size_t t0 = 0, k0 = 0, nb0 = 0;
+    g.sel.n_seq = n; g.sel.heads = a.B * a.Hq; g.sel.g = a.Hq / a.Hkv;
+    for (int i = 0; i < n; ++i) {
+        const int L = a.lengths[s + i], k = a.k_per_seq[s + i];
+        seq[i] = tc_ragged_seq(x, L, k, t0, k0, nb0);
+        SelSeq& q = g.sel.seq[i] = SelSeq{};
+        q.q = a.q ? static_cast<const __nv_bfloat16*>(a.q[s + i]) : nullptr;
+        q.k = a.k_ ? static_cast<const __nv_bfloat16*>(a.k_[s + i]) : nullptr;
+        q.Lq = q.Lk = L; q.t = a.n_tail ? a.n_tail : (a.window < L ? a.window : L);
+        q.P = k > 0 && L > a.window ? L - a.window : 0;
+        q.k_sel = k; q.idx0 = (long)a.Hq * (long)k0;
+        t0 += (size_t)L; k0 += (size_t)k; nb0 += (size_t)((L + a.block_tokens - 1) / a.block_tokens);
+    }
+    if (!tc_make_plan(x, seq, n, a.B * a.Hq, a.Hq / a.Hkv, g.plan)) return false;
+    g.sel_at = align_up(g.plan.w.total, 256);
+    g.total = g.sel_at + select_scratch_bytes(g.sel);
+    return true;
+}
+// as many sequences from s on as one round of launches within `bytes` of workspace can hold (halved until it fits; 0: not one)
+static int next_prefill_group(const hyq_prefill_args& a, int s, size_t bytes, PrefillGroup& g) {
+    int n = a.n_seq - s < TC_MAX_SEQ ? a.n_seq - s : TC_MAX_SEQ;
+    while (!(plan_prefill(a, s, n, g) && g.total <= bytes)) {
+        if (n == 1) return 0;
+        n = (n + 1) / 2;
+    }
+    return n;
+}
+
+int hyq_hybrid_prefill_workspace(const hyq_prefill_args* args, size_t* bytes) {
+    if (!bytes) return HYQ_ERR_INVALID_ARG;
+    const int rc = check_prefill(args, false);
+    if (rc != HYQ_OK) return rc;
+    size_t most = 0;
+    PrefillGroup g;
+    for (int s = 0, n; s < args->n_seq; s += n) {
+        n = next_prefill_group(*args, s, (size_t)-1, g);
+        if (n == 0) return HYQ_ERR_UNSUPPORTED;
+        most = g.total > most ? g.total : most;
+    }
+    *bytes = most;
+    return HYQ_OK;
+}
+
+int hyq_hybrid_prefill(const hyq_prefill_args* args, void* stream) {
+    int rc = check_prefill(args, true);
+    if (rc != HYQ_OK) return rc;
+    const hyq_prefill_args& a = *args;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    PrefillGroup g;
+    if (!a.workspace) return HYQ_ERR_INVALID_ARG;
+    if (a.n_seq > 1)                                            // (one sequence: its only group below says so)
+        for (int s = 0; s < a.n_seq; ++s)
+            if (!plan_prefill(a, s, 1, g) || g.total > a.workspace_bytes) return HYQ_ERR_WORKSPACE;
+    const float alpha = a.softmax_scale != 0.0f ? a.softmax_scale : 1.0f / sqrtf((float)a.D);
+    size_t t0 = 0, k0 = 0, nb0 = 0;
+    for (int s = 0, n; s < a.n_seq; s += n) {
+        n = next_prefill_group(a, s, a.workspace_bytes, g);
+        if (n == 0) return HYQ_ERR_WORKSPACE;
+        const hyq_attn_args x = attn_args_of(a, s, t0, k0, nb0);
+        char* base = static_cast<char*>(a.workspace);
+        QuantJobs jobs;
+        TcSources src;
+        jobs.n = 3 * n;
+        size_t tt = 0, nb = 0;
+        for (int i = 0; i < n; ++i) {
+            const int L = a.lengths[s + i];
+            src.q[i] = a.q[s + i]; src.k[i] = a.k_[s + i]; src.v[i] = a.v[s + i];
+            auto job = [&](int which, const void* data, int H, int format, const void* codes, const float* scales) -> QuantJob& {
+                QuantJob& j = jobs.job[3 * i + which] = QuantJob{};
+                const size_t row = format == HYQ_FMT_INT4 ? HYQ_D / 2 : HYQ_D;
+                j.x = static_cast<const uint4*>(data); j.L = L; j.heads = a.B * H; j.format = format;
+                j.codes = static_cast<uint8_t*>(const_cast<void*>(codes)) + H * row * tt;
+                j.scales = const_cast<float*>(scales) + H * nb;
+                return j;
+            };
+            QuantJob& jq = job(0, a.q[s + i], a.Hq, a.q_format, x.q_codes, x.q_scales);
+            QuantJob& jk = job(1, a.k_[s + i], a.Hkv, a.k_format, x.k_codes, x.k_scales);
+            QuantJob& jv = job(2, a.v[s + i], a.Hkv, a.v_format, x.v_codes, x.v_scales);
+            if (a.q_format == HYQ_FMT_INT4) {
+                jq.wide = reinterpret_cast<uint8_t*>(base + g.plan.w.q8) + a.Hq * tt * HYQ_D;
+                jk.wide = reinterpret_cast<uint8_t*>(base + g.plan.w.k8) + a.Hkv * tt * HYQ_D;
+            }
+            jv.v16 = reinterpret_cast<uint4*>(base + g.plan.w.v16) + a.Hkv * tt * (HYQ_D / 8);
+            jv.vh16 = reinterpret_cast<uint4*>(base + g.plan.w.vh16) + a.Hkv * tt * (HYQ_D / 8);
+            tt += (size_t)L; nb += (size_t)((L + a.block_tokens - 1) / a.block_tokens);
+            k0 += (size_t)a.k_per_seq[s + i];
+        }
+        rc = launch_quantize_jobs(jobs, a.block_tokens, st);
+        if (rc == HYQ_OK) rc = launch_select_table(g.sel, const_cast<int32_t*>(x.vl_idx), base + g.sel_at, st);
+        if (rc == HYQ_OK) rc = launch_planned(x, g.plan, &src, alpha, st);
+        if (rc != HYQ_OK) return rc;
+        t0 += tt; nb0 += nb;
+    }
+    return HYQ_OK;
 }
 
 }  // extern "C"

@@ -25,6 +25,7 @@ struct TcSeq {
     int levels;                             // units per head
     int split;                              // CTAs that share the sequence's units tile by tile (0: one CTA per unit)
     int cta0, slot0;                        // split: first CTA behind the unsplit units, first slot for partial results ...
+    int src;                                // the sequence's number in the caller's order
     int tiles;                              // ... and key tiles of all its units together (as tc_unit_tiles counts them)
 };
 
@@ -89,7 +90,18 @@ bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads
 bool tc_plain_plan(const hyq_attn_args& a, TcPlan& plan);
 // one sequence of a ragged call as tc_make_plan takes it; Hq / Hkv times the tokens, vertical keys and blocks before it
 TcSeq tc_ragged_seq(const hyq_attn_args& a, int L, int k, size_t tokens_before, size_t k_before, size_t nb_before);
-int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, cudaStream_t st);
+
+// A call that quantizes and attends in one: Q, K, V per sequence wherever they lie (in the caller's order), and the pre-pass's
+// fp16 values and widened codes already written by the quantizer.
+struct TcSources {
+    const void *q[TC_MAX_SEQ], *k[TC_MAX_SEQ], *v[TC_MAX_SEQ];
+};
+int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, const TcSources* src, cudaStream_t st);
+// the whole tensor-core attention of a planned call (64-token quantization blocks / the others); src: see there, may be null
+int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, const TcSources* src, float alpha, cudaStream_t st);
+namespace tcbt {
+int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, const TcSources* src, float alpha, cudaStream_t st);
+}
 
 // Test hooks of the tensor-core kernel (hyq_test_set_attention_hooks): the clock limit of a single barrier wait
 // (0: the default of about two seconds) and the walk position whose K/V load the producer leaves out (-1: none).

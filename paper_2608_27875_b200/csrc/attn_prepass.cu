@@ -34,7 +34,8 @@ struct PreParams {
     unsigned v_end, gather_end, mask_end, k_end, q_end;      // block ranges of the pieces
     int mask_blocks[TC_MAX_SEQ];                             // mask blocks before each sequence
     int bt_shift;                                      // log2(tokens per quantization block)
-    const uint4 *k, *v;                                      // bf16 rows of 16 x 16 bytes
+    const uint4* v;                                          // bf16 rows of 16 x 16 bytes
+    const uint4 *k_seq[TC_MAX_SEQ], *v_seq[TC_MAX_SEQ];      // the same per sequence
     const uint2* v_codes;
     const float* v_scales;
     const int32_t* vl_idx;
@@ -92,11 +93,12 @@ __device__ __forceinline__ void pre_values(const TcSeqTable& tab, const PreParam
 __device__ __forceinline__ void pre_gather(const TcSeqTable& tab, const PreParams& p, long e) {
     const long row = e >> 4;
     if (row >= tab.vl_rows) return;
-    const TcSeq& sq = tab.seq[HYQ_SEQ_OF(tab, vl_row0, tab.heads * tab.seq[s_].k, row)];
+    const int s = HYQ_SEQ_OF(tab, vl_row0, tab.heads * tab.seq[s_].k, row);
+    const TcSeq& sq = tab.seq[s];
     const int head = ((int)row - sq.vl_row0) / sq.k;
     const int j = min(max(__ldg(p.vl_idx + row), 0), sq.L - 1);
-    const long src = ((long)sq.kv_row0 + (long)(head / tab.g) * sq.L + j) * 16 + (e & 15);
-    const uint4 kw = __ldg(p.k + src), vw = __ldg(p.v + src);
+    const long src = ((long)(head / tab.g) * sq.L + j) * 16 + (e & 15);
+    const uint4 kw = __ldg(p.k_seq[s] + src), vw = __ldg(p.v_seq[s] + src);
     p.kvl[e] = kw;
     p.vvl[e] = make_uint4(f16x2_sat(bf16_lo(vw.x), bf16_hi(vw.x)), f16x2_sat(bf16_lo(vw.y), bf16_hi(vw.y)),
                           f16x2_sat(bf16_lo(vw.z), bf16_hi(vw.z)), f16x2_sat(bf16_lo(vw.w), bf16_hi(vw.w)));
@@ -208,6 +210,7 @@ bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads
     long kv_rows = 0, vl_rows = 0, q_rows = 0, words = 0, units = 0;
     for (int s = 0; s < n_seq; ++s) {
         TcSeq& q = all[s] = seq[s];
+        q.src = s;
         long total;
         q.levels = (q.Lq + TC_ROWS - 1) / TC_ROWS;
         q.nb = (q.L + bt - 1) / bt; q.nbq = (q.Lq + bt - 1) / bt;
@@ -292,13 +295,13 @@ TcSeq tc_ragged_seq(const hyq_attn_args& a, int L, int k, size_t tokens_before, 
     return q;
 }
 
-int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, cudaStream_t st) {
+int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, const TcSources* src, cudaStream_t st) {
     char* base = static_cast<char*>(a.workspace);
     const TcSeqTable& t = plan.t.tab;
     const TcWorkspace& w = plan.w;
     PreParams p{};
     auto blocks = [](long threads) { return (threads + PRE_THREADS - 1) / PRE_THREADS; };
-    long n = blocks((long)t.kv_rows * 16);
+    long n = src ? 0 : blocks((long)t.kv_rows * 16);
     p.v_end = (unsigned)n;
     p.gather_end = (unsigned)(n += blocks((long)t.vl_rows * 16));
     long mb = 0;
@@ -307,14 +310,19 @@ int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, cudaStream_t s
         mb += (long)t.heads * ((t.seq[s].mask_words + PRE_MASK_WORDS - 1) / PRE_MASK_WORDS);
     }
     p.mask_end = (unsigned)(n += mb);
-    const bool int4 = a.q_format == HYQ_FMT_INT4;
+    const bool int4 = a.q_format == HYQ_FMT_INT4 && !src;
     p.k_vecs = int4 ? (long)t.kv_rows * 8 : 0;
     p.q_vecs = int4 ? (long)t.q_rows * 8 : 0;
     p.k_end = (unsigned)(n += blocks(p.k_vecs));
     p.q_end = (unsigned)(n += blocks(p.q_vecs));
     if (n > 0x7fffffffL) return HYQ_ERR_UNSUPPORTED;
     p.bt_shift = a.block_tokens == 32 ? 5 : a.block_tokens == 64 ? 6 : 7;
-    p.k = static_cast<const uint4*>(a.k_); p.v = static_cast<const uint4*>(a.v);
+    p.v = static_cast<const uint4*>(a.v);
+    for (int s = 0; s < t.n_seq; ++s) {
+        const long row0 = (long)t.seq[s].kv_row0 * 16;
+        p.k_seq[s] = src ? static_cast<const uint4*>(src->k[t.seq[s].src]) : static_cast<const uint4*>(a.k_) + row0;
+        p.v_seq[s] = src ? static_cast<const uint4*>(src->v[t.seq[s].src]) : static_cast<const uint4*>(a.v) + row0;
+    }
     p.v_codes = static_cast<const uint2*>(a.v_codes); p.v_scales = a.v_scales;
     p.vl_idx = a.vl_idx;
     p.q_codes = static_cast<const uint2*>(a.q_codes); p.k_codes = static_cast<const uint2*>(a.k_codes);

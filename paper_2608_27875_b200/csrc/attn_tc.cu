@@ -130,8 +130,12 @@ struct Piece {
     int t0, t1;
     int slot;                    // -1: the output; otherwise the slot for partial results
 };
-template <bool GENERAL> struct Tables : TcTables {};
-template <> struct Tables<false> {};         // a plain whole prefill finds its work from the block index alone
+enum { PLAIN = 0, PACKED = 1, SEPARATE = 2 };  // whole prefill; flattened views; the same with Q and K (bf16) per sequence
+template <int KIND> struct Tables : TcTables {};
+template <> struct Tables<PLAIN> {};         // a plain whole prefill finds its work from the block index alone
+template <> struct Tables<SEPARATE> : TcTables {
+    CUtensorMap q[TC_MAX_SEQ], k[TC_MAX_SEQ];
+};
 
 // The unit that tile `pos` of a split sequence falls into, its first tile and its number of tiles (warp-collective; the
 // tiles of the sequence are counted unit by unit, longest units first)
@@ -395,7 +399,7 @@ __device__ __forceinline__ bool mma_issuer(int q, const QSched& sq, const Walk& 
 }
 
 // The two query tiles (one thread, before the CTA's first synchronisation: they need nothing but the barrier)
-__device__ __forceinline__ void load_queries(const TcMaps& maps, const QSched& qs0, const QSched& qs1, int q_y, int q_z,
+__device__ __forceinline__ void load_queries(const CUtensorMap* q_map, const CUtensorMap* qc_map, int qc_dy, const QSched& qs0, const QSched& qs1, int q_y, int q_z,
                                              TcBarriers& bars, unsigned char* smem) {
     const int live[QT] = {qs0.live, qs1.live}, qi0[QT] = {qs0.i0, qs1.i0};
     const bool codes = max(qs0.nA, qs1.nA) > 0;
@@ -405,15 +409,15 @@ __device__ __forceinline__ void load_queries(const TcMaps& maps, const QSched& q
     mbar_arrive_expect_tx(&bars.q_full, qbytes);
     for (int q = 0; q < QT; ++q) {
         if (!live[q]) continue;
-        if (codes) tma_load_3d(smem + SQC_OFF + q * QC_TILE_BYTES, &maps.qc, &bars.q_full, 0, q_y + qi0[q], q_z);
-        tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES, &maps.q, &bars.q_full, 0, q_y + qi0[q], q_z);
-        tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES + Q_TILE_BYTES / 2, &maps.q, &bars.q_full, 64, q_y + qi0[q], q_z);
+        if (codes) tma_load_3d(smem + SQC_OFF + q * QC_TILE_BYTES, qc_map, &bars.q_full, 0, q_y + qc_dy + qi0[q], q_z);
+        tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES, q_map, &bars.q_full, 0, q_y + qi0[q], q_z);
+        tma_load_3d(smem + SQ_OFF + q * Q_TILE_BYTES + Q_TILE_BYTES / 2, q_map, &bars.q_full, 64, q_y + qi0[q], q_z);
     }
 }
 
 // TMA producer (one thread): the K ring and the V ring along the CTA's walk
 template <int TBN>
-__device__ __forceinline__ bool tma_producer(const TcMaps& maps, const Walk& w, int kv_y, int kv_z, int vl_y, int vl_z, TcBarriers& bars, unsigned char* smem, volatile int* abort_flag,
+__device__ __forceinline__ bool tma_producer(const TcMaps& maps, const CUtensorMap* k_map, int k_dy, const Walk& w, int kv_y, int kv_z, int vl_y, int vl_z, TcBarriers& bars, unsigned char* smem, volatile int* abort_flag,
                                              long long limit, int drop_load, const uint8_t* vl_tiles, bool settle) {
     using G = Geo<TBN>;
     constexpr int BN = TBN, NST = G::NST;
@@ -433,11 +437,12 @@ __device__ __forceinline__ bool tma_producer(const TcMaps& maps, const Walk& w, 
             tma_load_3d(sk, &maps.kc, &bars.kv_full[st], 0, row, hd);
             if (vl_tiles) bulk_load_1d(sk + VLT_OFF, vl_tiles + (long)t * VL_TILE_BYTES, VL_TILE_BYTES, &bars.kv_full[st]);
         } else {
-            const CUtensorMap* m = vl ? &maps.kvl : &maps.k;
+            const CUtensorMap* m = vl ? &maps.kvl : k_map;
+            const int k_row = vl ? row : row + k_dy;
             mbar_arrive_expect_tx(&bars.kv_full[st], 2 * G::STAGE_BYTES);
             if (t == drop_load) continue;
-            tma_load_3d(sk, m, &bars.kv_full[st], 0, row, hd);
-            tma_load_3d(sk + G::STAGE_BYTES / 2, m, &bars.kv_full[st], 64, row, hd);
+            tma_load_3d(sk, m, &bars.kv_full[st], 0, k_row, hd);
+            tma_load_3d(sk + G::STAGE_BYTES / 2, m, &bars.kv_full[st], 64, k_row, hd);
         }
         const CUtensorMap* m = lowbit ? &maps.vh16 : (vl ? &maps.vvl : &maps.v16);
         tma_load_3d(sv, m, &bars.kv_full[st], 0, row, hd);
@@ -537,10 +542,11 @@ __device__ __forceinline__ void mask_cols32(uint32_t (&raw)[32], int c0, int lo_
     for (int e = 0; e < 32; ++e) raw[e] = ((unsigned)(c0 + e - lo_eff) <= span) ? raw[e] : knock;
 }
 
-// LOWBIT_FP8: the low-bit codes are e4m3 bytes (kind::f8f6f4), else int8 (kind::i8).  GENERAL: everything but a plain
+// LOWBIT_FP8: the low-bit codes are e4m3 bytes (kind::f8f6f4), else int8 (kind::i8).  KIND other than PLAIN: everything but a plain
 // whole prefill - a query block of the last Lq < L positions, the fixed window, several sequences in one launch, units
 // shared by several CTAs (which leave unnormalised partial results that attn_merge_kernel combines by their reference
 // maxima).  A CTA then finds its pieces of work in `tabs`, and rows are addressed in the flattened views of the buffers;
+// with KIND = SEPARATE Q and K of every sequence are read where they are;
 // the plain kernel keeps a position offset and these look-ups out of its registers (2.6 % on the benchmark workload).
 // EXACT = false is the kernel of the first launch.  After the first tiles of a row's low-bit pass
 // (and if their maxima lie close together) it takes the exponentials against the row's reference as it stands, without
@@ -548,9 +554,10 @@ __device__ __forceinline__ void mask_cols32(uint32_t (&raw)[32], int c0, int lo_
 // piece - a score more than 2^16 above everything the row had seen - the CTA writes no output for it and puts the piece
 // on a list.  EXACT = true is the kernel of the second launch, a small grid that goes through that list
 // (normally empty) with the maximum looked at in every tile.
-template <bool LOWBIT_FP8, bool GENERAL, bool EXACT = false>
+template <bool LOWBIT_FP8, int KIND, bool EXACT = false>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcParams p, const __grid_constant__ Tables<GENERAL> tabs) {
+attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcParams p, const __grid_constant__ Tables<KIND> tabs) {
+    constexpr bool GENERAL = KIND != PLAIN;
     constexpr int TBN = 64, BN = 64;
     pdl_wait();
     if (EXACT && p.redo[0].x == 0) return;
@@ -584,6 +591,8 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
     }
     const bool settle = EXACT || next >= 0 || (GENERAL && pc.slot >= 0);      // the barriers may be initialised again
     int qhead, kvhead, pt, L, off, lim0, k_vl, q_y, q_z, kv_y, kv_z, vl_y, vl_z;
+    int q_dy = 0, k_dy = 0;                                  // flattened row minus row in the sequence's own Q; the converse for K
+    const CUtensorMap *q_map = &maps.q, *k_map = &maps.k;
     long qs_at, ks_at, mask_at, lse_at;
     const int W = p.window, g = p.Hq / p.Hkv;
     if constexpr (GENERAL) {
@@ -598,6 +607,10 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
         qs_at = sq_.qs0 + (long)qhead * sq_.nbq; ks_at = sq_.ks0 + (long)kvhead * sq_.nb;
         mask_at = sq_.mask0 + (long)qhead * sq_.mask_words;
         lse_at = q_y;
+        if constexpr (KIND == SEPARATE) {
+            q_map = &tabs.q[pc.seq]; k_map = &tabs.k[pc.seq];
+            q_dy = sq_.q_row0; k_dy = -sq_.kv_row0;
+        }
     } else {
         // Block index -> (head, pair of query tiles): the longest pairs of all heads of a group come first
         // (launch_attn_tc says how large a group is)
@@ -656,7 +669,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 mbar_init(&bars.drain[q], 1);
             }
             fence_mbar_init();
-            load_queries(maps, qs0, qs1, q_y, q_z, bars, smem);
+            load_queries(q_map, &maps.qc, q_dy, qs0, qs1, q_y - q_dy, q_z, bars, smem);
             restart_s = 0;
             if (EXACT) atomicAdd(&g_tc_restarts, 1ull);
         }
@@ -707,7 +720,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
 
     // the single-thread roles sit in the lowest warps (the softmax warps 4..19 keep warp % 4 = TMEM lane quarter)
     if (warp == 0) {
-        if (lane == 0 && !tma_producer<TBN>(maps, w, kv_y, kv_z, vl_y, vl_z, bars, smem, abort_flag, limit, p.drop_load, vl_tiles_head, settle)) fail();
+        if (lane == 0 && !tma_producer<TBN>(maps, k_map, k_dy, w, kv_y, kv_z, vl_y, vl_z, bars, smem, abort_flag, limit, p.drop_load, vl_tiles_head, settle)) fail();
     } else if (warp == 1 || warp == 2) {
         if (lane == 0) {
             const int q = warp - 1;
@@ -1191,16 +1204,26 @@ int tc_restarts(unsigned long long* count, bool reset) {
     return HYQ_OK;
 }
 
-template <bool GENERAL>
+template <int KIND>
 static int launch_attn_tc_kernels(const hyq_attn_args& a, const TcPlan& plan, const TcMaps& maps, const TcParams& p, int n_ctas,
-                                  int pieces, cudaStream_t st) {
-    Tables<GENERAL> tabs;
-    if constexpr (GENERAL) static_cast<TcTables&>(tabs) = plan.t;
+                                  int pieces, const TcSources* src, cudaStream_t st) {
+    Tables<KIND> tabs;
+    if constexpr (KIND != PLAIN) static_cast<TcTables&>(tabs) = plan.t;
+    if constexpr (KIND == SEPARATE) {
+        bool ok = true;
+        for (int s = 0; s < plan.t.tab.n_seq; ++s) {
+            const TcSeq& q = plan.t.tab.seq[s];
+            ok &= make_tmap_3d(&tabs.q[s], src->q[q.src], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, (uint64_t)plan.t.tab.heads * q.Lq, 1, 64, BM);
+            ok &= make_tmap_3d(&tabs.k[s], src->k[q.src], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D,
+                               (uint64_t)(plan.t.tab.heads / plan.t.tab.g) * q.L, 1, 64, 64);
+        }
+        if (!ok) return HYQ_ERR_CUDA;
+    }
     // e4m3 bytes on the low-bit side: FP8 codes as they are, or INT4 codes widened by the pre-pass
     const bool lowbit_fp8 = a.q_format != HYQ_FMT_INT8;
-    auto kern = lowbit_fp8 ? attn_tc_kernel<true, GENERAL> : attn_tc_kernel<false, GENERAL>;
+    auto kern = lowbit_fp8 ? attn_tc_kernel<true, KIND> : attn_tc_kernel<false, KIND>;
     // the same instantiation for the second launch (every maximum looked at; works through the first launch's list)
-    auto kern_exact = lowbit_fp8 ? attn_tc_kernel<true, GENERAL, true> : attn_tc_kernel<false, GENERAL, true>;
+    auto kern_exact = lowbit_fp8 ? attn_tc_kernel<true, KIND, true> : attn_tc_kernel<false, KIND, true>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(kern_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_BYTES) != cudaSuccess)
         return HYQ_ERR_CUDA;
@@ -1209,24 +1232,26 @@ static int launch_attn_tc_kernels(const hyq_attn_args& a, const TcPlan& plan, co
     return launch_pdl(kern_exact, dim3((unsigned)(pieces < TC_SMS ? pieces : TC_SMS)), dim3(TC_THREADS), TC_SMEM_BYTES, st, maps, p, tabs);
 }
 
-int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, float alpha, cudaStream_t st) {
+int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, const TcSources* src, float alpha, cudaStream_t st) {
     constexpr int TBN = 64;                                             // keys per tile
     const TcWorkspace& w = plan.w;
     const TcSeqTable& tab = plan.t.tab;
-    int rc = launch_tc_prepass(a, plan, st);
+    int rc = launch_tc_prepass(a, plan, src, st);
     if (rc != HYQ_OK) return rc;
     char* base = static_cast<char*>(a.workspace);
     const bool packed = a.q_format == HYQ_FMT_INT4;
     // the general kernel addresses the flattened views (everything but a plain whole prefill, see there)
     const TcSeq& s0 = tab.seq[0];
     const bool general = tab.n_seq > 1 || s0.split > 0 || s0.Lq < s0.L || a.window_mode == HYQ_WINDOW_FIXED_TAIL;
+    const bool separate = src && tab.n_seq > 1;
     const uint64_t qh = general ? 1 : tab.heads, kvh = general ? 1 : tab.heads / tab.g;
     const uint64_t L = tab.kv_rows / kvh, Lq = tab.q_rows / qh, kk = tab.vl_rows > 0 ? tab.vl_rows / qh : 1;
 
     TcMaps maps;
     bool ok = true;
-    ok &= make_tmap_3d(&maps.q, a.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, Lq, qh, 64, BM);
-    ok &= make_tmap_3d(&maps.k, a.k_, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, L, kvh, 64, TBN);
+    const void *q0 = src ? src->q[s0.src] : a.q, *k0 = src ? src->k[s0.src] : a.k_;      // (separate: not used)
+    ok &= make_tmap_3d(&maps.q, q0, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, Lq, qh, 64, BM);
+    ok &= make_tmap_3d(&maps.k, k0, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, HYQ_D, L, kvh, 64, TBN);
     ok &= make_tmap_3d(&maps.qc, packed ? (const void*)(base + w.q8) : a.q_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, HYQ_D, Lq, qh, 128, BM);
     ok &= make_tmap_3d(&maps.kc, packed ? (const void*)(base + w.k8) : a.k_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, HYQ_D, L, kvh, 128, TBN);
     ok &= make_tmap_3d(&maps.v16, base + w.v16, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, HYQ_D, L, kvh, 64, TBN);
@@ -1272,8 +1297,9 @@ int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, float alpha, cuda
     p.head_group = (int)((kv_heads + groups - 1) / groups) * (a.Hq / a.Hkv);
     p.redo = reinterpret_cast<int4*>(base + w.redo);           // (its count starts at zero: the pre-pass)
     if (a.ev_kernel_start && cudaEventRecord(static_cast<cudaEvent_t>(a.ev_kernel_start), st) != cudaSuccess) return HYQ_ERR_CUDA;
-    rc = general ? launch_attn_tc_kernels<true>(a, plan, maps, p, tab.ctas, w.pieces, st)
-                 : launch_attn_tc_kernels<false>(a, plan, maps, p, tab.ctas, w.pieces, st);
+    rc = separate ? launch_attn_tc_kernels<SEPARATE>(a, plan, maps, p, tab.ctas, w.pieces, src, st)
+         : general ? launch_attn_tc_kernels<PACKED>(a, plan, maps, p, tab.ctas, w.pieces, src, st)
+                   : launch_attn_tc_kernels<PLAIN>(a, plan, maps, p, tab.ctas, w.pieces, src, st);
     for (int s = tab.n_unsplit; rc == HYQ_OK && s < tab.n_seq; ++s)
         rc = launch_pdl(attn_merge_kernel, dim3((unsigned)(tab.seq[s].levels * tab.heads * 32)), dim3(256), 0, st, tab.seq[s], tab.heads,
                         a.window, p.fixed_tail, reinterpret_cast<const float*>(base + w.part_o), static_cast<const float*>(p.part_ml),

@@ -64,34 +64,68 @@ def test_units_shared_by_several_ctas(fmts, Hq, Hkv, L, Lq, W, k, mode, out):
     _close(*_both_kernels(Q, K, V, fmts, W, k, out, window_mode=mode))
 
 
+def _packed_calls(qs, ks, vs, W, k_per, fmts, all_in_one):
+    """The three *_varlen calls on packed buffers; the attention's workspace for all prompts at once or the smallest accepted."""
+    import ctypes
+    lib = api.lib()
+    n, Hq, Hkv = len(qs), qs[0].shape[0], ks[0].shape[0]
+    (qp, cu), (kp, _), (vp, _) = (api.pack_sequences(t) for t in (qs, ks, vs))
+    lens = [cu[i + 1] - cu[i] for i in range(n)]
+    cu_c, k_c = api._i32(cu), api._i32(k_per)
+    empty = lambda m, dt=torch.uint8: torch.empty(max(m, 16), dtype=dt, device="cuda")       # noqa: E731
+    idx = empty(Hq * sum(k_per), torch.int32)
+    ws = empty(max(api.hyq_select_vertical_workspace(1, Hq, Hkv, L, L, 128, W, k) for L, k in zip(lens, k_per)) * (20 if all_in_one else 1))
+    api._check(lib.hyq_select_vertical_varlen(qp.data_ptr(), kp.data_ptr(), n, cu_c, Hq, Hkv, 128, W, 0, k_c, idx.data_ptr(),
+                                              ws.data_ptr(), ws.numel(), api._stream()), "select")
+    qz = []
+    for x, H, f in ((qp, Hq, fmts[0]), (kp, Hkv, fmts[1]), (vp, Hkv, fmts[2])):
+        c, sc = empty(H * cu[-1] * api.code_row_bytes(f, 128)), empty(H * sum(-(-L // 64) for L in lens), torch.float32)
+        api._check(lib.hyq_quantize_blocks_varlen(x.data_ptr(), n, cu_c, H, 128, 64, f, c.data_ptr(), sc.data_ptr(), api._stream()), "quantize")
+        qz.append((c, sc))
+    out = torch.empty(Hq * cu[-1] * 128, device="cuda")
+    a = api.AttnArgs()
+    a.struct_size = ctypes.sizeof(api.AttnArgs)
+    a.B, a.Hq, a.Hkv, a.L, a.D, a.window, a.block_tokens, a.out_dtype = 1, Hq, Hkv, max(lens), 128, W, 64, 1
+    a.q_format, a.k_format, a.v_format = fmts
+    a.k = k_per[lens.index(max(lens))]
+    a.q, a.k_, a.v, a.vl_idx, a.out = qp.data_ptr(), kp.data_ptr(), vp.data_ptr(), idx.data_ptr(), out.data_ptr()
+    a.q_codes, a.k_codes, a.v_codes = (c.data_ptr() for c, _ in qz)
+    a.q_scales, a.k_scales, a.v_scales = (sc.data_ptr() for _, sc in qz)
+    need = ctypes.c_size_t(0)
+    if all_in_one:
+        api._check(lib.hyq_hybrid_attention_prefill_varlen_workspace(ctypes.byref(a), n, cu_c, k_c, ctypes.byref(need)), "workspace")
+    else:
+        api._check(lib.hyq_hybrid_attention_prefill_workspace(ctypes.byref(a), ctypes.byref(need)), "workspace")
+    ws = empty(need.value)
+    a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+    api._check(lib.hyq_hybrid_attention_prefill_varlen(ctypes.byref(a), n, cu_c, k_c, api._stream()), "attention")
+    return [out[Hq * 128 * cu[i]:Hq * 128 * cu[i + 1]].view(Hq, lens[i], 128) for i in range(n)]
+
+
 @pytest.mark.parametrize("fmts", [INT8, INT4FP8])
-def test_ragged_batches_of_any_launch_grouping_give_the_same_bits(fmts, monkeypatch):
-    """40 prompts (more than one launch holds) with all the workspace, and with the longest prompt's alone (the smallest
-    the call accepts: launches of a few prompts each); among them prompts whose units are shared by several CTAs."""
+def test_ragged_batches_of_any_launch_grouping_give_the_same_bits(fmts):
+    """40 prompts (more than one launch holds; among them prompts whose units are shared by several CTAs): the whole path in
+    one call on the prompts where they lie, the three packed calls with all the workspace and with the longest prompt's alone
+    (launches of a few prompts each), and the plain calls on a prompt by itself."""
     ensure_built()
     rng = np.random.default_rng(5)
     lens = [int(x) for x in np.exp(rng.uniform(np.log(1), np.log(3000), 39))] + [3000]
     qs, ks, vs = ([_normal((h, L, 128), 100 * h + n) for n, L in enumerate(lens)] for h in (6, 2, 2))
     k_per = [max(0, L - 128) // 40 for L in lens]
     one = api.hybrid_prefill_varlen(qs, ks, vs, 128, k_per, fmts)
-    lib = api.lib()
-
-    class Small:                              # the same library, but the ragged query answers with the longest prompt's need
-        def __getattr__(self, name):
-            if name != "hyq_hybrid_attention_prefill_varlen_workspace":
-                return getattr(lib, name)
-
-            def longest(a, n, cu, kk, out):
-                return lib.hyq_hybrid_attention_prefill_workspace(a, out)
-            return longest
-    monkeypatch.setattr(api, "lib", lambda: Small())
-    few = api.hybrid_prefill_varlen(qs, ks, vs, 128, k_per, fmts)
-    monkeypatch.undo()
-    for a, b in zip(one, few):
-        assert torch.equal(a["out"], b["out"])
-    for n in (0, 17, 39):                     # and the plain call's
+    for all_in_one in (True, False):
+        for r, out in zip(one, _packed_calls(qs, ks, vs, 128, k_per, fmts, all_in_one)):
+            assert torch.equal(r["out"], out)
+    for n in (0, 17, 39):
         alone = api.hybrid_prefill(qs[n][None], ks[n][None], vs[n][None], 128, k_per[n], fmts)
-        assert torch.equal(alone["out"][0], one[n]["out"])
+        for name in alone:
+            assert torch.equal(alone[name][0], one[n][name]), name
+        # stage by stage
+        qz = [api.hyq_quantize_blocks(t[n][None], f) for t, f in zip((qs, ks, vs), fmts)]
+        idx = api.hyq_select_vertical(qs[n][None], ks[n][None], 128, k_per[n])
+        out = api.hyq_hybrid_attention_prefill(qs[n][None], ks[n][None], vs[n][None], qz[0][0], qz[1][0], qz[2][0], qz[0][1],
+                                               qz[1][1], qz[2][1], fmts, idx, 128)
+        assert torch.equal(out[0], one[n]["out"]) and torch.equal(idx[0], one[n]["idx"])
 
 
 # ---- selection: the oracle's index sets bit for bit ---------------------------------------------------------------
