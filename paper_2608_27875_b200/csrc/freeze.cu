@@ -1,22 +1,21 @@
 // Freeze (Algorithm 4): builds the hybrid KV cache of the decode stage from the prefill cache.
 //
-// Two kernels, both HBM-bound and read-once / write-once:
-//   gather_rows_kernel     copies the vertical rows (by index) and the window rows (a slice) as bf16;
-//   freeze_quantize_kernel one CTA per group of G (32, 64 or 128) COMPACTED rows of one (b, kv head) and one tensor
-//                          (K or V): finds the source rows (the complement of the ascending vertical
-//                          set, by binary search), quantizes the G x 128 group to INT4 with the
-//                          arithmetic of the per-tile quantizer (fp32, one rounding per operation), and
-//                          writes K row-major and V in the fragment-major tile layout the decode kernel
-//                          loads straight into matrix-instruction operand registers.
-#include <cuda_fp8.h>
-
-#include "common.cuh"
+// One kernel, HBM-bound and read-once / write-once; a block either
+//   - quantizes one group of G (32, 64 or 128) COMPACTED rows of one (b, kv head), K and V: finds the source rows (the
+//     complement of the ascending vertical set) once for both, quantizes the two G x 128 groups with the arithmetic of
+//     the per-tile quantizer, and writes K row-major and V in the fragment-major tile layout the decode kernel
+//     loads straight into matrix-instruction operand registers; or
+//   - copies vertical rows (by index) and window rows (a slice) as bf16.
+// What kept it from the memory's rate was the chain search -> row numbers -> loads of 16 KB per CTA, and one conversion
+// instruction per element.  One chain now serves 32 KB, all loads are issued before the first maximum, and rounding is an
+// addition: 8 x 8 heads x 32768 rows (1.38 GB moved), INT4: 295 -> 267 us.
 #include "decode_common.cuh"
+#include "quantize.cuh"
 
 namespace hyq {
 
-constexpr int FRZ_THREADS = 128;     // gather kernel; the quantizer runs 2 * G threads (64 elements per thread)
-constexpr int FRZ_QTHREADS_PER_SM = 896;   // quantizer threads resident per SM the register budget is set for (7 CTAs of 128)
+constexpr int FRZ_THREADS = 128;     // append kernel; the quantizer runs 2 * G threads (64 elements of K and of V per thread)
+constexpr int FRZ_QTHREADS_PER_SM = 640;    // quantizer threads resident per SM the register budget is set for
 
 // Source position of compacted row p: p + j with j the number of vertical indices below it,
 // i.e. the smallest j with idx[j] - j > p (idx ascending, so idx[j] - j never decreases).
@@ -29,38 +28,43 @@ __device__ __forceinline__ int source_row(const int32_t* __restrict__ idx, int k
     return p + lo;
 }
 
-__global__ void __launch_bounds__(FRZ_THREADS)
-gather_rows_kernel(const uint4* __restrict__ k_, const uint4* __restrict__ v, const int32_t* __restrict__ idx,
-                   int N, int W, int k_vl, long sK, long sW, uint4* __restrict__ k_vl_out, uint4* __restrict__ v_vl_out,
-                   uint4* __restrict__ k_win, uint4* __restrict__ v_win) {
-    const long head = blockIdx.y;
-    const int o = blockIdx.x * 8 + (threadIdx.x >> 4);
-    const int c = threadIdx.x & 15;                       // 16 x 16 bytes = one 256-byte row
-    if (o >= k_vl + W) return;
-    const int P = N - W;
-    const bool vl = o < k_vl;
+struct FreezeParams {
+    const uint4 *k, *v;
+    const int32_t* idx;
+    int N, W, k_vl, nQ, n_groups;
+    long nQp, sK, sW;
+    uint8_t *kq, *vq;
+    float *ks, *vs;
+    uint4 *k_vl_out, *v_vl_out, *k_win, *v_win;
+};
+
+// 16 bytes (piece c) of vertical or window row o
+__device__ __forceinline__ void gather_piece(const FreezeParams& p, long head, int o, int c) {
+    if (o >= p.k_vl + p.W) return;
+    const bool vl = o < p.k_vl;
     // (a vertical index outside [0, N) is clamped: it then names a wrong row instead of memory outside the tensor)
-    const int src = vl ? min(max(__ldg(idx + head * k_vl + o), 0), N - 1) : P + (o - k_vl);
-    const long s = (head * N + src) * 16 + c;
-    const long d = vl ? (head * sK + o) * 16 + c : (head * sW + (o - k_vl)) * 16 + c;
-    (vl ? k_vl_out : k_win)[d] = __ldg(k_ + s);
-    (vl ? v_vl_out : v_win)[d] = __ldg(v + s);
+    const int src = vl ? min(max(__ldg(p.idx + head * p.k_vl + o), 0), p.N - 1) : p.N - p.W + (o - p.k_vl);
+    const long s = (head * p.N + src) * 16 + c;
+    const long d = vl ? (head * p.sK + o) * 16 + c : (head * p.sW + (o - p.k_vl)) * 16 + c;
+    (vl ? p.k_vl_out : p.k_win)[d] = __ldg(p.k + s);
+    (vl ? p.v_vl_out : p.v_win)[d] = __ldg(p.v + s);
 }
 
 template <int G, int FMT>
 __global__ void __launch_bounds__(2 * G, FRZ_QTHREADS_PER_SM / (2 * G))
-freeze_quantize_kernel(const uint4* __restrict__ k_, const uint4* __restrict__ v, const int32_t* __restrict__ idx,
-                       int N, int k_vl, int nQ, long nQp, uint8_t* __restrict__ kq, uint8_t* __restrict__ vq,
-                       float* __restrict__ ks, float* __restrict__ vs) {
+freeze_kernel(const __grid_constant__ FreezeParams p) {
+    constexpr int NT = 2 * G;                                  // threads of this CTA
     const int grp = blockIdx.x;
     const long head = blockIdx.y;
-    const bool is_v = blockIdx.z == 1;
-    const uint4* x = (is_v ? v : k_) + head * N * 16;
-    const int32_t* hidx = idx + head * k_vl;
+    if (grp >= p.n_groups) {
+        gather_piece(p, head, (grp - p.n_groups) * (NT / 16) + (threadIdx.x >> 4), threadIdx.x & 15);
+        return;
+    }
+    const int N = p.N, k_vl = p.k_vl, nQ = p.nQ;
+    const int32_t* hidx = p.idx + head * k_vl;
 
-    constexpr int NT = 2 * G;                                  // threads of this CTA
     __shared__ int src[G];
-    __shared__ float warp_max[NT / 32];
+    __shared__ uint32_t warp_max[2][NT / 32];
     constexpr bool FMT8 = FMT != HYQ_FMT_INT4;                 // byte-wide codes (INT8 or FP8 e4m3)
     constexpr int ROW_BYTES = FMT8 ? HYQ_D : HYQ_D / 2;        // code bytes per row
     constexpr int TILE_BYTES = 16 * ROW_BYTES;                 // one 16-row V tile
@@ -90,91 +94,73 @@ freeze_quantize_kernel(const uint4* __restrict__ k_, const uint4* __restrict__ v
         j0 = lo;
     }
     if (threadIdx.x < G) {
-        const int p = p0 + threadIdx.x;
+        const int row = p0 + threadIdx.x;
         int s = -1;
-        if (p < nQ) {
-            int j = j0, steps = 0;                          // smallest j >= j0 with idx[j] - j > p
-            while (j < k_vl && steps < 16 && __ldg(hidx + j) - j <= p) { ++j; ++steps; }
-            s = (steps < 16) ? p + j : source_row(hidx, k_vl, p);
+        if (row < nQ) {
+            int j = j0, steps = 0;                          // smallest j >= j0 with idx[j] - j > row
+            while (j < k_vl && steps < 16 && __ldg(hidx + j) - j <= row) { ++j; ++steps; }
+            s = (steps < 16) ? row + j : source_row(hidx, k_vl, row);
             s = min(s, N - 1);                              // (only a malformed index list can reach the clamp)
         }
         src[threadIdx.x] = s;
     }
     __syncthreads();
 
-    uint4 r[4][2];
-    float amax = 0.0f;
+    // all loads of both tensors before the first use
+    uint4 r[2][4][2];
 #pragma unroll
-    for (int gi = 0; gi < 4; ++gi) {
-        const int u = threadIdx.x + gi * NT;              // 16-channel unit: row u >> 3, channels 16 * (u & 7)
-        const int s = src[u >> 3];
-        if (s >= 0) {
-            r[gi][0] = __ldg(x + (long)s * 16 + (u & 7) * 2);
-            r[gi][1] = __ldg(x + (long)s * 16 + (u & 7) * 2 + 1);
-        } else {
-            r[gi][0] = make_uint4(0, 0, 0, 0);
-            r[gi][1] = make_uint4(0, 0, 0, 0);
-        }
-        const uint32_t* w = reinterpret_cast<const uint32_t*>(&r[gi][0]);
+    for (int z = 0; z < 2; ++z) {
+        const uint4* x = (z ? p.v : p.k) + head * N * 16;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            amax = fmaxf(amax, fabsf(bf16_lo(w[c])));
-            amax = fmaxf(amax, fabsf(bf16_hi(w[c])));
+        for (int gi = 0; gi < 4; ++gi) {
+            const int u = threadIdx.x + gi * NT;              // 16-channel unit: row u >> 3, channels 16 * (u & 7)
+            const int s = src[u >> 3];
+            r[z][gi][0] = r[z][gi][1] = make_uint4(0, 0, 0, 0);
+            if (s >= 0) {
+                r[z][gi][0] = __ldg(x + (long)s * 16 + (u & 7) * 2);
+                r[z][gi][1] = __ldg(x + (long)s * 16 + (u & 7) * 2 + 1);
+            }
         }
     }
+    uint32_t mx[2];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = amax;
+    for (int z = 0; z < 2; ++z) {
+        mx[z] = 0u;
+#pragma unroll
+        for (int gi = 0; gi < 4; ++gi) {
+            const uint32_t* w = reinterpret_cast<const uint32_t*>(&r[z][gi][0]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) mx[z] = amax_pair(mx[z], w[c]);
+        }
+        mx[z] = amax_warp(mx[z]);
+        if ((threadIdx.x & 31) == 0) warp_max[z][threadIdx.x >> 5] = mx[z];
+    }
     __syncthreads();
-    amax = warp_max[0];
 #pragma unroll
-    for (int w = 1; w < NT / 32; ++w) amax = fmaxf(amax, warp_max[w]);
-
-    const bool dead = !(amax >= 0x1p-100f);
-    const float inv = dead ? 0.0f : __fdiv_rn(CB, amax);
-    if (threadIdx.x == 0) (is_v ? vs : ks)[head * (nQp / G) + grp] = dead ? 0.0f : __fdiv_rn(amax, CB);
-
+    for (int z = 0; z < 2; ++z) {
 #pragma unroll
-    for (int gi = 0; gi < 4; ++gi) {
-        const int u = threadIdx.x + gi * NT;
-        const int row = u >> 3, ch0 = (u & 7) * 16;
-        const uint32_t* w = reinterpret_cast<const uint32_t*>(&r[gi][0]);
-        if (FMT8) {
-            uint32_t o[4] = {0u, 0u, 0u, 0u};
+        for (int w = 0; w < NT / 32; ++w) mx[z] = max(mx[z], warp_max[z][w]);
+        const float amax = __uint_as_float(mx[z] << 16);
+        const bool dead = !(amax >= 0x1p-100f);
+        const float inv = dead ? 0.0f : __fdiv_rn(CB, amax);
+        if (threadIdx.x == 0) (z ? p.vs : p.ks)[head * (p.nQp / G) + grp] = dead ? 0.0f : __fdiv_rn(amax, CB);
 #pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                const float y0 = __fmul_rn(bf16_lo(w[m]), inv), y1 = __fmul_rn(bf16_hi(w[m]), inv);
-                uint32_t two;                                // codes of channels 2m (low byte) and 2m + 1
-                if (FMT == HYQ_FMT_FP8_E4M3) {
-                    two = dead ? 0u : __nv_cvt_float2_to_fp8x2(make_float2(y0, y1), __NV_SATFINITE, __NV_E4M3);   // no -0 in a zero group
-                } else {
-                    two = (uint32_t)(max(-127, min(127, __float2int_rn(y0))) & 0xFF) |
-                          ((uint32_t)(max(-127, min(127, __float2int_rn(y1))) & 0xFF) << 8);
-                }
-                o[m >> 1] |= (two & 0xFFFFu) << (16 * (m & 1));
-            }
-            uint4* d4 = is_v ? reinterpret_cast<uint4*>(vstage + row * VSTRIDE + ch0)
-                             : reinterpret_cast<uint4*>(kq + ((head * nQp + grp * G + row) * ROW_BYTES + ch0));
-            *d4 = make_uint4(o[0], o[1], o[2], o[3]);
-        } else {
-            uint32_t o[2] = {0u, 0u};
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                const int q0 = max(-7, min(7, __float2int_rn(__fmul_rn(bf16_lo(w[m]), inv))));
-                const int q1 = max(-7, min(7, __float2int_rn(__fmul_rn(bf16_hi(w[m]), inv))));
-                o[m >> 2] |= (uint32_t)((q0 & 0xF) | ((q1 & 0xF) << 4)) << (8 * (m & 3));
-            }
-            uint2* d2 = is_v ? reinterpret_cast<uint2*>(vstage + row * VSTRIDE + ch0 / 2)
-                             : reinterpret_cast<uint2*>(kq + ((head * nQp + grp * G + row) * ROW_BYTES + ch0 / 2));
-            *d2 = make_uint2(o[0], o[1]);
+        for (int gi = 0; gi < 4; ++gi) {
+            const int u = threadIdx.x + gi * NT;
+            const int row = u >> 3, at = (u & 7) * (ROW_BYTES / 8);
+            const uint32_t* w = reinterpret_cast<const uint32_t*>(&r[z][gi][0]);
+            uint8_t* d = z ? vstage + row * VSTRIDE + at : p.kq + (head * p.nQp + grp * G + row) * ROW_BYTES + at;
+            if (FMT == HYQ_FMT_INT8) *reinterpret_cast<uint4*>(d) = quant16_int8(w, inv);
+            else if (FMT == HYQ_FMT_FP8_E4M3) *reinterpret_cast<uint4*>(d) = quant16_e4m3(w, inv, dead);
+            else *reinterpret_cast<uint2*>(d) = quant16_int4(w, inv);
         }
     }
-    if (is_v) {
+    {
         // Fragment-major write-out (the layouts of vq_byte_offset / vq8_byte_offset): 16-byte piece number 32 * run + l
         // of a tile, l = 4r + j, is made of one 4-byte load from each of the rows 2j, 2j + 1, 2j + 8, 2j + 9 and
         // a 4 x 4 (INT4) or 2 x 2 (byte codes) transpose of their bytes.
         __syncthreads();
-        uint4* dst = reinterpret_cast<uint4*>(vq + (head * (nQp / 16) + grp * (G / 16)) * (long)TILE_BYTES);
+        uint4* dst = reinterpret_cast<uint4*>(p.vq + (head * (p.nQp / 16) + grp * (G / 16)) * (long)TILE_BYTES);
         constexpr int PIECES = TILE_BYTES / 16;
 #pragma unroll
         for (int i = 0; i < (G / 16) * PIECES / NT; ++i) {
@@ -228,26 +214,24 @@ int launch_cache_append(const void* k_new, const void* v_new, const hyq_kv_cache
 int launch_freeze(const void* k_, const void* v, const int32_t* vl_idx, const hyq_kv_cache& c, cudaStream_t st) {
     const CacheGeo g = cache_geo(c);
     const long heads = (long)c.B * c.Hkv;
-    const uint4* k4 = static_cast<const uint4*>(k_);
-    const uint4* v4 = static_cast<const uint4*>(v);
-    if (c.k + g.W > 0) {
-        const dim3 grid((unsigned)((c.k + g.W + 7) / 8), (unsigned)heads);
-        gather_rows_kernel<<<grid, FRZ_THREADS, 0, st>>>(k4, v4, vl_idx, c.N, g.W, c.k, g.sK, g.sW, static_cast<uint4*>(c.k_vl),
-                                                         static_cast<uint4*>(c.v_vl), static_cast<uint4*>(c.k_win),
-                                                         static_cast<uint4*>(c.v_win));
-    }
-    if (g.nQ > 0) {
-        const dim3 grid((unsigned)(g.nQp / c.group), (unsigned)heads, 2);
-        auto* kq = static_cast<uint8_t*>(c.kq_codes);
-        auto* vq = static_cast<uint8_t*>(c.vq_codes);
-#define HYQ_FRZ(G_, F8_) freeze_quantize_kernel<G_, F8_><<<grid, 2 * G_, 0, st>>>(k4, v4, vl_idx, c.N, c.k, (int)g.nQ, g.sQ, kq, vq, c.kq_scales, c.vq_scales)
+    FreezeParams p;
+    p.k = static_cast<const uint4*>(k_); p.v = static_cast<const uint4*>(v); p.idx = vl_idx;
+    p.N = c.N; p.W = g.W; p.k_vl = c.k; p.nQ = (int)g.nQ; p.n_groups = (int)(g.nQp / c.group);
+    p.nQp = g.sQ; p.sK = g.sK; p.sW = g.sW;
+    p.kq = static_cast<uint8_t*>(c.kq_codes); p.vq = static_cast<uint8_t*>(c.vq_codes);
+    p.ks = c.kq_scales; p.vs = c.vq_scales;
+    p.k_vl_out = static_cast<uint4*>(c.k_vl); p.v_vl_out = static_cast<uint4*>(c.v_vl);
+    p.k_win = static_cast<uint4*>(c.k_win); p.v_win = static_cast<uint4*>(c.v_win);
+    const int rows = 2 * c.group / 16;                          // rows a gathering block copies
+    const dim3 grid((unsigned)(p.n_groups + (c.k + g.W + rows - 1) / rows), (unsigned)heads);
+    if (grid.x == 0) return HYQ_OK;
+#define HYQ_FRZ(G_, F_) freeze_kernel<G_, F_><<<grid, 2 * G_, 0, st>>>(p)
 #define HYQ_FRZ_F(G_) do { if (c.format == HYQ_FMT_INT8) HYQ_FRZ(G_, HYQ_FMT_INT8); else if (c.format == HYQ_FMT_FP8_E4M3) HYQ_FRZ(G_, HYQ_FMT_FP8_E4M3); else HYQ_FRZ(G_, HYQ_FMT_INT4); } while (0)
-        if (c.group == 32) HYQ_FRZ_F(32);
-        else if (c.group == 64) HYQ_FRZ_F(64);
-        else HYQ_FRZ_F(128);
+    if (c.group == 32) HYQ_FRZ_F(32);
+    else if (c.group == 64) HYQ_FRZ_F(64);
+    else HYQ_FRZ_F(128);
 #undef HYQ_FRZ_F
 #undef HYQ_FRZ
-    }
     return launch_status();
 }
 

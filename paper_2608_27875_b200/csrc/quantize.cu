@@ -12,8 +12,6 @@
 //
 // Arithmetic is fp32 with one IEEE rounding per operation (no FMA contraction, no fast-math):
 //   scale = absmax / c ; inv = c / absmax ; code = rint(x * inv) clamped, or e4m3(x * inv).
-#include <cuda_fp8.h>
-
 #include "quantize.cuh"
 
 namespace hyq {
@@ -32,7 +30,7 @@ __device__ __forceinline__ void quantize_tile(const QuantJob& job, int tile) {  
     const uint4* src = job.x + elem0 / 8;
 
     uint4 r[QUANT_GROUPS][2];
-    float amax = 0.0f;
+    uint32_t mx = 0u;
 #pragma unroll
     for (int gi = 0; gi < QUANT_GROUPS; ++gi) {
         const int e = (threadIdx.x + gi * QUANT_THREADS) * 16;
@@ -45,19 +43,15 @@ __device__ __forceinline__ void quantize_tile(const QuantJob& job, int tile) {  
         }
         const uint32_t* w = reinterpret_cast<const uint32_t*>(&r[gi][0]);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            amax = fmaxf(amax, fabsf(bf16_lo(w[c])));
-            amax = fmaxf(amax, fabsf(bf16_hi(w[c])));
-        }
+        for (int c = 0; c < 8; ++c) mx = amax_pair(mx, w[c]);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    __shared__ float warp_max[QUANT_THREADS / 32];
-    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = amax;
+    mx = amax_warp(mx);
+    __shared__ uint32_t warp_max[QUANT_THREADS / 32];
+    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = mx;
     __syncthreads();
-    amax = warp_max[0];
 #pragma unroll
-    for (int w = 1; w < QUANT_THREADS / 32; ++w) amax = fmaxf(amax, warp_max[w]);
+    for (int w = 0; w < QUANT_THREADS / 32; ++w) mx = max(mx, warp_max[w]);
+    const float amax = __uint_as_float(mx << 16);
 
     constexpr float c = (FMT == HYQ_FMT_INT8) ? 127.0f : (FMT == HYQ_FMT_FP8_E4M3) ? 448.0f : 7.0f;
     const bool dead = !(amax >= 0x1p-100f);
@@ -73,51 +67,32 @@ __device__ __forceinline__ void quantize_tile(const QuantJob& job, int tile) {  
         const uint32_t* w = reinterpret_cast<const uint32_t*>(&r[gi][0]);
         uint32_t vh[8];                                  // V^ as fp16 pairs
         if (FMT == HYQ_FMT_FP8_E4M3) {
-            uint32_t o[4];
+            const uint4 o = quant16_e4m3(w, inv, dead);
+            *reinterpret_cast<uint4*>(dst + e) = o;
+            if (EXTRAS && job.vh16) {
+                const uint32_t oc[4] = {o.x, o.y, o.z, o.w};
 #pragma unroll
-            for (int c4 = 0; c4 < 4; ++c4) {
-                const float y0 = __fmul_rn(bf16_lo(w[2 * c4]), inv), y1 = __fmul_rn(bf16_hi(w[2 * c4]), inv);
-                const float y2 = __fmul_rn(bf16_lo(w[2 * c4 + 1]), inv), y3 = __fmul_rn(bf16_hi(w[2 * c4 + 1]), inv);
-                const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(y0, y1), __NV_SATFINITE, __NV_E4M3);
-                const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(y2, y3), __NV_SATFINITE, __NV_E4M3);
-                o[c4] = dead ? 0u : (lo | (hi << 16));      // an all-zero tile has all-zero codes (no -0)
-                if (EXTRAS && job.vh16) {
-#pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((o[c4] >> (16 * half)) & 0xFFFFu), __NV_E4M3);
-                        const float2 ff = __half22float2(__half2(hr));
-                        vh[2 * c4 + half] = f16x2_sat(ff.x * scale, ff.y * scale);
-                    }
+                for (int c2 = 0; c2 < 8; ++c2) {
+                    const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((oc[c2 >> 1] >> (16 * (c2 & 1))) & 0xFFFFu), __NV_E4M3);
+                    const float2 ff = __half22float2(__half2(hr));
+                    vh[c2] = f16x2_sat(ff.x * scale, ff.y * scale);
                 }
             }
-            *reinterpret_cast<uint4*>(dst + e) = make_uint4(o[0], o[1], o[2], o[3]);
+        } else if (FMT == HYQ_FMT_INT8) {
+            *reinterpret_cast<uint4*>(dst + e) = quant16_int8(w, inv);
+            if (EXTRAS && job.vh16) {
+#pragma unroll
+                for (int c2 = 0; c2 < 8; ++c2) {
+                    const uint2 q = round_pair(w[c2], inv);
+                    vh[c2] = f16x2_sat(rounded_value(q.x) * scale, rounded_value(q.y) * scale);
+                }
+            }
         } else {
-            int q[16];
-#pragma unroll
-            for (int c2 = 0; c2 < 8; ++c2) {
-                q[2 * c2] = max(-(int)c, min((int)c, __float2int_rn(__fmul_rn(bf16_lo(w[c2]), inv))));
-                q[2 * c2 + 1] = max(-(int)c, min((int)c, __float2int_rn(__fmul_rn(bf16_hi(w[c2]), inv))));
-            }
-            if (FMT == HYQ_FMT_INT8) {
-                uint32_t o[4];
-#pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4)
-                    o[c4] = (uint32_t)(q[4 * c4] & 0xFF) | ((uint32_t)(q[4 * c4 + 1] & 0xFF) << 8) |
-                            ((uint32_t)(q[4 * c4 + 2] & 0xFF) << 16) | ((uint32_t)(q[4 * c4 + 3] & 0xFF) << 24);
-                *reinterpret_cast<uint4*>(dst + e) = make_uint4(o[0], o[1], o[2], o[3]);
-                if (EXTRAS && job.vh16) {
-#pragma unroll
-                    for (int c2 = 0; c2 < 8; ++c2) vh[c2] = f16x2_sat((float)q[2 * c2] * scale, (float)q[2 * c2 + 1] * scale);
-                }
-            } else {
-                uint32_t o[2] = {0u, 0u};
-#pragma unroll
-                for (int c16 = 0; c16 < 16; ++c16) o[c16 >> 3] |= (uint32_t)(q[c16] & 0xF) << ((c16 & 7) * 4);
-                *reinterpret_cast<uint2*>(dst + e / 2) = make_uint2(o[0], o[1]);
-                if (EXTRAS && job.wide)
-                    *reinterpret_cast<uint4*>(job.wide + elem0 + e) = make_uint4(nibbles_to_e4m3(o[0]), nibbles_to_e4m3(o[0] >> 16),
-                                                                                 nibbles_to_e4m3(o[1]), nibbles_to_e4m3(o[1] >> 16));
-            }
+            const uint2 o = quant16_int4(w, inv);
+            *reinterpret_cast<uint2*>(dst + e / 2) = o;
+            if (EXTRAS && job.wide)
+                *reinterpret_cast<uint4*>(job.wide + elem0 + e) = make_uint4(nibbles_to_e4m3(o.x), nibbles_to_e4m3(o.x >> 16),
+                                                                             nibbles_to_e4m3(o.y), nibbles_to_e4m3(o.y >> 16));
         }
         if (EXTRAS && FMT != HYQ_FMT_INT4 && job.vh16) {
             uint4* dh = job.vh16 + (elem0 + e) / 8;

@@ -1,6 +1,7 @@
 // Declarations of the per-tile quantizer and the value conversions it shares with the attention pre-pass.
 #pragma once
 #include <cuda_fp16.h>
+#include <cuda_fp8.h>
 
 #include "common.cuh"
 
@@ -44,5 +45,60 @@ __device__ __forceinline__ uint32_t nibbles_to_e4m3(uint32_t w) {
     m &= 0x7F7F7F7Fu;                                         // 0x7F where the code is negative
     return ((pos & ~m) | (neg & m)) | ((m << 1) & 0x80808080u);
 }
+
+// ---- the quantizer's arithmetic (fp32, one IEEE rounding per operation) -------------------------------------------
+// fl(x * inv) of the two bf16 values of a word, one packed multiplication
+__device__ __forceinline__ float2 mul_pair(uint32_t w, float inv) {
+    float2 y;
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\tmul.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
+        : "=f"(y.x), "=f"(y.y) : "f"(bf16_lo(w)), "f"(bf16_hi(w)), "f"(inv));
+    return y;
+}
+// The same rounded to integers (half to even) by adding 1.5 * 2^23: the low byte of each result word is the two's complement
+// code.  No clamp is needed: |x| <= absmax and two roundings keep fl(x * fl(c / absmax)) below c + 1/2.  (The conversion
+// instruction runs at an eighth of this rate.  The addition is not packed: the compiler fuses a packed product and sum into
+// one rounding, which turns exact ties around.)
+constexpr float ROUND_MAGIC = 12582912.0f;
+__device__ __forceinline__ uint2 round_pair(uint32_t w, float inv) {
+    const float2 y = mul_pair(w, inv);
+    return make_uint2(__float_as_uint(__fadd_rn(y.x, ROUND_MAGIC)), __float_as_uint(__fadd_rn(y.y, ROUND_MAGIC)));
+}
+__device__ __forceinline__ float rounded_value(uint32_t r) { return __uint_as_float(r) - ROUND_MAGIC; }
+// low bytes of four words
+__device__ __forceinline__ uint32_t pack_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+}
+// 16 values (8 words) -> 16 INT8 codes / 16 INT4 codes (channel 2m in the low nibble of byte m) / 16 e4m3 codes
+__device__ __forceinline__ uint4 quant16_int8(const uint32_t* w, float inv) {
+    uint32_t o[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint2 a = round_pair(w[2 * c], inv), b = round_pair(w[2 * c + 1], inv);
+        o[c] = pack_bytes(a.x, a.y, b.x, b.y);
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+__device__ __forceinline__ uint2 quant16_int4(const uint32_t* w, float inv) {
+    uint32_t byte[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        const uint2 a = round_pair(w[m], inv);
+        byte[m] = (a.x & 0xFu) | ((a.y << 4) & ~0xFu);
+    }
+    return make_uint2(pack_bytes(byte[0], byte[1], byte[2], byte[3]), pack_bytes(byte[4], byte[5], byte[6], byte[7]));
+}
+__device__ __forceinline__ uint4 quant16_e4m3(const uint32_t* w, float inv, bool dead) {
+    uint32_t o[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t lo = __nv_cvt_float2_to_fp8x2(mul_pair(w[2 * c], inv), __NV_SATFINITE, __NV_E4M3);
+        const uint32_t hi = __nv_cvt_float2_to_fp8x2(mul_pair(w[2 * c + 1], inv), __NV_SATFINITE, __NV_E4M3);
+        o[c] = dead ? 0u : (lo | (hi << 16));            // an all-zero tile has all-zero codes (no -0)
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+// running maximum of the magnitudes of both halves; bf16 magnitudes order like their bits
+__device__ __forceinline__ uint32_t amax_pair(uint32_t m, uint32_t w) { return __vmaxu2(m, w & 0x7FFF7FFFu); }
+__device__ __forceinline__ uint32_t amax_warp(uint32_t m) { return __reduce_max_sync(0xffffffffu, max(m & 0xFFFFu, m >> 16)); }   // bf16 bits
 
 }  // namespace hyq
