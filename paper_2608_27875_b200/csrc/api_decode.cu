@@ -74,7 +74,11 @@ int hyq_hybrid_attention_decode_workspace(const hyq_kv_cache* cache, int splits,
     if (!bytes || splits < 0 || splits > 1024) return HYQ_ERR_INVALID_ARG;
     const int rc = check_cache(cache, false);
     if (rc != HYQ_OK) return rc;
-    *bytes = decode_workspace_bytes(*cache, splits > 0 ? splits : decode_auto_splits(*cache));
+    int s = splits > 0 ? splits : decode_auto_splits(*cache);
+    // (capacities: the description may be a ragged batch's)
+    if (splits == 0 && (cache->cap_quantized_rows || cache->cap_vertical || cache->cap_window) && decode_ragged_splits(*cache) > s)
+        s = decode_ragged_splits(*cache);
+    *bytes = decode_workspace_bytes(*cache, s);
     return HYQ_OK;
 }
 
@@ -88,7 +92,7 @@ int hyq_hybrid_attention_decode(const void* q, const hyq_kv_cache* cache, float 
     const int s = splits > 0 ? splits : decode_auto_splits(*cache);
     if (workspace_bytes < decode_workspace_bytes(*cache, s)) return HYQ_ERR_WORKSPACE;
     const float alpha = softmax_scale != 0.0f ? softmax_scale : 1.0f / std::sqrt((float)cache->D);
-    return launch_decode(q, *cache, nullptr, alpha, s, out_dtype, out, lse, workspace, static_cast<cudaStream_t>(stream));
+    return launch_decode(q, *cache, nullptr, alpha, s, splits == 0, out_dtype, out, lse, workspace, static_cast<cudaStream_t>(stream));
 }
 
 int hyq_hybrid_attention_decode_ragged(const void* q, const hyq_kv_cache* cache, const int32_t* lengths, float softmax_scale,
@@ -99,10 +103,12 @@ int hyq_hybrid_attention_decode_ragged(const void* q, const hyq_kv_cache* cache,
     if (!q || !out || !workspace || !lengths || splits < 0 || splits > 1024) return HYQ_ERR_INVALID_ARG;
     if (out_dtype != 0 && out_dtype != 1) return HYQ_ERR_INVALID_ARG;
     if (!aligned16(q) || !aligned16(out) || !aligned16(workspace) || !aligned16(lengths)) return HYQ_ERR_ALIGNMENT;
-    const int s = splits > 0 ? splits : decode_auto_splits(*cache);
+    // slices by share where the workspace has room for them, the same number for every sequence otherwise
+    const bool by_share = splits == 0 && workspace_bytes >= decode_workspace_bytes(*cache, decode_ragged_splits(*cache));
+    const int s = splits > 0 ? splits : by_share ? decode_ragged_splits(*cache) : decode_auto_splits(*cache);
     if (workspace_bytes < decode_workspace_bytes(*cache, s)) return HYQ_ERR_WORKSPACE;
     const float alpha = softmax_scale != 0.0f ? softmax_scale : 1.0f / std::sqrt((float)cache->D);
-    return launch_decode(q, *cache, lengths, alpha, s, out_dtype, out, lse, workspace, static_cast<cudaStream_t>(stream));
+    return launch_decode(q, *cache, lengths, alpha, s, by_share, out_dtype, out, lse, workspace, static_cast<cudaStream_t>(stream));
 }
 
 }  // extern "C"

@@ -20,8 +20,10 @@
 // The bf16 segments (vertical rows, staging, window) go through the same two products with bf16 operands;
 // there V^T's key pairs are formed from two rows' words with byte permutes.
 //
-// Grid: (splits, B * Hkv).  A CTA owns a contiguous slice of the head's INT4 tiles and one of its bf16 tiles
-// (the three bf16 segments form one tile list); its 4 warps take tiles round-robin, each with its own online-softmax state, which
+// Grid: (B * Hkv, splits).  A CTA owns a contiguous slice of the head's INT4 tiles and one of its bf16 tiles
+// (the three bf16 segments form one tile list); in a ragged batch the number of slices of a head follows its sequence's share
+// of the batch's bytes.  The copies of the first INT4 tiles are under way before anything else is looked at, the bf16 tiles go
+// first (their loads wait beside those copies); its 4 warps take tiles round-robin, each with its own online-softmax state, which
 // are merged through shared memory; the slices' (m, l, acc) go to the workspace and decode_merge_kernel
 // applies ReduceSoftmax.  Softmax is lazy: a tile only raises the running reference maximum when one of its
 // scores exceeds it by more than 2^DEC_RAISE (warp vote), so the usual tile costs four compares, four ex2
@@ -54,6 +56,8 @@ struct DecParams {
     long nQ, sQ;         // quantized rows per head (valid), rows between heads
     int k, W, n_s;       // valid rows of the vertical, window and staging buffers ...
     int sK, sW, Ws;      // ... and rows between heads
+    int B, ragged_ctas;  // ragged batch with slices cut by share: sequences, CTAs to share out (0: every head `splits` slices)
+    int tile_cost;       // KB of a quantized tile (a bf16 tile: 8)
     const int4* lens;    // optional per-sequence {quantized, vertical, window, staging} valid rows (ragged batch)
     float scale_log2;
     const uint8_t* kq; const uint8_t* vq; const float* ks; const float* vs;
@@ -157,6 +161,39 @@ __device__ __forceinline__ uint32_t word_of(const uint4& v, int i) {
 }
 // channel of accumulator row (m-tile x, lane row r, e = 0: row r, 1: row r + 8); also V's code layout
 __device__ __forceinline__ int acc_channel(int x, int r, int e) { return 64 * (x >> 2) + 8 * r + 2 * (x & 3) + e; }
+
+// valid rows of a sequence (ragged: clamped to the buffers' capacities - a bad length then shortens the walk instead of
+// leaving the allocation)
+struct DecRows {
+    long nQ;
+    int n_vl, n_win, n_stg;
+};
+__device__ __forceinline__ DecRows dec_rows(const DecParams& p, long b) {
+    DecRows d = {p.nQ, p.k, p.W, p.n_s};
+    if (p.lens) {
+        const int4 l = __ldg(p.lens + b);
+        d.nQ = min(max((long)l.x, 0L), p.sQ); d.n_vl = min(max(l.y, 0), p.sK); d.n_win = min(max(l.z, 0), p.sW); d.n_stg = min(max(l.w, 0), p.Ws);
+    }
+    return d;
+}
+__device__ __forceinline__ long dec_tiles_f(const DecRows& d) { return (d.n_vl + 15) / 16 + (d.n_stg + 15) / 16 + (d.n_win + 15) / 16; }
+// Slices of a head of sequence b: all of them, or (ragged) its share of the CTAs by bytes, at least two tiles per warp and
+// slice.  The whole warp takes part.  With the same number for every sequence the longest one held the batch up.
+__device__ __forceinline__ int dec_slices(const DecParams& p, long b) {
+    if (p.ragged_ctas == 0) return p.splits;
+    float total = 0.0f;
+    for (int s = threadIdx.x & 31; s < p.B; s += 32) {
+        const DecRows d = dec_rows(p, s);
+        total += (float)((d.nQ + 15) / 16 * p.tile_cost + dec_tiles_f(d) * 8);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+    const DecRows d = dec_rows(p, b);
+    const float mine = (float)((d.nQ + 15) / 16 * p.tile_cost + dec_tiles_f(d) * 8);
+    const int most = min(p.splits, max(1, (int)(((d.nQ + 15) / 16 + dec_tiles_f(d)) / 8)));
+    const int want = (int)(mine * (float)p.ragged_ctas / (fmaxf(total, 1.0f) * (float)(p.Hkv * p.hgroups)) + 0.5f);
+    return min(max(want, 1), most);
+}
 
 struct SoftmaxState {
     float m0, m1, l0, l1;      // heads 2j and 2j+1 of this lane: reference maximum (log2 units), partial row sum
@@ -333,14 +370,20 @@ __global__ void __launch_bounds__(DEC_THREADS, DEC_CTAS_PER_SM)
 decode_kernel(const DecParams p) {
     constexpr bool FMT8 = KVF != HYQ_FMT_INT4;             // byte-wide codes
     constexpr bool FP8 = KVF == HYQ_FMT_FP8_E4M3;
-    const int split = blockIdx.x;
-    // blockIdx.y = (b * Hkv + kv head) * hgroups + head group: up to 8 of the KV head's g query heads per CTA
-    const long unit = blockIdx.y / p.hgroups;
-    const int h_base = (int)(blockIdx.y % p.hgroups) * DEC_MAX_GROUP, g_here = min(DEC_MAX_GROUP, p.g - h_base);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 2, j = lane & 3;
+    pdl_wait();
     // the merge kernel may be made resident while this grid runs (programmatic dependent launch): it waits for
     // this grid's completion before it reads anything, so only its launch latency is taken off the path
-    asm volatile("griddepcontrol.launch_dependents;");
+    pdl_launch_dependents();
+    const int split = blockIdx.y;
+    // blockIdx.x = (b * Hkv + kv head) * hgroups + head group: up to 8 of the KV head's g query heads per CTA
+    const long unit = blockIdx.x / p.hgroups;
+    const int h_base = (int)(blockIdx.x % p.hgroups) * DEC_MAX_GROUP, g_here = min(DEC_MAX_GROUP, p.g - h_base);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 2, j = lane & 3;
+    const DecRows rows = dec_rows(p, unit / p.Hkv);
+    const long nQ = rows.nQ;
+    const int n_vl = rows.n_vl, n_win = rows.n_win, n_stg = rows.n_stg;
+    const int slices = dec_slices(p, unit / p.Hkv);
+    if (split >= slices) return;
 
     __shared__ __align__(16) uint16_t qs[DEC_MAX_GROUP][HYQ_D];      // bf16 bits, heads >= g zero
     __shared__ float red_ml[DEC_WARPS][DEC_MAX_GROUP][2];
@@ -351,6 +394,47 @@ decode_kernel(const DecParams p) {
     extern __shared__ __align__(16) uint8_t ring_mem[];
     float (*red_acc)[DEC_MAX_GROUP][HYQ_D] = reinterpret_cast<float (*)[DEC_MAX_GROUP][HYQ_D]>(ring_mem);
     static_assert(DEC_STAGES * DEC_STAGE_BYTES >= DEC_MAX_GROUP * HYQ_D * 4, "rings too small for the merge");
+
+    const long Tq = (nQ + 15) / 16;
+    const int Tvl = (n_vl + 15) / 16, Ts = (n_stg + 15) / 16;
+    // Every slice takes the same share of the INT4 tiles AND of the bf16 tiles (a bf16 tile moves four times the
+    // bytes and goes through a different loop), so all CTAs of a head carry the same mix of work.
+    const long Tf = dec_tiles_f(rows);
+    const long q_lo = Tq * split / slices, q_hi = Tq * (split + 1) / slices;
+    const long f_lo = Tf * split / slices, f_hi = Tf * (split + 1) / slices;
+
+    // This warp's quantized tiles: t0, t0 + 4, ... (behind the bf16 tiles' round-robin, so that the warps stay balanced).
+    // Tile i is copied into ring stage i % NST NST tiles ahead of its use; one commit group per tile (empty past the end)
+    // keeps the group arithmetic uniform.
+    constexpr int NST = FMT8 ? 2 : DEC_STAGES, ST_BYTES = DEC_STAGES * DEC_STAGE_BYTES / NST;
+    static_assert(!FMT8 || ST_BYTES == 4096, "an INT8 tile is 2 KB of K and 2 KB of V");
+    const long t0 = q_lo + (int)((warp - (f_hi - f_lo)) & (DEC_WARPS - 1));
+    const int n_my = t0 < q_hi ? (int)((q_hi - t0 + DEC_WARPS - 1) / DEC_WARPS) : 0;
+    const bool has_ragged = n_my > 0 && (nQ & 15) && t0 + (long)(n_my - 1) * DEC_WARPS == Tq - 1;
+    constexpr int TILE = FMT8 ? 2048 : 1024;                // bytes of K (and of V) per tile
+    const uint8_t* gk = p.kq + unit * p.sQ * (TILE / 16) + t0 * TILE + (FMT8 ? r * 128 + j * 16 : lane * 16);   // (byte codes: [16j, +16) and [64 + 16j, +16) of row r)
+    const uint8_t* gv = p.vq + unit * (p.sQ / 16) * TILE + t0 * TILE + lane * 16;
+    const int gshift = p.gshift;
+    const float* pks = p.ks + unit * (p.sQ >> (p.gshift + 4));
+    const float* pvs = p.vs + unit * (p.sQ >> (p.gshift + 4));
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(ring_mem) + warp * (DEC_STAGES * DEC_STAGE_BYTES) + lane * 16;
+    auto issue = [&](uint32_t sa) {
+        if (FMT8) {
+            cp_async16(sa, gk); cp_async16(sa + 512, gk + 64);
+            cp_async16(sa + 1024, gk + 1024); cp_async16(sa + 1536, gk + 1088);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cp_async16(sa + 2048 + i * 512, gv + i * 512);
+        } else {
+            cp_async16(sa, gk); cp_async16(sa + 512, gk + 512);
+            cp_async16(sa + 1024, gv); cp_async16(sa + 1536, gv + 512);
+        }
+        gk += DEC_WARPS * TILE; gv += DEC_WARPS * TILE;
+    };
+#pragma unroll
+    for (int s = 0; s < NST; ++s) {
+        if (s < n_my) issue(ring + s * ST_BYTES);
+        cp_async_commit();
+    }
 
     {   // q of the g heads of this KV head: thread t loads 8 channels of head t >> 4
         const int h = threadIdx.x >> 4, c8 = threadIdx.x & 15;
@@ -372,28 +456,71 @@ decode_kernel(const DecParams p) {
     }
     __syncthreads();
 
-    long nQ = p.nQ;
-    int n_vl = p.k, n_win = p.W, n_stg = p.n_s;
-    if (p.lens) {                                           // ragged batch: this sequence's own row counts
-        // (clamped to the buffers' capacities: a bad length then shortens the walk instead of leaving the allocation)
-        const int4 l = __ldg(p.lens + unit / p.Hkv);
-        nQ = min(max((long)l.x, 0L), p.sQ); n_vl = min(max(l.y, 0), p.sK); n_win = min(max(l.z, 0), p.sW); n_stg = min(max(l.w, 0), p.Ws);
-    }
-    const long Tq = (nQ + 15) / 16;
-    const int Tvl = (n_vl + 15) / 16, Ts = (n_stg + 15) / 16, Tw = (n_win + 15) / 16;
-    // Every slice takes the same share of the INT4 tiles AND of the bf16 tiles (a bf16 tile moves four times the
-    // bytes and goes through a different loop), so all CTAs of a head carry the same mix of work.
-    const long Tf = Tvl + Ts + Tw;
-    const long q_lo = Tq * split / p.splits, q_hi = Tq * (split + 1) / p.splits;
-    const long f_lo = Tq + Tf * split / p.splits, f_hi = Tq + Tf * (split + 1) / p.splits;
-
     SoftmaxState st = {-INFINITY, -INFINITY, 0.0f, 0.0f};
     float acc[8][4];
 #pragma unroll
     for (int x = 0; x < 8; ++x) acc[x][0] = acc[x][1] = acc[x][2] = acc[x][3] = 0.0f;
 
+    // ---------------- bf16 segments: vertical rows, staging, window ----------------
+    long t = f_lo + warp;
+    if (t < f_hi) {
+        uint32_t qb[16];                                   // q^T operand, bf16
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int base = 32 * (c >> 1) + 8 * j + 4 * (c & 1);
+            qb[2 * c] = *reinterpret_cast<const uint32_t*>(&qs[r][base]);
+            qb[2 * c + 1] = *reinterpret_cast<const uint32_t*>(&qs[r][base + 2]);
+        }
+        for (; t < f_hi; t += DEC_WARPS) {
+            long u = t;
+            const uint4 *kseg, *vseg;
+            int n;
+            if (u < Tvl) { kseg = p.k_vl + unit * p.sK * 16; vseg = p.v_vl + unit * p.sK * 16; n = n_vl; }
+            else if ((u -= Tvl) < Ts) { kseg = p.k_s + unit * p.Ws * 16; vseg = p.v_s + unit * p.Ws * 16; n = n_stg; }
+            else { u -= Ts; kseg = p.k_win + unit * p.sW * 16; vseg = p.v_win + unit * p.sW * 16; n = n_win; }
+            const int row0 = (int)u * 16;
+            const int ra = min(row0 + r, n - 1), rb = min(row0 + r + 8, n - 1);
+            uint4 ka[4], kb[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { ka[i] = __ldg(kseg + (long)ra * 16 + 4 * i + j); kb[i] = __ldg(kseg + (long)rb * 16 + 4 * i + j); }
+            uint4 vv[4][2];
+#pragma unroll
+            for (int sIdx = 0; sIdx < 4; ++sIdx) {
+                const int key = min(row0 + 2 * j + (sIdx & 1) + 8 * (sIdx >> 1), n - 1);
+                vv[sIdx][0] = __ldg(vseg + (long)key * 16 + r);
+                vv[sIdx][1] = __ldg(vseg + (long)key * 16 + 8 + r);
+            }
+            float c4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const int wd = 2 * (c & 1);
+                mma_bf16(c4, word_of(ka[c >> 1], wd), word_of(kb[c >> 1], wd), word_of(ka[c >> 1], wd + 1),
+                         word_of(kb[c >> 1], wd + 1), qb[2 * c], qb[2 * c + 1]);
+            }
+            float pw[4];
+            if (row0 + 16 > n) softmax_tile<true>(st, acc, c4, p.scale_log2, 0.0f, 0.0f, row0 + r < n, row0 + r + 8 < n, pw);
+            else softmax_tile<false>(st, acc, c4, p.scale_log2, 0.0f, 0.0f, true, true, pw);
+            // The weights go into the bf16 product as a sum of two bf16 numbers (p = hi + lo, 16 significant bits):
+            // with one bf16 the 2^-9 rounding of a dominant full-precision key would show in the output.
+            const uint32_t h01 = pack_bf16(pw[0], pw[1]), h23 = pack_bf16(pw[2], pw[3]);
+            const uint32_t l01 = pack_bf16(pw[0] - bf16_lo(h01), pw[1] - bf16_hi(h01));
+            const uint32_t l23 = pack_bf16(pw[2] - bf16_lo(h23), pw[3] - bf16_hi(h23));
+            const uint32_t b0 = movmatrix_trans(h01), b1 = movmatrix_trans(h23);
+            const uint32_t b0l = movmatrix_trans(l01), b1l = movmatrix_trans(l23);
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+                const uint32_t w0 = word_of(vv[0][x >> 2], x & 3), w1 = word_of(vv[1][x >> 2], x & 3);
+                const uint32_t w2 = word_of(vv[2][x >> 2], x & 3), w3 = word_of(vv[3][x >> 2], x & 3);
+                const uint32_t a0 = __byte_perm(w0, w1, 0x5410), a1 = __byte_perm(w0, w1, 0x7632);
+                const uint32_t a2 = __byte_perm(w2, w3, 0x5410), a3 = __byte_perm(w2, w3, 0x7632);
+                mma_bf16(acc[x], a0, a1, a2, a3, b0, b1);
+                mma_bf16(acc[x], a0, a1, a2, a3, b0l, b1l);
+            }
+        }
+    }
+
     // ---------------- quantized prefix ----------------
-    if (!FMT8 && q_lo + warp < q_hi) {
+    if (!FMT8 && n_my > 0) {
         uint32_t qf[16];                                   // q^T operand, fp16: k-step c -> qf[2c], qf[2c+1]
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
@@ -409,27 +536,6 @@ decode_kernel(const DecParams p) {
 #endif
             qf[2 * c] = *reinterpret_cast<const uint32_t*>(&h0);
             qf[2 * c + 1] = *reinterpret_cast<const uint32_t*>(&h1);
-        }
-        // this warp's tiles: t0, t0 + 4, ...  Tile i is copied into ring stage i % DEC_STAGES DEC_STAGES tiles ahead
-        // of its use; one commit group per tile (empty past the end) keeps the group arithmetic uniform.
-        const long t0 = q_lo + warp;
-        const int n_my = (int)((q_hi - t0 + DEC_WARPS - 1) / DEC_WARPS);
-        const bool has_ragged = (nQ & 15) && t0 + (long)(n_my - 1) * DEC_WARPS == Tq - 1;
-        const uint8_t* gk = p.kq + unit * p.sQ * 64 + t0 * 1024 + lane * 16;
-        const uint8_t* gv = p.vq + unit * (p.sQ / 16) * DEC_VTILE_BYTES + t0 * 1024 + lane * 16;
-        const int gshift = p.gshift;
-        const float* pks = p.ks + unit * (p.sQ >> (p.gshift + 4));
-        const float* pvs = p.vs + unit * (p.sQ >> (p.gshift + 4));
-        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(ring_mem) + warp * (DEC_STAGES * DEC_STAGE_BYTES) + lane * 16;
-        auto issue = [&](uint32_t stage_addr) {
-            cp_async16(stage_addr, gk); cp_async16(stage_addr + 512, gk + 512);
-            cp_async16(stage_addr + 1024, gv); cp_async16(stage_addr + 1536, gv + 512);
-            gk += DEC_WARPS * 1024; gv += DEC_WARPS * 1024;
-        };
-#pragma unroll
-        for (int s = 0; s < DEC_STAGES; ++s) {
-            if (s < n_my) issue(ring + s * DEC_STAGE_BYTES);
-            cp_async_commit();
         }
         uint32_t stage_addr = ring;
         const float kscale = p.scale_log2 * DEC_K_UNIT;
@@ -463,7 +569,7 @@ decode_kernel(const DecParams p) {
             else quant_tile<false>(A, qf, kscale, b0, b1, 16, r, st, acc);
         }
     }
-    if (FMT8 && q_lo + warp < q_hi) {
+    if (FMT8 && n_my > 0) {
         uint32_t qf[16];                                   // k-step c: channels 64 (c >> 2) + 16 j + 4 (c & 3) + {0,1} and + {2,3}
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
@@ -474,106 +580,24 @@ decode_kernel(const DecParams p) {
             qf[2 * c] = *reinterpret_cast<const uint32_t*>(&h0);
             qf[2 * c + 1] = *reinterpret_cast<const uint32_t*>(&h1);
         }
-        constexpr int ST8 = 2, ST8_BYTES = DEC_STAGES * DEC_STAGE_BYTES / ST8;      // the same ring as two 4 KB stages
-        static_assert(ST8_BYTES == 4096, "an INT8 tile is 2 KB of K and 2 KB of V");
-        const long t0 = q_lo + warp;
-        const int n_my = (int)((q_hi - t0 + DEC_WARPS - 1) / DEC_WARPS);
-        const bool has_ragged = (nQ & 15) && t0 + (long)(n_my - 1) * DEC_WARPS == Tq - 1;
-        const uint8_t* gk = p.kq + unit * p.sQ * 128 + t0 * 2048 + r * 128 + j * 16;       // bytes [16j, +16) and [64 + 16j, +16) of row r
-        const uint8_t* gv = p.vq + unit * (p.sQ / 16) * 2048 + t0 * 2048 + lane * 16;
-        const int gshift = p.gshift;
-        const float* pks = p.ks + unit * (p.sQ >> (p.gshift + 4));
-        const float* pvs = p.vs + unit * (p.sQ >> (p.gshift + 4));
-        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(ring_mem) + warp * (DEC_STAGES * DEC_STAGE_BYTES) + lane * 16;
-        auto issue = [&](uint32_t sa) {
-            cp_async16(sa, gk); cp_async16(sa + 512, gk + 64);
-            cp_async16(sa + 1024, gk + 1024); cp_async16(sa + 1536, gk + 1088);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) cp_async16(sa + 2048 + i * 512, gv + i * 512);
-            gk += DEC_WARPS * 2048; gv += DEC_WARPS * 2048;
-        };
-#pragma unroll
-        for (int s = 0; s < ST8; ++s) {
-            if (s < n_my) issue(ring + s * ST8_BYTES);
-            cp_async_commit();
-        }
         // INT8: subnormal operand (2^-24) and the +128 offset; FP8: the 2^-8 of the exponent-bias trick, no offset
         const float kscale = p.scale_log2 * (FP8 ? 256.0f : 16777216.0f);
         const float b0 = FP8 ? 0.0f : q_sum[2 * j] * (128.0f / 16777216.0f), b1 = FP8 ? 0.0f : q_sum[2 * j + 1] * (128.0f / 16777216.0f);
         for (int i = 0; i < n_my; ++i) {
-            cp_async_wait<ST8 - 1>();                       // tile i has landed
-            const uint32_t sa = ring + (i & 1) * ST8_BYTES;
+            cp_async_wait<NST - 1>();                       // tile i has landed
+            const uint32_t sa = ring + (i & 1) * ST_BYTES;
             QTile8 A;
 #pragma unroll
             for (int u = 0; u < 4; ++u) { A.k[u] = lds128(sa + u * 512); A.v[u] = lds128(sa + 2048 + u * 512); }
             const int grp = ((int)t0 + i * DEC_WARPS) >> gshift;
             A.fk = __ldg(pks + grp); A.fv = __ldg(pvs + grp);
-            if (i + ST8 < n_my) issue(sa);                  // own bytes only: no barrier
+            if (i + NST < n_my) issue(sa);                  // own bytes only: no barrier
             cp_async_commit();
             if (has_ragged && i == n_my - 1) quant_tile8<true, FP8>(A, qf, kscale, b0, b1, (int)(nQ & 15), r, st, acc);
             else quant_tile8<false, FP8>(A, qf, kscale, b0, b1, 16, r, st, acc);
         }
     }
     cp_async_wait<0>();
-
-    // ---------------- bf16 segments: vertical rows, staging, window ----------------
-    // continue the round-robin where the INT4 tiles left off so that the warps stay balanced
-    long t = f_lo + ((warp - (q_hi - q_lo)) % DEC_WARPS + DEC_WARPS) % DEC_WARPS;
-    if (t < f_hi) {
-        uint32_t qb[16];                                   // q^T operand, bf16
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int base = 32 * (c >> 1) + 8 * j + 4 * (c & 1);
-            qb[2 * c] = *reinterpret_cast<const uint32_t*>(&qs[r][base]);
-            qb[2 * c + 1] = *reinterpret_cast<const uint32_t*>(&qs[r][base + 2]);
-        }
-        for (; t < f_hi; t += DEC_WARPS) {
-            long u = t - Tq;
-            const uint4 *kseg, *vseg;
-            int n;
-            if (u < Tvl) { kseg = p.k_vl + unit * p.sK * 16; vseg = p.v_vl + unit * p.sK * 16; n = n_vl; }
-            else if ((u -= Tvl) < Ts) { kseg = p.k_s + unit * p.Ws * 16; vseg = p.v_s + unit * p.Ws * 16; n = n_stg; }
-            else { u -= Ts; kseg = p.k_win + unit * p.sW * 16; vseg = p.v_win + unit * p.sW * 16; n = n_win; }
-            const int row0 = (int)u * 16;
-            const int ra = min(row0 + r, n - 1), rb = min(row0 + r + 8, n - 1);
-            uint4 ka[4], kb[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { ka[i] = __ldg(kseg + (long)ra * 16 + 4 * i + j); kb[i] = __ldg(kseg + (long)rb * 16 + 4 * i + j); }
-            float c4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const int wd = 2 * (c & 1);
-                mma_bf16(c4, word_of(ka[c >> 1], wd), word_of(kb[c >> 1], wd), word_of(ka[c >> 1], wd + 1),
-                         word_of(kb[c >> 1], wd + 1), qb[2 * c], qb[2 * c + 1]);
-            }
-            uint4 vv[4][2];
-#pragma unroll
-            for (int sIdx = 0; sIdx < 4; ++sIdx) {
-                const int key = min(row0 + 2 * j + (sIdx & 1) + 8 * (sIdx >> 1), n - 1);
-                vv[sIdx][0] = __ldg(vseg + (long)key * 16 + r);
-                vv[sIdx][1] = __ldg(vseg + (long)key * 16 + 8 + r);
-            }
-            float pw[4];
-            if (row0 + 16 > n) softmax_tile<true>(st, acc, c4, p.scale_log2, 0.0f, 0.0f, row0 + r < n, row0 + r + 8 < n, pw);
-            else softmax_tile<false>(st, acc, c4, p.scale_log2, 0.0f, 0.0f, true, true, pw);
-            // The weights go into the bf16 product as a sum of two bf16 numbers (p = hi + lo, 16 significant bits):
-            // with one bf16 the 2^-9 rounding of a dominant full-precision key would show in the output.
-            const uint32_t h01 = pack_bf16(pw[0], pw[1]), h23 = pack_bf16(pw[2], pw[3]);
-            const uint32_t l01 = pack_bf16(pw[0] - bf16_lo(h01), pw[1] - bf16_hi(h01));
-            const uint32_t l23 = pack_bf16(pw[2] - bf16_lo(h23), pw[3] - bf16_hi(h23));
-            const uint32_t b0 = movmatrix_trans(h01), b1 = movmatrix_trans(h23);
-            const uint32_t b0l = movmatrix_trans(l01), b1l = movmatrix_trans(l23);
-#pragma unroll
-            for (int x = 0; x < 8; ++x) {
-                const uint32_t w0 = word_of(vv[0][x >> 2], x & 3), w1 = word_of(vv[1][x >> 2], x & 3);
-                const uint32_t w2 = word_of(vv[2][x >> 2], x & 3), w3 = word_of(vv[3][x >> 2], x & 3);
-                const uint32_t a0 = __byte_perm(w0, w1, 0x5410), a1 = __byte_perm(w0, w1, 0x7632);
-                const uint32_t a2 = __byte_perm(w2, w3, 0x5410), a3 = __byte_perm(w2, w3, 0x7632);
-                mma_bf16(acc[x], a0, a1, a2, a3, b0, b1);
-                mma_bf16(acc[x], a0, a1, a2, a3, b0l, b1l);
-            }
-        }
-    }
 
     // ---------------- merge the warps' states, write the slice's partial result ----------------
     __syncthreads();                                       // every warp is done with its ring
@@ -594,7 +618,7 @@ decode_kernel(const DecParams p) {
         red_acc[warp][2 * j + 1][acc_channel(x, r, 1)] = acc[x][3];
     }
     __syncthreads();
-    const long slot = (long)blockIdx.y * p.splits + split;
+    const long slot = (long)blockIdx.x * p.splits + split;
     for (int h = 0; h < g_here; ++h) {
         float M = -INFINITY;
 #pragma unroll
@@ -620,16 +644,18 @@ decode_kernel(const DecParams p) {
 // independent loads (the kernel is pure latency otherwise: it moves a few hundred KB).
 constexpr int DEC_MAX_SPLITS = 1024;
 __global__ void __launch_bounds__(HYQ_D)
-decode_merge_kernel(const float* __restrict__ part_acc, const float* __restrict__ part_ml, int g, int hgroups, int splits,
-                    int out_fp32, void* __restrict__ out, float* __restrict__ lse) {
+decode_merge_kernel(const DecParams p, int out_fp32, void* __restrict__ out, float* __restrict__ lse) {
     const long unit = blockIdx.x;                                  // (b * Hkv + kv head) * hgroups + head group
-    const int h = blockIdx.y;                                      // head within the group
+    const int h = blockIdx.y, g = p.g, hgroups = p.hgroups;        // h: head within the group
     const int h_base = (int)(unit % hgroups) * DEC_MAX_GROUP;
+    const float* part_acc = p.part_acc;
+    const float* part_ml = p.part_ml;
+    pdl_wait();                                              // the slice kernel has completed and its results are visible
     if (h_base + h >= g) return;
-    asm volatile("griddepcontrol.wait;" ::: "memory");       // the slice kernel has completed and its results are visible
+    const int splits = dec_slices(p, unit / hgroups / p.Hkv);
     __shared__ float wt[DEC_MAX_SPLITS];
     __shared__ float red[2][HYQ_D / 32];
-    const long slot0 = unit * splits * DEC_MAX_GROUP + h;          // slice s sits at slot0 + s * DEC_MAX_GROUP
+    const long slot0 = unit * p.splits * DEC_MAX_GROUP + h;        // slice s sits at slot0 + s * DEC_MAX_GROUP
     float M = -INFINITY;
     for (int s = threadIdx.x; s < splits; s += HYQ_D) {
         wt[s] = __ldg(part_ml + (slot0 + (long)s * DEC_MAX_GROUP) * 2);
@@ -683,18 +709,30 @@ int decode_auto_splits(const hyq_kv_cache& c) {
     return (int)(s < 1 ? 1 : s);
 }
 
+// Slices the grid of a ragged batch provides for: up to four times the even share, so that a sequence much longer than the
+// others can be cut as finely as its share asks (blocks beyond a head's own number of slices end at once).
+int decode_ragged_splits(const hyq_kv_cache& c) {
+    const long units = (long)c.B * c.Hkv * ((c.Hq / c.Hkv + DEC_MAX_GROUP - 1) / DEC_MAX_GROUP);
+    const long s = 4 * (148L * DEC_CTAS_PER_SM / units) + 2, T = decode_tiles(c);
+    const long most = T / 8 > 1 ? T / 8 : 1;
+    const long v = s < most ? s : most;
+    return (int)(v > 64 ? 64 : v);
+}
+
 size_t decode_workspace_bytes(const hyq_kv_cache& c, int splits) {
     const size_t slots = (size_t)c.B * c.Hkv * ((c.Hq / c.Hkv + DEC_MAX_GROUP - 1) / DEC_MAX_GROUP) * splits * DEC_MAX_GROUP;
     return align_up(slots * HYQ_D * sizeof(float), 16) + align_up(slots * 2 * sizeof(float), 16);
 }
 
-int launch_decode(const void* q, const hyq_kv_cache& c, const int32_t* lengths, float alpha, int splits, int out_dtype,
+int launch_decode(const void* q, const hyq_kv_cache& c, const int32_t* lengths, float alpha, int splits, bool auto_splits, int out_dtype,
                   void* out, float* lse, void* workspace, cudaStream_t st) {
     const CacheGeo geo = cache_geo(c);
     DecParams p;
     p.g = c.Hq / c.Hkv; p.splits = splits;
     p.hgroups = (p.g + DEC_MAX_GROUP - 1) / DEC_MAX_GROUP;
     const long units = (long)c.B * c.Hkv * p.hgroups;         // CTA rows of the grid: (b, kv head, head group)
+    p.B = c.B; p.ragged_ctas = (lengths && auto_splits) ? 148 * DEC_CTAS_PER_SM : 0;
+    p.tile_cost = c.format == HYQ_FMT_INT4 ? 2 : 4;
     p.gshift = c.group == 32 ? 1 : c.group == 64 ? 2 : 3;
     p.Hkv = c.Hkv; p.lens = reinterpret_cast<const int4*>(lengths);
     p.nQ = geo.nQ; p.sQ = geo.sQ; p.k = c.k; p.W = geo.W; p.n_s = c.n_staging;
@@ -722,23 +760,13 @@ int launch_decode(const void* q, const hyq_kv_cache& c, const int32_t* lengths, 
             return HYQ_ERR_CUDA;
         attr_set[dev] = true;
     }
-    const dim3 grid((unsigned)splits, (unsigned)units);
-    if (c.format == HYQ_FMT_INT8) decode_kernel<HYQ_FMT_INT8><<<grid, DEC_THREADS, ring_bytes, st>>>(p);
-    else if (c.format == HYQ_FMT_FP8_E4M3) decode_kernel<HYQ_FMT_FP8_E4M3><<<grid, DEC_THREADS, ring_bytes, st>>>(p);
-    else decode_kernel<HYQ_FMT_INT4><<<grid, DEC_THREADS, ring_bytes, st>>>(p);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)units, (unsigned)(p.g < DEC_MAX_GROUP ? p.g : DEC_MAX_GROUP));
-    cfg.blockDim = dim3(HYQ_D);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const float* pa = p.part_acc;
-    const float* pm = p.part_ml;
-    if (cudaLaunchKernelEx(&cfg, decode_merge_kernel, pa, pm, p.g, p.hgroups, splits, out_dtype, out, lse) != cudaSuccess) return HYQ_ERR_CUDA;
-    return launch_status();
+    const dim3 grid((unsigned)units, (unsigned)splits);
+    auto kern = c.format == HYQ_FMT_INT8 ? decode_kernel<HYQ_FMT_INT8> : c.format == HYQ_FMT_FP8_E4M3 ? decode_kernel<HYQ_FMT_FP8_E4M3>
+                                                                                                    : decode_kernel<HYQ_FMT_INT4>;
+    const int rc = launch_pdl(kern, grid, dim3(DEC_THREADS), ring_bytes, st, p);
+    if (rc != HYQ_OK) return rc;
+    return launch_pdl(decode_merge_kernel, dim3((unsigned)units, (unsigned)(p.g < DEC_MAX_GROUP ? p.g : DEC_MAX_GROUP)), dim3(HYQ_D), 0, st,
+                      p, out_dtype, out, lse);
 }
 
 }  // namespace hyq
