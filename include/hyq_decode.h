@@ -115,6 +115,17 @@ int hyq_freeze(const void* k_, const void* v, const int32_t* vl_idx, const hyq_k
 int hyq_kv_cache_append(const void* k_new, const void* v_new, const hyq_kv_cache* cache, void* stream);
 
 /* ---------------------------------------------------------------------------------------------
+ * hyq_kv_cache_append_ragged - hyq_kv_cache_append for sequence b of a ragged batch (see
+ * hyq_hybrid_attention_decode_ragged): `cache` describes the batch's allocation, k_new, v_new [Hkv,D] bf16 (device) go to
+ * row lengths_host[b][3] of the sequence's staging buffer.  lengths_host [B][4] int32 (HOST): on success its entry [b][3] is
+ * counted up, and the whole table, as it then is, is written to `lengths` [B][4] int32 (device, 16-byte aligned) by the
+ * same enqueued work; the host array is read during the call.  Errors: as hyq_kv_cache_append; b outside [0, B), or a
+ * staging fill outside [0, staging_capacity) -> INVALID_ARG (nothing is changed).
+ * ------------------------------------------------------------------------------------------- */
+int hyq_kv_cache_append_ragged(const void* k_new, const void* v_new, const hyq_kv_cache* cache, int b,
+                               int32_t* lengths_host /* host, in and out */, int32_t* lengths /* device */, void* stream);
+
+/* ---------------------------------------------------------------------------------------------
  * hyq_hybrid_attention_decode - Algorithm 3 / Section 3.3 for one token per sequence:
  *     s_j   = softmax_scale * <q[b,h], key_j>      over every cached row j of KV head h / g, where
  *             key_j / value_j = scale(group) * code for quantized rows, the bf16 row otherwise

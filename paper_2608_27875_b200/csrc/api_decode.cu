@@ -70,6 +70,19 @@ int hyq_kv_cache_append(const void* k_new, const void* v_new, const hyq_kv_cache
     return launch_cache_append(k_new, v_new, *cache, static_cast<cudaStream_t>(stream));
 }
 
+int hyq_kv_cache_append_ragged(const void* k_new, const void* v_new, const hyq_kv_cache* cache, int b, int32_t* lengths_host,
+                               int32_t* lengths, void* stream) {
+    const int rc = check_cache(cache, false);
+    if (rc != HYQ_OK) return rc;
+    if (!k_new || !v_new || !cache->k_s || !cache->v_s || !lengths_host || !lengths || b < 0 || b >= cache->B) return HYQ_ERR_INVALID_ARG;
+    const int row = lengths_host[4 * b + 3];
+    if (row < 0 || row >= cache->staging_capacity) return HYQ_ERR_INVALID_ARG;
+    if (!aligned16(k_new) || !aligned16(v_new) || !aligned16(cache->k_s) || !aligned16(cache->v_s) || !aligned16(lengths)) return HYQ_ERR_ALIGNMENT;
+    const int done = launch_cache_append_ragged(k_new, v_new, *cache, b, lengths_host, row, lengths, static_cast<cudaStream_t>(stream));
+    if (done == HYQ_OK) lengths_host[4 * b + 3] = row + 1;
+    return done;
+}
+
 int hyq_hybrid_attention_decode_workspace(const hyq_kv_cache* cache, int splits, size_t* bytes) {
     if (!bytes || splits < 0 || splits > 1024) return HYQ_ERR_INVALID_ARG;
     const int rc = check_cache(cache, false);

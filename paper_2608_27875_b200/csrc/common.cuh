@@ -24,7 +24,8 @@ static inline int launch_status() { return cudaGetLastError() == cudaSuccess ? H
 
 // Launch whose grid may be set up while the kernel before it on the stream still runs (programmatic dependent launch):
 // the kernel calls pdl_wait() before it touches memory, which returns when the one before has completed.  Every kernel of
-// this library that is launched this way calls it, so that completion is passed on along the stream.
+// this library that is launched this way calls it, so that completion is passed on along the stream; pdl_launch_dependents()
+// behind it lets the next kernel's blocks take the places that this one's last blocks leave.
 template <typename... P, typename... A>
 static inline int launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {
     cudaLaunchConfig_t cfg = {};

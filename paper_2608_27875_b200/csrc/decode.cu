@@ -651,6 +651,7 @@ decode_merge_kernel(const DecParams p, int out_fp32, void* __restrict__ out, flo
     const float* part_acc = p.part_acc;
     const float* part_ml = p.part_ml;
     pdl_wait();                                              // the slice kernel has completed and its results are visible
+    pdl_launch_dependents();
     if (h_base + h >= g) return;
     const int splits = dec_slices(p, unit / hgroups / p.Hkv);
     __shared__ float wt[DEC_MAX_SPLITS];
@@ -698,14 +699,15 @@ int decode_auto_splits(const hyq_kv_cache& c) {
     const long T = decode_tiles(c);
     long s = 148L * DEC_CTAS_PER_SM / units;            // one full wave of resident CTAs, never a second partial one
     // Few heads (small batches) cannot fill the wave with slices long enough to pay for a CTA's prologue, its partial
-    // results and their merge: aim at 64 tiles per slice (measured at batch 1: 32 slices 20.4 us, 64 slices 22.6 us),
-    // but keep at least 8 slices of two tiles per warp for short caches.
-    const long cap = T / 8 > 1 ? T / 8 : 1;
-    const long floor_s = cap < 8 ? cap : 8;
-    long want = T / 64;
+    // results and their merge: aim at 32 tiles per slice, at least 16 slices of two tiles per warp, and no more than 32 slices
+    // (64 for a few heads).  Measured, batch 1, 8 KV heads, us by slices: 2048 rows 8: 7.8, 16: 7.5, 32: 8.9; 8192 rows
+    // 8: 11.4, 16: 9.4, 32: 10.5; 32768 rows 16: 16.8, 32: 15.7, 64: 18.8; 65536 rows (INT8) 16: 36.0, 32: 30.9, 64: 35.2.
+    const long floor_s = T / 8 < 16 ? (T / 8 > 1 ? T / 8 : 1) : 16;
+    long want = T / 32, cap = 256 / units;
+    cap = cap < 32 ? 32 : cap > 64 ? 64 : cap;
     if (want < floor_s) want = floor_s;
     if (s > want) s = want;
-    if (s > 64) s = 64;
+    if (s > cap) s = cap;
     return (int)(s < 1 ? 1 : s);
 }
 

@@ -48,6 +48,8 @@ __host__ __device__ __forceinline__ int vq8_byte_offset(int key, int d) {
 
 int launch_freeze(const void* k_, const void* v, const int32_t* vl_idx, const hyq_kv_cache& c, cudaStream_t st);
 int launch_cache_append(const void* k_new, const void* v_new, const hyq_kv_cache& c, cudaStream_t st);
+int launch_cache_append_ragged(const void* k_new, const void* v_new, const hyq_kv_cache& c, int b, const int32_t* lengths_host,
+                               int row, int32_t* lengths, cudaStream_t st);
 int decode_auto_splits(const hyq_kv_cache& c);
 int decode_ragged_splits(const hyq_kv_cache& c);
 size_t decode_workspace_bytes(const hyq_kv_cache& c, int splits);

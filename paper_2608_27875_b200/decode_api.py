@@ -11,7 +11,7 @@ import torch
 from . import api
 from .workloads import FMT_INT4, FMT_INT8
 
-EXPORTS = ("hyq_kv_cache_query_sizes", "hyq_freeze", "hyq_kv_cache_append", "hyq_hybrid_attention_decode_workspace",
+EXPORTS = ("hyq_kv_cache_query_sizes", "hyq_freeze", "hyq_kv_cache_append", "hyq_kv_cache_append_ragged", "hyq_hybrid_attention_decode_workspace",
            "hyq_hybrid_attention_decode", "hyq_hybrid_attention_decode_ragged")
 
 
@@ -42,6 +42,7 @@ def _lib():
         L.hyq_kv_cache_query_sizes.argtypes = [ctypes.POINTER(KvCacheDesc), ctypes.POINTER(KvCacheSizes)]
         L.hyq_freeze.argtypes = [ctypes.c_void_p] * 3 + [ctypes.POINTER(KvCacheDesc), ctypes.c_void_p]
         L.hyq_kv_cache_append.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTER(KvCacheDesc), ctypes.c_void_p]
+        L.hyq_kv_cache_append_ragged.argtypes = [ctypes.c_void_p] * 2 + [ctypes.POINTER(KvCacheDesc), ctypes.c_int] + [ctypes.c_void_p] * 3
         L.hyq_hybrid_attention_decode_workspace.argtypes = [ctypes.POINTER(KvCacheDesc), ctypes.c_int,
                                                             ctypes.POINTER(ctypes.c_size_t)]
         L.hyq_hybrid_attention_decode.argtypes = [ctypes.c_void_p, ctypes.POINTER(KvCacheDesc), ctypes.c_float,
@@ -193,16 +194,13 @@ class RaggedKvCache:
 
     def append(self, b: int, k_new: torch.Tensor, v_new: torch.Tensor) -> None:
         """One token's rows ([Hkv,D] bf16) of sequence b into its staging buffer."""
-        n = int(self.lengths_host[b, 3])
         api._dev(k_new, torch.bfloat16, "k_new"), api._dev(v_new, torch.bfloat16, "v_new")
-        one = KvCacheDesc()
-        ctypes.memmove(ctypes.byref(one), ctypes.byref(self.batch.desc), ctypes.sizeof(KvCacheDesc))
-        one.B, one.n_staging = 1, n                      # sequence b's staging buffers as a batch of one
-        one.k_s, one.v_s = self.batch.buffers["k_s"][b].data_ptr(), self.batch.buffers["v_s"][b].data_ptr()
-        api._check(_lib().hyq_kv_cache_append(k_new.data_ptr(), v_new.data_ptr(), ctypes.byref(one), api._stream()),
-                   "hyq_kv_cache_append")
-        self.lengths_host[b, 3] = n + 1
-        self.lengths.copy_(self.lengths_host)
+        B = self.batch.desc.B
+        if not -B <= b < B:
+            raise IndexError(f"sequence {b} of a batch of {B}")
+        api._check(_lib().hyq_kv_cache_append_ragged(k_new.data_ptr(), v_new.data_ptr(), ctypes.byref(self.batch.desc), b % B,
+                                                     self.lengths_host.data_ptr(), self.lengths.data_ptr(), api._stream()),
+                   "hyq_kv_cache_append_ragged")
 
 
 def hyq_hybrid_attention_decode_ragged(q: torch.Tensor, cache: RaggedKvCache, softmax_scale: float = 0.0, splits: int = 0,

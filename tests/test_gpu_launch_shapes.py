@@ -183,3 +183,35 @@ def test_tail_mean_in_any_order_and_in_row_order(t, spread):
     Q = (Q * torch.exp2(e.float())).bfloat16()
     Q[0, 0, -1, :7] = 0.0
     _select_is_the_oracles(Q, K, 100, 150, n_tail=t)
+
+
+# ---- ragged decode ------------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("lens", [
+    [300] * 3 + [9000],                       # one sequence with almost all of the bytes: slices by share
+    [40 + 7 * i for i in range(131)],         # more sequences than one table of lengths holds, some shorter than the window
+    [17],
+])
+def test_ragged_steps_with_slices_by_share(lens):
+    """Appends to the first and the last sequence, then the attention: slices by share against the same slices for all
+    (bounds: the suite's for the decode attention), and with a workspace that has room for the latter only."""
+    from paper_2608_27875_b200 import decode_api as dapi
+    ensure_built()
+    B, Hq, Hkv, W = len(lens), 4, 2, 64
+    rc = dapi.RaggedKvCache(B, Hq, Hkv, max(lens), W, 8, staging_capacity=4)
+    for b, n in enumerate(lens):
+        rc.freeze_sequence(b, _normal((1, Hkv, n, 128), b), _normal((1, Hkv, n, 128), 500 + b), None)
+    for i, b in enumerate((0, B - 1, -1)):
+        rc.append(b, _normal((Hkv, 128), 900 + i), _normal((Hkv, 128), 950 + i))
+    assert torch.equal(rc.lengths.cpu(), rc.lengths_host) and int(rc.lengths_host[:, 3].sum()) == 3
+    with pytest.raises(IndexError):
+        rc.append(B, _normal((Hkv, 128), 1), _normal((Hkv, 128), 2))
+    q = _normal((B, Hq, 128), 7)
+    share, even = (dapi.hyq_hybrid_attention_decode_ragged(q, rc, splits=n, out_dtype=torch.float32) for n in (0, 2))
+    n = dapi.hyq_hybrid_attention_decode_workspace(rc.batch, 1)
+    small = torch.empty(n if B == 1 else max(n, dapi.hyq_hybrid_attention_decode_workspace(rc.batch, 0) // 2), dtype=torch.uint8, device="cuda")
+    outs = [share]
+    if B > 1:
+        outs.append(dapi.hyq_hybrid_attention_decode_ragged(q, rc, out_dtype=torch.float32, workspace=small))
+    for out in outs:
+        d = (out - even).abs()
+        assert float(d.max()) <= MAX_ABS_TOL and float(d.sum() / even.abs().sum()) <= MEAN_REL_TOL
