@@ -45,6 +45,7 @@ struct PreParams {
     uint8_t* tiles;
     uint32_t* redo;
     long q_vecs, k_vecs;
+    int window, fixed_tail;
 };
 
 // sequence that a row of a flattened view belongs to (member `row0`: its first row; LEN: its number of rows)
@@ -55,21 +56,29 @@ struct PreParams {
         return s_;                                                                                          \
     }())
 
-// V (bf16) -> fp16 and V^ = code * scale -> fp16; one thread per 8 channels
+// V (bf16) -> fp16 for the keys that some row's window holds and V^ = code * scale -> fp16 for those that some row sees
+// low-bit (the last 1024 rows of 32768 keys with window 1024: 52 -> 43 us); one thread per 8 channels
 template <int V_FMT>
 __device__ __forceinline__ void pre_values(const TcSeqTable& tab, const PreParams& p, long e) {
     const long row = e >> 4;
     if (row >= tab.kv_rows) return;
     const TcSeq& sq = tab.seq[HYQ_SEQ_OF(tab, kv_row0, tab.heads / tab.g * tab.seq[s_].L, row)];
     const int local = (int)row - sq.kv_row0, head = local / sq.L, tok = local - head * sq.L;
+    // The rows at positions L - Lq .. L - 1 visit window tiles from the one of `lo16` on and low-bit tiles up to the one of
+    // `hi_lq` (the kernel's tile lists).  Whole tiles, and the first tile of every head, which a ragged last tile of the head
+    // before it reaches into: a key with weight zero still enters the product, so every value row of a tile has to be finite.
+    const int a0 = sq.L - sq.Lq, lim = sq.L - p.window - 1;
+    const int lo16 = (p.fixed_tail ? min(a0, lim) : a0 - p.window) + 1, hi_lq = p.fixed_tail ? min(sq.L - 1, lim) : sq.L - 1 - p.window;
+    if (tok >= (max(lo16, 0) & ~63) || tok < 64) {
+        const uint4 w = __ldg(p.v + e);
+        p.v16[e] = make_uint4(f16x2_sat(bf16_lo(w.x), bf16_hi(w.x)), f16x2_sat(bf16_lo(w.y), bf16_hi(w.y)),
+                              f16x2_sat(bf16_lo(w.z), bf16_hi(w.z)), f16x2_sat(bf16_lo(w.w), bf16_hi(w.w)));
+    }
+    if (tok >= 64 && (hi_lq < 0 || tok > (hi_lq | 63))) return;
     const float sc = __ldg(p.v_scales + sq.ks0 + (long)head * sq.nb + (tok >> p.bt_shift));
-    const uint4 w = __ldg(p.v + e);
-    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-    uint32_t o[4], oh[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) o[c] = f16x2_sat(bf16_lo(ws[c]), bf16_hi(ws[c]));
     const uint2 cw = __ldg(p.v_codes + e);
     const uint32_t cs[2] = {cw.x, cw.y};
+    uint32_t oh[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         const uint32_t two = (cs[c >> 1] >> ((c & 1) * 16)) & 0xFFFFu;
@@ -85,7 +94,6 @@ __device__ __forceinline__ void pre_values(const TcSeqTable& tab, const PreParam
         }
         oh[c] = f16x2_sat(f0 * sc, f1 * sc);
     }
-    p.v16[e] = make_uint4(o[0], o[1], o[2], o[3]);
     p.vh16[e] = make_uint4(oh[0], oh[1], oh[2], oh[3]);
 }
 
@@ -318,6 +326,7 @@ int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, const TcSource
     if (n > 0x7fffffffL) return HYQ_ERR_UNSUPPORTED;
     p.bt_shift = a.block_tokens == 32 ? 5 : a.block_tokens == 64 ? 6 : 7;
     p.v = static_cast<const uint4*>(a.v);
+    p.window = a.window; p.fixed_tail = a.window_mode == HYQ_WINDOW_FIXED_TAIL;
     for (int s = 0; s < t.n_seq; ++s) {
         const long row0 = (long)t.seq[s].kv_row0 * 16;
         p.k_seq[s] = src ? static_cast<const uint4*>(src->k[t.seq[s].src]) : static_cast<const uint4*>(a.k_) + row0;

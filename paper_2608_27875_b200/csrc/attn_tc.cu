@@ -467,9 +467,10 @@ __device__ __forceinline__ bool tma_producer(const TcMaps& maps, const CUtensorM
 // 64 probabilities as fp16 pairs over the first 32 columns of the buffer it read.
 constexpr int TC_THREADS = 384;                     // TMA producer, 2 MMA issuers, 1 idle warp, 8 softmax warps
 constexpr float P_SUM_LIMIT = 65504.0f;             // a tile's row sum below the largest fp16 number: none of its P overflowed
-constexpr int WARM_TILES = 8;                       // tiles at the start of a walk whose maximum is always looked at, and ...
-constexpr float WARM_SPREAD = 6.0f;                 // ... how far apart (log2 units) their maxima may lie for the rest to go without
-// the same for short pieces of a shared unit (four tiles and more): two maxima say less than eight, so they have to lie
+constexpr int WARM_TILES = 4;                       // tiles at the start of a walk whose maximum is always looked at, and ...
+constexpr float WARM_SPREAD = 5.0f;                 // ... how far apart (log2 units) their maxima may lie for the rest to go without
+// (eight tiles within 6 units: the steady state starts 5 k clocks later in a CTA's 141 k at L = 8192; 535 -> 531 us)
+// the same for short pieces of a shared unit (four tiles and more): two maxima say less than four, so they have to lie
 // closer (rows with heavy tails, sigma of 7 to 10 log2 units, practically never pass: they differ by 5 on average)
 constexpr int WARM_TILES_SHORT = 2;
 constexpr float WARM_SPREAD_SHORT = 3.0f;

@@ -18,7 +18,8 @@ def _normal(shape, seed):
 
 
 def _both_kernels(Q, K, V, fmts, W, k, out_dtype=torch.float32, **kw):
-    """The tensor-core kernel's output and LSE and the CUDA-core kernel's, on the same codes and index sets."""
+    """The tensor-core kernel's output and LSE and the CUDA-core kernel's, on the same codes and index sets.  The workspace
+    starts out full of NaN patterns: nothing that the pre-pass leaves out may be read."""
     idx = api.hyq_select_vertical(Q, K, W, k) if k else None
     qz = [api.hyq_quantize_blocks(t, f) for t, f in zip((Q, K, V), fmts)]
     res = []
@@ -26,6 +27,7 @@ def _both_kernels(Q, K, V, fmts, W, k, out_dtype=torch.float32, **kw):
         lse = torch.empty(Q.shape[:3], dtype=torch.float32, device="cuda")
         status = torch.zeros(1, dtype=torch.int32, device="cuda")
         out = api.hyq_hybrid_attention_prefill(Q, K, V, qz[0][0], qz[1][0], qz[2][0], qz[0][1], qz[1][1], qz[2][1], fmts, idx, W,
+                                               workspace=torch.full((400 << 20,), 0xFF, dtype=torch.uint8, device="cuda"),
                                                out_dtype=out_dtype, lse=lse, status_word=status, impl=impl, **kw)
         assert int(status.item()) == 0
         res += [out.float(), lse]
@@ -56,6 +58,8 @@ def test_heads_interleaved_in_groups(B, Hq, Hkv, L, Lq):
     (1, 1, 3333, 3333, 100, 70, 0, torch.bfloat16),     # ragged last tile, bf16 rows from the merge and from whole pieces
     (4, 2, 9000, 777, 256, 200, 0, torch.float32),      # a query block, last unit of 9 rows
     (4, 1, 6000, 1500, 512, 100, 1, torch.bfloat16),    # fixed window: equal units
+    (2, 2, 5003, 900, 1000, 50, 1, torch.float32),      # fixed window wider than the block, ragged last key tile
+    (2, 2, 5003, 300, 2000, 50, 0, torch.float32),      # a window from the middle of a key tile on
     (1, 1, 20000, 1, 64, 300, 0, torch.float32),        # one row: most pieces have one live query tile
 ])
 def test_units_shared_by_several_ctas(fmts, Hq, Hkv, L, Lq, W, k, mode, out):
