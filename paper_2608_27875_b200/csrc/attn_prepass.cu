@@ -203,7 +203,7 @@ static int split_ctas(const hyq_attn_args& a, const TcSeq& q, int heads, long& t
     const long mean = (total + units * CTA_COST) / TC_SMS;
     if (mean > bound) bound = mean;
     long ctas = total / MIN_TILES < TC_SMS ? total / MIN_TILES : TC_SMS;
-    if (ctas < 2) return 0;
+    if (ctas < 2 || total >= 0xffffffffL / TC_SMS) return 0;     // (tile * CTAs in 32 bits)
     const long split = (total + ctas - 1) / ctas + 2 * CTA_COST + MERGE_COST;
     return split * 100 < bound * 93 ? (int)ctas : 0;
 }

@@ -166,8 +166,8 @@ __device__ __forceinline__ UnitAt unit_at(const TcSeq& q, int heads, int window,
     return u;
 }
 // first tile of CTA c of a sequence whose tiles are shared by `split` CTAs, and the CTA that works on tile x
-__host__ __device__ inline int split_begin(int tiles, int split, int c) { return (int)((long)tiles * c / split); }
-__host__ __device__ inline int split_of(int tiles, int split, int x) { return (int)((((long)x + 1) * split - 1) / tiles); }
+__host__ __device__ inline int split_begin(int tiles, int split, int c) { return (int)((uint32_t)tiles * (uint32_t)c / (uint32_t)split); }
+__host__ __device__ inline int split_of(int tiles, int split, int x) { return (int)((((uint32_t)x + 1u) * (uint32_t)split - 1u) / (uint32_t)tiles); }
 
 // Work of a CTA of a general launch, from tile `pos` of its share on (-1: from the start).  Returns in `next` the tile to
 // go on from, -1 when nothing is left.
@@ -1145,7 +1145,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
 
 // Combines the partial results of a split sequence's units: every piece s of a unit left, per row, its accumulator O_s
 // relative to its own reference maximum m_s (log2 units) and its row sum l_s; the row's result is
-// sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s with M = max_s m_s.  One warp per row; units that one CTA did alone are
+// sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s with M = max_s m_s.  A warp per row; units that one CTA did alone are
 // complete already.
 __global__ void __launch_bounds__(256)
 attn_merge_kernel(const __grid_constant__ TcSeq q, int heads, int window, int fixed_tail, const float* __restrict__ part_o,
@@ -1169,20 +1169,45 @@ attn_merge_kernel(const __grid_constant__ TcSeq q, int heads, int window, int fi
     const int row = (blockIdx.x & 31) * 8 + (threadIdx.x >> 5), i = (q.levels - 1 - level) * TC_ROWS + row;
     if (i >= q.Lq) return;
     // the unit's first piece is its CTA's first or a later one, all others are their CTAs' first
-    const int s0 = q.slot0 + 2 * c0 + (split_begin(q.tiles, q.split, c0) == first ? 0 : 1);
-    auto slot = [&](int c) -> long { return (long)(c == c0 ? s0 : q.slot0 + 2 * c) * TC_ROWS + row; };
-    float m = -INFINITY;
-    for (int c = c0; c <= c1; ++c) m = fmaxf(m, __ldg(part_ml + slot(c) * 2));
+    const int s0 = q.slot0 + 2 * c0 + (split_begin(q.tiles, q.split, c0) == first ? 0 : 1), n_pc = c1 - c0 + 1;
+    auto slot = [&](int c) -> long { return (long)(c == 0 ? s0 : q.slot0 + 2 * (c0 + c)) * TC_ROWS + row; };
+    // Lane c looks after the reference and the row sum of piece c (+ 32 ...), the first four accumulators are loaded beside them:
+    // piece by piece their latencies, and 64-bit divisions in the look-up above, were the kernel (2 heads x 2048 rows in 91
+    // pieces 7.1 us, now 4.8; 32 x 1024 rows in 148 19.1, now 17.8)
+    const float2* ml_at = reinterpret_cast<const float2*>(part_ml);
+    const float2 ml = lane < n_pc ? __ldg(ml_at + slot(lane)) : make_float2(-INFINITY, 0.0f);
+    float4 o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)                                 // (an empty piece's accumulator was not written: its weight is zero)
+        o[j] = j < n_pc ? __ldg(reinterpret_cast<const float4*>(part_o + slot(j) * HYQ_D) + lane) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    float m = ml.x;
+    for (int c = 32 + lane; c < n_pc; c += 32) m = fmaxf(m, __ldg(ml_at + slot(c)).x);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
     float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    float l = 0.0f;
-    for (int c = c0; c <= c1; ++c) {
-        const float2 ml = __ldg(reinterpret_cast<const float2*>(part_ml) + slot(c));
-        if (!(ml.y > 0.0f)) continue;                           // empty piece: its accumulator was not written
-        const float wgt = exp2f(ml.x - m);
-        const float4 o = __ldg(reinterpret_cast<const float4*>(part_o + slot(c) * HYQ_D) + lane);
-        acc.x = fmaf(wgt, o.x, acc.x); acc.y = fmaf(wgt, o.y, acc.y); acc.z = fmaf(wgt, o.z, acc.z); acc.w = fmaf(wgt, o.w, acc.w);
-        l = fmaf(wgt, ml.y, l);
+    float l = 0.0f, wgt = 0.0f;
+    for (int j0 = 0; j0 < n_pc; j0 += 4) {
+        if ((j0 & 31) == 0) {
+            const float2 v = j0 == 0 ? ml : j0 + lane < n_pc ? __ldg(ml_at + slot(j0 + lane)) : make_float2(-INFINITY, 0.0f);
+            wgt = v.y > 0.0f ? exp2f(v.x - m) : 0.0f;
+            l = fmaf(wgt, v.y, l);
+        }
+        if (j0 > 0) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (j0 + j < n_pc) o[j] = __ldg(reinterpret_cast<const float4*>(part_o + slot(j0 + j) * HYQ_D) + lane);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float wj = __shfl_sync(0xffffffffu, wgt, (j0 + j) & 31);
+            if (j0 + j < n_pc && wj > 0.0f) {
+                acc.x = fmaf(wj, o[j].x, acc.x); acc.y = fmaf(wj, o[j].y, acc.y);
+                acc.z = fmaf(wj, o[j].z, acc.z); acc.w = fmaf(wj, o[j].w, acc.w);
+            }
+        }
     }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) l += __shfl_xor_sync(0xffffffffu, l, d);
     const float inv = (l > 0.0f) ? 1.0f / l : 0.0f;
     acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
     const long orow = q.q_row0 + (long)(unit - level * heads) * q.Lq + i;
