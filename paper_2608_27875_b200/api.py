@@ -4,8 +4,10 @@ step of the path runs in the library's kernels.  There is no CPU fallback: the
 first call raises if ``libhyq.so`` has not been built."""
 from __future__ import annotations
 
+import array
 import ctypes
 import os
+import struct
 
 import torch
 
@@ -92,8 +94,8 @@ def lib() -> ctypes.CDLL:
         L.hyq_hybrid_attention_prefill_varlen.argtypes = [ctypes.POINTER(AttnArgs), ctypes.c_int, i32p, i32p, ctypes.c_void_p]
         L.hyq_hybrid_attention_prefill_varlen_workspace.argtypes = [ctypes.POINTER(AttnArgs), ctypes.c_int, i32p, i32p,
                                                                     ctypes.POINTER(ctypes.c_size_t)]
-        L.hyq_hybrid_prefill_workspace.argtypes = [ctypes.POINTER(PrefillArgs), ctypes.POINTER(ctypes.c_size_t)]
-        L.hyq_hybrid_prefill.argtypes = [ctypes.POINTER(PrefillArgs), ctypes.c_void_p]
+        L.hyq_hybrid_prefill_workspace.argtypes = [ctypes.c_void_p, ctypes.POINTER(ctypes.c_size_t)]      # (a PrefillArgs' address)
+        L.hyq_hybrid_prefill.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
         _lib = L
     return _lib
 
@@ -107,9 +109,12 @@ def _check(code: int, where: str):
         raise HyqError(code, where)
 
 
+_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
 def _stream() -> int:
     # the current stream's handle (torch.cuda.current_stream() builds a Stream object for it: 2-3 us a call)
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream(_device())
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
@@ -283,29 +288,41 @@ def hyq_hybrid_attention_prefill(q, k, v, q_codes, k_codes, v_codes, q_scales, k
     return out
 
 
-def _prefill(qs, ks, vs, B, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens, out_dtype, dev, status=None):
-    """hyq_hybrid_prefill on prompts where they lie; returns the packed results: idx, codes, scales (three each), out."""
-    n, D, total = len(lens), 128, sum(lens)
-    nb = sum([-(-L_ // block_tokens) for L_ in lens])
-    empty = torch.empty
-    idx = empty(B * Hq * sum(k_per_seq), dtype=torch.int32, device=dev)
-    codes = [empty(B * H * total * code_row_bytes(f, D), dtype=torch.uint8, device=dev) for H, f in zip((Hq, Hkv, Hkv), fmts)]
-    scales = [empty(B * H * nb, dtype=torch.float32, device=dev) for H in (Hq, Hkv, Hkv)]
-    out = empty(B * Hq * total * D, dtype=out_dtype, device=dev)
-    a = PrefillArgs(ctypes.sizeof(PrefillArgs), n, B, Hq, Hkv, D, window, 0, block_tokens, *fmts,
-                    1 if out_dtype == torch.float32 else 0, 0.0)
-    host = [_i32(lens), _i32(k_per_seq)] + [(ctypes.c_void_p * n)(*[t.data_ptr() for t in ts]) for ts in (qs, ks, vs)]   # (outlives the call)
-    a.lengths, a.k_per_seq, a.q, a.k_, a.v = (ctypes.addressof(h) for h in host)
-    a.idx, a.out = idx.data_ptr() or None, out.data_ptr()
-    a.q_codes, a.k_codes, a.v_codes = (c.data_ptr() for c in codes)
-    a.q_scales, a.k_scales, a.v_scales = (c.data_ptr() for c in scales)
-    a.status_word = None if status is None else status.data_ptr()
+# hyq_prefill_args as it lies in memory: packed at once, which takes a tenth of the time of setting a ctypes structure's fields
+_PREFILL = struct.Struct("@I12if5P11PN")
+assert _PREFILL.size == ctypes.sizeof(PrefillArgs)
+
+
+def _prefill(qs, ks, vs, B, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens, out_dtype, dev, shapes, status=None):
+    """hyq_hybrid_prefill on prompts where they lie.  Returns the packed results idx, codes (three), scales (three) and out in
+    the given shapes."""
+    n, empty = len(lens), torch.empty
+    s_idx, s_codes, s_scales, s_out = shapes
+    idx = empty(s_idx, dtype=torch.int32, device=dev)
+    qc, kc, vc = (empty(x, dtype=torch.uint8, device=dev) for x in s_codes)
+    qs_, ks_, vs_ = (empty(x, dtype=torch.float32, device=dev) for x in s_scales)
+    out = empty(s_out, dtype=out_dtype, device=dev)
+    # the argument block, and behind it the arrays that it points at
+    head = _PREFILL.size
+    buf = array.array("Q", bytes(head + 32 * n))
+    at = buf.buffer_info()[0]
+    struct.pack_into(f"@{2 * n}i{3 * n}P", buf, head, *lens, *k_per_seq, *(t.data_ptr() for ts in (qs, ks, vs) for t in ts))
+    lists = at + head + 8 * n
+
+    def pack(ws, ws_bytes):
+        _PREFILL.pack_into(buf, 0, head, n, B, Hq, Hkv, 128, window, 0, block_tokens, *fmts, 1 if out_dtype == torch.float32 else 0, 0.0,
+                           at + head, at + head + 4 * n, lists, lists + 8 * n, lists + 16 * n, idx.data_ptr(), qc.data_ptr(), kc.data_ptr(),
+                           vc.data_ptr(), qs_.data_ptr(), ks_.data_ptr(), vs_.data_ptr(), out.data_ptr(), 0,
+                           0 if status is None else status.data_ptr(), ws, ws_bytes)
+    L = lib()
     need = ctypes.c_size_t(0)
-    _check(lib().hyq_hybrid_prefill_workspace(ctypes.byref(a), ctypes.byref(need)), "hyq_hybrid_prefill_workspace")
-    ws = empty(max(need.value, 16), dtype=torch.uint8, device=dev)
-    a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
-    _check(lib().hyq_hybrid_prefill(ctypes.byref(a), _stream()), "hyq_hybrid_prefill")
-    return idx, codes, scales, out
+    pack(0, 0)
+    _check(L.hyq_hybrid_prefill_workspace(at, ctypes.byref(need)), "hyq_hybrid_prefill_workspace")
+    ws_bytes = max(need.value, 16)
+    ws = empty(ws_bytes, dtype=torch.uint8, device=dev)
+    pack(ws.data_ptr(), ws_bytes)
+    _check(L.hyq_hybrid_prefill(at, _stream()), "hyq_hybrid_prefill")
+    return idx, (qc, kc, vc), (qs_, ks_, vs_), out
 
 
 def hybrid_prefill(q, k, v, window: int, k_sel: int, fmts=(FMT_INT8, FMT_INT8, FMT_INT8), impl: int = IMPL_AUTO,
@@ -326,11 +343,12 @@ def hybrid_prefill(q, k, v, window: int, k_sel: int, fmts=(FMT_INT8, FMT_INT8, F
     if D != 128:
         raise HyqError(2, "hybrid_prefill")
     k_eff = k_sel if L - window > 0 else 0
-    idx, c, s, out = _prefill((q,), (k,), (v,), B, Hq, Hkv, (L,), window, (k_eff,), fmts, 64, out_dtype, q.device)
     nb = -(-L // 64)
-    return dict(idx=idx.view(B, Hq, k_eff), q_codes=c[0].view(B, Hq, L, -1), k_codes=c[1].view(B, Hkv, L, -1),
-                v_codes=c[2].view(B, Hkv, L, -1), q_scales=s[0].view(B, Hq, nb), k_scales=s[1].view(B, Hkv, nb),
-                v_scales=s[2].view(B, Hkv, nb), out=out.view(B, Hq, L, D))
+    row = [64 if f == FMT_INT4 else 128 for f in fmts]
+    idx, c, s, out = _prefill((q,), (k,), (v,), B, Hq, Hkv, (L,), window, (k_eff,), fmts, 64, out_dtype, q.device,
+                              ((B, Hq, k_eff), ((B, Hq, L, row[0]), (B, Hkv, L, row[1]), (B, Hkv, L, row[2])),
+                               ((B, Hq, nb), (B, Hkv, nb), (B, Hkv, nb)), (B, Hq, L, D)))
+    return dict(idx=idx, q_codes=c[0], k_codes=c[1], v_codes=c[2], q_scales=s[0], k_scales=s[1], v_scales=s[2], out=out)
 
 
 # ---- ragged batches --------------------------------------------------------------------------------------------
@@ -371,7 +389,10 @@ def hybrid_prefill_varlen(qs, ks, vs, window: int, k_per_seq, fmts=(FMT_INT8, FM
     k_per_seq = [int(k) if L_ - window > 0 else 0 for L_, k in zip(lens, k_per_seq)]
     nbs = [-(-L_ // block_tokens) for L_ in lens]
     status = torch.zeros(1, dtype=torch.int32, device=dev)
-    idx, codes, scales, out = _prefill(qs, ks, vs, 1, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens, out_dtype, dev, status)
+    total, blocks = cu[-1], sum(nbs)
+    idx, codes, scales, out = _prefill(qs, ks, vs, 1, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens, out_dtype, dev,
+                                       (Hq * sum(k_per_seq), [H * total * code_row_bytes(f, D) for H, f in zip((Hq, Hkv, Hkv), fmts)],
+                                        [H * blocks for H in (Hq, Hkv, Hkv)], Hq * total * D), status)
     res, ko, no = [], 0, 0
     for s in range(n):
         L_, k_, nb = lens[s], k_per_seq[s], nbs[s]

@@ -195,17 +195,18 @@ freeze_kernel(const __grid_constant__ FreezeParams p) {
 
 // part of a ragged batch's host table of lengths on its way to the device: by value, so that an append needs no copy from
 // pageable memory, which waits for the stream (30 us each for the 16 sequences of a step)
-constexpr int LENGTH_ROWS = 128;
-struct LengthTable {
+constexpr int LENGTH_ROWS = 128, LENGTH_FEW = 32;       // (a launch costs by the size of its parameters, too)
+template <int ROWS> struct LengthTable {
     int n;
     int4* dst;
-    int4 rows[LENGTH_ROWS];
+    int4 rows[ROWS];
 };
 
 // one new token per sequence: rows [B*Hkv][128] bf16 -> row `row` of every head's staging buffer
+template <int ROWS>
 __global__ void __launch_bounds__(FRZ_THREADS)
 append_rows_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_new, long heads, int row, int Ws,
-                   uint4* __restrict__ k_s, uint4* __restrict__ v_s, const __grid_constant__ LengthTable table) {
+                   uint4* __restrict__ k_s, uint4* __restrict__ v_s, const __grid_constant__ LengthTable<ROWS> table) {
     pdl_wait();
     pdl_launch_dependents();                 // (the attention that follows waits for this grid's end before it reads anything)
     for (int s = blockIdx.x * FRZ_THREADS + threadIdx.x; s < table.n; s += gridDim.x * FRZ_THREADS) table.dst[s] = table.rows[s];
@@ -217,32 +218,39 @@ append_rows_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_
     v_s[d] = __ldg(v_new + e);
 }
 
+template <int ROWS>
 static int launch_append(const void* k_new, const void* v_new, long heads, int row, int Ws, void* k_s, void* v_s,
-                         const LengthTable& table, cudaStream_t st) {
-    return launch_pdl(append_rows_kernel, dim3((unsigned)((heads * 16 + FRZ_THREADS - 1) / FRZ_THREADS)), dim3(FRZ_THREADS), 0, st,
+                         const LengthTable<ROWS>& table, cudaStream_t st) {
+    return launch_pdl(append_rows_kernel<ROWS>, dim3((unsigned)((heads * 16 + FRZ_THREADS - 1) / FRZ_THREADS)), dim3(FRZ_THREADS), 0, st,
                       static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), heads, row, Ws, static_cast<uint4*>(k_s),
                       static_cast<uint4*>(v_s), table);
 }
 
 int launch_cache_append(const void* k_new, const void* v_new, const hyq_kv_cache& c, cudaStream_t st) {
-    LengthTable none;
-    none.n = 0; none.dst = nullptr;
+    LengthTable<1> none{};
     return launch_append(k_new, v_new, (long)c.B * c.Hkv, c.n_staging, c.staging_capacity, c.k_s, c.v_s, none, st);
 }
 
-int launch_cache_append_ragged(const void* k_new, const void* v_new, const hyq_kv_cache& c, int b, const int32_t* lengths_host,
-                               int row, int32_t* lengths, cudaStream_t st) {
+template <int ROWS>
+static int launch_append_ragged(const void* k_new, const void* v_new, const hyq_kv_cache& c, int b, const int32_t* lengths_host,
+                                int row, int32_t* lengths, cudaStream_t st) {
     const size_t at = (size_t)b * c.Hkv * c.staging_capacity * HYQ_D * 2;
     int rc = HYQ_OK;
-    for (int s0 = 0; s0 < c.B && rc == HYQ_OK; s0 += LENGTH_ROWS) {     // (the rows themselves with the first part of the table)
-        LengthTable t;
-        t.n = c.B - s0 < LENGTH_ROWS ? c.B - s0 : LENGTH_ROWS;
+    for (int s0 = 0; s0 < c.B && rc == HYQ_OK; s0 += ROWS) {    // (the rows themselves with every part of the table)
+        LengthTable<ROWS> t;
+        t.n = c.B - s0 < ROWS ? c.B - s0 : ROWS;
         t.dst = reinterpret_cast<int4*>(lengths) + s0;
         memcpy(t.rows, lengths_host + 4 * s0, (size_t)t.n * sizeof(int4));
         if (b >= s0 && b < s0 + t.n) t.rows[b - s0].w = row + 1;
         rc = launch_append(k_new, v_new, c.Hkv, row, c.staging_capacity, static_cast<char*>(c.k_s) + at, static_cast<char*>(c.v_s) + at, t, st);
     }
     return rc;
+}
+
+int launch_cache_append_ragged(const void* k_new, const void* v_new, const hyq_kv_cache& c, int b, const int32_t* lengths_host,
+                               int row, int32_t* lengths, cudaStream_t st) {
+    return c.B <= LENGTH_FEW ? launch_append_ragged<LENGTH_FEW>(k_new, v_new, c, b, lengths_host, row, lengths, st)
+                             : launch_append_ragged<LENGTH_ROWS>(k_new, v_new, c, b, lengths_host, row, lengths, st);
 }
 
 int launch_freeze(const void* k_, const void* v, const int32_t* vl_idx, const hyq_kv_cache& c, cudaStream_t st) {

@@ -33,10 +33,11 @@ class KvCacheSizes(ctypes.Structure):
 
 
 _bound = False
+_append_ragged = None          # the library's function, once bound (a step of a batch calls it for every sequence)
 
 
 def _lib():
-    global _bound
+    global _bound, _append_ragged
     L = api.lib()
     if not _bound:
         L.hyq_kv_cache_query_sizes.argtypes = [ctypes.POINTER(KvCacheDesc), ctypes.POINTER(KvCacheSizes)]
@@ -51,6 +52,7 @@ def _lib():
         L.hyq_hybrid_attention_decode_ragged.argtypes = [ctypes.c_void_p, ctypes.POINTER(KvCacheDesc), ctypes.c_void_p,
                                                          ctypes.c_float, ctypes.c_int, ctypes.c_int, ctypes.c_void_p,
                                                          ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]
+        _append_ragged = L.hyq_kv_cache_append_ragged
         _bound = True
     return L
 
@@ -194,13 +196,18 @@ class RaggedKvCache:
 
     def append(self, b: int, k_new: torch.Tensor, v_new: torch.Tensor) -> None:
         """One token's rows ([Hkv,D] bf16) of sequence b into its staging buffer."""
-        api._dev(k_new, torch.bfloat16, "k_new"), api._dev(v_new, torch.bfloat16, "v_new")
-        B = self.batch.desc.B
+        for t, n in ((k_new, "k_new"), (v_new, "v_new")):
+            if not (t.is_cuda and t.dtype is torch.bfloat16 and t.is_contiguous()):
+                api._dev(t, torch.bfloat16, n)
+        desc = self.batch.desc
+        B = desc.B
         if not -B <= b < B:
             raise IndexError(f"sequence {b} of a batch of {B}")
-        api._check(_lib().hyq_kv_cache_append_ragged(k_new.data_ptr(), v_new.data_ptr(), ctypes.byref(self.batch.desc), b % B,
-                                                     self.lengths_host.data_ptr(), self.lengths.data_ptr(), api._stream()),
-                   "hyq_kv_cache_append_ragged")
+        rc = (_append_ragged or _lib().hyq_kv_cache_append_ragged)(
+            k_new.data_ptr(), v_new.data_ptr(), ctypes.byref(desc), b % B, self.lengths_host.data_ptr(), self.lengths.data_ptr(),
+            api._stream())
+        if rc:
+            api._check(rc, "hyq_kv_cache_append_ragged")
 
 
 def hyq_hybrid_attention_decode_ragged(q: torch.Tensor, cache: RaggedKvCache, softmax_scale: float = 0.0, splits: int = 0,
