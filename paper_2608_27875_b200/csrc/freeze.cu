@@ -8,7 +8,7 @@
 //   - copies vertical rows (by index) and window rows (a slice) as bf16.
 // What kept it from the memory's rate was the chain search -> row numbers -> loads of 16 KB per CTA, and one conversion
 // instruction per element.  One chain now serves 32 KB, all loads are issued before the first maximum, and rounding is an
-// addition: 8 x 8 heads x 32768 rows (1.38 GB moved), INT4: 295 -> 267 us.
+// addition: 8 x 8 heads x 32768 rows (1.38 GB moved), INT4: 295 -> 242 us.
 #include <string.h>
 
 #include "decode_common.cuh"
@@ -17,7 +17,7 @@
 namespace hyq {
 
 constexpr int FRZ_THREADS = 128;     // append kernel; the quantizer runs 2 * G threads (64 elements of K and of V per thread)
-constexpr int FRZ_QTHREADS_PER_SM = 640;    // quantizer threads resident per SM the register budget is set for
+constexpr int FRZ_QTHREADS_PER_SM = 768;    // quantizer threads resident per SM the register budget is set for (512: 285 us, 640: 272, 896: 262)
 
 // Source position of compacted row p: p + j with j the number of vertical indices below it,
 // i.e. the smallest j with idx[j] - j > p (idx ascending, so idx[j] - j never decreases).
