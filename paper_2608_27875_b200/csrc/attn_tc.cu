@@ -656,6 +656,10 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
     // tensor memory (warp 0), the counts of vertical keys (warps 1 and 2), the constant operand (all).
     if (warp == 0) {
         if (lane == 0) {
+            if (EXACT ? item != (int)blockIdx.x : (GENERAL && next_s >= 0)) {      // (a later piece: barriers in use may not be initialised as they are)
+                uint64_t* all = reinterpret_cast<uint64_t*>(&bars);
+                for (int i = 0; i < (int)(sizeof(TcBarriers) / sizeof(uint64_t)); ++i) mbar_inval(all + i);
+            }
             mbar_init(&bars.q_full, 1);
             for (int s = 0; s < NST; ++s) {
                 mbar_init(&bars.kv_full[s], 1);
