@@ -817,7 +817,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             // one tile of the online softmax for this thread's row: all 64 columns, in two register halves.  Returns
             // false when this warp ran into an expired wait.
             float tile_max = -INFINITY;                         // maximum of the tile last looked at (this row, log2 units)
-            auto do_tile = [&](auto range_tag, int n, float cs, uint64_t vl, bool int_scores, int lo_eff, unsigned span) -> bool {
+            auto do_tile = [&](auto range_tag, int n, float cs, uint64_t vl, bool int_scores, int lo, int hi, bool look = true) -> bool {
                 constexpr bool NEED_RANGE = decltype(range_tag)::value;
                 const uint32_t knock = int_scores ? KNOCKOUT_S32 : KNOCKOUT_F32;
                 const int nl = n - n0;                          // tile number within this CTA's slice
@@ -837,9 +837,16 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 tmem_ld32(ts, ra);
                 tmem_ld32(ts + 32, rb);
                 tmem_wait_ld();
+                // A boundary crosses the 64 columns of two tiles for the 128 rows of a query tile, so three in eight of these
+                // half tiles hold nothing for any row of the warp: their P is zero without exponentials.  Halves that
+                // every row uses in full go without the mask (8192 x 32 heads, window 512: 530.5 -> 525.3 us).
+                const bool some_a = !NEED_RANGE || __any_sync(0xffffffffu, hi >= lo && lo < 32 && hi >= 0);
+                const bool some_b = !NEED_RANGE || __any_sync(0xffffffffu, hi >= lo && hi >= 32);
                 if (NEED_RANGE) {
-                    mask_cols32(ra, 0, lo_eff, span, knock);
-                    mask_cols32(rb, 32, lo_eff, span, knock);
+                    const int lo_eff = (hi >= lo) ? lo : 4096;
+                    const unsigned span = (hi >= lo) ? (unsigned)(hi - lo) : 0u;
+                    if (!__all_sync(0xffffffffu, lo == 0 && hi >= 31)) mask_cols32(ra, 0, lo_eff, span, knock);
+                    if (!__all_sync(0xffffffffu, lo <= 32 && hi == BN - 1)) mask_cols32(rb, 32, lo_eff, span, knock);
                 }
                 // integer scores become the floats 2^23 + 2^22 + s by one integer add each (knocked-out entries
                 // become -inf); the offset is taken out again by the bias of the exponent
@@ -850,7 +857,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
 #if HYQ_TC_VARIANT_BT
                 const float csb = cs_hi;                        // the second half's factor (its own K scale with 32-token blocks)
 #endif
-                {
+                if (look) {
 #if HYQ_TC_VARIANT_BT
                 const float fa = row_max32(ra) - (int_scores ? INT_MAGIC_F : 0.0f), fb = row_max32(rb) - (int_scores ? INT_MAGIC_F : 0.0f);
                 const float mt = fmaxf((fa == -INFINITY) ? -INFINITY : fa * cs, (fb == -INFINITY) ? -INFINITY : fb * csb);
@@ -892,14 +899,21 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 const float m_eff = (m_used == -INFINITY) ? 0.0f : m_used;
                 const float bias = int_scores ? fmaf(-INT_MAGIC_F, cs, -m_eff) : -m_eff;
                 uint32_t pa[16], pb[16];
-                const float t_a = row_exp32(ra, cs, bias, pa);
+                auto exp_half = [&](bool some, const uint32_t (&raw)[32], float sc, float bi, uint32_t (&pk)[16]) -> float {
+                    if (some) return row_exp32(raw, sc, bi, pk);
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) pk[e] = 0u;
+                    return 0.0f;
+                };
+                const float t_a = exp_half(some_a, ra, cs, bias, pa);
                 tmem_st16(ts, pa);
 #if HYQ_TC_VARIANT_BT
-                const float t_b = row_exp32(rb, csb, int_scores ? fmaf(-INT_MAGIC_F, csb, -m_eff) : -m_eff, pb);
+                const float t_b = exp_half(some_b, rb, csb, int_scores ? fmaf(-INT_MAGIC_F, csb, -m_eff) : -m_eff, pb);
 #else
-                const float t_b = row_exp32(rb, cs, bias, pb);
+                const float t_b = exp_half(some_b, rb, cs, bias, pb);
 #endif
                 l_h += t_a + t_b;
+                if (!look) over |= !(t_a + t_b < P_SUM_LIMIT);
                 tmem_st16(ts + 16, pb);
                 tmem_wait_st();
                 tc_fence_before();
@@ -925,7 +939,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
 #endif
                 const auto vl = nvl;
                 prefetch_tile(n + 1);
-                return do_tile(std::false_type{}, n, cs, vl, !LOWBIT_FP8, 0, 0u);
+                return do_tile(std::false_type{}, n, cs, vl, !LOWBIT_FP8, 0, 0);
             };
             const bool brief = GENERAL && pc.slot >= 0 && n_plain_end - n0 <= 2 * WARM_TILES;
             const int n_warm = n0 + (brief ? WARM_TILES_SHORT : WARM_TILES);
@@ -1040,15 +1054,14 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
 #if HYQ_TC_VARIANT_BT
                 cs_hi = lowbit ? fmaxf(qs2 * ks_b, 1e-37f) : cs;
 #endif
-                const int lo_eff = (hi >= lo) ? lo : 4096;
-                const unsigned span = (hi >= lo) ? (unsigned)(hi - lo) : 0u;
                 // tiles that every row of this warp uses in full (most window and vertical-line tiles) need no range mask
-                // (with two threads per row both warps of a pair still meet at the same named barriers)
+                // and, in the window of a row whose low-bit pass went without them, no maximum (525.3 -> 523.3 us; vertical-line keys
+                // are the ones with the large scores, so their tiles are always looked at)
                 if (__all_sync(0xffffffffu, lo == 0 && hi == BN - 1)) {
-                    if (!do_tile(std::false_type{}, n, cs, vl, lowbit && !LOWBIT_FP8, 0, 0u)) aborted = true;
+                    if (!do_tile(std::false_type{}, n, cs, vl, lowbit && !LOWBIT_FP8, 0, 0, !warm || t < own.b_end)) aborted = true;
                     continue;
                 }
-                if (!do_tile(std::true_type{}, n, cs, vl, lowbit && !LOWBIT_FP8, lo_eff, span)) aborted = true;
+                if (!do_tile(std::true_type{}, n, cs, vl, lowbit && !LOWBIT_FP8, lo, hi)) aborted = true;
             }
 
             // ---- epilogue: the last P.V (MMAs complete in order), sum of the two halves' row sums, O / l
