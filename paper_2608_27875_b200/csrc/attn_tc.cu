@@ -839,14 +839,15 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 tmem_wait_ld();
                 // A boundary crosses the 64 columns of two tiles for the 128 rows of a query tile, so three in eight of these
                 // half tiles hold nothing for any row of the warp: their P is zero without exponentials.  Halves that
-                // every row uses in full go without the mask (8192 x 32 heads, window 512: 530.5 -> 525.3 us).
-                const bool some_a = !NEED_RANGE || __any_sync(0xffffffffu, hi >= lo && lo < 32 && hi >= 0);
-                const bool some_b = !NEED_RANGE || __any_sync(0xffffffffu, hi >= lo && hi >= 32);
+                // every row uses in full go without the mask (8192 x 32 heads, window 512: 530.5 -> 525.3 us; in the other kernels the
+                // main loop comes out slower for it: 168 rows against 32062 keys, 32 heads 378 -> 396 us).
+                const bool some_a = !NEED_RANGE || GENERAL || __any_sync(0xffffffffu, hi >= lo && lo < 32 && hi >= 0);
+                const bool some_b = !NEED_RANGE || GENERAL || __any_sync(0xffffffffu, hi >= lo && hi >= 32);
                 if (NEED_RANGE) {
                     const int lo_eff = (hi >= lo) ? lo : 4096;
                     const unsigned span = (hi >= lo) ? (unsigned)(hi - lo) : 0u;
-                    if (!__all_sync(0xffffffffu, lo == 0 && hi >= 31)) mask_cols32(ra, 0, lo_eff, span, knock);
-                    if (!__all_sync(0xffffffffu, lo <= 32 && hi == BN - 1)) mask_cols32(rb, 32, lo_eff, span, knock);
+                    if (GENERAL || !__all_sync(0xffffffffu, lo == 0 && hi >= 31)) mask_cols32(ra, 0, lo_eff, span, knock);
+                    if (GENERAL || !__all_sync(0xffffffffu, lo <= 32 && hi == BN - 1)) mask_cols32(rb, 32, lo_eff, span, knock);
                 }
                 // integer scores become the floats 2^23 + 2^22 + s by one integer add each (knocked-out entries
                 // become -inf); the offset is taken out again by the bias of the exponent
@@ -857,7 +858,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
 #if HYQ_TC_VARIANT_BT
                 const float csb = cs_hi;                        // the second half's factor (its own K scale with 32-token blocks)
 #endif
-                if (look) {
+                if (GENERAL || look) {
 #if HYQ_TC_VARIANT_BT
                 const float fa = row_max32(ra) - (int_scores ? INT_MAGIC_F : 0.0f), fb = row_max32(rb) - (int_scores ? INT_MAGIC_F : 0.0f);
                 const float mt = fmaxf((fa == -INFINITY) ? -INFINITY : fa * cs, (fb == -INFINITY) ? -INFINITY : fb * csb);
@@ -913,7 +914,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 const float t_b = exp_half(some_b, rb, cs, bias, pb);
 #endif
                 l_h += t_a + t_b;
-                if (!look) over |= !(t_a + t_b < P_SUM_LIMIT);
+                if (!GENERAL && !look) over |= !(t_a + t_b < P_SUM_LIMIT);
                 tmem_st16(ts + 16, pb);
                 tmem_wait_st();
                 tc_fence_before();
