@@ -233,3 +233,17 @@ def test_ragged_steps_with_slices_by_share(lens):
     for out in outs:
         d = (out - even).abs()
         assert float(d.max()) <= MAX_ABS_TOL and float(d.sum() / even.abs().sum()) <= MEAN_REL_TOL
+
+
+# ---- column-mass selector: query counts by which the warps share the keys, key counts around its blocks ------------
+@pytest.mark.parametrize("Hq,Hkv,Lq,Lk,W,nT,k", [
+    (2, 1, 64, 700, 64, 4, 30), (2, 2, 64, 513, 64, 5, 449), (4, 2, 64, 512, 40, 8, 20), (2, 1, 64, 769, 30, 9, 40),
+    (3, 1, 33, 1025, 33, 33, 60),
+    (2, 1, 512, 16640, 512, 512, 300),                          # a head's scores fill a group: one round of launches each
+])
+def test_mass_selector_by_query_count(Hq, Hkv, Lq, Lk, W, nT, k):
+    ensure_built()
+    import oracle
+    Q, K = _normal((1, Hq, Lq, 128), Lk).cpu(), _normal((1, Hkv, Lk, 128), Lk + 1).cpu()
+    got = api.hyq_select_vertical_mass(Q.cuda(), K.cuda(), W, k, nT).cpu().numpy()
+    np.testing.assert_array_equal(got, oracle.select_vertical_mass(wl.bits(Q), wl.bits(K), W, k, nT))
