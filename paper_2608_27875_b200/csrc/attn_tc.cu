@@ -1131,6 +1131,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                                 for (int rr = lane >> 3; rr < rows; rr += 4)
                                     *reinterpret_cast<uint4*>(static_cast<char*>(p.out) + (long)(o_y + rr) * row_bytes + col) =
                                         *reinterpret_cast<const uint4*>(buf + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
+                                if (GENERAL) fence_proxy_async();   // (the CTA's next piece loads its queries over these rows by TMA)
                                 __syncwarp();
                             }
                         }

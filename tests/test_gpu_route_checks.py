@@ -1,0 +1,18 @@
+"""GPU checks that calls keep their results, their workspaces and their pace whatever launch the library picks for them."""
+import pytest
+import torch
+
+from gpu_util import ensure_built
+from test_gpu_launch_shapes import FP8ALL, INT4FP8, INT8, _both_kernels, _close, _normal
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("fmts,out", [(INT8, torch.float32), (INT4FP8, torch.bfloat16)])
+def test_ctas_that_go_on_from_a_unit_with_a_ragged_end(fmts, out):
+    """160 units of 200 rows (eight of their last warp's 32) shared by 148 CTAs: most CTAs write such a unit's rows from the
+    buffers that their next unit's queries are loaded into."""
+    ensure_built()
+    Q, K, V = _normal((4, 40, 200, 128), 1), _normal((4, 8, 3000, 128), 2), _normal((4, 8, 3000, 128), 3)
+    for _ in range(3):
+        _close(*_both_kernels(Q, K, V, fmts, 256, 40, out))
