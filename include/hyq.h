@@ -178,8 +178,9 @@ int hyq_quantize_blocks(const void* x, int B, int H, int L, int D, int block_tok
  *   hyq_quantize_blocks writes them for a [B,Hq,Lq,D] tensor) and lse Lq entries; K, V and vl_idx are those
  *   of the whole context.  Lq = 0 or Lq = L is the whole prefill.  Lq > L -> HYQ_ERR_INVALID_ARG.
  *   (Where 256-row units of query rows are too few or too unequal to fill the GPU, the tensor-core path shares their
- *   keys out over several CTAs and merges the partial results; the workspace query accounts for their buffers.  Results do not depend on the split up to
- *   fp32 rounding.)
+ *   keys out over several CTAs and merges the partial results.  Results do not depend on the split up to fp32 rounding.)
+ *   Workspace: hyq_hybrid_attention_prefill_workspace bytes.  What the query returns is enough for the call described and for
+ *   every smaller one - fewer sequences, heads, keys, query rows or vertical keys, with the same formats and block size.
  *
  *   Window form: HYQ_WINDOW_SLIDING - key j is a window key of the row at position i iff i - j < window (every
  *   row has its own last `window` positions; the form the whole prefill needs).  HYQ_WINDOW_FIXED_TAIL -

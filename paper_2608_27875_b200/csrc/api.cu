@@ -197,7 +197,7 @@ int hyq_hybrid_attention_prefill_workspace(const hyq_attn_args* args, size_t* by
     }
     TcPlan plan;
     if (!tc_plain_plan(*args, plan)) return HYQ_ERR_UNSUPPORTED;
-    *bytes = plan.w.total;
+    *bytes = tc_query_bytes(plan);
     return HYQ_OK;
 }
 

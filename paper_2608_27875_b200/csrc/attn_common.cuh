@@ -88,6 +88,8 @@ struct TcPlan {
 bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads, int g, TcPlan& plan);
 // the plan of a plain call
 bool tc_plain_plan(const hyq_attn_args& a, TcPlan& plan);
+// workspace for a plain call and for any smaller one
+size_t tc_query_bytes(const TcPlan& plan);
 // one sequence of a ragged call as tc_make_plan takes it; Hq / Hkv times the tokens, vertical keys and blocks before it
 TcSeq tc_ragged_seq(const hyq_attn_args& a, int L, int k, size_t tokens_before, size_t k_before, size_t nb_before);
 

@@ -186,8 +186,9 @@ int launch_vl_bitmask(const int32_t* idx, long n_heads, int k, int L, int mask_w
 // mean load of an SM, and for every w at least w times the shortest of the longest 148 (w - 1) + 1 units.  Measured (attention launches, INT8, 2 heads x
 // 2048 tokens): one CTA per unit 54.6 us, shared 34.8; the last 1024 rows of 32 heads x 32768 keys (INT4): three equal
 // slices per unit 499 us, shared 435.
+constexpr long SPLIT_MIN_TILES = 4;                             // tiles per CTA at least
 static int split_ctas(const hyq_attn_args& a, const TcSeq& q, int heads, long& total) {
-    constexpr long CTA_COST = 10, MERGE_COST = 8, MIN_TILES = 4;
+    constexpr long CTA_COST = 10, MERGE_COST = 8;
     const bool ft = a.window_mode == HYQ_WINDOW_FIXED_TAIL;
     const long units = (long)q.levels * heads;
     total = 0;
@@ -202,7 +203,7 @@ static int split_ctas(const hyq_attn_args& a, const TcSeq& q, int heads, long& t
     }
     const long mean = (total + units * CTA_COST) / TC_SMS;
     if (mean > bound) bound = mean;
-    long ctas = total / MIN_TILES < TC_SMS ? total / MIN_TILES : TC_SMS;
+    long ctas = total / SPLIT_MIN_TILES < TC_SMS ? total / SPLIT_MIN_TILES : TC_SMS;
     if (ctas < 2 || total >= 0xffffffffL / TC_SMS) return 0;     // (tile * CTAs in 32 bits)
     const long split = (total + ctas - 1) / ctas + 2 * CTA_COST + MERGE_COST;
     return split * 100 < bound * 93 ? (int)ctas : 0;
@@ -287,6 +288,21 @@ bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads
     w.part_ml = slots ? take((size_t)slots * TC_ROWS * 2 * 4) : 0;
     w.total = off;
     return true;
+}
+
+// Workspace that a plain call's query returns: enough for the call itself and for every smaller one (fewer heads, keys, query
+// rows or vertical keys), so that one buffer of the largest call's size serves them all.  Everything but the partial results grows
+// with the call; those are taken at the most CTAs that a smaller call's units may be shared by, whether or not this call's are.
+size_t tc_query_bytes(const TcPlan& plan) {
+    const TcSeq& q = plan.t.tab.seq[0];
+    const long units = (long)q.levels * plan.t.tab.heads;
+    // (units of another length or alignment may have a low-bit, a vertical and a window tile more each)
+    const long by_tiles = units > 4 * TC_SMS ? TC_SMS : ((long)q.tiles + 3 * units) / SPLIT_MIN_TILES + 1;
+    const size_t slots = 2 * (size_t)(by_tiles < TC_SMS ? by_tiles : TC_SMS);
+    const TcWorkspace& w = plan.w;
+    const size_t most = (w.slots ? w.part_o : w.total) + align_up(slots * TC_ROWS * HYQ_D * 4, 1024) + align_up(slots * TC_ROWS * 2 * 4, 1024) +
+                        align_up(slots * 16, 1024);              // (the last term: their entries in the redo list)
+    return most > w.total ? most : w.total;
 }
 
 bool tc_plain_plan(const hyq_attn_args& a, TcPlan& plan) {

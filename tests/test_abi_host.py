@@ -161,3 +161,28 @@ def test_decode_side_argument_checks(lib):
     full.n_staging = 3
     assert L.hyq_kv_cache_append(0x30008, 0x40000, ctypes.byref(full), None) == 4          # misaligned rows
     assert L.hyq_hybrid_attention_decode(None, ctypes.byref(d), 0.0, 0, 0, None, None, None, 0, None) == 1
+
+
+@pytest.mark.parametrize("fmts", [(0, 0, 0), (2, 2, 1)])
+@pytest.mark.parametrize("Hq,Hkv", [(2, 2), (8, 8), (6, 2), (32, 8)])
+def test_a_workspace_for_the_longest_prompt_holds_every_shorter_one(lib, fmts, Hq, Hkv):
+    """What the varlen call demands of each prompt alone (its own query with one prompt says) against the plain query of the
+    longest.  Between them lie the lengths at which units begin and cease to be shared out over CTAs with partial results."""
+    W, pct = 256, 0.02
+    lens = [1, 63, 64, 300, 1000, 1536, 2500, 4000, 6016, 9000, 20000, 40000]
+    k_of = lambda L: int(max(0, L - W) * pct)       # noqa: E731
+    def args(L, Hq, Hkv):
+        a = _args(Hq=Hq, Hkv=Hkv, L=L, window=W, k=k_of(L), impl=api.IMPL_AUTO)
+        a.q_format, a.k_format, a.v_format = fmts
+        return a
+    n = ctypes.c_size_t(0)
+    alone = []
+    for i, L in enumerate(lens):
+        a = args(L, Hq, Hkv)
+        assert lib.hyq_hybrid_attention_prefill_varlen_workspace(ctypes.byref(a), 1, (ctypes.c_int32 * 2)(0, L),
+                                                                 (ctypes.c_int32 * 1)(k_of(L)), ctypes.byref(n)) == 0
+        alone.append(n.value)
+        for more in (1, 3):                                                   # (the query of more heads covers them, too)
+            a = args(L, more * Hq, more * Hkv)
+            assert lib.hyq_hybrid_attention_prefill_workspace(ctypes.byref(a), ctypes.byref(n)) == 0
+            assert n.value >= max(alone), (L, more)

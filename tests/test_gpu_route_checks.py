@@ -3,7 +3,8 @@ import pytest
 import torch
 
 from gpu_util import ensure_built
-from test_gpu_launch_shapes import FP8ALL, INT4FP8, INT8, _both_kernels, _close, _normal
+from paper_2608_27875_b200 import api
+from test_gpu_launch_shapes import FP8ALL, INT4FP8, INT8, _both_kernels, _close, _normal, _packed_calls
 
 pytestmark = pytest.mark.gpu
 
@@ -16,3 +17,14 @@ def test_ctas_that_go_on_from_a_unit_with_a_ragged_end(fmts, out):
     Q, K, V = _normal((4, 40, 200, 128), 1), _normal((4, 8, 3000, 128), 2), _normal((4, 8, 3000, 128), 3)
     for _ in range(3):
         _close(*_both_kernels(Q, K, V, fmts, 256, 40, out))
+
+
+def test_the_longest_prompts_workspace_is_enough_for_a_batch_with_shorter_ones():
+    """The longest prompt's units are not shared by several CTAs and leave no partial results, the shorter one's are."""
+    ensure_built()
+    Hq, W, lens = 8, 256, [6016, 1536]
+    qs, ks, vs = ([_normal((Hq, L, 128), 10 * h + n) for n, L in enumerate(lens)] for h in range(3))
+    k_per = [(L - W) // 50 for L in lens]
+    one = api.hybrid_prefill_varlen(qs, ks, vs, W, k_per, INT8)
+    for r, out in zip(one, _packed_calls(qs, ks, vs, W, k_per, INT8, False)):
+        assert torch.equal(r["out"], out)
