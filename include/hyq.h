@@ -134,7 +134,8 @@ int hyq_select_vertical_static(const void* q, const void* k_, int B, int Hq, int
  *   meant for a handful of tail queries (tens), not for the whole window.
  *
  *   Arguments, outputs and errors as hyq_select_vertical, plus: n_queries > min(window, Lq) or Lq > Lk ->
- *   INVALID_ARG.  softmax_scale 0 => 1/sqrt(D).  workspace: hyq_select_vertical_mass_workspace bytes.
+ *   INVALID_ARG.  softmax_scale 0 => 1/sqrt(D).  workspace: hyq_select_vertical_mass_workspace bytes
+ *   (enough for any call with fewer heads, keys or queries, too).
  * ------------------------------------------------------------------------------------------- */
 int hyq_select_vertical_mass_workspace(int B, int Hq, int Hkv, int Lq, int Lk, int D, int window, int n_queries,
                                        int k, size_t* bytes /* host, out */);

@@ -125,7 +125,7 @@ int hyq_select_vertical_mass_workspace(int B, int Hq, int Hkv, int Lq, int Lk, i
     int nT = 0;
     const int rc = check_select_mass(B, Hq, Hkv, Lq, Lk, D, window, n_queries, k, &nT);
     if (rc != HYQ_OK) return rc;
-    *bytes = select_mass_workspace_bytes(B, Hq, Lk, window, nT);
+    *bytes = select_mass_query_bytes(B, Hq, Lk, window, nT);
     return HYQ_OK;
 }
 

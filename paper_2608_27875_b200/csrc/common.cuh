@@ -45,7 +45,8 @@ static inline bool block_tokens_ok(int bt) { return bt == 32 || bt == 64 || bt =
 int launch_select(const void* q, const void* k, int B, int Hq, int Hkv, int Lq, int Lk, int window, int n_tail,
                   int k_sel, int32_t* idx_out, void* ws, cudaStream_t st);
 size_t select_workspace_bytes(int B, int Hq, int Lk, int window);
-size_t select_mass_workspace_bytes(int B, int Hq, int Lk, int window, int n_queries);
+size_t select_mass_workspace_bytes(int B, int Hq, int Lk, int window, int n_queries);      // of a call ...
+size_t select_mass_query_bytes(int B, int Hq, int Lk, int window, int n_queries);          // ... and of any smaller one
 int launch_select_mass(const void* q, const void* k, int B, int Hq, int Hkv, int Lq, int Lk, int window, int n_queries,
                        int k_sel, double alpha, int32_t* idx_out, void* ws, cudaStream_t st);
 int launch_select_static(const void* q, const void* k, int B, int Hq, int Hkv, int Lq, int Lk, int window, int n_tail,

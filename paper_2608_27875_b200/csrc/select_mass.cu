@@ -277,6 +277,14 @@ static MassPlan mass_plan(int B, int Hq, int Lk, int window, int n_queries) {
     return m;
 }
 size_t select_mass_workspace_bytes(int B, int Hq, int Lk, int window, int n_queries) { return mass_plan(B, Hq, Lk, window, n_queries).total(); }
+// The query's answer: never less than that of a call with fewer heads, keys or queries.  (A group's heads are a whole number, so
+// that a longer call may need less than a shorter one; here the groups are full and the statistics those of all heads.)
+size_t select_mass_query_bytes(int B, int Hq, int Lk, int window, int n_queries) {
+    const size_t P = Lk > window ? Lk - window : 0, all = (size_t)B * Hq, per_head = (size_t)n_queries * P * sizeof(double);
+    const size_t n_chunks = (Lk + MASS_KEYS - 1) / MASS_KEYS, group = per_head > (size_t)MASS_GROUP_BYTES ? per_head : (size_t)MASS_GROUP_BYTES;
+    return align_up(all * P * sizeof(double), 256) + align_up(all * per_head < group ? all * per_head : group, 256) +
+           2 * align_up(all * n_queries * n_chunks * sizeof(double), 256) + align_up(all * n_queries * 2 * sizeof(double), 256);
+}
 
 int launch_select_mass(const void* q, const void* k, int B, int Hq, int Hkv, int Lq, int Lk, int window, int n_queries,
                        int k_sel, double alpha, int32_t* idx_out, void* ws, cudaStream_t st) {

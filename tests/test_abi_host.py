@@ -186,3 +186,15 @@ def test_a_workspace_for_the_longest_prompt_holds_every_shorter_one(lib, fmts, H
             a = args(L, more * Hq, more * Hkv)
             assert lib.hyq_hybrid_attention_prefill_workspace(ctypes.byref(a), ctypes.byref(n)) == 0
             assert n.value >= max(alone), (L, more)
+
+
+def test_the_mass_selectors_workspace_grows_with_the_call(lib):
+    n = ctypes.c_size_t(0)
+    def need(Hq, Lk, nT):       # noqa: E306
+        assert lib.hyq_select_vertical_mass_workspace(1, Hq, 1, 2048, Lk, 128, 2048, nT, 100, ctypes.byref(n)) == 0
+        return n.value
+    for nT in (1, 16, 512, 2048):
+        for Hq in (1, 2, 8, 32):
+            got = [need(Hq, Lk, nT) for Lk in range(2200, 60000, 700)]
+            assert got == sorted(got), (nT, Hq)
+            assert need(Hq, 59900, nT) >= need(max(1, Hq // 2), 59900, nT) and need(Hq, 30000, nT) >= need(Hq, 30000, max(1, nT - 3))

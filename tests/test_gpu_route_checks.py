@@ -1,4 +1,6 @@
 """GPU checks that calls keep their results, their workspaces and their pace whatever launch the library picks for them."""
+import ctypes
+
 import pytest
 import torch
 
@@ -28,3 +30,14 @@ def test_the_longest_prompts_workspace_is_enough_for_a_batch_with_shorter_ones()
     one = api.hybrid_prefill_varlen(qs, ks, vs, W, k_per, INT8)
     for r, out in zip(one, _packed_calls(qs, ks, vs, W, k_per, INT8, False)):
         assert torch.equal(r["out"], out)
+
+
+def test_the_mass_selectors_workspace_of_a_longer_context_is_enough_for_a_shorter_one():
+    """512 queries: the kept scores of two heads fit a group at 11000 keys, those of one do at 15000."""
+    ensure_built()
+    q, k = _normal((1, 2, 512, 128), 1), _normal((1, 1, 15000, 128), 2)
+    n = ctypes.c_size_t(0)
+    api._check(api.lib().hyq_select_vertical_mass_workspace(1, 2, 1, 512, 15000, 128, 512, 512, 200, ctypes.byref(n)), "workspace")
+    ws = torch.empty(n.value, dtype=torch.uint8, device="cuda")
+    short = k[:, :, :11000].contiguous()
+    assert torch.equal(api.hyq_select_vertical_mass(q, short, 512, 200, 512, workspace=ws), api.hyq_select_vertical_mass(q, short, 512, 200, 512))
