@@ -858,7 +858,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
 #if HYQ_TC_VARIANT_BT
                 const float csb = cs_hi;                        // the second half's factor (its own K scale with 32-token blocks)
 #endif
-                if (GENERAL || look) {
+                if (look) {
 #if HYQ_TC_VARIANT_BT
                 const float fa = row_max32(ra) - (int_scores ? INT_MAGIC_F : 0.0f), fb = row_max32(rb) - (int_scores ? INT_MAGIC_F : 0.0f);
                 const float mt = fmaxf((fa == -INFINITY) ? -INFINITY : fa * cs, (fb == -INFINITY) ? -INFINITY : fb * csb);
@@ -914,7 +914,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 const float t_b = exp_half(some_b, rb, cs, bias, pb);
 #endif
                 l_h += t_a + t_b;
-                if (!GENERAL && !look) over |= !(t_a + t_b < P_SUM_LIMIT);
+                if (!look) over |= !(t_a + t_b < P_SUM_LIMIT);
                 tmem_st16(ts + 16, pb);
                 tmem_wait_st();
                 tc_fence_before();

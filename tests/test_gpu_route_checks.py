@@ -41,3 +41,22 @@ def test_the_mass_selectors_workspace_of_a_longer_context_is_enough_for_a_shorte
     ws = torch.empty(n.value, dtype=torch.uint8, device="cuda")
     short = k[:, :, :11000].contiguous()
     assert torch.equal(api.hyq_select_vertical_mass(q, short, 512, 200, 512, workspace=ws), api.hyq_select_vertical_mass(q, short, 512, 200, 512))
+
+
+@pytest.mark.parametrize("fmts", [INT8, FP8ALL])
+def test_a_window_key_a_little_above_the_reference_gives_the_same_bits_alone_and_in_a_batch(fmts):
+    """One window key whose score lies 12 to 16 log2 units above a row's reference: above what raises the reference where the
+    maximum is looked at, and not enough to have the piece done again where it is not.  64 heads x 2560: not shared by CTAs."""
+    ensure_built()
+    u = torch.ones(128, device="cuda") / 128 ** 0.5
+    def queries(L, seed):                                       # noqa: E306 (each query 6 units along u: one score for all rows)
+        q = _normal((64, L, 128), seed).float()
+        return (q + (6.0 - q @ u).unsqueeze(-1) * u).bfloat16()
+    lens, W = [2560, 700], 512
+    qs, (ks, vs) = [queries(L, n) for n, L in enumerate(lens)], ([_normal((1, L, 128), 10 * h + n) for n, L in enumerate(lens)] for h in (1, 2))
+    ks[0][:, 2300] = (23.0 * u).bfloat16()
+    api.hyq_test_read_attention_restarts(reset=True)
+    alone = api.hybrid_prefill(qs[0][None], ks[0][None], vs[0][None], W, 0, fmts)
+    batch = api.hybrid_prefill_varlen(qs, ks, vs, W, [0, 0], fmts)
+    assert api.hyq_test_read_attention_restarts(reset=True) == 0
+    assert torch.equal(alone["out"][0], batch[0]["out"])
