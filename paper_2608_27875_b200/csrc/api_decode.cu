@@ -116,8 +116,9 @@ int hyq_hybrid_attention_decode_ragged(const void* q, const hyq_kv_cache* cache,
     if (!q || !out || !workspace || !lengths || splits < 0 || splits > 1024) return HYQ_ERR_INVALID_ARG;
     if (out_dtype != 0 && out_dtype != 1) return HYQ_ERR_INVALID_ARG;
     if (!aligned16(q) || !aligned16(out) || !aligned16(workspace) || !aligned16(lengths)) return HYQ_ERR_ALIGNMENT;
-    // slices by share where the workspace has room for them, the same number for every sequence otherwise
-    const bool by_share = splits == 0 && workspace_bytes >= decode_workspace_bytes(*cache, decode_ragged_splits(*cache));
+    // slices by share where a wave of CTAs has more than one per head and the workspace room for them, the same number for every
+    // sequence otherwise
+    const bool by_share = splits == 0 && decode_cuts_by_share(*cache) && workspace_bytes >= decode_workspace_bytes(*cache, decode_ragged_splits(*cache));
     const int s = splits > 0 ? splits : by_share ? decode_ragged_splits(*cache) : decode_auto_splits(*cache);
     if (workspace_bytes < decode_workspace_bytes(*cache, s)) return HYQ_ERR_WORKSPACE;
     const float alpha = softmax_scale != 0.0f ? softmax_scale : 1.0f / std::sqrt((float)cache->D);

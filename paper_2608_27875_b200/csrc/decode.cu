@@ -177,58 +177,70 @@ __device__ __forceinline__ DecRows dec_rows(const DecParams& p, long b) {
     return d;
 }
 __device__ __forceinline__ long dec_tiles_f(const DecRows& d) { return (d.n_vl + 15) / 16 + (d.n_stg + 15) / 16 + (d.n_win + 15) / 16; }
-// Slices of a head of sequence b: all of them, or (ragged) as many as its bytes take in pieces of one size - the smallest size,
-// in steps of 4 %, with which the batch fits the CTAs that run at once - and at least two tiles per warp and slice.  The whole
-// warp takes part.  With the same number for every sequence the longest one held the batch up, with shares rounded to the
-// nearest a few slices too many ran alone at the end (16 sequences of 668 to 19474 rows: 51 us, 46 us, now 39).
-__device__ __forceinline__ float dec_cost(const DecParams& p, const DecRows& d) { return (float)((d.nQ + 15) / 16 * p.tile_cost + dec_tiles_f(d) * 8); }
-__device__ __forceinline__ int dec_count(const DecParams& p, const DecRows& d, float piece) {
-    const int most = min(p.splits, max(1, (int)(((d.nQ + 15) / 16 + dec_tiles_f(d)) / 8)));
-    return min(max((int)ceilf(dec_cost(p, d) / piece), 1), most);
-}
-__device__ __forceinline__ float dec_piece(const DecParams& p) {
-    const int lane = threadIdx.x & 31, heads = p.Hkv * p.hgroups;
-    const DecRows first = dec_rows(p, min(lane, p.B - 1));
-    float total = 0.0f;
-    for (int s = lane; s < p.B; s += 32) total += dec_cost(p, s == lane ? first : dec_rows(p, s));
+// Slices of a head of a ragged batch's sequence: as many as its bytes take in pieces of one size, at least two tiles per warp and
+// slice.  With the same number for every sequence the longest one held the batch up (16 x 8 heads of 4000 to 24000 rows: 52 us,
+// now 42).  The size is the one with which the batch comes to about as many slices as CTAs run at once: rounding up adds half a slice
+// per head on average, and a few too many would run alone at the end, so that 0.6 per head are taken off (16 x 8 heads of 300 to
+// 6000 rows: 0.5 19.9 us, 0.6 16.5).  Pieces below 80 KB don't pay for a CTA's prologue, its partial results and their merge (2 x 2 heads
+// of 4000 to 24000 rows: 48 KB 15.7 us, 80 14.4; 128 and more make short batches wait for their longest slice).
+constexpr float DEC_ROUND_UP = 0.6f, DEC_MIN_PIECE = 80.0f;
+__device__ __forceinline__ float dec_cost(const DecParams& p, const DecRows& d) { return (float)(((int)d.nQ + 15) / 16 * p.tile_cost + (int)dec_tiles_f(d) * 8); }
+__device__ __forceinline__ int dec_most(const DecParams& p, const DecRows& d) { return min(p.splits, max(1, (((int)d.nQ + 15) / 16 + (int)dec_tiles_f(d)) / 8)); }
+__device__ __forceinline__ int dec_count(float cost, int most, float per_piece) { return min(max((int)ceilf(cost * per_piece), 1), most); }
+// What a CTA of the slice kernel works on: unit row x = (b * Hkv + kv head) * hgroups + head group, slice `split` of `slices`
+// (0: nothing).  Ragged: the slices of all sequences are numbered through, heads innermost, so that every CTA that is started at
+// first has work.  A warp looks through the lengths once, 1 / 32 of the sequences per lane; the merge kernel does not (see there).
+// A search for the smallest piece with which the slices fit one wave exactly, by every warp and once more in the merge kernel, took
+// longer than the attention from 40 sequences on (64 x 8 heads of 100 to 700 rows: 51.0 us, with one slice for each 17.8, now 18.8).
+struct DecWork {
+    int x, split, slices;
+};
+constexpr int DEC_LANE_SEQS = 4;             // sequences per lane whose lengths stay in registers (longer batches are read twice)
+__device__ __forceinline__ DecWork dec_work(const DecParams& p) {
+    if (p.ragged_ctas == 0) return {(int)blockIdx.x, (int)blockIdx.y, p.splits};
+    const int lane = threadIdx.x & 31, heads = p.Hkv * p.hgroups, per = (p.B + 31) >> 5, s0 = lane * per;
+    float cost[DEC_LANE_SEQS], total = 0.0f;
+    int most[DEC_LANE_SEQS];
+    auto look = [&](int i, float& c, int& m) {
+        c = 0.0f; m = 0;
+        if (i < per && s0 + i < p.B) { const DecRows d = dec_rows(p, s0 + i); c = dec_cost(p, d); m = dec_most(p, d); }
+    };
+#pragma unroll
+    for (int i = 0; i < DEC_LANE_SEQS; ++i) { look(i, cost[i], most[i]); total += cost[i]; }
+    for (int i = DEC_LANE_SEQS; i < per; ++i) { float c; int m; look(i, c, m); total += c; }
+    const int at = (int)blockIdx.x / heads, h = (int)blockIdx.x - at * heads;      // the at-th slice of all sequences
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-    float piece = fmaxf(total * (float)heads / (float)p.ragged_ctas, 1.0f);
-    for (int i = 0; i < 16; ++i, piece *= 1.04f) {
-        int n = 0;
-        for (int s = lane; s < p.B; s += 32) n += dec_count(p, s == lane ? first : dec_rows(p, s), piece);
-        if (__reduce_add_sync(0xffffffffu, n) * heads <= p.ragged_ctas) break;
-    }
-    return piece;
-}
-// What a CTA of the slice kernel works on: unit row x = (b * Hkv + kv head) * hgroups + head group, slice `split` of `slices`
-// (0: nothing).  Ragged: the slices of all sequences are numbered through, so that every CTA that is started at first has work.
-struct DecWork {
-    long x;
-    int split, slices;
-};
-__device__ __forceinline__ DecWork dec_work(const DecParams& p) {
-    if (p.ragged_ctas == 0) return {(long)blockIdx.x, (int)blockIdx.y, p.splits};
-    const int lane = threadIdx.x & 31, heads = p.Hkv * p.hgroups;
-    const float piece = dec_piece(p);
-    int base = 0;
-    for (int s0 = 0; s0 < p.B; s0 += 32) {
-        const int n = s0 + lane < p.B ? dec_count(p, dec_rows(p, s0 + lane), piece) : 0;
-        int incl = n * heads;
+    const float ctas = fmaxf((float)p.ragged_ctas - DEC_ROUND_UP * (float)(p.B * heads), 0.25f * (float)p.ragged_ctas);
+    const float per_piece = fminf(__fdividef(ctas, total * (float)heads), 1.0f / DEC_MIN_PIECE);
+    int n[DEC_LANE_SEQS], sum = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const unsigned hit = __ballot_sync(0xffffffffu, base + incl > (int)blockIdx.x);
-        if (hit) {
-            const int f = __ffs(hit) - 1, slices = __shfl_sync(0xffffffffu, n, f);
-            const int r = (int)blockIdx.x - base - (__shfl_sync(0xffffffffu, incl, f) - slices * heads);
-            return {(long)(s0 + f) * heads + r % heads, r / heads, slices};
-        }
-        base += __shfl_sync(0xffffffffu, incl, 31);
+    for (int i = 0; i < DEC_LANE_SEQS; ++i) sum += n[i] = dec_count(cost[i], most[i], per_piece);
+    for (int i = DEC_LANE_SEQS; i < per; ++i) { float c; int m; look(i, c, m); sum += dec_count(c, m, per_piece); }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
     }
-    return {0, 0, 0};
+    const unsigned hit = __ballot_sync(0xffffffffu, incl > at);
+    if (hit == 0) return {0, 0, 0};
+    const int f = __ffs(hit) - 1;
+    int begin = incl - sum, seq = s0, slices = 0;             // (lane f: the sequence whose slices hold number `at`)
+#pragma unroll
+    for (int i = 0; i < DEC_LANE_SEQS; ++i)
+        if (slices == 0 && n[i] > 0) {
+            if (begin + n[i] > at) { slices = n[i]; seq = s0 + i; }
+            else begin += n[i];
+        }
+    for (int i = DEC_LANE_SEQS; lane == f && slices == 0 && i < per; ++i) {
+        float c; int m; look(i, c, m);
+        const int k = dec_count(c, m, per_piece);
+        if (begin + k > at) { slices = k; seq = s0 + i; }
+        else begin += k;
+    }
+    slices = __shfl_sync(0xffffffffu, slices, f);
+    return {__shfl_sync(0xffffffffu, seq, f) * heads + h, at - __shfl_sync(0xffffffffu, begin, f), slices};
 }
 
 struct SoftmaxState {
@@ -415,7 +427,7 @@ decode_kernel(const DecParams p) {
     const int split = wk.split, slices = wk.slices;
     // up to 8 of the KV head's g query heads per CTA
     const long unit = wk.x / p.hgroups;
-    const int h_base = (int)(wk.x % p.hgroups) * DEC_MAX_GROUP, g_here = min(DEC_MAX_GROUP, p.g - h_base);
+    const int h_base = (wk.x % p.hgroups) * DEC_MAX_GROUP, g_here = min(DEC_MAX_GROUP, p.g - h_base);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 2, j = lane & 3;
     const DecRows rows = dec_rows(p, unit / p.Hkv);
     const long nQ = rows.nQ;
@@ -654,7 +666,8 @@ decode_kernel(const DecParams p) {
         red_acc[warp][2 * j + 1][acc_channel(x, r, 1)] = acc[x][3];
     }
     __syncthreads();
-    const long slot = wk.x * p.splits + split;
+    const bool last = p.ragged_ctas && split == slices - 1;
+    const long slot = (long)wk.x * p.splits + split;
     for (int h = 0; h < g_here; ++h) {
         float M = -INFINITY;
 #pragma unroll
@@ -670,7 +683,7 @@ decode_kernel(const DecParams p) {
         p.part_acc[(slot * DEC_MAX_GROUP + h) * HYQ_D + threadIdx.x] = A;
         if (threadIdx.x == 0) {
             p.part_ml[(slot * DEC_MAX_GROUP + h) * 2] = M;
-            p.part_ml[(slot * DEC_MAX_GROUP + h) * 2 + 1] = L;
+            p.part_ml[(slot * DEC_MAX_GROUP + h) * 2 + 1] = last ? -L : L;     // (sign: the head's last slice)
         }
     }
 }
@@ -679,6 +692,7 @@ decode_kernel(const DecParams p) {
 // The slices' (m, l) pairs are staged in shared memory first so that the channel loop is a run of
 // independent loads (the kernel is pure latency otherwise: it moves a few hundred KB).
 constexpr int DEC_MAX_SPLITS = 1024;
+constexpr int DEC_RAGGED_SPLITS = 64;       // ... of a ragged batch cut by share
 __global__ void __launch_bounds__(HYQ_D)
 decode_merge_kernel(const DecParams p, int out_fp32, void* __restrict__ out, float* __restrict__ lse) {
     const long unit = blockIdx.x;                                  // (b * Hkv + kv head) * hgroups + head group
@@ -689,10 +703,21 @@ decode_merge_kernel(const DecParams p, int out_fp32, void* __restrict__ out, flo
     pdl_wait();                                              // the slice kernel has completed and its results are visible
     pdl_launch_dependents();
     if (h_base + h >= g) return;
-    const int splits = p.ragged_ctas ? dec_count(p, dec_rows(p, unit / hgroups / p.Hkv), dec_piece(p)) : p.splits;
+    int splits = p.splits;
     __shared__ float wt[DEC_MAX_SPLITS];
     __shared__ float red[2][HYQ_D / 32];
+    __shared__ int n_end[2];
     const long slot0 = unit * p.splits * DEC_MAX_GROUP + h;        // slice s sits at slot0 + s * DEC_MAX_GROUP
+    if (p.ragged_ctas) {                                           // the first entry with the sign is the last one written
+        static_assert(DEC_RAGGED_SPLITS <= 64, "two warps look");
+        if (threadIdx.x < 64) {
+            const bool end = (int)threadIdx.x < p.splits && (__float_as_uint(__ldg(part_ml + (slot0 + (long)threadIdx.x * DEC_MAX_GROUP) * 2 + 1)) >> 31);
+            const unsigned b = __ballot_sync(0xffffffffu, end);
+            if ((threadIdx.x & 31) == 0) n_end[threadIdx.x >> 5] = b ? (int)threadIdx.x + __ffs(b) : p.splits;
+        }
+        __syncthreads();
+        splits = min(n_end[0], n_end[1]);
+    }
     float M = -INFINITY;
     for (int s = threadIdx.x; s < splits; s += HYQ_D) {
         wt[s] = __ldg(part_ml + (slot0 + (long)s * DEC_MAX_GROUP) * 2);
@@ -706,7 +731,7 @@ decode_merge_kernel(const DecParams p, int out_fp32, void* __restrict__ out, flo
     float L = 0.0f;
     for (int s = threadIdx.x; s < splits; s += HYQ_D) {
         const float w = wt[s] == -INFINITY ? 0.0f : ex2(wt[s] - M);
-        L += __ldg(part_ml + (slot0 + (long)s * DEC_MAX_GROUP) * 2 + 1) * w;
+        L += fabsf(__ldg(part_ml + (slot0 + (long)s * DEC_MAX_GROUP) * 2 + 1)) * w;
         wt[s] = w;
     }
 #pragma unroll
@@ -747,6 +772,12 @@ int decode_auto_splits(const hyq_kv_cache& c) {
     return (int)(s < 1 ? 1 : s);
 }
 
+// With more heads than CTAs run at once a head gets one slice either way, unless it is several times the average, and looking through
+// the lengths in every CTA costs more than it gives (150 x 8 heads of 100 to 700 rows: 41.8 us by share, 34.5; 300 x 2: 27.6, 18.6).
+bool decode_cuts_by_share(const hyq_kv_cache& c) {
+    return (long)c.B * c.Hkv * ((c.Hq / c.Hkv + DEC_MAX_GROUP - 1) / DEC_MAX_GROUP) <= 148L * DEC_CTAS_PER_SM;
+}
+
 // Slices the grid of a ragged batch provides for: up to four times the even share, so that a sequence much longer than the
 // others can be cut as finely as its share asks.
 int decode_ragged_splits(const hyq_kv_cache& c) {
@@ -754,7 +785,7 @@ int decode_ragged_splits(const hyq_kv_cache& c) {
     const long s = 4 * (148L * DEC_CTAS_PER_SM / units) + 2, T = decode_tiles(c);
     const long most = T / 8 > 1 ? T / 8 : 1;
     const long v = s < most ? s : most;
-    return (int)(v > 64 ? 64 : v);
+    return (int)(v > DEC_RAGGED_SPLITS ? DEC_RAGGED_SPLITS : v);
 }
 
 size_t decode_workspace_bytes(const hyq_kv_cache& c, int splits) {
@@ -798,7 +829,9 @@ int launch_decode(const void* q, const hyq_kv_cache& c, const int32_t* lengths, 
             return HYQ_ERR_CUDA;
         attr_set[dev] = true;
     }
-    const dim3 grid = p.ragged_ctas ? dim3((unsigned)(p.ragged_ctas + units)) : dim3((unsigned)units, (unsigned)splits);   // (no more than that: dec_piece)
+    // (ragged: rounding up adds less than a slice per head to the CTAs that run at once, and no head has more than `splits`)
+    const long most = p.ragged_ctas + units < units * splits ? p.ragged_ctas + units : units * splits;
+    const dim3 grid = p.ragged_ctas ? dim3((unsigned)most) : dim3((unsigned)units, (unsigned)splits);
     auto kern = c.format == HYQ_FMT_INT8 ? decode_kernel<HYQ_FMT_INT8> : c.format == HYQ_FMT_FP8_E4M3 ? decode_kernel<HYQ_FMT_FP8_E4M3>
                                                                                                     : decode_kernel<HYQ_FMT_INT4>;
     const int rc = launch_pdl(kern, grid, dim3(DEC_THREADS), ring_bytes, st, p);

@@ -52,6 +52,7 @@ int launch_cache_append_ragged(const void* k_new, const void* v_new, const hyq_k
                                int row, int32_t* lengths, cudaStream_t st);
 int decode_auto_splits(const hyq_kv_cache& c);
 int decode_ragged_splits(const hyq_kv_cache& c);
+bool decode_cuts_by_share(const hyq_kv_cache& c);      // whether a ragged batch's heads get slices by their share of the bytes
 size_t decode_workspace_bytes(const hyq_kv_cache& c, int splits);
 int launch_decode(const void* q, const hyq_kv_cache& c, const int32_t* lengths, float alpha, int splits, bool auto_splits, int out_dtype,
                   void* out, float* lse, void* workspace, cudaStream_t st);

@@ -4,8 +4,8 @@ import ctypes
 import pytest
 import torch
 
-from gpu_util import ensure_built
-from paper_2608_27875_b200 import api
+from gpu_util import MAX_ABS_TOL, MEAN_REL_TOL, ensure_built
+from paper_2608_27875_b200 import api, decode_api as dapi
 from test_gpu_launch_shapes import FP8ALL, INT4FP8, INT8, _both_kernels, _close, _normal, _packed_calls
 
 pytestmark = pytest.mark.gpu
@@ -60,3 +60,41 @@ def test_a_window_key_a_little_above_the_reference_gives_the_same_bits_alone_and
     batch = api.hybrid_prefill_varlen(qs, ks, vs, W, [0, 0], fmts)
     assert api.hyq_test_read_attention_restarts(reset=True) == 0
     assert torch.equal(alone["out"][0], batch[0]["out"])
+
+
+def _ragged_cache(lens, Hkv, W=128):
+    rc = dapi.RaggedKvCache(len(lens), 4 * Hkv, Hkv, max(lens), W, 8)
+    for b, n in enumerate(lens):
+        rc.freeze_sequence(b, _normal((1, Hkv, n, 128), b), _normal((1, Hkv, n, 128), 1000 + b), None)
+    return rc, _normal((len(lens), 4 * Hkv, 128), 7)
+
+
+def _median_us(calls, n=20, rounds=5):
+    """Median device time of each call, the calls in turn."""
+    times = [[] for _ in calls]
+    for r in range(rounds + 1):
+        for t, f in zip(times, calls):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(n):
+                f()
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b) / n * 1e3)
+    return [sorted(t[1:])[rounds // 2] for t in times]
+
+
+@pytest.mark.parametrize("n,Hkv", [(64, 8), (74, 8), (100, 8), (300, 2)])
+def test_large_ragged_batches_take_no_longer_than_with_one_slice_each(n, Hkv):
+    """Sequences of 100 to 700 rows, a slice per head whichever way they are cut: what a CTA spends on finding its slice may not
+    show (bound: half as long again; the search that every CTA once made took 1.9 to 25 times as long)."""
+    ensure_built()
+    lens = [100 + (97 * b) % 600 for b in range(n)]
+    rc, q = _ragged_cache(lens, Hkv)
+    outs = [torch.empty(n, 4 * Hkv, 128, device="cuda") for _ in range(2)]
+    ws = [torch.empty(dapi.hyq_hybrid_attention_decode_workspace(rc.batch, s), dtype=torch.uint8, device="cuda") for s in (0, 1)]
+    calls = [lambda s=s: dapi.hyq_hybrid_attention_decode_ragged(q, rc, splits=s, out=outs[s], workspace=ws[s]) for s in (0, 1)]
+    share, one = _median_us(calls)
+    assert share <= 1.5 * one, (share, one)
+    d = (outs[0] - outs[1]).abs()
+    assert float(d.max()) <= MAX_ABS_TOL and float(d.sum() / outs[1].abs().sum()) <= MEAN_REL_TOL
