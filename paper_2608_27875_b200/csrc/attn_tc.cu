@@ -766,7 +766,6 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             const int i = sq.i0 + r;                           // row of the query block ...
             const int ia = i + off;                             // ... and its position among the keys
             const bool row_live = i < L;
-            const bool ragged = sq.i0 + BM > L;
             const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
             const uint32_t to = tmem + tm_o(q) + lane_addr, ts0 = tmem + tm_s(q) + lane_addr;
 #if HYQ_TC_VARIANT_BT
@@ -923,8 +922,11 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 return true;
             };
 
-            // ---- low-bit tiles that lie wholly below every row's window: no range mask, no bounds to compute
-            const int n_plain = ragged ? 0 : min(own.a_end, max(0, (qhi(sq.i0 + off) + 1) / BN));
+            // ---- low-bit tiles that lie wholly below every row's window: no range mask, no bounds to compute.  (Rows past the end
+            // take part: their scale is zero, so their scores are too, and nothing of them is stored.  Masked, a last query tile went
+            // through all its keys at half the pace, and its CTA with it: the last 2000 rows of 20000 keys, 32 heads 1101 us, of
+            // 2048 rows 647.)
+            const int n_plain = min(own.a_end, max(0, (qhi(sq.i0 + off) + 1) / BN));
             int n = n0;
             // First launch: the first WARM_TILES tiles are looked at in full.  If the maxima of these tiles lie close together
             // for every row of the warp (scores without heavy tails: none of the later ones will be 2^16 above the reference),

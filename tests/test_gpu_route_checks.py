@@ -98,3 +98,19 @@ def test_large_ragged_batches_take_no_longer_than_with_one_slice_each(n, Hkv):
     assert share <= 1.5 * one, (share, one)
     d = (outs[0] - outs[1]).abs()
     assert float(d.max()) <= MAX_ABS_TOL and float(d.sum() / outs[1].abs().sum()) <= MEAN_REL_TOL
+
+
+def _block_call(Q, K, V, fmts, W, k):
+    idx = api.hyq_select_vertical(Q, K, W, k)
+    qz = [api.hyq_quantize_blocks(t, f) for t, f in zip((Q, K, V), fmts)]
+    out = torch.empty(Q.shape, device="cuda")
+    return lambda: api.hyq_hybrid_attention_prefill(Q, K, V, qz[0][0], qz[1][0], qz[2][0], qz[0][1], qz[1][1], qz[2][1], fmts, idx, W, out=out)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,L,Lq,fmts", [(1, 32, 8, 20000, 2000, INT8), (2, 32, 4, 20000, 1000, FP8ALL), (1, 40, 8, 12000, 3001, INT4FP8)])
+def test_a_query_block_with_a_ragged_last_tile_takes_no_longer_than_a_full_one(B, Hq, Hkv, L, Lq, fmts):
+    """Against the next multiple of 256 rows (bound: a fifth more; with its ragged tiles at half the pace 1.6 to 1.9 times)."""
+    ensure_built()
+    K, V = _normal((B, Hkv, L, 128), 2), _normal((B, Hkv, L, 128), 3)
+    short, full = _median_us([_block_call(_normal((B, Hq, n, 128), 1), K, V, fmts, 512, 390) for n in (Lq, -(-Lq // 256) * 256)], n=5, rounds=5)
+    assert short <= 1.2 * full, (short, full)
