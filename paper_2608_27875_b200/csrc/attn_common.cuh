@@ -26,7 +26,8 @@ struct TcSeq {
     int split;                              // CTAs that share the sequence's units tile by tile (0: one CTA per unit)
     int cta0, slot0;                        // split: first CTA behind the unsplit units, first slot for partial results ...
     int src;                                // the sequence's number in the caller's order
-    int tiles;                              // ... and key tiles of all its units together (as tc_unit_tiles counts them)
+    int tiles;                              // ... and key tiles of all its units together (as tc_unit_tiles counts them),
+    int lead;                               // each unit counted `lead` tiles longer than it is: the cost of beginning it
 };
 
 struct TcSeqTable {

@@ -181,32 +181,40 @@ int launch_vl_bitmask(const int32_t* idx, long n_heads, int k, int L, int mask_w
 
 // ---------------------------------------------------------------------------------------------
 // Whether a sequence's units are shared out over CTAs tile by tile (each CTA a contiguous share of the sequence's key
-// tiles, units longest first), and over how many CTAs.  In units of a key tile (about 0.75 us): a CTA costs about 10 tiles
-// beside its keys, a split about as much again for partial results and their merge.  One CTA per unit takes at least the
+// tiles, units longest first), and over how many CTAs.  In units of a key tile (about 0.75 us): beginning a piece of work costs about
+// 10 tiles beside its keys, so a unit counts for that much more in the shares (without it a CTA at the end of the list got a dozen
+// short units: 16 heads x 7282 tokens 452 us, one CTA per unit 222) - unless the shares are small, with two pieces each at
+// most; the merge costs by the partial results that it reads.  One CTA per unit takes at least the
 // mean load of an SM, and for every w at least w times the shortest of the longest 148 (w - 1) + 1 units.  Measured (attention launches, INT8, 2 heads x
-// 2048 tokens): one CTA per unit 54.6 us, shared 34.8; the last 1024 rows of 32 heads x 32768 keys (INT4): three equal
-// slices per unit 499 us, shared 435.
+// 2048 tokens): one CTA per unit 54.6 us, shared 34.8; over 60 blocks and prompts of 2 to 80 heads the rule's choice takes at most
+// 1.05 times the better one's time.  Fills q.split, q.tiles and q.lead.
 constexpr long SPLIT_MIN_TILES = 4;                             // tiles per CTA at least
-static int split_ctas(const hyq_attn_args& a, const TcSeq& q, int heads, long& total) {
-    constexpr long CTA_COST = 10, MERGE_COST = 8;
+static void plan_split(const hyq_attn_args& a, TcSeq& q, int heads) {
+    constexpr long PIECE_COST = 10, LEAD_MIN_TILES = 20;
     const bool ft = a.window_mode == HYQ_WINDOW_FIXED_TAIL;
     const long units = (long)q.levels * heads;
-    total = 0;
-    if (units > 4 * TC_SMS) return 0;                           // enough units for the longest-first order to balance
-    long bound = 0, seen = 0;
+    q.split = q.tiles = q.lead = 0;
+    if (units > 4 * TC_SMS) return;                             // enough units for the longest-first order to balance
+    long bound = 0, seen = 0, total = 0;
     for (int l = 0; l < q.levels; ++l) {
         const long t = tc_unit_tiles(q.L, q.Lq, q.k, a.window, ft, q.levels - 1 - l);
         const long waves = (seen + heads + TC_SMS - 1) / TC_SMS;         // some SM runs as many of the units seen so far
-        if (waves * (t + CTA_COST) > bound) bound = waves * (t + CTA_COST);
+        if (waves * (t + PIECE_COST) > bound) bound = waves * (t + PIECE_COST);
         total += heads * t;
         seen += heads;
     }
-    const long mean = (total + units * CTA_COST) / TC_SMS;
+    const long mean = (total + units * PIECE_COST) / TC_SMS;
     if (mean > bound) bound = mean;
-    long ctas = total / SPLIT_MIN_TILES < TC_SMS ? total / SPLIT_MIN_TILES : TC_SMS;
-    if (ctas < 2 || total >= 0xffffffffL / TC_SMS) return 0;     // (tile * CTAs in 32 bits)
-    const long split = (total + ctas - 1) / ctas + 2 * CTA_COST + MERGE_COST;
-    return split * 100 < bound * 93 ? (int)ctas : 0;
+    const long ctas = total / SPLIT_MIN_TILES < TC_SMS ? total / SPLIT_MIN_TILES : TC_SMS;
+    const long lead = ctas > 0 && total / ctas >= LEAD_MIN_TILES ? PIECE_COST : 0;
+    total += lead * units;
+    const bool fits = total < 0xffffffffL / TC_SMS;             // (tile * CTAs in 32 bits)
+    q.tiles = fits ? (int)total : 0x7fffffff;
+    if (ctas < 2 || !fits) return;
+    const long merge = 3 + (ctas + (units < ctas ? units : ctas)) / 16;
+    const long split = (total + ctas - 1) / ctas + (lead ? 1 : 2) * PIECE_COST + merge;
+    if (split * 100 >= bound * 93) return;
+    q.split = (int)ctas; q.lead = (int)lead;
 }
 
 bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads, int g, TcPlan& plan) {
@@ -220,12 +228,10 @@ bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads
     for (int s = 0; s < n_seq; ++s) {
         TcSeq& q = all[s] = seq[s];
         q.src = s;
-        long total;
         q.levels = (q.Lq + TC_ROWS - 1) / TC_ROWS;
         q.nb = (q.L + bt - 1) / bt; q.nbq = (q.Lq + bt - 1) / bt;
         q.mask_words = (q.L + 127) / 128 * 4;
-        q.split = split_ctas(a, q, heads, total);
-        q.tiles = (int)total;
+        plan_split(a, q, heads);
         if (q.split == 0 && n_seq > 1 && q.levels > TC_MAX_LEVELS) return false;
         kv_rows += (long)(heads / g) * q.L; vl_rows += (long)heads * q.k; q_rows += (long)heads * q.Lq; words += (long)heads * q.mask_words;
         units += (long)heads * q.levels;

@@ -138,7 +138,7 @@ template <> struct Tables<SEPARATE> : TcTables {
 };
 
 // The unit that tile `pos` of a split sequence falls into, its first tile and its number of tiles (warp-collective; the
-// tiles of the sequence are counted unit by unit, longest units first)
+// tiles of the sequence are counted unit by unit, longest units first, a unit's lead before its own)
 struct UnitAt {
     int unit, first, tiles;
 };
@@ -147,7 +147,7 @@ __device__ __forceinline__ UnitAt unit_at(const TcSeq& q, int heads, int window,
     int base = 0;
     for (int l0 = 0; l0 < q.levels; l0 += 32) {
         const int l = l0 + (int)(threadIdx.x & 31);
-        const int t = l < q.levels ? tc_unit_tiles(q.L, q.Lq, q.k, window, fixed_tail, q.levels - 1 - l) : 0;
+        const int t = l < q.levels ? q.lead + tc_unit_tiles(q.L, q.Lq, q.k, window, fixed_tail, q.levels - 1 - l) : 0;
         int incl = t * heads;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -197,11 +197,11 @@ __device__ __forceinline__ Piece find_piece(const TcTables& t, int window, int f
     if (pos < 0) pos = begin;
     const UnitAt u = unit_at(q, tab.heads, window, fixed_tail, pos);
     pc.seq = s; pc.unit = u.unit;
-    pc.t0 = pos - u.first;
-    pc.t1 = min(u.tiles, end - u.first);
-    if (pc.t0 == 0 && pc.t1 == u.tiles) pc.t1 = 0x7fffffff;
+    pc.t0 = max(pos - u.first - q.lead, 0);
+    pc.t1 = min(u.tiles, end - u.first) - q.lead;            // (positive: a share is longer than a lead, and see below)
+    if (pc.t0 == 0 && pc.t1 == u.tiles - q.lead) pc.t1 = 0x7fffffff;
     else pc.slot = q.slot0 + 2 * c + (pos == begin ? 0 : 1);
-    if (u.first + u.tiles < end) next = u.first + u.tiles;
+    if (u.first + u.tiles + q.lead < end) next = u.first + u.tiles;     // (nothing but the next unit's lead: not begun)
     return pc;
 }
 
@@ -1177,7 +1177,7 @@ attn_merge_kernel(const __grid_constant__ TcSeq q, int heads, int window, int fi
     int first = 0, tiles = 0;
     for (int l0 = 0; l0 <= level; l0 += 32) {
         const int l = l0 + lane;
-        const int t = l <= level ? tc_unit_tiles(q.L, q.Lq, q.k, window, fixed_tail, q.levels - 1 - l) : 0;
+        const int t = l <= level ? q.lead + tc_unit_tiles(q.L, q.Lq, q.k, window, fixed_tail, q.levels - 1 - l) : 0;
         int sum = l < level ? t * heads : 0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -1185,12 +1185,12 @@ attn_merge_kernel(const __grid_constant__ TcSeq q, int heads, int window, int fi
         if (level - l0 < 32) tiles = __shfl_sync(0xffffffffu, t, level - l0);
     }
     first += (unit - level * heads) * tiles;
-    const int c0 = split_of(q.tiles, q.split, first), c1 = split_of(q.tiles, q.split, first + tiles - 1);
+    const int c0 = split_of(q.tiles, q.split, first + q.lead), c1 = split_of(q.tiles, q.split, first + tiles - 1);
     if (c0 == c1) return;
     const int row = (blockIdx.x & 31) * 8 + (threadIdx.x >> 5), i = (q.levels - 1 - level) * TC_ROWS + row;
     if (i >= q.Lq) return;
     // the unit's first piece is its CTA's first or a later one, all others are their CTAs' first
-    const int s0 = q.slot0 + 2 * c0 + (split_begin(q.tiles, q.split, c0) == first ? 0 : 1), n_pc = c1 - c0 + 1;
+    const int s0 = q.slot0 + 2 * c0 + (split_begin(q.tiles, q.split, c0) >= first ? 0 : 1), n_pc = c1 - c0 + 1;
     auto slot = [&](int c) -> long { return (long)(c == 0 ? s0 : q.slot0 + 2 * (c0 + c)) * TC_ROWS + row; };
     // Lane c looks after the reference and the row sum of piece c (+ 32 ...), the first four accumulators are loaded beside them:
     // piece by piece their latencies, and 64-bit divisions in the look-up above, were the kernel (2 heads x 2048 rows in 91

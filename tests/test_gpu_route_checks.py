@@ -114,3 +114,26 @@ def test_a_query_block_with_a_ragged_last_tile_takes_no_longer_than_a_full_one(B
     K, V = _normal((B, Hkv, L, 128), 2), _normal((B, Hkv, L, 128), 3)
     short, full = _median_us([_block_call(_normal((B, Hq, n, 128), 1), K, V, fmts, 512, 390) for n in (Lq, -(-Lq // 256) * 256)], n=5, rounds=5)
     assert short <= 1.2 * full, (short, full)
+
+
+@pytest.mark.parametrize("fmts", [INT8, INT4FP8])
+@pytest.mark.parametrize("B,Hq,Hkv,L,Lq,W,k", [
+    (1, 2, 2, 20010, 20010, 256, 395),      # a whole prefill: CTAs with one piece at the long end, a dozen short units at the other
+    (1, 4, 1, 9000, 9000, 0, 0),            # no window: units down to four tiles, shorter than the cost of beginning them
+    (3, 16, 4, 5000, 700, 200, 60),         # a query block, three units per head
+    (1, 1, 1, 30000, 3, 64, 300),           # one unit for all CTAs
+])
+def test_shares_that_count_what_a_unit_costs_to_begin(fmts, B, Hq, Hkv, L, Lq, W, k):
+    ensure_built()
+    Q, K, V = _normal((B, Hq, Lq, 128), L), _normal((B, Hkv, L, 128), L + 1), _normal((B, Hkv, L, 128), L + 2)
+    if W == 0:                              # (the selector's tail mean needs a window or a count)
+        idx = torch.arange(0, L, 97, dtype=torch.int32, device="cuda").expand(B, Hq, -1).contiguous()
+    else:
+        idx = api.hyq_select_vertical(Q, K, W, k)
+    qz = [api.hyq_quantize_blocks(t, f) for t, f in zip((Q, K, V), fmts)]
+    res = []
+    for impl in (api.IMPL_TCGEN05, api.IMPL_SIMT):
+        lse = torch.empty(Q.shape[:3], dtype=torch.float32, device="cuda")
+        out = api.hyq_hybrid_attention_prefill(Q, K, V, qz[0][0], qz[1][0], qz[2][0], qz[0][1], qz[1][1], qz[2][1], fmts, idx, W, lse=lse, impl=impl)
+        res += [out, lse]
+    _close(*res)
