@@ -184,7 +184,7 @@ int launch_vl_bitmask(const int32_t* idx, long n_heads, int k, int L, int mask_w
 // tiles, units longest first), and over how many CTAs.  In units of a key tile (about 0.75 us): beginning a piece of work costs about
 // 10 tiles beside its keys, so a unit counts for that much more in the shares (without it a CTA at the end of the list got a dozen
 // short units: 16 heads x 7282 tokens 452 us, one CTA per unit 222) - unless the shares are small, with two pieces each at
-// most; the merge costs by the partial results that it reads.  One CTA per unit takes at least the
+// most; the merge costs by the partial results that it reads (8 tiles where the shares are small).  One CTA per unit takes at least the
 // mean load of an SM, and for every w at least w times the shortest of the longest 148 (w - 1) + 1 units.  Measured (attention launches, INT8, 2 heads x
 // 2048 tokens): one CTA per unit 54.6 us, shared 34.8; over 60 blocks and prompts of 2 to 80 heads the rule's choice takes at most
 // 1.05 times the better one's time.  Fills q.split, q.tiles and q.lead.
@@ -211,7 +211,7 @@ static void plan_split(const hyq_attn_args& a, TcSeq& q, int heads) {
     const bool fits = total < 0xffffffffL / TC_SMS;             // (tile * CTAs in 32 bits)
     q.tiles = fits ? (int)total : 0x7fffffff;
     if (ctas < 2 || !fits) return;
-    const long merge = 3 + (ctas + (units < ctas ? units : ctas)) / 16;
+    const long merge = lead ? 3 + (ctas + (units < ctas ? units : ctas)) / 16 : 8;
     const long split = (total + ctas - 1) / ctas + (lead ? 1 : 2) * PIECE_COST + merge;
     if (split * 100 >= bound * 93) return;
     q.split = (int)ctas; q.lead = (int)lead;
