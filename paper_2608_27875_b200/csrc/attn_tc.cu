@@ -171,6 +171,7 @@ __host__ __device__ inline int split_of(int tiles, int split, int x) { return (i
 
 // Work of a CTA of a general launch, from tile `pos` of its share on (-1: from the start).  Returns in `next` the tile to
 // go on from, -1 when nothing is left.
+template <bool SHARED>                           // (false: no sequence of the launch is split)
 __device__ __forceinline__ Piece find_piece(const TcTables& t, int window, int fixed_tail, int pos, int& next) {
     const TcSeqTable& tab = t.tab;
     Piece pc = {0, 0, 0, 0x7fffffff, -1};
@@ -190,6 +191,7 @@ __device__ __forceinline__ Piece find_piece(const TcTables& t, int window, int f
         }
         return pc;
     }
+    if (!SHARED) return pc;
     int s = tab.n_unsplit;
     while (s + 1 < tab.n_seq && tab.seq[s + 1].cta0 <= cta) ++s;
     const TcSeq& q = tab.seq[s];
@@ -549,16 +551,20 @@ __device__ __forceinline__ void mask_cols32(uint32_t (&raw)[32], int c0, int lo_
 // maxima).  A CTA then finds its pieces of work in `tabs`, and rows are addressed in the flattened views of the buffers;
 // with KIND = SEPARATE Q and K of every sequence are read where they are;
 // the plain kernel keeps a position offset and these look-ups out of its registers (2.6 % on the benchmark workload).
+// SHARED: some sequence's units are shared out tile by tile, and a CTA goes through several pieces of them.  Launches without such a
+// sequence have one unit per CTA and a kernel of their own: what the loop over pieces keeps in registers (167 instead of 150) makes the
+// softmax warps slower (4096 rows against 65536 keys, 32 heads, INT8, one CTA per unit: 4170 -> 3990 us; against 20000 keys 1540 -> 1362).
 // EXACT = false is the kernel of the first launch.  After the first tiles of a row's low-bit pass
 // (and if their maxima lie close together) it takes the exponentials against the row's reference as it stands, without
 // looking for the tile's maximum, and every tile's row sum tells afterwards whether that was safe (no P beyond fp16).  If it was not for any row of the
 // piece - a score more than 2^16 above everything the row had seen - the CTA writes no output for it and puts the piece
 // on a list.  EXACT = true is the kernel of the second launch, a small grid that goes through that list
 // (normally empty) with the maximum looked at in every tile.
-template <bool LOWBIT_FP8, int KIND, bool EXACT = false>
+template <bool LOWBIT_FP8, int KIND, bool EXACT = false, bool SHARED = false>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcParams p, const __grid_constant__ Tables<KIND> tabs) {
     constexpr bool GENERAL = KIND != PLAIN;
+    constexpr bool PIECES = GENERAL && (SHARED || EXACT);       // parts of units, several of them per CTA
     constexpr int TBN = 64, BN = 64;
     pdl_wait();
     if (EXACT && p.redo[0].x == 0) return;
@@ -576,8 +582,8 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
         tmem_relinquish();
     }
     if (threadIdx.x == 0) abort_s = 0;
-    if (GENERAL && !EXACT && threadIdx.x == 0) next_s = -1;
-    if (GENERAL && !EXACT) __syncthreads();
+    if (SHARED && threadIdx.x == 0) next_s = -1;
+    if (SHARED) __syncthreads();
     int item = blockIdx.x;                                   // second launch: place on the list
 #pragma unroll 1
     for (;;) {
@@ -588,9 +594,9 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
         const int4 r = p.redo[1 + item];
         pc.seq = r.x & 0xff; pc.slot = (r.x >> 8) - 1; pc.unit = r.y; pc.t0 = r.z; pc.t1 = r.w;
     } else if constexpr (GENERAL) {
-        pc = find_piece(tabs, p.window, p.fixed_tail, next_s, next);
+        pc = find_piece<SHARED>(tabs, p.window, p.fixed_tail, SHARED ? next_s : -1, next);
     }
-    const bool settle = EXACT || next >= 0 || (GENERAL && pc.slot >= 0);      // the barriers may be initialised again
+    const bool settle = EXACT || next >= 0 || (PIECES && pc.slot >= 0);      // the barriers may be initialised again
     int qhead, kvhead, pt, L, off, lim0, k_vl, q_y, q_z, kv_y, kv_z, vl_y, vl_z;
     int q_dy = 0, k_dy = 0;                                  // flattened row minus row in the sequence's own Q; the converse for K
     const CUtensorMap *q_map = &maps.q, *k_map = &maps.k;
@@ -656,7 +662,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
     // tensor memory (warp 0), the counts of vertical keys (warps 1 and 2), the constant operand (all).
     if (warp == 0) {
         if (lane == 0) {
-            if (EXACT ? item != (int)blockIdx.x : (GENERAL && next_s >= 0)) {      // (a later piece: barriers in use may not be initialised as they are)
+            if (EXACT ? item != (int)blockIdx.x : (SHARED && next_s >= 0)) {      // (a later piece: barriers in use may not be initialised as they are)
                 uint64_t* all = reinterpret_cast<uint64_t*>(&bars);
                 for (int i = 0; i < (int)(sizeof(TcBarriers) / sizeof(uint64_t)); ++i) mbar_inval(all + i);
             }
@@ -679,7 +685,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             if (EXACT) atomicAdd(&g_tc_restarts, 1ull);
         }
         __syncwarp();
-        if (!EXACT && (!GENERAL || next_s < 0)) {            // (once: the first piece)
+        if (!EXACT && (!SHARED || next_s < 0)) {            // (once: the first piece)
             tmem_alloc(&tmem_base_s, TM_COLS);
             tmem_relinquish();
         }
@@ -704,7 +710,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
-    if (GENERAL && !EXACT && threadIdx.x == 0) next_s = next;    // (read again behind the synchronisation that ends this piece)
+    if (SHARED && threadIdx.x == 0) next_s = next;    // (read again behind the synchronisation that ends this piece)
     qs0.nB = (cnt_b_s[0] + BN - 1) / BN;
     qs1.nB = (cnt_b_s[1] + BN - 1) / BN;
     Walk w;
@@ -713,8 +719,8 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
     w.tC0 = qs0.tC0;
     w.nC = (W > 0) ? max(qs0.tC1, qs1.tC1) - w.tC0 + 1 : 0;
     w.T = w.nA + w.nB + w.nC;
-    w.t0 = GENERAL ? pc.t0 : 0;
-    w.t1 = GENERAL ? max(pc.t0, min(pc.t1, w.T)) : w.T;
+    w.t0 = PIECES ? pc.t0 : 0;
+    w.t1 = PIECES ? max(pc.t0, min(pc.t1, w.T)) : w.T;
 
     volatile int* abort_flag = &abort_s;
     volatile int* restart_flag = &restart_s;
@@ -757,9 +763,9 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             return again;
         };
         // own tiles of this CTA: numbers [n0, n_total) in the query tile's own list (all of it unless the keys are split)
-        const int n0 = GENERAL ? own_before(own, w.t0) : 0;
-        const int n_total = GENERAL ? own_before(own, w.t1) : own.a_end + (own.b_end - own.b_beg) + (own.c_end - own.c_beg);
-        if (GENERAL && pc.slot >= 0 && sq.live && n_total <= n0)   // nothing of this query tile lies in the piece: an empty partial result
+        const int n0 = PIECES ? own_before(own, w.t0) : 0;
+        const int n_total = PIECES ? own_before(own, w.t1) : own.a_end + (own.b_end - own.b_beg) + (own.c_end - own.c_beg);
+        if (PIECES && pc.slot >= 0 && sq.live && n_total <= n0)   // nothing of this query tile lies in the piece: an empty partial result
             reinterpret_cast<float2*>(p.part_ml)[(long)pc.slot * TC_ROWS + q * BM + (warp & 3) * 32 + lane] = make_float2(-INFINITY, 0.0f);
         if (sq.live && n_total > n0) {
             const int r = (warp & 3) * 32 + lane;               // query row inside the tile = TMEM lane
@@ -944,7 +950,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 prefetch_tile(n + 1);
                 return do_tile(std::false_type{}, n, cs, vl, !LOWBIT_FP8, 0, 0);
             };
-            const bool brief = GENERAL && pc.slot >= 0 && n_plain_end - n0 <= 2 * WARM_TILES;
+            const bool brief = PIECES && pc.slot >= 0 && n_plain_end - n0 <= 2 * WARM_TILES;
             const int n_warm = n0 + (brief ? WARM_TILES_SHORT : WARM_TILES);
             if (!EXACT && n_plain_end > n_warm) {
                 float mt_lo = INFINITY, mt_hi = -INFINITY;
@@ -1079,7 +1085,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 // average CTA's 141 k at L = 8192, fp32; now 5.0 k).  Per warp three 4 KB buffers of 32 rows x 128 bytes, pieces swizzled as the
                 // tensor map expects them.  Rows past the end are clipped by the plain kernel's map; in the flattened view they would be
                 // the next head's, so a warp with such rows copies its own ones instead.
-                const bool part = GENERAL && pc.slot >= 0;      // (a partial result leaves O as accumulated, relative to m_used)
+                const bool part = PIECES && pc.slot >= 0;      // (a partial result leaves O as accumulated, relative to m_used)
                 const float inv = part ? 1.0f : (l_run > 0.0f) ? 1.0f / l_run : 0.0f;
                 if (ok) {
                     unsigned char* buf0 = smem + SQ_OFF + q * Q_TILE_BYTES + (warp & 3) * 8192;
@@ -1133,7 +1139,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                                 for (int rr = lane >> 3; rr < rows; rr += 4)
                                     *reinterpret_cast<uint4*>(static_cast<char*>(p.out) + (long)(o_y + rr) * row_bytes + col) =
                                         *reinterpret_cast<const uint4*>(buf + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
-                                if (GENERAL) fence_proxy_async();   // (the CTA's next piece loads its queries over these rows by TMA)
+                                if (PIECES) fence_proxy_async();   // (the CTA's next piece loads its queries over these rows by TMA)
                                 __syncwarp();
                             }
                         }
@@ -1152,7 +1158,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (!EXACT && !GENERAL) break;
+    if (!EXACT && !SHARED) break;
     if (abort_s || (!EXACT && next_s < 0)) break;
     item += gridDim.x;
     }
@@ -1269,6 +1275,8 @@ static int launch_attn_tc_kernels(const hyq_attn_args& a, const TcPlan& plan, co
     // e4m3 bytes on the low-bit side: FP8 codes as they are, or INT4 codes widened by the pre-pass
     const bool lowbit_fp8 = a.q_format != HYQ_FMT_INT8;
     auto kern = lowbit_fp8 ? attn_tc_kernel<true, KIND> : attn_tc_kernel<false, KIND>;
+    if constexpr (KIND != PLAIN)
+        if (plan.t.tab.n_unsplit < plan.t.tab.n_seq) kern = lowbit_fp8 ? attn_tc_kernel<true, KIND, false, true> : attn_tc_kernel<false, KIND, false, true>;
     // the same instantiation for the second launch (every maximum looked at; works through the first launch's list)
     auto kern_exact = lowbit_fp8 ? attn_tc_kernel<true, KIND, true> : attn_tc_kernel<false, KIND, true>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_BYTES) != cudaSuccess ||
