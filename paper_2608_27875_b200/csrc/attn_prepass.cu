@@ -189,7 +189,8 @@ int launch_vl_bitmask(const int32_t* idx, long n_heads, int k, int L, int mask_w
 // 2048 tokens): one CTA per unit 54.6 us, shared 34.8; over 60 blocks and prompts of 2 to 80 heads the rule's choice takes at most
 // 1.05 times the better one's time.  Fills q.split, q.tiles and q.lead.
 constexpr long SPLIT_MIN_TILES = 4;                             // tiles per CTA at least
-static void plan_split(const hyq_attn_args& a, TcSeq& q, int heads) {
+constexpr long SPLIT_L2_BYTES = 96L << 20;                      // codes and values that stay in L2 (126 MB, beside the queries and outputs)
+static void plan_split(const hyq_attn_args& a, TcSeq& q, int heads, int g) {
     constexpr long PIECE_COST = 10, LEAD_MIN_TILES = 20;
     const bool ft = a.window_mode == HYQ_WINDOW_FIXED_TAIL;
     const long units = (long)q.levels * heads;
@@ -213,7 +214,13 @@ static void plan_split(const hyq_attn_args& a, TcSeq& q, int heads) {
     if (ctas < 2 || !fits) return;
     const long merge = lead ? 3 + (ctas + (units < ctas ? units : ctas)) / 16 : 8;
     const long split = (total + ctas - 1) / ctas + (lead ? 1 : 2) * PIECE_COST + merge;
-    if (split * 100 >= bound * 93) return;
+    // CTAs that share units are at different keys at any time, those with one unit each walk their KV head's keys together.  Where
+    // the keys and values don't stay in L2 the former read them from memory 148 times over: up to 1.14 times the estimate, so that
+    // it has to pay more (4096 rows against 65536 keys of 8 KV heads: estimate 0.89 of one CTA per unit, measured 1.10; 2048 against
+    // 131072 0.87, 1.13; 3000 x 40 heads against 65536 0.82, 0.88).  Not with one unit per CTA at most, where SMs would be idle
+    // (1024 rows against 65536: 0.89, 0.91).
+    const long kv_bytes = (long)(heads / g) * q.L * (HYQ_D + 2 * HYQ_D);
+    if (split * 100 >= bound * (kv_bytes > SPLIT_L2_BYTES && units > TC_SMS ? 86 : 93)) return;
     q.split = (int)ctas; q.lead = (int)lead;
 }
 
@@ -231,7 +238,7 @@ bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads
         q.levels = (q.Lq + TC_ROWS - 1) / TC_ROWS;
         q.nb = (q.L + bt - 1) / bt; q.nbq = (q.Lq + bt - 1) / bt;
         q.mask_words = (q.L + 127) / 128 * 4;
-        plan_split(a, q, heads);
+        plan_split(a, q, heads, g);
         if (q.split == 0 && n_seq > 1 && q.levels > TC_MAX_LEVELS) return false;
         kv_rows += (long)(heads / g) * q.L; vl_rows += (long)heads * q.k; q_rows += (long)heads * q.Lq; words += (long)heads * q.mask_words;
         units += (long)heads * q.levels;
