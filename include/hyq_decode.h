@@ -137,7 +137,8 @@ int hyq_kv_cache_append_ragged(const void* k_new, const void* v_new, const hyq_k
  *   q [B,Hq,D] bf16 (device).  out [B,Hq,D]: bf16 (out_dtype 0) or fp32 (1).  lse: optional [B,Hq] fp32,
  *   natural-log-sum-exp of the scaled scores (NULL to skip).  softmax_scale 0 => 1/sqrt(D).
  *   splits: 1 <= S <= 1024, or 0 for a choice that fills the GPU.  workspace: hyq_hybrid_attention_decode_workspace
- *   bytes (the slices' partial results).  The cache must hold at least one row in total.
+ *   bytes (the slices' partial results; the query's answer holds for every fill of the staging buffer).  The cache must hold at
+ *   least one row in total.
  *   Errors: as hyq_freeze, plus WORKSPACE.
  * ------------------------------------------------------------------------------------------- */
 int hyq_hybrid_attention_decode_workspace(const hyq_kv_cache* cache, int splits, size_t* bytes /* host, out */);

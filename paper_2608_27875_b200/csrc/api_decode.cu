@@ -87,10 +87,13 @@ int hyq_hybrid_attention_decode_workspace(const hyq_kv_cache* cache, int splits,
     if (!bytes || splits < 0 || splits > 1024) return HYQ_ERR_INVALID_ARG;
     const int rc = check_cache(cache, false);
     if (rc != HYQ_OK) return rc;
-    int s = splits > 0 ? splits : decode_auto_splits(*cache);
+    // the number of slices grows with the staged rows: the answer is for a full staging buffer, so that it holds for every step
+    hyq_kv_cache full = *cache;
+    full.n_staging = full.staging_capacity;
+    int s = splits > 0 ? splits : decode_auto_splits(full);
     // (capacities: the description may be a ragged batch's)
-    if (splits == 0 && (cache->cap_quantized_rows || cache->cap_vertical || cache->cap_window) && decode_ragged_splits(*cache) > s)
-        s = decode_ragged_splits(*cache);
+    if (splits == 0 && (cache->cap_quantized_rows || cache->cap_vertical || cache->cap_window) && decode_ragged_splits(full) > s)
+        s = decode_ragged_splits(full);
     *bytes = decode_workspace_bytes(*cache, s);
     return HYQ_OK;
 }

@@ -198,3 +198,18 @@ def test_the_mass_selectors_workspace_grows_with_the_call(lib):
             got = [need(Hq, Lk, nT) for Lk in range(2200, 60000, 700)]
             assert got == sorted(got), (nT, Hq)
             assert need(Hq, 59900, nT) >= need(max(1, Hq // 2), 59900, nT) and need(Hq, 30000, nT) >= need(Hq, 30000, max(1, nT - 3))
+
+
+def test_the_decode_workspace_holds_for_every_fill_of_the_staging_buffer(lib):
+    """Queried before the first token, used until the buffer is full: more staged rows may ask for another slice."""
+    L = decode_api._lib()
+    n = ctypes.c_size_t(0)
+    for Hkv in (1, 2, 8):
+        for N in list(range(200, 3000, 90)) + list(range(15000, 17000, 90)):
+            d = decode_api.make_desc(B=1, Hq=4 * Hkv, Hkv=Hkv, N=N, window=128, k=N // 100)
+            need = []
+            for staged in range(0, 129, 8):
+                d.n_staging = staged
+                assert L.hyq_hybrid_attention_decode_workspace(ctypes.byref(d), 0, ctypes.byref(n)) == 0
+                need.append(n.value)
+            assert need[0] == max(need), (Hkv, N)
