@@ -328,6 +328,9 @@ def _prefill(qs, ks, vs, B, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens
 def hybrid_prefill(q, k, v, window: int, k_sel: int, fmts=(FMT_INT8, FMT_INT8, FMT_INT8), impl: int = IMPL_AUTO,
                    out_dtype=torch.float32):
     """The whole path on device tensors: select -> quantize Q, K, V -> fused attention."""
+    # (the library sees pointers only)
+    if v.shape != k.shape or k.shape[0] != q.shape[0] or k.shape[3] != q.shape[3]:
+        raise ValueError(f"q, k, v: {tuple(q.shape)}, {tuple(k.shape)} and {tuple(v.shape)} don't belong together")
     if impl == IMPL_SIMT or q.shape[2] != k.shape[2]:        # stage by stage
         idx = hyq_select_vertical(q, k, window, k_sel)
         qc, qs = hyq_quantize_blocks(q, fmts[0])
@@ -383,6 +386,13 @@ def hybrid_prefill_varlen(qs, ks, vs, window: int, k_per_seq, fmts=(FMT_INT8, FM
         raise HyqError(2, "hybrid_prefill_varlen")
     dev = qs[0].device
     lens = [t.shape[1] for t in qs]
+    # (the library sees pointers only: every prompt's K and V as long as its Q, all with the first prompt's heads)
+    k_per_seq = list(k_per_seq)
+    if not n == len(ks) == len(vs) == len(k_per_seq):
+        raise ValueError(f"{n} prompts of q, {len(ks)} of k, {len(vs)} of v, {len(k_per_seq)} vertical counts")
+    for q, k, v, L_ in zip(qs, ks, vs, lens):
+        if q.shape != (Hq, L_, D) or k.shape != (Hkv, L_, D) or v.shape != k.shape:
+            raise ValueError(f"q, k, v of a prompt: {tuple(q.shape)}, {tuple(k.shape)}, {tuple(v.shape)}, not {(Hq, L_, D)} and twice {(Hkv, L_, D)}")
     cu = [0]
     for L_ in lens:
         cu.append(cu[-1] + L_)

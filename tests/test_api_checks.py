@@ -1,0 +1,48 @@
+"""Argument checks of the Python calls that end before a pointer reaches the library (CPU tensors stand in for the device's)."""
+import pytest
+import torch
+
+from paper_2608_27875_b200 import api
+
+
+@pytest.fixture
+def any_device(monkeypatch):
+    """Tensors of any device pass, and a call that gets as far as the library fails with another error."""
+    def reached():
+        raise RuntimeError("the library was called")
+    monkeypatch.setattr(api, "_dev", lambda t, dtype, name: t)
+    monkeypatch.setattr(api, "lib", reached)
+
+
+def _t(*shape):
+    return torch.zeros(*shape, dtype=torch.bfloat16)
+
+
+def test_hybrid_prefill_takes_shapes_that_belong_together(any_device):
+    q, k = _t(2, 4, 300, 128), _t(2, 2, 300, 128)
+    with pytest.raises(RuntimeError, match="library"):
+        api.hybrid_prefill(q, k, k.clone(), 64, 5)
+    for bad_k, bad_v in ((k, _t(2, 2, 299, 128)), (k, _t(2, 1, 300, 128)), (_t(1, 2, 300, 128), _t(1, 2, 300, 128)), (_t(2, 2, 300, 64),) * 2):
+        for impl in (api.IMPL_AUTO, api.IMPL_SIMT):
+            with pytest.raises(ValueError):
+                api.hybrid_prefill(q, bad_k, bad_v, 64, 5, impl=impl)
+
+
+def test_hybrid_prefill_varlen_takes_prompts_that_belong_together(any_device):
+    lens = [100, 70]
+    good = lambda: tuple([_t(h, n, 128) for n in lens] for h in (4, 2, 2)) + ([1, 0],)       # noqa: E731
+    qs, ks, vs, kp = good()
+    with pytest.raises(RuntimeError, match="library"):
+        api.hybrid_prefill_varlen(qs, ks, vs, 64, kp)
+    for which, s, t in ((0, 1, _t(5, 70, 128)), (1, 1, _t(2, 69, 128)), (2, 0, _t(2, 99, 128)), (1, 1, _t(1, 70, 128)), (2, 1, _t(2, 70, 64))):
+        args = good()
+        args[which][s] = t
+        with pytest.raises(ValueError):
+            api.hybrid_prefill_varlen(*args[:3], 64, kp)
+    for short in range(4):
+        args = [list(a) for a in good()]
+        args[short].pop()
+        with pytest.raises(ValueError):
+            api.hybrid_prefill_varlen(*args[:3], 64, args[3])
+    with pytest.raises(ValueError):
+        api.hybrid_prefill_varlen(qs, ks, vs, 64, [1, 0, 0])
