@@ -331,7 +331,7 @@ def hybrid_prefill(q, k, v, window: int, k_sel: int, fmts=(FMT_INT8, FMT_INT8, F
     # (the library sees pointers only)
     if v.shape != k.shape or k.shape[0] != q.shape[0] or k.shape[3] != q.shape[3]:
         raise ValueError(f"q, k, v: {tuple(q.shape)}, {tuple(k.shape)} and {tuple(v.shape)} don't belong together")
-    if impl == IMPL_SIMT or q.shape[2] != k.shape[2]:        # stage by stage
+    if impl not in (IMPL_AUTO, IMPL_TCGEN05) or q.shape[2] != k.shape[2]:        # stage by stage (an unknown kernel is refused there)
         idx = hyq_select_vertical(q, k, window, k_sel)
         qc, qs = hyq_quantize_blocks(q, fmts[0])
         kc, ks = hyq_quantize_blocks(k, fmts[1])

@@ -137,3 +137,12 @@ def test_shares_that_count_what_a_unit_costs_to_begin(fmts, B, Hq, Hkv, L, Lq, W
         out = api.hyq_hybrid_attention_prefill(Q, K, V, qz[0][0], qz[1][0], qz[2][0], qz[0][1], qz[1][1], qz[2][1], fmts, idx, W, lse=lse, impl=impl)
         res += [out, lse]
     _close(*res)
+
+
+def test_an_unknown_attention_kernel_is_refused():
+    ensure_built()
+    q, k = _normal((1, 2, 200, 128), 1), _normal((1, 1, 200, 128), 2)
+    for impl in (-1, 3):
+        with pytest.raises(api.HyqError) as e:
+            api.hybrid_prefill(q, k, k, 64, 3, impl=impl)
+        assert e.value.code == 1
