@@ -401,7 +401,7 @@ def hybrid_prefill_varlen(qs, ks, vs, window: int, k_per_seq, fmts=(FMT_INT8, FM
     status = torch.zeros(1, dtype=torch.int32, device=dev)
     total, blocks = cu[-1], sum(nbs)
     idx, codes, scales, out = _prefill(qs, ks, vs, 1, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens, out_dtype, dev,
-                                       (Hq * sum(k_per_seq), [H * total * code_row_bytes(f, D) for H, f in zip((Hq, Hkv, Hkv), fmts)],
+                                       (max(0, Hq * sum(k_per_seq)), [H * total * code_row_bytes(f, D) for H, f in zip((Hq, Hkv, Hkv), fmts)],
                                         [H * blocks for H in (Hq, Hkv, Hkv)], Hq * total * D), status)
     res, ko, no = [], 0, 0
     for s in range(n):

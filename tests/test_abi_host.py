@@ -213,3 +213,15 @@ def test_the_decode_workspace_holds_for_every_fill_of_the_staging_buffer(lib):
                 assert L.hyq_hybrid_attention_decode_workspace(ctypes.byref(d), 0, ctypes.byref(n)) == 0
                 need.append(n.value)
             assert need[0] == max(need), (Hkv, N)
+
+
+def test_a_negative_vertical_count_is_an_invalid_argument(lib):
+    a = api.PrefillArgs()
+    a.struct_size = ctypes.sizeof(api.PrefillArgs)
+    a.n_seq, a.B, a.Hq, a.Hkv, a.D, a.window, a.block_tokens = 1, 1, 4, 2, 128, 64, 64
+    lens, k = (ctypes.c_int32 * 1)(100), (ctypes.c_int32 * 1)(-1)
+    a.lengths, a.k_per_seq = ctypes.addressof(lens), ctypes.addressof(k)
+    n = ctypes.c_size_t(0)
+    assert lib.hyq_hybrid_prefill_workspace(ctypes.byref(a), ctypes.byref(n)) == 1
+    k[0] = 3
+    assert lib.hyq_hybrid_prefill_workspace(ctypes.byref(a), ctypes.byref(n)) == 0

@@ -46,3 +46,10 @@ def test_hybrid_prefill_varlen_takes_prompts_that_belong_together(any_device):
             api.hybrid_prefill_varlen(*args[:3], 64, args[3])
     with pytest.raises(ValueError):
         api.hybrid_prefill_varlen(qs, ks, vs, 64, [1, 0, 0])
+
+
+def test_negative_vertical_counts_are_the_librarys_to_refuse(any_device):
+    """(its code INVALID_ARG, not torch's complaint about a negative size)"""
+    ts = [[_t(h, 100, 128)] for h in (4, 2, 2)]
+    with pytest.raises(RuntimeError, match="library"):
+        api.hybrid_prefill_varlen(*ts, 64, [-1])
