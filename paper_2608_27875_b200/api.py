@@ -109,11 +109,14 @@ def _check(code: int, where: str):
         raise HyqError(code, where)
 
 
-_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# the current stream's handle: torch.cuda.current_stream() builds a Stream object for it, 2-3 us a call (a torch without CUDA has
+# neither function, and no use for the handle)
+_raw_stream, _device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream() -> int:
-    # the current stream's handle (torch.cuda.current_stream() builds a Stream object for it: 2-3 us a call)
+    if _raw_stream is None or _device is None:
+        return torch.cuda.current_stream().cuda_stream
     return _raw_stream(_device())
 
 

@@ -1,4 +1,8 @@
 """Argument checks of the Python calls that end before a pointer reaches the library (CPU tensors stand in for the device's)."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -53,3 +57,10 @@ def test_negative_vertical_counts_are_the_librarys_to_refuse(any_device):
     ts = [[_t(h, 100, 128)] for h in (4, 2, 2)]
     with pytest.raises(RuntimeError, match="library"):
         api.hybrid_prefill_varlen(*ts, 64, [-1])
+
+
+def test_the_package_imports_with_a_torch_that_has_no_cuda_functions():
+    code = ("import torch\nfor n in ('_cuda_getCurrentRawStream', '_cuda_getDevice'): delattr(torch._C, n)\n"
+            "from paper_2608_27875_b200 import api, decode_api\nassert api._stream is not None")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    assert subprocess.run([sys.executable, "-c", code], cwd=root, timeout=300).returncode == 0
