@@ -75,6 +75,25 @@ def test_second_pass_of_a_short_query_block_with_split_keys():
     assert float((tc - simt).abs().max()) <= MAX_ABS_TOL
 
 
+@pytest.mark.parametrize("fmts,bt", [(INT8, 64), (INT4FP8, 64), (FP8, 64), (INT8, 32), (INT4FP8, 128)])
+def test_second_pass_of_the_kernel_of_plain_prefills(fmts, bt):
+    """More units than are shared out over CTAs (64 heads of ten), a dominant low-bit key in half of them; against the CUDA-core
+    kernel, and the same bits twice (the second launch goes through its list in any order)."""
+    ensure_built()
+    Hq, Hkv, L, W, k = 64, 4, 2560, 128, 16
+    Q, K, V, idx = _inputs(1, Hq, Hkv, L, L, W, k, 1200, seed=5 + bt)
+    Qd, Kd, Vd, idx_t = Q.cuda(), K.cuda(), V.cuda(), torch.from_numpy(idx).cuda()
+    qz = [api.hyq_quantize_blocks(t, f, bt) for t, f in zip((Qd, Kd, Vd), fmts)]
+    api.hyq_test_read_attention_restarts(reset=True)
+    outs = [api.hyq_hybrid_attention_prefill(Qd, Kd, Vd, qz[0][0], qz[1][0], qz[2][0], qz[0][1], qz[1][1], qz[2][1], fmts, idx_t, W,
+                                             impl=impl, block_tokens=bt) for impl in (api.IMPL_TCGEN05, api.IMPL_TCGEN05, api.IMPL_SIMT)]
+    n_second = api.hyq_test_read_attention_restarts(reset=True)
+    assert n_second >= 2 * Hq, n_second
+    assert torch.isfinite(outs[0]).all() and torch.equal(outs[0], outs[1])
+    assert float((outs[0] - outs[2]).abs().max()) <= MAX_ABS_TOL
+    assert float((outs[0] - outs[2]).abs().sum() / outs[2].abs().sum()) <= MEAN_REL_TOL
+
+
 def test_heavy_tailed_rows_keep_looking_for_the_maximum_instead_of_taking_the_second_pass():
     """The outlier-stress workload (four K channels x 20): rows whose scores spread widely raise their reference often.
     Their warps see that in the first tiles' maxima and keep looking for the maximum, so that (almost) no CTA has to be

@@ -80,3 +80,30 @@ def test_benchmark_shape_heads_and_argument_checks():
         api.hyq_select_vertical_mass(Qt.cuda(), K.cuda(), w.window, w.k, 65)       # more queries than rows given
     with pytest.raises(api.HyqError):
         api.hyq_select_vertical_mass(Q[:, :, -8:].contiguous().cuda(), K[:, :, :4].contiguous().cuda(), 2, 1, 2)   # Lq > Lk
+
+
+def _near_ties(Hq, Hkv, Lk, nT, seed):
+    """Keys that agree in the channels that carry the scores and differ in channels 50 binary orders below: their scores lie closer
+    together than the rounding of the 128 additions, so that the set depends on the order of the additions."""
+    g = torch.Generator().manual_seed(seed)
+    big = torch.randperm(128, generator=g)[:64]
+    small = torch.full((128,), 2.0**-50)
+    small[big] = 1.0
+    K = torch.randn(1, Hkv, Lk, 128, generator=g) * small
+    K[:, :, :, big] = (torch.randn(1, Hkv, 1, 64, generator=g) / 8).bfloat16().float()
+    Q = torch.randn(1, Hq, nT, 128, generator=g) * torch.exp2(torch.randint(-6, 7, (1, Hq, nT, 128), generator=g).float())
+    return Q.bfloat16(), K.bfloat16()
+
+
+@pytest.mark.parametrize("nT", [1, 4, 8, 9, 16, 23])
+@pytest.mark.parametrize("Hq,Hkv,Lk", [(8, 2, 3000), (6, 6, 777)])
+def test_sums_that_depend_on_the_order_of_the_channels_are_the_recipes(nT, Hq, Hkv, Lk):
+    """The recipe adds the channels in ascending order; the matrix instruction's own order is not specified by its manual."""
+    W, k = 64, 100
+    Q, K = _near_ties(Hq, Hkv, Lk, nT, seed=100 * nT + Hq)
+    want = oracle.select_vertical_mass(wl.bits(Q), wl.bits(K), W, k, nT)
+    order = torch.randperm(128, generator=torch.Generator().manual_seed(1))
+    other = oracle.select_vertical_mass(wl.bits(Q[..., order].contiguous()), wl.bits(K[..., order].contiguous()), W, k, nT)
+    assert not np.array_equal(want, other)                     # (these inputs tell the orders apart)
+    got = api.hyq_select_vertical_mass(Q.cuda(), K.cuda(), W, k, nT).cpu().numpy()
+    assert np.array_equal(got, want)

@@ -50,6 +50,29 @@ def test_a_missing_copy_ends_in_a_timeout_status_and_the_next_call_is_fine(fmts,
     assert torch.equal(again, good)
 
 
+@pytest.mark.parametrize("fmts", [(0, 0, 0), (2, 2, 1)])
+@pytest.mark.parametrize("drop", [0, 3, 9])
+def test_the_kernel_of_plain_prefills_ends_in_a_timeout_status_too(fmts, drop):
+    """More units than are shared out over CTAs (64 heads of ten): the kernel that ordinary prompts run."""
+    ensure_built()
+    B, Hq, Hkv, L, W, k = 1, 64, 4, 2560, 128, 32
+    Q, K, V = (rand_bf16((B, h, L, 128), seed=950 + n).cuda() for n, h in enumerate((Hq, Hkv, Hkv)))
+    idx = api.hyq_select_vertical(Q, K, W, k)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    good = _run(Q, K, V, fmts, idx, W, status)
+    assert int(status.item()) == 0
+    try:
+        api.hyq_test_set_attention_hooks(wait_limit_clocks=200_000, drop_load_position=drop)
+        _run(Q, K, V, fmts, idx, W, status)
+        assert int(status.item()) == HYQ_ERR_TIMEOUT
+    finally:
+        api.hyq_test_set_attention_hooks(0, -1)
+    status.zero_()
+    again = _run(Q, K, V, fmts, idx, W, status)
+    assert int(status.item()) == 0
+    assert torch.equal(again, good)
+
+
 def test_hook_arguments_are_checked():
     lib = ensure_built()
     assert lib.hyq_test_set_attention_hooks(-1, -1) == 1
