@@ -31,7 +31,7 @@ constexpr int PRE_THREADS = 256;
 constexpr int PRE_MASK_WORDS = 32;           // bitmask words (16 tiles of 64 keys) a block builds
 
 struct PreParams {
-    unsigned v_end, gather_end, mask_end, k_end, q_end;      // block ranges of the pieces
+    unsigned v_end, gather_end, mask_end, k_end;             // block ranges of the pieces (the Q codes behind them)
     int mask_blocks[TC_MAX_SEQ];                             // mask blocks before each sequence
     int bt_shift;                                      // log2(tokens per quantization block)
     const uint4* v;                                          // bf16 rows of 16 x 16 bytes
@@ -351,7 +351,7 @@ int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, const TcSource
     p.k_vecs = int4 ? (long)t.kv_rows * 8 : 0;
     p.q_vecs = int4 ? (long)t.q_rows * 8 : 0;
     p.k_end = (unsigned)(n += blocks(p.k_vecs));
-    p.q_end = (unsigned)(n += blocks(p.q_vecs));
+    n += blocks(p.q_vecs);
     if (n > 0x7fffffffL) return HYQ_ERR_UNSUPPORTED;
     p.bt_shift = a.block_tokens == 32 ? 5 : a.block_tokens == 64 ? 6 : 7;
     p.v = static_cast<const uint4*>(a.v);

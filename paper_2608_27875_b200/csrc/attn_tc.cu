@@ -72,8 +72,6 @@ template <int TBN> struct Geo {
     static constexpr uint32_t STAGE_BYTES = TBN * HYQ_D * 2;            // one bf16 / fp16 tile
     static constexpr uint32_t KC_TILE_BYTES = TBN * HYQ_D;              // one tile of 8-bit codes
     static constexpr int NST = RING_BYTES / STAGE_BYTES;                // ring depth
-    static constexpr int NSC = TBN / 64;                                // K scales (quantization blocks) per tile
-    static constexpr int NVW = TBN / 32;                                // vertical-line bitmask words per tile
 };
 constexpr uint32_t TC_SMEM_BYTES = TILE_SMEM + 1024;                // + slack for 1024-byte alignment
 
@@ -729,7 +727,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
         if (p.status) atomicExch(p.status, HYQ_ERR_TIMEOUT);
     };
 
-    // the single-thread roles sit in the lowest warps (the softmax warps 4..19 keep warp % 4 = TMEM lane quarter)
+    // the single-thread roles sit in the lowest warps (the softmax warps 4..11 keep warp % 4 = TMEM lane quarter)
     if (warp == 0) {
         if (lane == 0 && !tma_producer<TBN>(maps, k_map, k_dy, w, kv_y, kv_z, vl_y, vl_z, bars, smem, abort_flag, limit, p.drop_load, vl_tiles_head, settle)) fail();
     } else if (warp == 1 || warp == 2) {

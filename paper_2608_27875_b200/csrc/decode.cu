@@ -36,16 +36,8 @@ namespace hyq {
 
 constexpr int DEC_THREADS = 128;
 constexpr int DEC_WARPS = DEC_THREADS / 32;
-#ifndef DEC_CTAS_PER_SM
-#define DEC_CTAS_PER_SM 4                   // resident CTAs per SM the register budget is set for
-#endif
-#ifndef DEC_PAIR
-#define DEC_PAIR 1                           // INT4 tiles are processed two at a time
-#endif
-#ifndef DEC_STAGES_N
-#define DEC_STAGES_N 4
-#endif
-constexpr int DEC_STAGES = DEC_STAGES_N;    // tiles in flight per warp (cp.async ring)
+constexpr int DEC_CTAS_PER_SM = 4;          // resident CTAs per SM the register budget is set for
+constexpr int DEC_STAGES = 4;               // tiles in flight per warp (cp.async ring)
 constexpr int DEC_STAGE_BYTES = 2048;       // 1 KB K codes + 1 KB V codes
 constexpr float DEC_RAISE = 8.0f;          // log2 units; P <= 2^8 stays far inside fp16 / bf16 range
 
@@ -107,28 +99,17 @@ __device__ __forceinline__ uint32_t dq4_hi(uint32_t w) {
 // common 2^-24 goes into the score scale, and the +8 becomes 8 * sum_d q_d per head, subtracted from the score
 // (a cancellation of a few units against a dot product of eight k-steps: harmless in fp32).  The products
 // fp16 x fp16 are exact in the instruction's fp32 accumulation.
-#ifndef DEC_K_SUBNORMAL
-#define DEC_K_SUBNORMAL 1
-#endif
 __device__ __forceinline__ uint32_t kq4_lo(uint32_t w) {
-#if DEC_K_SUBNORMAL
     uint32_t h;
     asm("lop3.b32 %0, %1, 0x000F000F, 0x00080008, 0x6A;" : "=r"(h) : "r"(w));
     return h;
-#else
-    return dq4_lo(w);
-#endif
 }
 __device__ __forceinline__ uint32_t kq4_hi(uint32_t w) {
-#if DEC_K_SUBNORMAL
     uint32_t h;
     asm("lop3.b32 %0, %1, 0x00F000F0, 0x00800080, 0x6A;" : "=r"(h) : "r"(w));
     return h;
-#else
-    return dq4_hi(w);
-#endif
 }
-constexpr float DEC_K_UNIT = DEC_K_SUBNORMAL ? 16777216.0f : 1.0f;      // 2^24: undoes the subnormal placement
+constexpr float DEC_K_UNIT = 16777216.0f;                               // 2^24: undoes the subnormal placement
 __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
     uint32_t d;
     asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
@@ -576,19 +557,15 @@ decode_kernel(const DecParams p) {
             const uint16_t* qr = qs[r];
             auto f16 = [&](int ch) { return __float2half_rn(__uint_as_float((uint32_t)qr[ch] << 16)); };
             const __half2 h0 = __halves2half2(f16(base), f16(base + 4));
-#if DEC_K_SUBNORMAL
             auto f16s = [&](int ch) { return __float2half_rn(__uint_as_float((uint32_t)qr[ch] << 16) * 0.0625f); };
             const __half2 h1 = __halves2half2(f16s(base + 1), f16s(base + 5));
-#else
-            const __half2 h1 = __halves2half2(f16(base + 1), f16(base + 5));
-#endif
             qf[2 * c] = *reinterpret_cast<const uint32_t*>(&h0);
             qf[2 * c + 1] = *reinterpret_cast<const uint32_t*>(&h1);
         }
         uint32_t stage_addr = ring;
         const float kscale = p.scale_log2 * DEC_K_UNIT;
-        const float b0 = DEC_K_SUBNORMAL ? q_sum[2 * j] * (8.0f / DEC_K_UNIT) : 0.0f;
-        const float b1 = DEC_K_SUBNORMAL ? q_sum[2 * j + 1] * (8.0f / DEC_K_UNIT) : 0.0f;
+        const float b0 = q_sum[2 * j] * (8.0f / DEC_K_UNIT);
+        const float b1 = q_sum[2 * j + 1] * (8.0f / DEC_K_UNIT);
         const int n_full = n_my - (has_ragged ? 1 : 0);
         auto fetch = [&](QTile& d, int i) {                 // ring stage of tile i -> registers, then refill it
             d.ka = lds128(stage_addr); d.kb = lds128(stage_addr + 512);
@@ -600,7 +577,6 @@ decode_kernel(const DecParams p) {
             stage_addr = (i % DEC_STAGES == DEC_STAGES - 1) ? ring : stage_addr + DEC_STAGE_BYTES;
         };
         int i = 0;
-#if DEC_PAIR
         for (; i + 2 <= n_full; i += 2) {
             cp_async_wait<DEC_STAGES - 2>();                // tiles i and i + 1 have landed
             QTile A, B;
@@ -608,7 +584,6 @@ decode_kernel(const DecParams p) {
             fetch(B, i + 1);
             quant_tile_pair(A, B, qf, kscale, b0, b1, st, acc);
         }
-#endif
         for (; i < n_my; ++i) {
             cp_async_wait<DEC_STAGES - 1>();                // tile i has landed
             QTile A;

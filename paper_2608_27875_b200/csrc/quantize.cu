@@ -11,7 +11,7 @@
 // attention kernel streams - V and V^ = code * scale as fp16, INT4 codes widened to e4m3 bytes - while the tile is in registers.
 //
 // Arithmetic is fp32 with one IEEE rounding per operation (no FMA contraction, no fast-math):
-//   scale = absmax / c ; inv = c / absmax ; code = rint(x * inv) clamped, or e4m3(x * inv).
+//   scale = absmax / c ; inv = c / absmax ; code = rint(x * inv), which cannot leave [-c, c], or e4m3(x * inv).
 #include "quantize.cuh"
 
 namespace hyq {
