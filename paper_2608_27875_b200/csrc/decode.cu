@@ -668,6 +668,10 @@ decode_kernel(const DecParams p) {
 // independent loads (the kernel is pure latency otherwise: it moves a few hundred KB).
 constexpr int DEC_MAX_SPLITS = 1024;
 constexpr int DEC_RAGGED_SPLITS = 64;       // ... of a ragged batch cut by share
+// SHARE: slices cut by share, a head's last one marked.  AHEAD: accumulators in flight, the first ones beside the (m, l) pairs: 24 where there
+// are more than eight slices (18 slices, 4 x 8 heads, INT8: 8 34.5 us a step, 12 34.1, 24 32.6), eight where there are few and many heads
+// (256 x 8 heads of one slice: 8 55.9, 24 59.8).
+template <bool SHARE, int AHEAD>
 __global__ void __launch_bounds__(HYQ_D)
 decode_merge_kernel(const DecParams p, int out_fp32, void* __restrict__ out, float* __restrict__ lse) {
     const long unit = blockIdx.x;                                  // (b * Hkv + kv head) * hgroups + head group
@@ -683,21 +687,25 @@ decode_merge_kernel(const DecParams p, int out_fp32, void* __restrict__ out, flo
     __shared__ float red[2][HYQ_D / 32];
     __shared__ int n_end[2];
     const long slot0 = unit * p.splits * DEC_MAX_GROUP + h;        // slice s sits at slot0 + s * DEC_MAX_GROUP
-    if (p.ragged_ctas) {                                           // the first entry with the sign is the last one written
+    const float2* ml_at = reinterpret_cast<const float2*>(part_ml) + slot0;
+    const float* acc_at = part_acc + slot0 * HYQ_D + threadIdx.x;
+    float acc[AHEAD];
+    auto load = [&](int s0) {
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i) acc[i] = s0 + i < splits ? __ldg(acc_at + (long)(s0 + i) * (DEC_MAX_GROUP * HYQ_D)) : 0.0f;
+    };
+    float2 ml = (int)threadIdx.x < splits ? __ldg(ml_at + (long)threadIdx.x * DEC_MAX_GROUP) : make_float2(-INFINITY, 0.0f);
+    load(0);
+    if (SHARE) {                                                   // the first entry with the sign is the last one written
         static_assert(DEC_RAGGED_SPLITS <= 64, "two warps look");
-        if (threadIdx.x < 64) {
-            const bool end = (int)threadIdx.x < p.splits && (__float_as_uint(__ldg(part_ml + (slot0 + (long)threadIdx.x * DEC_MAX_GROUP) * 2 + 1)) >> 31);
-            const unsigned b = __ballot_sync(0xffffffffu, end);
-            if ((threadIdx.x & 31) == 0) n_end[threadIdx.x >> 5] = b ? (int)threadIdx.x + __ffs(b) : p.splits;
-        }
+        const unsigned b = __ballot_sync(0xffffffffu, (int)threadIdx.x < splits && (__float_as_uint(ml.y) >> 31));
+        if ((threadIdx.x & 31) == 0 && threadIdx.x < 64) n_end[threadIdx.x >> 5] = b ? (int)threadIdx.x + __ffs(b) : splits;
         __syncthreads();
         splits = min(n_end[0], n_end[1]);
+        ml = (int)threadIdx.x < splits ? make_float2(ml.x, fabsf(ml.y)) : make_float2(-INFINITY, 0.0f);
     }
-    float M = -INFINITY;
-    for (int s = threadIdx.x; s < splits; s += HYQ_D) {
-        wt[s] = __ldg(part_ml + (slot0 + (long)s * DEC_MAX_GROUP) * 2);
-        M = fmaxf(M, wt[s]);
-    }
+    float M = ml.x;
+    for (int s = threadIdx.x + HYQ_D; s < splits; s += HYQ_D) M = fmaxf(M, __ldg(ml_at + (long)s * DEC_MAX_GROUP).x);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
     if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = M;
@@ -705,8 +713,9 @@ decode_merge_kernel(const DecParams p, int out_fp32, void* __restrict__ out, flo
     M = fmaxf(fmaxf(red[0][0], red[0][1]), fmaxf(red[0][2], red[0][3]));
     float L = 0.0f;
     for (int s = threadIdx.x; s < splits; s += HYQ_D) {
-        const float w = wt[s] == -INFINITY ? 0.0f : ex2(wt[s] - M);
-        L += fabsf(__ldg(part_ml + (slot0 + (long)s * DEC_MAX_GROUP) * 2 + 1)) * w;
+        if (s >= HYQ_D) ml = __ldg(ml_at + (long)s * DEC_MAX_GROUP);
+        const float w = ml.x == -INFINITY ? 0.0f : ex2(ml.x - M);
+        L += ml.y * w;
         wt[s] = w;
     }
 #pragma unroll
@@ -715,8 +724,12 @@ decode_merge_kernel(const DecParams p, int out_fp32, void* __restrict__ out, flo
     __syncthreads();
     L = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
     float A = 0.0f;
-#pragma unroll 8
-    for (int s = 0; s < splits; ++s) A += __ldg(part_acc + (slot0 + (long)s * DEC_MAX_GROUP) * HYQ_D + threadIdx.x) * wt[s];
+    for (int s0 = 0; s0 < splits; s0 += AHEAD) {
+        if (s0 > 0) load(s0);
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i)
+            if (s0 + i < splits) A += acc[i] * wt[s0 + i];
+    }
     const float o = L > 0.0f ? A / L : 0.0f;               // a sequence with no cached row at all: zeros
     const long head = (unit / hgroups) * g + h_base + h;
     const long oi = head * HYQ_D + threadIdx.x;
@@ -811,7 +824,7 @@ int launch_decode(const void* q, const hyq_kv_cache& c, const int32_t* lengths, 
                                                                                                     : decode_kernel<HYQ_FMT_INT4>;
     const int rc = launch_pdl(kern, grid, dim3(DEC_THREADS), ring_bytes, st, p);
     if (rc != HYQ_OK) return rc;
-    return launch_pdl(decode_merge_kernel, dim3((unsigned)units, (unsigned)(p.g < DEC_MAX_GROUP ? p.g : DEC_MAX_GROUP)), dim3(HYQ_D), 0, st,
+    return launch_pdl(p.ragged_ctas ? decode_merge_kernel<true, 8> : splits > 8 ? decode_merge_kernel<false, 24> : decode_merge_kernel<false, 8>, dim3((unsigned)units, (unsigned)(p.g < DEC_MAX_GROUP ? p.g : DEC_MAX_GROUP)), dim3(HYQ_D), 0, st,
                       p, out_dtype, out, lse);
 }
 
