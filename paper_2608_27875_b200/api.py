@@ -331,10 +331,11 @@ def _prefill(qs, ks, vs, B, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens
 def hybrid_prefill(q, k, v, window: int, k_sel: int, fmts=(FMT_INT8, FMT_INT8, FMT_INT8), impl: int = IMPL_AUTO,
                    out_dtype=torch.float32):
     """The whole path on device tensors: select -> quantize Q, K, V -> fused attention."""
-    # (the library sees pointers only)
-    if v.shape != k.shape or k.shape[0] != q.shape[0] or k.shape[3] != q.shape[3]:
-        raise ValueError(f"q, k, v: {tuple(q.shape)}, {tuple(k.shape)} and {tuple(v.shape)} don't belong together")
-    if impl not in (IMPL_AUTO, IMPL_TCGEN05) or q.shape[2] != k.shape[2]:        # stage by stage (an unknown kernel is refused there)
+    B, Hq, L, D = q.shape
+    Bk, Hkv, Lk, Dk = sk = k.shape
+    if v.shape != sk or Bk != B or Dk != D:                  # (the library sees pointers only)
+        raise ValueError(f"q, k, v: {tuple(q.shape)}, {tuple(sk)} and {tuple(v.shape)} don't belong together")
+    if impl not in (IMPL_AUTO, IMPL_TCGEN05) or L != Lk:     # stage by stage (an unknown kernel is refused there)
         idx = hyq_select_vertical(q, k, window, k_sel)
         qc, qs = hyq_quantize_blocks(q, fmts[0])
         kc, ks = hyq_quantize_blocks(k, fmts[1])
@@ -344,8 +345,6 @@ def hybrid_prefill(q, k, v, window: int, k_sel: int, fmts=(FMT_INT8, FMT_INT8, F
         return dict(idx=idx, q_codes=qc, k_codes=kc, v_codes=vc, q_scales=qs, k_scales=ks, v_scales=vs, out=out)
     for t, n in ((q, "q"), (k, "k"), (v, "v")):
         _dev(t, torch.bfloat16, n)
-    B, Hq, L, D = q.shape
-    Hkv = k.shape[1]
     if D != 128:
         raise HyqError(2, "hybrid_prefill")
     k_eff = k_sel if L - window > 0 else 0
