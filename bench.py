@@ -46,6 +46,16 @@ NCU_TRAFFIC_BYTES = {"c2": 733547008 + 503056896}
 NCU_DECODE_TRAFFIC_BYTES_B4 = 157169152 + 3803392
 
 
+def same_result(a, b) -> bool:
+    """The same bits; or, where the few heads of one call have their units shared out over CTAs and the other call's are not (the
+    partial sums are then added in another order), equal within the bounds that the tests hold the kernel to."""
+    if torch.equal(a, b):
+        return True
+    d, ref = (a.float() - b.float()).abs(), b.float().abs()
+    # (a bf16 output may lie a rounding step, 2^-8 of the value, apart)
+    return bool((d <= 1e-2 + (2.0**-8 * ref if a.dtype == torch.bfloat16 else 0.0)).all()) and float(d.sum() / ref.sum()) <= 2e-3
+
+
 def workload_config(w, world: int = 1, strong: bool = False) -> dict:
     """The `config` object of the JSON line: the same keys and values from both arms (hyq and reference)."""
     return {"workload": w.name, "B": w.B * (1 if strong else max(1, world)), "Hq": w.Hq, "Hkv": w.Hkv, "L": w.L, "D": w.D,
@@ -683,9 +693,9 @@ def run_hyq(args, w):
         if n > 0:
             e2e_ms.append((time.perf_counter() - t0) * 1e3)
     assert pipe.status() == 0, "attention kernel reported a device-side error"
-    # the pipelined units must reproduce the whole-batch result bit for bit (checked on the last unit)
+    # the pipelined units must reproduce the whole-batch result (checked on the last unit)
     g_ = wr.Hq // wr.Hkv
-    assert torch.equal(out_host[wr.B - 1:, wr.Hq - g_:].to(dev), path.out[wr.B - 1:, wr.Hq - g_:]), "pipelined e2e differs"
+    assert same_result(out_host[wr.B - 1:, wr.Hq - g_:].to(dev), path.out[wr.B - 1:, wr.Hq - g_:]), "pipelined e2e differs"
     e2e_ms_max = sharding.max_over_ranks(float(np.mean(e2e_ms)), dev)
     e2e_val = world * flops / (e2e_ms_max * 1e-3) / 1e12
     # the same with the output stored as bf16 (RNE of the fp32 result, the dtype of Q, K, V): half the D2H bytes
@@ -700,7 +710,7 @@ def run_hyq(args, w):
         if n > 0:
             e2e16_ms.append((time.perf_counter() - t0) * 1e3)
     assert pipe16.status() == 0, "attention kernel reported a device-side error"
-    assert torch.equal(out_host16[wr.B - 1:, wr.Hq - g_:].to(dev), path.out[wr.B - 1:, wr.Hq - g_:].to(torch.bfloat16)), "bf16 e2e differs"
+    assert same_result(out_host16[wr.B - 1:, wr.Hq - g_:].to(dev), path.out[wr.B - 1:, wr.Hq - g_:].to(torch.bfloat16)), "bf16 e2e differs"
     e2e16_ms_max = sharding.max_over_ranks(float(np.mean(e2e16_ms)), dev)
     h2d = sum(t.numel() * t.element_size() for t in (Q, K, V))
     d2h = out_host.numel() * out_host.element_size()
