@@ -128,10 +128,10 @@ int hyq_select_vertical_static(const void* q, const void* k_, int B, int Hq, int
  *   S[p] = sum over t in T of a_tp,    p in the non-window prefix [0, P),  P = max(0, Lk - window)
  *   idx_out[b, h, :] = positions of the k largest S, ties towards the lower position, ASCENDING.
  *
- *   All arithmetic is fp64 with a fixed order of operations (fma chain over channels, a polynomial exp,
- *   row sums as 64-key chunk trees combined in ascending order, queries added in ascending order), so the
- *   selected set is reproducible bit for bit.  Cost: two passes of n_queries * Lk * D fp64 fma per head -
- *   meant for a handful of tail queries (tens), not for the whole window.
+ *   All arithmetic is fp64 with a fixed order of operations (products added in ascending channel order, as by
+ *   a chain of fma; a polynomial exp, row sums as 64-key chunk trees combined in ascending order, queries added
+ *   in ascending order), so the selected set is reproducible bit for bit.  Cost: n_queries * Lk * D fp64 fma per
+ *   head - meant for a handful of tail queries (tens), not for the whole window.
  *
  *   Arguments, outputs and errors as hyq_select_vertical, plus: n_queries > min(window, Lq) or Lq > Lk ->
  *   INVALID_ARG.  softmax_scale 0 => 1/sqrt(D).  workspace: hyq_select_vertical_mass_workspace bytes

@@ -16,7 +16,8 @@
 // through its heads in groups whose scores fit in L2.
 //
 // The score kernel multiplies with the fp64 matrix instruction, whose results are those of the fma chain in ascending order of
-// the contraction index, bit for bit (the index sets of the tests depend on it).  It runs at 18.4 T fma/s, the plain instruction
+// the contraction index, bit for bit (not promised by its manual: the tests hold keys that agree up to 50 binary orders below
+// their scores against it).  It runs at 18.4 T fma/s, the plain instruction
 // at 15.3, of which its kernels saw half beside their conversions of bf16 bits and shared-memory loads (and doubles staged in shared
 // memory, 8 x 4 instead of 2 x 8 chains per thread or twice the warps did not change that): one conversion now serves 16 queries.
 // A warp owns a chunk of 64 keys against up to 16 queries.  12007 keys, 32 heads, 16 queries: 124 + 8 + 125 us for the three kernels
