@@ -9,7 +9,10 @@ __host__ __device__ inline int query_rows(const hyq_attn_args& a) { return a.Lq 
 
 constexpr int TC_ROWS = 256;                // query rows of a work unit (two 128-row tiles of one query head)
 constexpr int TC_SMS = 148;
-constexpr int VL_TILE_BYTES = 2048;
+constexpr int VL_TILE_BYTES = 1024;
+// element 0 of a key's row in the vertical-line operand: e4m3 scores get -inf in e5m2 added for a vertical-line key (0 otherwise);
+// integer scores start from 2^63 times a bf16 number, 1.5 * 2^23 or, for a vertical-line key, -1.5 * 2^127 (attn_tc.cu, LIFT)
+constexpr uint32_t VL_KNOCK_E5M2 = 0xFCu, VL_KNOCK_BF16 = 0xDFC0u, VL_PLAIN_BF16 = 0x2BC0u;
 constexpr int TC_MAX_SEQ = 32;              // sequences of one ragged launch (the table travels as a kernel parameter) ...
 constexpr int TC_MAX_LEVELS = 512;          // ... and units per head of its longest sequence
 
@@ -67,9 +70,8 @@ struct TcWorkspace {
     size_t vvl;         // fp16 [vl_rows][D]            gathered vertical-line V rows
     size_t q8;          // u8   [q_rows][D]             INT4 only: Q codes as e4m3 bytes
     size_t k8;          // u8   [kv_rows][D]            INT4 only: K codes as e4m3 bytes
-    size_t vl_tiles;    // u8   [mask_words/2][2048] per head, FP8 / INT4 scores only: per 64-key tile a 64 x 32 e5m2 operand, -inf
-                        //                              in element 0 of a vertical-line key's row, zero elsewhere (two 16-byte
-                        //                              column chunks, each [64 keys][16 bytes])
+    size_t vl_tiles;    // u8   [mask_words/2][1024] per head: the first 16 bytes of every key's row of the vertical-line operand
+                        //                              (element 0 as above, zero elsewhere), [64 keys][16 bytes] per tile
     size_t redo;        // i32x4 [1 + pieces]           pieces of work the second launch does again, behind their count
     size_t part_o;      // f32  [slots][256][D]         split sequences only: partial accumulators ...
     size_t part_ml;     // f32  [slots][256][2]         ... and (reference maximum, row sum) per row
@@ -78,6 +80,9 @@ struct TcWorkspace {
     int slots;          // partial results
     int pieces;         // pieces of work at most (entries of the redo list)
 };
+
+// e4m3 scores need the vertical-line operand only where there are vertical-line keys; integer scores are lifted by it
+inline bool tc_has_vl_tiles(const hyq_attn_args& a, long vl_rows) { return a.q_format == HYQ_FMT_INT8 || vl_rows > 0; }
 
 struct TcPlan {
     TcTables t;

@@ -1,7 +1,7 @@
 // Pre-pass of the fused attention: lays out in the caller's workspace what the tensor-core kernel
 // streams with TMA.  One launch; its blocks take one of five independent pieces of work each, all coalesced and bound by
 // memory traffic (separate launches cost a short prompt 5 launches and 2 memsets of 2-4 us each).
-//   - vertical-line bitmask per (b, h) over key positions and, with e4m3 scores, the operand tiles made from it
+//   - vertical-line bitmask per (b, h) over key positions and the operand tiles made from it
 //   - gathered vertical-line K rows (bf16) and V rows (fp16) per query head, in ascending position
 //     order (the physical "reorder" of Algorithm 2 Stage 1, done per query head because under
 //     GQA the heads that share a KV head select different keys)
@@ -43,6 +43,7 @@ struct PreParams {
     uint4 *v16, *vh16, *kvl, *vvl, *q8, *k8;
     uint32_t* bits;
     uint8_t* tiles;
+    uint32_t vl_plain, vl_knock;                             // element 0 of an operand tile's rows
     uint32_t* redo;
     long q_vecs, k_vecs;
     int window, fixed_tail;
@@ -112,8 +113,7 @@ __device__ __forceinline__ void pre_gather(const TcSeqTable& tab, const PreParam
                           f16x2_sat(bf16_lo(vw.z), bf16_hi(vw.z)), f16x2_sat(bf16_lo(vw.w), bf16_hi(vw.w)));
 }
 
-// 32 bitmask words (1024 keys) of one head, and with e4m3 scores their 16 operand tiles: the byte 0xFC (-inf in e5m2) in
-// element 0 of a vertical key's row, zero elsewhere
+// 32 bitmask words (1024 keys) of one head and their 16 operand tiles (the first 16 bytes of every key's row)
 __device__ __forceinline__ void pre_masks(const TcSeqTable& tab, const PreParams& p, int block) {
     __shared__ uint32_t words[PRE_MASK_WORDS];
     int s = 0;
@@ -144,9 +144,9 @@ __device__ __forceinline__ void pre_masks(const TcSeqTable& tab, const PreParams
     if (p.tiles) {
         uint4* dst = reinterpret_cast<uint4*>(p.tiles + (word0 >> 1) * VL_TILE_BYTES);
         for (int c = threadIdx.x; c < (n_words >> 1) * (VL_TILE_BYTES / 16); c += PRE_THREADS) {
-            const int tile = c >> 7, chunk = c & 127;        // chunks 0..63: elements 0..15 of key `chunk`; 64..127: zeros
-            const bool on = chunk < 64 && ((words[2 * tile + (chunk >> 5)] >> (chunk & 31)) & 1u);
-            dst[c] = make_uint4(on ? 0xFCu : 0u, 0u, 0u, 0u);
+            const int key = c & 63;
+            const bool on = (words[2 * (c >> 6) + (key >> 5)] >> (key & 31)) & 1u;
+            dst[c] = make_uint4(on ? p.vl_knock : p.vl_plain, 0u, 0u, 0u);
         }
     }
 }
@@ -295,7 +295,7 @@ bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads
     const bool int4 = a.q_format == HYQ_FMT_INT4;
     w.q8 = int4 ? take(q_elems) : 0;
     w.k8 = int4 ? take(kv_elems) : 0;
-    w.vl_tiles = (a.q_format != HYQ_FMT_INT8 && vl_rows > 0) ? take((size_t)(words / 2) * VL_TILE_BYTES) : 0;
+    w.vl_tiles = tc_has_vl_tiles(a, vl_rows) ? take((size_t)(words / 2) * VL_TILE_BYTES) : 0;
     w.redo = take((size_t)(1 + pieces) * 16);
     w.part_o = slots ? take((size_t)slots * TC_ROWS * HYQ_D * 4) : 0;
     w.part_ml = slots ? take((size_t)slots * TC_ROWS * 2 * 4) : 0;
@@ -368,7 +368,9 @@ int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, const TcSource
     p.kvl = reinterpret_cast<uint4*>(base + w.kvl); p.vvl = reinterpret_cast<uint4*>(base + w.vvl);
     p.q8 = reinterpret_cast<uint4*>(base + w.q8); p.k8 = reinterpret_cast<uint4*>(base + w.k8);
     p.bits = reinterpret_cast<uint32_t*>(base + w.vl_bits);
-    p.tiles = (a.q_format != HYQ_FMT_INT8 && t.vl_rows > 0) ? reinterpret_cast<uint8_t*>(base + w.vl_tiles) : nullptr;
+    p.tiles = tc_has_vl_tiles(a, t.vl_rows) ? reinterpret_cast<uint8_t*>(base + w.vl_tiles) : nullptr;
+    p.vl_plain = a.q_format == HYQ_FMT_INT8 ? VL_PLAIN_BF16 : 0u;
+    p.vl_knock = a.q_format == HYQ_FMT_INT8 ? VL_KNOCK_BF16 : VL_KNOCK_E5M2;
     p.redo = reinterpret_cast<uint32_t*>(base + w.redo);
     auto kern = a.v_format == HYQ_FMT_INT8 ? tc_prepass_kernel<HYQ_FMT_INT8> : tc_prepass_kernel<HYQ_FMT_FP8_E4M3>;
     return launch_pdl(kern, dim3((unsigned)n), dim3(PRE_THREADS), 0, st, t, p);

@@ -20,12 +20,11 @@
 // one thread per query row (row r = TMEM lane r of every score tile; the thread holds the 64 scores
 // of its row in two register halves), so a row's reference maximum needs no agreement between
 // threads.  The exponentials are taken against that reference, which is only raised when
-// a tile exceeds it by more than 2^14 (the rescale of O is then rare); integer scores become floats
-// by a magic-number add.  The vertical-line keys inside a low-bit tile are taken out of pass A before the
-// softmax sees the scores: with e4m3 codes by a fifth MMA step per tile, S += ones . mask^T in e5m2 (the one
-// 8-bit format with an infinity), whose 64 x 32 operand - -inf in element 0 of a vertical key's row - is copied
-// in with the K codes; with int8 codes (no infinity) by the softmax warps, which store -inf over those columns
-// of S before they read the tile.  The attention call launches the kernel twice: the first launch takes most low-bit
+// a tile exceeds it by more than 2^14 (the rescale of O is then rare).  The vertical-line keys inside a
+// low-bit tile are taken out of pass A before the softmax sees the scores, by a fifth MMA step per tile whose
+// operand is copied in with the K codes: with e4m3 codes S += ones . mask^T in e5m2 (the one 8-bit format with an
+// infinity) behind the four steps, with int8 codes S = 2^63 . mask^T in bf16 before them, which turns integer scores
+// into floats as well (LIFT below).  The attention call launches the kernel twice: the first launch takes most low-bit
 // tiles without looking for their maximum and checks the tiles' row sums instead, the second redoes the CTAs (normally
 // none) in which that check failed - see the comment at attn_tc_kernel.  Every mbarrier wait is bounded; when one expires the CTA records
 // HYQ_ERR_TIMEOUT in the status word, waits (bounded) for its own copies and MMAs in flight and unwinds.
@@ -61,8 +60,9 @@ constexpr uint32_t SV_OFF = SK_OFF + RING_BYTES;
 constexpr uint32_t TILE_SMEM = SV_OFF + RING_BYTES;                 // 229376
 constexpr int MAX_STAGES = 4;
 // In the low-bit pass a K ring slot holds 8 KB of codes; behind them sit the vertical-line operand of the tile
-// (64 keys x 32 e5m2 elements, copied in with the codes) and this slot's copy of the constant 128 x 32 operand whose
-// element 0 of every row is one.
+// (64 keys x 32 bytes, of which the first 16 of every key are copied in with the codes) and this slot's copy of the constant
+// 128 x 32 byte operand, zero but for element 0 of every row.  The second 16 bytes of every key are zero: they are read from the
+// constant operand's second half.
 constexpr uint32_t VLT_OFF = 8192, ONES_OFF = 10240, ONES_BYTES = 4096;
 
 // geometry that follows from the keys per tile (64: 4-stage ring, two S buffers per query tile)
@@ -79,10 +79,19 @@ constexpr uint32_t TM_COLS = 512;
 __device__ __forceinline__ uint32_t tm_s(int q) { return q * 128; }      // + buffer * BN
 __device__ __forceinline__ uint32_t tm_o(int q) { return 256 + q * 128; }
 
-constexpr uint32_t INT_MAGIC = 0x4B400000u;          // float(2^23 + 2^22): int -> float by integer add
+// LIFT: integer scores arrive as floats.  An accumulator that holds the bits of 2^23 + 2^22 is an integer to which kind::i8 adds
+// the score s, and the bits of the float 2^23 + 2^22 + s afterwards (|s| <= 127 * 127 * 128 < 2^21); the offset is taken out again by the bias of
+// the exponent.  A vertical-line key's accumulator holds -1.5 * 2^127 instead: the score only moves its mantissa, whatever it
+// is, and the exponential is zero (its bits may not be those of -inf: +1 would make them a NaN).  Both are products of the
+// bf16 step's operands: LIFT_A in element 0 of every row of the constant operand, VL_PLAIN_BF16 / VL_KNOCK_BF16 in the tile's.
+// Before, the softmax warps added the offset to 64 scores per row and tile and stored -inf over vertical keys' columns, on
+// their critical path: whole calls at 8192 x 32 heads 611 -> 570 us, 4 x 16384 x 40 heads 11164 -> 10149 us, the same bits.
 constexpr float INT_MAGIC_F = 12582912.0f;
+constexpr uint32_t LIFT_A_BF16 = 0x5F00u;            // 2^63
+constexpr float LIFT_KNOCKED = -1.0e30f;             // a lifted score below this belongs to a vertical-line key
 constexpr uint32_t KNOCKOUT_F32 = 0xFF800000u;       // -inf
-constexpr uint32_t KNOCKOUT_S32 = KNOCKOUT_F32 - INT_MAGIC;   // becomes -inf after the magic add
+// smallest score factor: a zero scale (all-zero tile) still has to let -inf and -1.5 * 2^127 pass through the multiply
+constexpr float MIN_FACTOR = 1e-20f;
 
 // CTAs whose work was done a second time by the exact kernel (read and reset by the test hook)
 __device__ unsigned long long g_tc_restarts = 0ull;
@@ -109,7 +118,7 @@ struct TcParams {
     int4* redo;                  // [0].x: pieces of work of the optimistic kernel that it gave up, [1 + i]: what they are (Piece)
     int grid_x;                  // plain whole prefill: units per head
     int head_group;              // heads whose items are interleaved, longest first (a whole number of KV heads)
-    const uint8_t* vl_tiles;     // FP8 / INT4 scores: the vertical-line operand tiles [B*Hq][mask_words/2][2048] (null: none)
+    const uint8_t* vl_tiles;     // the vertical-line operand tiles [B*Hq][mask_words/2][VL_TILE_BYTES] (null: none)
     void* out;
     float* lse;
     int32_t* status;
@@ -286,10 +295,22 @@ __device__ __forceinline__ bool mma_issuer(int q, const QSched& sq, const Walk& 
     const uint64_t dqc = make_smem_desc(smem_u32(smem + SQC_OFF + q * QC_TILE_BYTES), 0, 1024);
     const uint64_t dk0 = make_smem_desc(smem_u32(smem + SK_OFF), 0, 1024);
     const uint64_t dv0 = make_smem_desc(smem_u32(smem + SV_OFF), G::STAGE_BYTES / 2, 1024);
-    // S += ones . mask^T: -inf on the columns of vertical-line keys, +0 elsewhere (e5m2 has an infinity, e4m3 has not)
+    // The step with the vertical-line operand.  e4m3 scores: S += ones . mask^T behind the four steps of the codes, -inf on the
+    // columns of vertical-line keys, +0 elsewhere (e5m2 has an infinity, e4m3 has not).  Integer scores: S = 2^63 . mask^T in bf16
+    // before them, so that the integer steps accumulate on the bits of a float (see LIFT below).
     const uint32_t idesc_vl = make_idesc(ACC_F32, FMT_E5M2, FMT_E5M2, 0, 0, BM, BN);
     const uint64_t dones0 = make_smem_desc_plain(smem_u32(smem + SK_OFF + ONES_OFF), BM * 16, 128);
-    const uint64_t dvlt0 = make_smem_desc_plain(smem_u32(smem + SK_OFF + VLT_OFF), BN * 16, 128);
+    const uint64_t dvlt0 = make_smem_desc_plain(smem_u32(smem + SK_OFF + VLT_OFF), ONES_OFF + BM * 16 - VLT_OFF, 128);
+    // scores of a low-bit tile in ring stage `st` (in units of STAGE16)
+    auto qk_low = [&](uint32_t d, uint64_t st) {
+        if (!LOWBIT_FP8) umma_ss_f16(d, dones0 + st, dvlt0 + st, idesc_qk, 0u);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            if (LOWBIT_FP8) umma_ss_f8f6f4(d, dqc + kk * 2, dk0 + st + kk * 2, idesc_lq, kk > 0);
+            else umma_ss_i8(d, dqc + kk * 2, dk0 + st + kk * 2, idesc_lq, 1u);
+        }
+        if (LOWBIT_FP8 && vl_mma) umma_ss_f8f6f4(d, dones0 + st, dvlt0 + st, idesc_vl, 1u);
+    };
     const uint32_t ts0 = tmem + tm_s(q), to = tmem + tm_o(q);
     const OwnTiles own = own_tiles(sq, w);
     const int nA = w.nA;
@@ -304,17 +325,12 @@ __device__ __forceinline__ bool mma_issuer(int q, const QSched& sq, const Walk& 
         if (!k_ready && !mbar_wait(&bars.kv_full[kst], kpar, limit)) return false;
         if (own.has(tq)) {
             tc_fence_after();
-            const uint64_t dk = dk0 + (uint64_t)(kst * STAGE16);
             const uint32_t buf = n_qk % NBUF;
             const uint32_t d = ts0 + buf * BN;
             if (tq < nA) {
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    if (LOWBIT_FP8) umma_ss_f8f6f4(d, dqc + kk * 2, dk + kk * 2, idesc_lq, kk > 0);
-                    else umma_ss_i8(d, dqc + kk * 2, dk + kk * 2, idesc_lq, kk > 0);
-                }
-                if (LOWBIT_FP8 && vl_mma) umma_ss_f8f6f4(d, dones0 + (uint64_t)(kst * STAGE16), dvlt0 + (uint64_t)(kst * STAGE16), idesc_vl, 1u);
+                qk_low(d, (uint64_t)(kst * STAGE16));
             } else {
+                const uint64_t dk = dk0 + (uint64_t)(kst * STAGE16);
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk)
                     umma_ss_f16(d, dq + ((kk >> 2) * (Q_TILE_BYTES / 32) + (kk & 3) * 2),
@@ -359,12 +375,7 @@ __device__ __forceinline__ bool mma_issuer(int q, const QSched& sq, const Walk& 
                 umma_commit_a(a_bars + (uint32_t)offsetof(TcBarriers, kv_free) + i * 8);
                 if (!(done & 2u) && !mbar_wait_a(a_kf, kpi, limit)) { ok = false; break; }
                 tc_fence_after();
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    if (LOWBIT_FP8) umma_ss_f8f6f4(ts0 + bf * BN, dqc + kk * 2, dk0 + (uint64_t)(ks * STAGE16 + kk * 2), idesc_lq, kk > 0);
-                    else umma_ss_i8(ts0 + bf * BN, dqc + kk * 2, dk0 + (uint64_t)(ks * STAGE16 + kk * 2), idesc_lq, kk > 0);
-                }
-                if (LOWBIT_FP8 && vl_mma) umma_ss_f8f6f4(ts0 + bf * BN, dones0 + (uint64_t)(ks * STAGE16), dvlt0 + (uint64_t)(ks * STAGE16), idesc_vl, 1u);
+                qk_low(ts0 + bf * BN, (uint64_t)(ks * STAGE16));
                 umma_commit_a(a_bars + (uint32_t)offsetof(TcBarriers, s_full) + (q * 2 + bf) * 8);
             }
             if (!ok) return false;
@@ -537,10 +548,10 @@ __device__ __forceinline__ float row_exp32(const uint32_t (&raw)[32], float sc, 
     return (s0 + s1) + (s2 + s3);
 }
 
-// columns [c0, c0 + 32) of a boundary tile: entries outside [lo_eff, lo_eff + span] of this row become `knock`
-__device__ __forceinline__ void mask_cols32(uint32_t (&raw)[32], int c0, int lo_eff, unsigned span, uint32_t knock) {
+// columns [c0, c0 + 32) of a boundary tile: entries outside [lo_eff, lo_eff + span] of this row become -inf
+__device__ __forceinline__ void mask_cols32(uint32_t (&raw)[32], int c0, int lo_eff, unsigned span) {
 #pragma unroll
-    for (int e = 0; e < 32; ++e) raw[e] = ((unsigned)(c0 + e - lo_eff) <= span) ? raw[e] : knock;
+    for (int e = 0; e < 32; ++e) raw[e] = ((unsigned)(c0 + e - lo_eff) <= span) ? raw[e] : KNOCKOUT_F32;
 }
 
 // LOWBIT_FP8: the low-bit codes are e4m3 bytes (kind::f8f6f4), else int8 (kind::i8).  KIND other than PLAIN: everything but a plain
@@ -653,8 +664,8 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
         return s;
     };
     QSched qs0 = make_sched(0), qs1 = make_sched(1);
-    // vertical-line keys of the low-bit pass: with e4m3 scores an extra MMA step per tile adds -inf to their columns
-    const uint8_t* vl_tiles_head = (LOWBIT_FP8 && p.vl_tiles) ? p.vl_tiles + (mask_at >> 1) * VL_TILE_BYTES : nullptr;
+    // vertical-line keys of the low-bit pass: an extra MMA step per tile takes their columns out (integer scores: lifts the others, too)
+    const uint8_t* vl_tiles_head = p.vl_tiles ? p.vl_tiles + (mask_at >> 1) * VL_TILE_BYTES : nullptr;
 
     // Everything up to the first synchronisation is independent work on different warps: barriers, query loads and
     // tensor memory (warp 0), the counts of vertical keys (warps 1 and 2), the constant operand (all).
@@ -700,7 +711,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
         for (int c = threadIdx.x; c < n_slots * (int)(ONES_BYTES / 16); c += TC_THREADS) {
             const int slot = c / (int)(ONES_BYTES / 16), chunk = c % (int)(ONES_BYTES / 16);   // chunks 0..127: element 0..15 of row `chunk`
             *reinterpret_cast<uint4*>(smem + SK_OFF + slot * G::STAGE_BYTES + ONES_OFF + chunk * 16) =
-                make_uint4(chunk < BM ? 0x3Cu : 0u, 0u, 0u, 0u);                               // 0x3C = 1.0 in e5m2
+                make_uint4(chunk < BM ? (LOWBIT_FP8 ? 0x3Cu : LIFT_A_BF16) : 0u, 0u, 0u, 0u);  // 0x3C = 1.0 in e5m2
         }
         fence_proxy_async();
     }
@@ -778,7 +789,6 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
 #else
             const float q_scale = row_live ? __ldg(p.q_scales + qs_at + i / HYQ_BLOCK_TOKENS) : 0.0f;
 #endif
-            constexpr uint32_t knock_lq = LOWBIT_FP8 ? KNOCKOUT_F32 : KNOCKOUT_S32;
             float m_used = -INFINITY, l_h = 0.0f;               // reference maximum of the row; row sum
             bool over = false;                                  // a tile taken without its maximum had a row sum beyond fp16
             bool dead = false;                                  // this warp ran into an expired wait
@@ -790,18 +800,16 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 const int tb = own.b_beg + (n - own.a_end);
                 return (tb < own.b_end) ? tb : own.c_beg + (n - own.a_end - (own.b_end - own.b_beg));
             };
-            // K scale and this half's vertical-line bitmask word of a low-bit tile, fetched one tile ahead of their use
-            // (tile n of the low-bit pass sits at walk position n; its block and mask words exist for n < a_end)
+            // K scale of a low-bit tile, fetched one tile ahead of its use (tile n of the low-bit pass sits at walk position n; its
+            // block exists for n < a_end)
             // (other block sizes: a 64-key tile n lies in block n / 2 or in blocks 2n and 2n + 1, one per column half)
             const float* ks_ptr = p.k_scales + ks_at;
-            const uint32_t* vl_ptr = p.vl_bits + mask_at;
             float nks = 0.0f;
 #if HYQ_TC_VARIANT_BT
             float nks_b = 0.0f, cs_hi = 0.0f;                   // K scale and score factor of columns 32-63 (32-token blocks: their own block)
 #endif
-            uint64_t nvl = 0u;                                  // both mask words of the tile (columns 0-31 low, 32-63 high)
             auto prefetch_tile = [&](int n) {
-                nks = 0.0f; nvl = 0u;
+                nks = 0.0f;
 #if HYQ_TC_VARIANT_BT
                 nks_b = 0.0f;
 #endif
@@ -812,7 +820,6 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
 #else
                 nks = __ldg(ks_ptr + n);
 #endif
-                if (!LOWBIT_FP8) nvl = (uint64_t)__ldg(vl_ptr + 2 * n) | ((uint64_t)__ldg(vl_ptr + 2 * n + 1) << 32);
             };
             prefetch_tile(n0);
             const float qs2 = q_scale * p.scale_log2;
@@ -820,9 +827,8 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             // one tile of the online softmax for this thread's row: all 64 columns, in two register halves.  Returns
             // false when this warp ran into an expired wait.
             float tile_max = -INFINITY;                         // maximum of the tile last looked at (this row, log2 units)
-            auto do_tile = [&](auto range_tag, int n, float cs, uint64_t vl, bool int_scores, int lo, int hi, bool look = true) -> bool {
+            auto do_tile = [&](auto range_tag, int n, float cs, bool int_scores, int lo, int hi, bool look = true) -> bool {
                 constexpr bool NEED_RANGE = decltype(range_tag)::value;
-                const uint32_t knock = int_scores ? KNOCKOUT_S32 : KNOCKOUT_F32;
                 const int nl = n - n0;                          // tile number within this CTA's slice
                 const int buf = nl & 1;
                 const uint32_t ts = ts0 + buf * BN;
@@ -831,11 +837,6 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                     return false;
                 }
                 tc_fence_after();
-                // vertical-line keys of a low-bit tile: -inf into their S columns before the row is read
-                if (!LOWBIT_FP8 && vl != 0ull) {                 // uniform over the warp (e4m3 scores: the issuer's extra MMA step did it)
-                    while (vl) { const int c = __ffsll((long long)vl) - 1; vl &= vl - 1; tmem_st1(ts + c, knock_lq); }
-                    tmem_wait_st();
-                }
                 uint32_t ra[32], rb[32];
                 tmem_ld32(ts, ra);
                 tmem_ld32(ts + 32, rb);
@@ -849,25 +850,20 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 if (NEED_RANGE) {
                     const int lo_eff = (hi >= lo) ? lo : 4096;
                     const unsigned span = (hi >= lo) ? (unsigned)(hi - lo) : 0u;
-                    if (GENERAL || !__all_sync(0xffffffffu, lo == 0 && hi >= 31)) mask_cols32(ra, 0, lo_eff, span, knock);
-                    if (GENERAL || !__all_sync(0xffffffffu, lo <= 32 && hi == BN - 1)) mask_cols32(rb, 32, lo_eff, span, knock);
-                }
-                // integer scores become the floats 2^23 + 2^22 + s by one integer add each (knocked-out entries
-                // become -inf); the offset is taken out again by the bias of the exponent
-                if (int_scores) {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) { ra[e] += INT_MAGIC; rb[e] += INT_MAGIC; }
+                    if (GENERAL || !__all_sync(0xffffffffu, lo == 0 && hi >= 31)) mask_cols32(ra, 0, lo_eff, span);
+                    if (GENERAL || !__all_sync(0xffffffffu, lo <= 32 && hi == BN - 1)) mask_cols32(rb, 32, lo_eff, span);
                 }
 #if HYQ_TC_VARIANT_BT
                 const float csb = cs_hi;                        // the second half's factor (its own K scale with 32-token blocks)
 #endif
                 if (look) {
 #if HYQ_TC_VARIANT_BT
+                const float none = int_scores ? LIFT_KNOCKED : -INFINITY;              // (nothing left of the half: at most this)
                 const float fa = row_max32(ra) - (int_scores ? INT_MAGIC_F : 0.0f), fb = row_max32(rb) - (int_scores ? INT_MAGIC_F : 0.0f);
-                const float mt = fmaxf((fa == -INFINITY) ? -INFINITY : fa * cs, (fb == -INFINITY) ? -INFINITY : fb * csb);
+                const float mt = fmaxf((fa <= none) ? -INFINITY : fa * cs, (fb <= none) ? -INFINITY : fb * csb);
 #else
                 const float f = fmaxf(row_max32(ra), row_max32(rb)) - (int_scores ? INT_MAGIC_F : 0.0f);
-                const float mt = (f == -INFINITY) ? -INFINITY : f * cs;
+                const float mt = (f <= (int_scores ? LIFT_KNOCKED : -INFINITY)) ? -INFINITY : f * cs;
 #endif
                 tile_max = mt;
                 const bool raise = mt > m_used + RAISE_THRESHOLD;
@@ -939,14 +935,12 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             bool warm = false;
             const int n_plain_end = min(n_plain, n_total);
             auto plain_tile = [&]() -> bool {
-                // a zero scale (all-zero tile) still has to let -inf pass through the multiply
-                const float cs = fmaxf(qs2 * nks, 1e-37f);
+                const float cs = fmaxf(qs2 * nks, MIN_FACTOR);
 #if HYQ_TC_VARIANT_BT
-                cs_hi = fmaxf(qs2 * nks_b, 1e-37f);
+                cs_hi = fmaxf(qs2 * nks_b, MIN_FACTOR);
 #endif
-                const auto vl = nvl;
                 prefetch_tile(n + 1);
-                return do_tile(std::false_type{}, n, cs, vl, !LOWBIT_FP8, 0, 0);
+                return do_tile(std::false_type{}, n, cs, !LOWBIT_FP8, 0, 0);
             };
             const bool brief = PIECES && pc.slot >= 0 && n_plain_end - n0 <= 2 * WARM_TILES;
             const int n_warm = n0 + (brief ? WARM_TILES_SHORT : WARM_TILES);
@@ -971,31 +965,22 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 uint32_t ra[32], rb[32];
                 bool have_a = false;
                 for (; n < n_end; ++n) {
-                    const float cs = fmaxf(qs2 * nks, 1e-37f);
+                    const float cs = fmaxf(qs2 * nks, MIN_FACTOR);
 #if HYQ_TC_VARIANT_BT
-                    const float csb = fmaxf(qs2 * nks_b, 1e-37f);
+                    const float csb = fmaxf(qs2 * nks_b, MIN_FACTOR);
 #else
                     const float csb = cs;
 #endif
-                    uint64_t vl = nvl;                         // this tile's vertical-line columns (integer scores only)
                     prefetch_tile(n + 1);
                     const int nl = n - n0, buf = nl & 1;
                     const uint32_t ts = ts0 + buf * BN;
                     if (!have_a) {
                         if (!__all_sync(0xffffffffu, mbar_wait(&bars.s_full[q][buf], (uint32_t)(nl >> 1) & 1u, limit))) { dead = true; aborted = true; break; }
                         tc_fence_after();
-                        if (!LOWBIT_FP8 && vl != 0ull) {
-                            while (vl) { const int c = __ffsll((long long)vl) - 1; vl &= vl - 1; tmem_st1(ts + c, knock_lq); }
-                            tmem_wait_st();
-                        }
                         tmem_ld32(ts, ra);
                     }
                     tmem_wait_ld();
                     tmem_ld32(ts + 32, rb);
-                    if (!LOWBIT_FP8) {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) ra[e] += INT_MAGIC;
-                    }
                     const float bias = LOWBIT_FP8 ? -m_used : fmaf(-INT_MAGIC_F, cs, -m_used);
                     const float bias_b = LOWBIT_FP8 ? -m_used : fmaf(-INT_MAGIC_F, csb, -m_used);
                     uint32_t pa[16], pb[16];
@@ -1007,18 +992,9 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                         const int nl1 = nl + 1, buf1 = nl1 & 1;
                         if (__all_sync(0xffffffffu, mbar_test_wait(&bars.s_full[q][buf1], (uint32_t)(nl1 >> 1) & 1u))) {
                             tc_fence_after();
-                            if (!LOWBIT_FP8 && nvl != 0ull) {     // (nvl: the next tile's columns by now)
-                                uint64_t v1 = nvl;
-                                while (v1) { const int c = __ffsll((long long)v1) - 1; v1 &= v1 - 1; tmem_st1(ts0 + buf1 * BN + c, knock_lq); }
-                                tmem_wait_st();
-                            }
                             tmem_ld32(ts0 + buf1 * BN, ra);
                             have_a = true;
                         }
-                    }
-                    if (!LOWBIT_FP8) {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) rb[e] += INT_MAGIC;
                     }
                     const float t_b = row_exp32(rb, csb, bias_b, pb);
                     tmem_st16(ts + 16, pb);
@@ -1034,21 +1010,20 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             // ---- the remaining low-bit tiles, the vertical-line tiles and the window tiles
             // (number of vertical-line keys this row may use: only needed from here on)
             const int cnt_r = (!aborted && sq.nB > 0 && row_live && qhi(ia) >= 0)
-                                  ? cnt_b_s[q] - vl_between(vl_ptr, qhi(ia), qhi(sq.i1 + off)) : 0;
+                                  ? cnt_b_s[q] - vl_between(p.vl_bits + mask_at, qhi(ia), qhi(sq.i1 + off)) : 0;
             for (; n < n_total && !aborted; ++n) {
                 const int t = walk_pos(n);
                 const float ks = nks;
 #if HYQ_TC_VARIANT_BT
                 const float ks_b = nks_b;
 #endif
-                const auto vl = nvl;
                 prefetch_tile(n + 1);
                 int lo = 0, hi = -1;
                 float cs;
                 const bool lowbit = t < own.a_end;
                 if (lowbit) {
                     hi = row_live ? min(qhi(ia) - t * BN, BN - 1) : -1;
-                    cs = fmaxf(qs2 * ks, 1e-37f);
+                    cs = fmaxf(qs2 * ks, MIN_FACTOR);
                 } else if (t < own.b_end) {
                     hi = min(cnt_r - (t - own.b_beg) * BN - 1, BN - 1);
                     cs = p.scale_log2;
@@ -1059,16 +1034,16 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                     cs = p.scale_log2;
                 }
 #if HYQ_TC_VARIANT_BT
-                cs_hi = lowbit ? fmaxf(qs2 * ks_b, 1e-37f) : cs;
+                cs_hi = lowbit ? fmaxf(qs2 * ks_b, MIN_FACTOR) : cs;
 #endif
                 // tiles that every row of this warp uses in full (most window and vertical-line tiles) need no range mask
                 // and, in the window of a row whose low-bit pass went without them, no maximum (525.3 -> 523.3 us; vertical-line keys
                 // are the ones with the large scores, so their tiles are always looked at)
                 if (__all_sync(0xffffffffu, lo == 0 && hi == BN - 1)) {
-                    if (!do_tile(std::false_type{}, n, cs, vl, lowbit && !LOWBIT_FP8, 0, 0, !warm || t < own.b_end)) aborted = true;
+                    if (!do_tile(std::false_type{}, n, cs, lowbit && !LOWBIT_FP8, 0, 0, !warm || t < own.b_end)) aborted = true;
                     continue;
                 }
-                if (!do_tile(std::true_type{}, n, cs, vl, lowbit && !LOWBIT_FP8, lo, hi)) aborted = true;
+                if (!do_tile(std::true_type{}, n, cs, lowbit && !LOWBIT_FP8, lo, hi)) aborted = true;
             }
 
             // ---- epilogue: the last P.V (MMAs complete in order), sum of the two halves' row sums, O / l
@@ -1334,7 +1309,7 @@ int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, const TcSources* 
     p.scale_log2 = alpha * 1.4426950408889634f;
     p.q_scales = a.q_scales; p.k_scales = a.k_scales; p.vl_idx = a.vl_idx;
     p.vl_bits = reinterpret_cast<const uint32_t*>(base + w.vl_bits);
-    p.vl_tiles = (a.q_format != HYQ_FMT_INT8 && tab.vl_rows > 0) ? reinterpret_cast<const uint8_t*>(base + w.vl_tiles) : nullptr;
+    p.vl_tiles = tc_has_vl_tiles(a, tab.vl_rows) ? reinterpret_cast<const uint8_t*>(base + w.vl_tiles) : nullptr;
     p.out = a.out; p.lse = a.lse; p.status = a.status_word;
     const TcTestHooks hooks = tc_test_hooks();
     p.wait_limit = hooks.wait_limit > 0 ? hooks.wait_limit : WAIT_LIMIT_DEFAULT;
@@ -1344,7 +1319,7 @@ int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, const TcSources* 
     // head" the last heads' long CTAs ran beside idle SMs (L = 8192, 32 heads: the busiest SM 14 % above the mean).
     // Whole KV heads, at most 48 MB of keys and values (half of L2), the heads shared out evenly over the groups.
     p.grid_x = s0.levels;
-    const long kv_bytes = (long)s0.L * (HYQ_D + 2 * HYQ_D + (p.vl_tiles ? 32 * (a.Hq / a.Hkv) : 0));   // codes, V^, vertical-line operands
+    const long kv_bytes = (long)s0.L * (HYQ_D + 2 * HYQ_D + (p.vl_tiles ? VL_TILE_BYTES / 64 * (a.Hq / a.Hkv) : 0));   // codes, V^, vertical-line operands
     const long kv_heads = tab.heads / tab.g, cap = (48L << 20) / kv_bytes > 1 ? (48L << 20) / kv_bytes : 1;
     const long groups = (kv_heads + cap - 1) / cap;
     p.head_group = (int)((kv_heads + groups - 1) / groups) * (a.Hq / a.Hkv);

@@ -86,6 +86,24 @@ def test_vertical_keys_inside_the_window_and_beyond_the_diagonal(impl):
     _check(Q, K, V, INT8, idx, W, impl)
 
 
+@pytest.mark.parametrize("fmts", [INT8, INT4FP8])
+def test_extreme_code_sums_and_zero_tiles_around_vertical_keys(fmts):
+    """Scores whose code products sum to the largest and the smallest number there is (every code +-127: the bits that a
+    vertical-line key's score starts from may reach neither a finite number nor a NaN), a tile of vertical keys only, and
+    all-zero tiles (scale 0) with vertical keys in them."""
+    L, W = 700, 64
+    sign = torch.where(torch.arange(L) % 3 == 0, -1.0, 1.0).view(1, 1, L, 1)
+    pattern = torch.where(rand_bf16((128,), seed=5) > 0, 0.25, -0.25).view(1, 1, 1, 128)
+    Q = (torch.ones(1, 2, L, 1) * pattern).to(torch.bfloat16)
+    K = (sign * pattern).expand(1, 2, L, 128).clone().to(torch.bfloat16)
+    K[:, :, 256:320] = 0
+    K[:, 1, 384:448] = 0
+    V = rand_bf16((1, 2, L, 128), seed=6)
+    a = list(range(64, 128)) + [130, 131, 260, 400, 500, 503]
+    b = [0, 1, 2] + list(range(256, 320)) + [384, 447, 635]
+    _check(Q, K, V, fmts, np.array([[a, b]], dtype=np.int32), W, api.IMPL_TCGEN05)
+
+
 @pytest.mark.parametrize("impl", IMPLS)
 def test_config0_full_output(impl):
     w = wl.CONFIGS["c0"]
