@@ -543,6 +543,7 @@ int hyq_hybrid_prefill(const hyq_prefill_args* args, void* stream) {
             }
             jv.v16 = reinterpret_cast<uint4*>(base + g.plan.w.v16) + a.Hkv * tt * (HYQ_D / 8);
             jv.vh16 = reinterpret_cast<uint4*>(base + g.plan.w.vh16) + a.Hkv * tt * (HYQ_D / 8);
+            jk.kv_fac = jv.kv_fac = reinterpret_cast<float4*>(base + g.plan.w.kv_fac) + a.Hkv * nb;
             tt += (size_t)L; nb += (size_t)((L + a.block_tokens - 1) / a.block_tokens);
             k0 += (size_t)a.k_per_seq[s + i];
         }

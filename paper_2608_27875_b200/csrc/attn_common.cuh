@@ -65,7 +65,8 @@ __host__ __device__ inline int tc_unit_tiles(int L, int Lq, int k, int window, i
 struct TcWorkspace {
     size_t vl_bits;     // uint32 [heads][mask_words] per sequence: vertical-line bitmask over key positions
     size_t v16;         // fp16 [kv_rows][D]            V
-    size_t vh16;        // fp16 [kv_rows][D]            V^ = code * scale
+    size_t vh16;        // fp16 [kv_rows][D]            V^ without the mantissa of its scale: code * 2^e (value_factor)
+    size_t kv_fac;      // f32x4, a block each          K scale, log2 of that mantissa and its reciprocal
     size_t kvl;         // bf16 [vl_rows][D]            gathered vertical-line K rows
     size_t vvl;         // fp16 [vl_rows][D]            gathered vertical-line V rows
     size_t q8;          // u8   [q_rows][D]             INT4 only: Q codes as e4m3 bytes

@@ -5,12 +5,14 @@
 //   - gathered vertical-line K rows (bf16) and V rows (fp16) per query head, in ascending position
 //     order (the physical "reorder" of Algorithm 2 Stage 1, done per query head because under
 //     GQA the heads that share a KV head select different keys)
-//   - V in fp16 (full-precision class) and dequantized V^ = code * scale in fp16 (low-bit class):
+//   - V in fp16 (full-precision class) and V^ (code times the power of two of its scale) in fp16 (low-bit class):
 //     the P.V products run as fp16 x fp16 MMAs
 //   - INT4 codes widened to one e4m3 byte each (-7..7 are exact in e4m3), so that the score MMA
 //     returns fp32 sums that are exact integers
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
+
+#include <algorithm>
 
 #include "attn_common.cuh"
 #include "quantize.cuh"
@@ -41,6 +43,8 @@ struct PreParams {
     const int32_t* vl_idx;
     const uint2 *q_codes, *k_codes;                          // packed INT4
     uint4 *v16, *vh16, *kvl, *vvl, *q8, *k8;
+    float4* kv_fac;
+    const float* k_scales;
     uint32_t* bits;
     uint8_t* tiles;
     uint32_t vl_plain, vl_knock;                             // element 0 of an operand tile's rows
@@ -57,7 +61,7 @@ struct PreParams {
         return s_;                                                                                          \
     }())
 
-// V (bf16) -> fp16 for the keys that some row's window holds and V^ = code * scale -> fp16 for those that some row sees
+// V (bf16) -> fp16 for the keys that some row's window holds and V^ -> fp16 for those that some row sees
 // low-bit (the last 1024 rows of 32768 keys with window 1024: 52 -> 43 us); one thread per 8 channels
 template <int V_FMT>
 __device__ __forceinline__ void pre_values(const TcSeqTable& tab, const PreParams& p, long e) {
@@ -76,7 +80,12 @@ __device__ __forceinline__ void pre_values(const TcSeqTable& tab, const PreParam
                               f16x2_sat(bf16_lo(w.z), bf16_hi(w.z)), f16x2_sat(bf16_lo(w.w), bf16_hi(w.w)));
     }
     if (tok >= 64 && (hi_lq < 0 || tok > (hi_lq | 63))) return;
-    const float sc = __ldg(p.v_scales + sq.ks0 + (long)head * sq.nb + (tok >> p.bt_shift));
+    const long block = sq.ks0 + (long)head * sq.nb + (tok >> p.bt_shift);
+    const float scale = __ldg(p.v_scales + block), sc = value_factor(scale);
+    if ((e & 15) == 0 && (tok & ((1 << p.bt_shift) - 1)) == 0) {
+        const float2 rest = value_rest(scale);
+        p.kv_fac[block] = make_float4(__ldg(p.k_scales + block), rest.x, rest.y, 0.0f);
+    }
     const uint2 cw = __ldg(p.v_codes + e);
     const uint32_t cs[2] = {cw.x, cw.y};
     uint32_t oh[4];
@@ -231,7 +240,7 @@ bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads
     t.n_unsplit = t.unsplit_ctas = 0;
     const int bt = a.block_tokens;
     TcSeq all[TC_MAX_SEQ];
-    long kv_rows = 0, vl_rows = 0, q_rows = 0, words = 0, units = 0;
+    long kv_rows = 0, vl_rows = 0, q_rows = 0, words = 0, units = 0, blocks = 0;
     for (int s = 0; s < n_seq; ++s) {
         TcSeq& q = all[s] = seq[s];
         q.src = s;
@@ -242,6 +251,7 @@ bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads
         if (q.split == 0 && n_seq > 1 && q.levels > TC_MAX_LEVELS) return false;
         kv_rows += (long)(heads / g) * q.L; vl_rows += (long)heads * q.k; q_rows += (long)heads * q.Lq; words += (long)heads * q.mask_words;
         units += (long)heads * q.levels;
+        blocks = std::max(blocks, (long)q.ks0 + (long)(heads / g) * q.nb);
     }
     if (q_rows > 0x7fffffffL || kv_rows > 0x7fffffffL || words > 0x7fffffffL || units > 0x3fffffffL) return false;
     t.kv_rows = (int)kv_rows; t.vl_rows = (int)vl_rows; t.q_rows = (int)q_rows;
@@ -290,6 +300,7 @@ bool tc_make_plan(const hyq_attn_args& a, const TcSeq* seq, int n_seq, int heads
     w.vl_bits = take((size_t)words * 4);
     w.v16 = take(kv_elems * 2);
     w.vh16 = take(kv_elems * 2);
+    w.kv_fac = take((size_t)blocks * 16);
     w.kvl = take(vl_elems * 2);
     w.vvl = take(vl_elems * 2);
     const bool int4 = a.q_format == HYQ_FMT_INT4;
@@ -367,6 +378,7 @@ int launch_tc_prepass(const hyq_attn_args& a, const TcPlan& plan, const TcSource
     p.v16 = reinterpret_cast<uint4*>(base + w.v16); p.vh16 = reinterpret_cast<uint4*>(base + w.vh16);
     p.kvl = reinterpret_cast<uint4*>(base + w.kvl); p.vvl = reinterpret_cast<uint4*>(base + w.vvl);
     p.q8 = reinterpret_cast<uint4*>(base + w.q8); p.k8 = reinterpret_cast<uint4*>(base + w.k8);
+    p.kv_fac = reinterpret_cast<float4*>(base + w.kv_fac); p.k_scales = a.k_scales;
     p.bits = reinterpret_cast<uint32_t*>(base + w.vl_bits);
     p.tiles = tc_has_vl_tiles(a, t.vl_rows) ? reinterpret_cast<uint8_t*>(base + w.vl_tiles) : nullptr;
     p.vl_plain = a.q_format == HYQ_FMT_INT8 ? VL_PLAIN_BF16 : 0u;

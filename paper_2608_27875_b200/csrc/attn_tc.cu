@@ -112,7 +112,7 @@ struct TcParams {
     int out_fp32;
     float scale_log2;            // softmax_scale * log2(e)
     const float* q_scales;
-    const float* k_scales;
+    const float4* kv_fac;        // per quantization block: K scale, log2 of the V scale's mantissa and its reciprocal (quantize.cuh)
     const int32_t* vl_idx;
     const uint32_t* vl_bits;
     int4* redo;                  // [0].x: pieces of work of the optimistic kernel that it gave up, [1 + i]: what they are (Piece)
@@ -803,23 +803,27 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             // K scale of a low-bit tile, fetched one tile ahead of its use (tile n of the low-bit pass sits at walk position n; its
             // block exists for n < a_end)
             // (other block sizes: a 64-key tile n lies in block n / 2 or in blocks 2n and 2n + 1, one per column half)
-            const float* ks_ptr = p.k_scales + ks_at;
-            float nks = 0.0f;
+            // The same for the V block's factor: V^ carries the scale's power of two, the weights its mantissa as an addend of
+            // their exponent (lr), which the row sum takes out again (ir).
+            const float4* fac_ptr = p.kv_fac + ks_at;
+            float nks = 0.0f, nlr = 0.0f, nir = 1.0f;
 #if HYQ_TC_VARIANT_BT
             float nks_b = 0.0f, cs_hi = 0.0f;                   // K scale and score factor of columns 32-63 (32-token blocks: their own block)
+            float nlr_b = 0.0f, nir_b = 1.0f, lr_hi = 0.0f, ir_hi = 1.0f;
 #endif
             auto prefetch_tile = [&](int n) {
-                nks = 0.0f;
+                float4 f = make_float4(0.0f, 0.0f, 1.0f, 0.0f);
 #if HYQ_TC_VARIANT_BT
-                nks_b = 0.0f;
-#endif
-                if (n >= own.a_end) return;
-#if HYQ_TC_VARIANT_BT
-                nks = __ldg(ks_ptr + ((n << 6) >> bsh));
-                nks_b = (bsh == 5) ? __ldg(ks_ptr + 2 * n + 1) : nks;
+                float4 fb = f;
+                if (n < own.a_end) {
+                    f = __ldg(fac_ptr + ((n << 6) >> bsh));
+                    fb = (bsh == 5) ? __ldg(fac_ptr + 2 * n + 1) : f;
+                }
+                nks_b = fb.x; nlr_b = fb.y; nir_b = fb.z;
 #else
-                nks = __ldg(ks_ptr + n);
+                if (n < own.a_end) f = __ldg(fac_ptr + n);
 #endif
+                nks = f.x; nlr = f.y; nir = f.z;
             };
             prefetch_tile(n0);
             const float qs2 = q_scale * p.scale_log2;
@@ -827,7 +831,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             // one tile of the online softmax for this thread's row: all 64 columns, in two register halves.  Returns
             // false when this warp ran into an expired wait.
             float tile_max = -INFINITY;                         // maximum of the tile last looked at (this row, log2 units)
-            auto do_tile = [&](auto range_tag, int n, float cs, bool int_scores, int lo, int hi, bool look = true) -> bool {
+            auto do_tile = [&](auto range_tag, int n, float cs, float lr, float ir, bool int_scores, int lo, int hi, bool look = true) -> bool {
                 constexpr bool NEED_RANGE = decltype(range_tag)::value;
                 const int nl = n - n0;                          // tile number within this CTA's slice
                 const int buf = nl & 1;
@@ -897,7 +901,7 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 }
                 // ---- P = 2^(s - m) as fp16 pairs over the first 32 columns of the buffer; row sum
                 const float m_eff = (m_used == -INFINITY) ? 0.0f : m_used;
-                const float bias = int_scores ? fmaf(-INT_MAGIC_F, cs, -m_eff) : -m_eff;
+                const float bias = int_scores ? fmaf(-INT_MAGIC_F, cs, lr - m_eff) : lr - m_eff;
                 uint32_t pa[16], pb[16];
                 auto exp_half = [&](bool some, const uint32_t (&raw)[32], float sc, float bi, uint32_t (&pk)[16]) -> float {
                     if (some) return row_exp32(raw, sc, bi, pk);
@@ -908,11 +912,12 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 const float t_a = exp_half(some_a, ra, cs, bias, pa);
                 tmem_st16(ts, pa);
 #if HYQ_TC_VARIANT_BT
-                const float t_b = exp_half(some_b, rb, csb, int_scores ? fmaf(-INT_MAGIC_F, csb, -m_eff) : -m_eff, pb);
+                const float t_b = exp_half(some_b, rb, csb, int_scores ? fmaf(-INT_MAGIC_F, csb, lr_hi - m_eff) : lr_hi - m_eff, pb);
+                l_h = fmaf(t_a, ir, fmaf(t_b, ir_hi, l_h));
 #else
                 const float t_b = exp_half(some_b, rb, cs, bias, pb);
+                l_h = fmaf(t_a + t_b, ir, l_h);                 // (the row sum is that of the weights without the value factor)
 #endif
-                l_h += t_a + t_b;
                 if (!look) over |= !(t_a + t_b < P_SUM_LIMIT);
                 tmem_st16(ts + 16, pb);
                 tmem_wait_st();
@@ -935,12 +940,13 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
             bool warm = false;
             const int n_plain_end = min(n_plain, n_total);
             auto plain_tile = [&]() -> bool {
-                const float cs = fmaxf(qs2 * nks, MIN_FACTOR);
+                const float cs = fmaxf(qs2 * nks, MIN_FACTOR), lr = nlr, ir = nir;
 #if HYQ_TC_VARIANT_BT
                 cs_hi = fmaxf(qs2 * nks_b, MIN_FACTOR);
+                lr_hi = nlr_b; ir_hi = nir_b;
 #endif
                 prefetch_tile(n + 1);
-                return do_tile(std::false_type{}, n, cs, !LOWBIT_FP8, 0, 0);
+                return do_tile(std::false_type{}, n, cs, lr, ir, !LOWBIT_FP8, 0, 0);
             };
             const bool brief = PIECES && pc.slot >= 0 && n_plain_end - n0 <= 2 * WARM_TILES;
             const int n_warm = n0 + (brief ? WARM_TILES_SHORT : WARM_TILES);
@@ -965,11 +971,11 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 uint32_t ra[32], rb[32];
                 bool have_a = false;
                 for (; n < n_end; ++n) {
-                    const float cs = fmaxf(qs2 * nks, MIN_FACTOR);
+                    const float cs = fmaxf(qs2 * nks, MIN_FACTOR), lr = nlr, ir = nir;
 #if HYQ_TC_VARIANT_BT
-                    const float csb = fmaxf(qs2 * nks_b, MIN_FACTOR);
+                    const float csb = fmaxf(qs2 * nks_b, MIN_FACTOR), lrb = nlr_b, irb = nir_b;
 #else
-                    const float csb = cs;
+                    const float csb = cs, lrb = lr;
 #endif
                     prefetch_tile(n + 1);
                     const int nl = n - n0, buf = nl & 1;
@@ -981,8 +987,8 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                     }
                     tmem_wait_ld();
                     tmem_ld32(ts + 32, rb);
-                    const float bias = LOWBIT_FP8 ? -m_used : fmaf(-INT_MAGIC_F, cs, -m_used);
-                    const float bias_b = LOWBIT_FP8 ? -m_used : fmaf(-INT_MAGIC_F, csb, -m_used);
+                    const float bias = LOWBIT_FP8 ? lr - m_used : fmaf(-INT_MAGIC_F, cs, lr - m_used);
+                    const float bias_b = LOWBIT_FP8 ? lrb - m_used : fmaf(-INT_MAGIC_F, csb, lrb - m_used);
                     uint32_t pa[16], pb[16];
                     const float t_a = row_exp32(ra, cs, bias, pa);
                     tmem_st16(ts, pa);
@@ -998,7 +1004,11 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                     }
                     const float t_b = row_exp32(rb, csb, bias_b, pb);
                     tmem_st16(ts + 16, pb);
-                    l_h += t_a + t_b;
+#if HYQ_TC_VARIANT_BT
+                    l_h = fmaf(t_a, ir, fmaf(t_b, irb, l_h));
+#else
+                    l_h = fmaf(t_a + t_b, ir, l_h);
+#endif
                     over |= !(t_a + t_b < P_SUM_LIMIT);
                     tmem_wait_st();
                     tc_fence_before();
@@ -1013,9 +1023,10 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                                   ? cnt_b_s[q] - vl_between(p.vl_bits + mask_at, qhi(ia), qhi(sq.i1 + off)) : 0;
             for (; n < n_total && !aborted; ++n) {
                 const int t = walk_pos(n);
-                const float ks = nks;
+                const float ks = nks, lr = nlr, ir = nir;       // (0 and 1 for the full-precision tiles)
 #if HYQ_TC_VARIANT_BT
                 const float ks_b = nks_b;
+                lr_hi = nlr_b; ir_hi = nir_b;
 #endif
                 prefetch_tile(n + 1);
                 int lo = 0, hi = -1;
@@ -1040,10 +1051,10 @@ attn_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcPa
                 // and, in the window of a row whose low-bit pass went without them, no maximum (525.3 -> 523.3 us; vertical-line keys
                 // are the ones with the large scores, so their tiles are always looked at)
                 if (__all_sync(0xffffffffu, lo == 0 && hi == BN - 1)) {
-                    if (!do_tile(std::false_type{}, n, cs, lowbit && !LOWBIT_FP8, 0, 0, !warm || t < own.b_end)) aborted = true;
+                    if (!do_tile(std::false_type{}, n, cs, lr, ir, lowbit && !LOWBIT_FP8, 0, 0, !warm || t < own.b_end)) aborted = true;
                     continue;
                 }
-                if (!do_tile(std::true_type{}, n, cs, lowbit && !LOWBIT_FP8, lo, hi)) aborted = true;
+                if (!do_tile(std::true_type{}, n, cs, lr, ir, lowbit && !LOWBIT_FP8, lo, hi)) aborted = true;
             }
 
             // ---- epilogue: the last P.V (MMAs complete in order), sum of the two halves' row sums, O / l
@@ -1307,7 +1318,7 @@ int launch_attn_tc(const hyq_attn_args& a, const TcPlan& plan, const TcSources* 
     p.mask_words = s0.mask_words;
     p.out_fp32 = a.out_dtype == 1;
     p.scale_log2 = alpha * 1.4426950408889634f;
-    p.q_scales = a.q_scales; p.k_scales = a.k_scales; p.vl_idx = a.vl_idx;
+    p.q_scales = a.q_scales; p.kv_fac = reinterpret_cast<const float4*>(base + w.kv_fac); p.vl_idx = a.vl_idx;
     p.vl_bits = reinterpret_cast<const uint32_t*>(base + w.vl_bits);
     p.vl_tiles = tc_has_vl_tiles(a, tab.vl_rows) ? reinterpret_cast<const uint8_t*>(base + w.vl_tiles) : nullptr;
     p.out = a.out; p.lse = a.lse; p.status = a.status_word;

@@ -8,7 +8,7 @@
 //
 // One launch covers any number of tensors (QuantJob: the Q, K and V of a call, of every prompt of a ragged batch), whose
 // tiles are numbered through; a tile looks its tensor up.  Inside the whole-path call a job may also write what the
-// attention kernel streams - V and V^ = code * scale as fp16, INT4 codes widened to e4m3 bytes - while the tile is in registers.
+// attention kernel streams - V and V^ as fp16, INT4 codes widened to e4m3 bytes - while the tile is in registers.
 //
 // Arithmetic is fp32 with one IEEE rounding per operation (no FMA contraction, no fast-math):
 //   scale = absmax / c ; inv = c / absmax ; code = rint(x * inv), which cannot leave [-c, c], or e4m3(x * inv).
@@ -56,7 +56,19 @@ __device__ __forceinline__ void quantize_tile(const QuantJob& job, int tile) {  
     constexpr float c = (FMT == HYQ_FMT_INT8) ? 127.0f : (FMT == HYQ_FMT_FP8_E4M3) ? 448.0f : 7.0f;
     const bool dead = !(amax >= 0x1p-100f);
     const float inv = dead ? 0.0f : __fdiv_rn(c, amax), scale = dead ? 0.0f : __fdiv_rn(amax, c);
-    if (threadIdx.x == 0) job.scales[tile] = scale;
+    if (threadIdx.x == 0) {
+        job.scales[tile] = scale;
+        if (EXTRAS && job.kv_fac) {
+            float* fac = reinterpret_cast<float*>(job.kv_fac + tile);
+            if (FMT != HYQ_FMT_INT4 && job.vh16) {
+                const float2 rest = value_rest(scale);
+                fac[1] = rest.x; fac[2] = rest.y;
+            } else {
+                fac[0] = scale;
+            }
+        }
+    }
+    const float vf = value_factor(scale);
 
     constexpr int ROW_BYTES = (FMT == HYQ_FMT_INT4) ? HYQ_D / 2 : HYQ_D;
     uint8_t* dst = job.codes + (head * job.L + t0) * (long)ROW_BYTES;
@@ -75,7 +87,7 @@ __device__ __forceinline__ void quantize_tile(const QuantJob& job, int tile) {  
                 for (int c2 = 0; c2 < 8; ++c2) {
                     const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((oc[c2 >> 1] >> (16 * (c2 & 1))) & 0xFFFFu), __NV_E4M3);
                     const float2 ff = __half22float2(__half2(hr));
-                    vh[c2] = f16x2_sat(ff.x * scale, ff.y * scale);
+                    vh[c2] = f16x2_sat(ff.x * vf, ff.y * vf);
                 }
             }
         } else if (FMT == HYQ_FMT_INT8) {
@@ -84,7 +96,7 @@ __device__ __forceinline__ void quantize_tile(const QuantJob& job, int tile) {  
 #pragma unroll
                 for (int c2 = 0; c2 < 8; ++c2) {
                     const uint2 q = round_pair(w[c2], inv);
-                    vh[c2] = f16x2_sat(rounded_value(q.x) * scale, rounded_value(q.y) * scale);
+                    vh[c2] = f16x2_sat(rounded_value(q.x) * vf, rounded_value(q.y) * vf);
                 }
             }
         } else {
@@ -146,7 +158,7 @@ static int launch_quantize_fmt(const QuantJobs& all, int block_tokens, cudaStrea
         q.tile0 = (int)tiles;
         tiles += (long)q.heads * ((q.L + block_tokens - 1) / block_tokens);
         if (tiles > 0x7fffffffL) return HYQ_ERR_INVALID_ARG;
-        extras |= q.vh16 != nullptr || q.wide != nullptr;
+        extras |= q.vh16 != nullptr || q.wide != nullptr || q.kv_fac != nullptr;
     }
     if (tiles == 0) return HYQ_OK;
 #define HYQ_QUANT(BT_) (extras ? launch_quantize_bt<FMT, BT_, true>(jobs, tiles, st) : launch_quantize_bt<FMT, BT_, false>(jobs, tiles, st))

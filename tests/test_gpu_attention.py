@@ -104,6 +104,29 @@ def test_extreme_code_sums_and_zero_tiles_around_vertical_keys(fmts):
     _check(Q, K, V, fmts, np.array([[a, b]], dtype=np.int32), W, api.IMPL_TCGEN05)
 
 
+@pytest.mark.parametrize("whole_call", [False, True])
+@pytest.mark.parametrize("bt", [32, 64, 128])
+@pytest.mark.parametrize("fmts", [INT8, INT4FP8, FP8ALL])
+def test_value_blocks_of_very_different_scale(fmts, bt, whole_call):
+    """A V block's scale is split between the values (its power of two) and the weights (its mantissa): neighbouring blocks
+    with unrelated scales, one of zeros, through the pre-pass and through the quantizer of the whole call."""
+    ensure_built()
+    L, W, k = 900, 100, 20
+    Q, K, V = (rand_bf16((1, h, L, 128), seed=70 + n) for n, h in enumerate((4, 2, 2)))
+    factor = torch.tensor([1.0, 1.9, 0.0, 0.013, 2.7, 0.31])[(torch.arange(L) // bt) % 6].view(1, 1, L, 1)
+    V = (V.float() * factor).to(torch.bfloat16)
+    qz = oracle_quant_all(Q, K, V, fmts, bt)
+    if whole_call:
+        res = api.hybrid_prefill_varlen([Q[0].cuda()], [K[0].cuda()], [V[0].cuda()], W, [k], fmts, block_tokens=bt)[0]
+        got, idx = res["out"][None].cpu().numpy(), res["idx"][None].cpu().numpy()
+    else:
+        idx = _rand_idx(1, 4, L - W, k, seed=9)
+        got = gpu_attention(Q, K, V, qz, fmts, idx, W, api.IMPL_TCGEN05, block_tokens=bt).numpy()
+    ref = _ref(Q, K, V, qz, fmts, idx, W, None, block_tokens=bt)
+    max_abs, mean_rel = errors(got, ref)
+    assert np.isfinite(got).all() and max_abs <= MAX_ABS_TOL and mean_rel <= MEAN_REL_TOL, (max_abs, mean_rel)
+
+
 @pytest.mark.parametrize("impl", IMPLS)
 def test_config0_full_output(impl):
     w = wl.CONFIGS["c0"]
