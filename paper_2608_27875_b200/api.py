@@ -58,11 +58,14 @@ class PrefillArgs(ctypes.Structure):
 
 
 _lib = None
+# csrc/binding.cpp: the marshalling of calls that wait for their host thread, in native code, once the library is loaded.  What it hands
+# back (tensors that it does not take) goes through the general paths of this file and decode_api, which report what is wrong with it.
+_native = None
 
 
 def lib() -> ctypes.CDLL:
     """The loaded shared library; raises if it is missing (no fallback)."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(f"{LIB_PATH} is missing: run `python -m paper_2608_27875_b200.build`")
@@ -96,6 +99,11 @@ def lib() -> ctypes.CDLL:
                                                                     ctypes.POINTER(ctypes.c_size_t)]
         L.hyq_hybrid_prefill_workspace.argtypes = [ctypes.c_void_p, ctypes.POINTER(ctypes.c_size_t)]      # (a PrefillArgs' address)
         L.hyq_hybrid_prefill.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+        try:
+            from . import _binding as native
+            _native = native
+        except ImportError:                          # (a torch without CUDA)
+            pass
         _lib = L
     return _lib
 
@@ -328,9 +336,18 @@ def _prefill(qs, ks, vs, B, Hq, Hkv, lens, window, k_per_seq, fmts, block_tokens
     return idx, (qc, kc, vc), (qs_, ks_, vs_), out
 
 
+_FP32_OUT = {torch.float32: 1, torch.bfloat16: 0}
+
+
 def hybrid_prefill(q, k, v, window: int, k_sel: int, fmts=(FMT_INT8, FMT_INT8, FMT_INT8), impl: int = IMPL_AUTO,
                    out_dtype=torch.float32):
     """The whole path on device tensors: select -> quantize Q, K, V -> fused attention."""
+    if _native and impl in (IMPL_AUTO, IMPL_TCGEN05) and out_dtype in _FP32_OUT:
+        res = _native.prefill(q, k, v, window, k_sel, fmts, _FP32_OUT[out_dtype])
+        if type(res) is dict:
+            return res
+        if res is not None:
+            raise HyqError(res, "hyq_hybrid_prefill")
     B, Hq, L, D = q.shape
     Bk, Hkv, Lk, Dk = sk = k.shape
     if v.shape != sk or Bk != B or Dk != D:                  # (the library sees pointers only)
@@ -375,6 +392,12 @@ def hybrid_prefill_varlen(qs, ks, vs, window: int, k_per_seq, fmts=(FMT_INT8, FM
     """The whole path over a ragged batch: ``qs[s]`` is [Hq, L_s, D], ``ks[s]`` / ``vs[s]`` are [Hkv, L_s, D] (bf16,
     CUDA).  Runs hyq_hybrid_prefill on the prompts where they lie and returns per-sequence views of the packed results:
     a list of dicts with idx [Hq, k_s], codes, scales and out [Hq, L_s, D]."""
+    if _native and out_dtype in _FP32_OUT:
+        res = _native.prefill_varlen(qs, ks, vs, window, k_per_seq, fmts, block_tokens, _FP32_OUT[out_dtype])
+        if type(res) is tuple:
+            return _checked(*res)
+        if res is not None:
+            raise HyqError(res, "hyq_hybrid_prefill")
     n = len(qs)
     # (a prompt that is a view of the caller's buffer may be strided or lie off a 16-byte boundary: copied then)
     qs, ks, vs = ([t if t.is_contiguous() and t.data_ptr() % 16 == 0 else t.clone(memory_format=torch.contiguous_format) for t in ts]
@@ -417,6 +440,10 @@ def hybrid_prefill_varlen(qs, ks, vs, window: int, k_per_seq, fmts=(FMT_INT8, FM
             v_scales=scales[2][Hkv * no:Hkv * (no + nb)].view(Hkv, nb), out=view(out, Hq, D)))
         ko += k_
         no += nb
+    return _checked(res, status)
+
+
+def _checked(res, status):
     code = int(status.item())                                # (waits for the results)
     if code != 0:
         raise HyqError(code, "hybrid_prefill_varlen (device)")

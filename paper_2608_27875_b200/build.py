@@ -3,7 +3,8 @@
     python -m paper_2608_27875_b200.build [--force] [--verbose]
 
 Each .cu becomes an object under build/ (recompiled only when it or a header
-changed, in parallel), then everything is linked into one shared library.
+changed, in parallel), then everything is linked into one shared library.  csrc/binding.cpp
+becomes the Python module _binding beside it (the marshalling of calls that wait for their host thread).
 """
 from __future__ import annotations
 
@@ -12,12 +13,14 @@ import os
 import re
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 OBJ = os.path.join(_HERE, "build")
 LIB = os.path.join(_HERE, "libhyq.so")
+BINDING = os.path.join(_HERE, "_binding.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -61,7 +64,26 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + f".{os.getpid()}.tmp"
         subprocess.check_call([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp] + objs)
         os.replace(tmp, LIB)
+    build_binding(force, hdr_time)
     return LIB
+
+
+def build_binding(force: bool, hdr_time: float) -> None:
+    src = os.path.join(CSRC, "binding.cpp")
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= max(os.path.getmtime(src), hdr_time):
+        return
+    import torch
+    inc, lib = (os.path.join(os.path.dirname(torch.__file__), d) for d in ("include", "lib"))
+    if not os.path.exists(os.path.join(lib, "libc10_cuda.so")):
+        return                                   # a torch without CUDA: nothing that these calls would run on
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    dirs = (inc, os.path.join(inc, "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"], cuda)
+    tmp = BINDING + f".{os.getpid()}.tmp"
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] +
+                          [a for d in dirs for a in ("-isystem", d)] +
+                          [src, "-o", tmp, "-L" + _HERE, "-l:" + os.path.basename(LIB), "-L" + lib, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda",
+                           "-lc10", "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, BINDING)
 
 
 if __name__ == "__main__":

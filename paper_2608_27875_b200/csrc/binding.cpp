@@ -1,0 +1,298 @@
+// Argument marshalling of the calls that wait for the thread that launches them: decode steps, the whole prefill.  Reading tensors
+// and allocating results through the interpreter and converting arguments through ctypes took longer than the kernels of a small
+// call: one decode step 12.0 -> 9.9 us, 16 appends and the attention of a ragged batch 128 -> 93, a prefill of 2048 tokens on 2 heads
+// 57.5 -> 45.5, eight prompts of 130 to 6000 tokens 674 -> 626.
+// Nothing here decides anything: what is not a plain, contiguous CUDA tensor of the expected type and shape is handed back to
+// the caller, whose general path takes or refuses it.
+#include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
+
+#include <ATen/ATen.h>
+#include <c10/cuda/CUDAStream.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "../../include/hyq.h"
+#include "../../include/hyq_decode.h"
+
+namespace {
+
+constexpr int64_t HEAD_DIM = 128;
+constexpr long NOT_PLAIN = -1;               // the caller takes its general path (no status code is negative)
+
+bool plain(PyObject* o, const at::Tensor** t) {
+    if (!THPVariable_CheckExact(o)) return false;
+    *t = &THPVariable_Unpack(o);
+    return (*t)->is_cuda() && (*t)->is_contiguous();
+}
+bool rows_bf16(PyObject* o, const void** data) {
+    const at::Tensor* t;
+    if (!plain(o, &t) || t->scalar_type() != at::kBFloat16) return false;
+    *data = t->const_data_ptr();
+    return true;
+}
+
+// the description that a ctypes structure holds
+struct Desc {
+    Py_buffer view{};
+    hyq_kv_cache* d = nullptr;
+    explicit Desc(PyObject* o) {
+        if (PyObject_GetBuffer(o, &view, PyBUF_WRITABLE) != 0) PyErr_Clear();
+        else if (view.len == (Py_ssize_t)sizeof(hyq_kv_cache)) d = static_cast<hyq_kv_cache*>(view.buf);
+    }
+    Desc(const Desc&) = delete;
+    ~Desc() { if (view.obj) PyBuffer_Release(&view); }
+};
+
+void* current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
+
+// append(desc, k_new, v_new): hyq_kv_cache_append on the current stream; the staged row is counted in the description
+PyObject* append(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (n != 3) return PyErr_Format(PyExc_TypeError, "append takes 3 arguments");
+    Desc c(a[0]);
+    const void *k, *v;
+    if (!c.d || !rows_bf16(a[1], &k) || !rows_bf16(a[2], &v)) return PyLong_FromLong(NOT_PLAIN);
+    void* st = current_stream();
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = hyq_kv_cache_append(k, v, c.d, st);
+    Py_END_ALLOW_THREADS
+    if (rc == HYQ_OK) ++c.d->n_staging;
+    return PyLong_FromLong(rc);
+    END_HANDLE_TH_ERRORS
+}
+
+// append_ragged(desc, k_new, v_new, b, lengths_host, lengths): hyq_kv_cache_append_ragged on the current stream
+PyObject* append_ragged(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (n != 6) return PyErr_Format(PyExc_TypeError, "append_ragged takes 6 arguments");
+    Desc c(a[0]);
+    const void *k, *v;
+    if (!c.d || !rows_bf16(a[1], &k) || !rows_bf16(a[2], &v) || !THPVariable_CheckExact(a[4]) || !THPVariable_CheckExact(a[5]))
+        return PyLong_FromLong(NOT_PLAIN);
+    const long b = PyLong_AsLong(a[3]);
+    if (b == -1 && PyErr_Occurred()) return nullptr;
+    int32_t *host = static_cast<int32_t*>(THPVariable_Unpack(a[4]).data_ptr()), *lengths = static_cast<int32_t*>(THPVariable_Unpack(a[5]).data_ptr());
+    void* st = current_stream();
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = hyq_kv_cache_append_ragged(k, v, c.d, (int)b, host, lengths, st);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(rc);
+    END_HANDLE_TH_ERRORS
+}
+
+// decode(desc, q, out, workspace, lse or None, lengths or None, softmax_scale, splits): one token's attention on the current stream
+PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (n != 8) return PyErr_Format(PyExc_TypeError, "decode takes 8 arguments");
+    Desc c(a[0]);
+    const void* q;
+    if (!c.d || !rows_bf16(a[1], &q) || THPVariable_Unpack(a[1]).dim() != 3 || !THPVariable_CheckExact(a[2]) || !THPVariable_CheckExact(a[3]))
+        return PyLong_FromLong(NOT_PLAIN);
+    const at::Tensor &out = THPVariable_Unpack(a[2]), &ws = THPVariable_Unpack(a[3]);
+    float* lse = nullptr;
+    const int32_t* lengths = nullptr;
+    if (a[4] != Py_None) {
+        if (!THPVariable_CheckExact(a[4])) return PyLong_FromLong(NOT_PLAIN);
+        lse = static_cast<float*>(THPVariable_Unpack(a[4]).data_ptr());
+    }
+    if (a[5] != Py_None) {
+        if (!THPVariable_CheckExact(a[5])) return PyLong_FromLong(NOT_PLAIN);
+        lengths = static_cast<const int32_t*>(THPVariable_Unpack(a[5]).const_data_ptr());
+    }
+    const double scale = PyFloat_AsDouble(a[6]);
+    const long splits = PyErr_Occurred() ? 0 : PyLong_AsLong(a[7]);
+    if (PyErr_Occurred()) return nullptr;
+    const int out_dtype = out.scalar_type() == at::kFloat ? 1 : 0;
+    void *o = out.data_ptr(), *w = ws.data_ptr(), *st = current_stream();
+    const size_t ws_bytes = (size_t)ws.numel();
+    const bool ragged = a[5] != Py_None;
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = ragged ? hyq_hybrid_attention_decode_ragged(q, c.d, lengths, (float)scale, (int)splits, out_dtype, o, lse, w, ws_bytes, st)
+                : hyq_hybrid_attention_decode(q, c.d, (float)scale, (int)splits, out_dtype, o, lse, w, ws_bytes, st);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(rc);
+    END_HANDLE_TH_ERRORS
+}
+
+// ---- the whole prefill in one call ----------------------------------------------------------------------------------
+bool as_int(PyObject* o, long* x) {
+    if (!PyLong_CheckExact(o)) return false;
+    *x = PyLong_AsLong(o);
+    if (*x == -1 && PyErr_Occurred()) { PyErr_Clear(); return false; }
+    return *x >= 0 && *x <= 0x7fffffffL;
+}
+int64_t code_row_bytes(long fmt) { return fmt == HYQ_FMT_INT4 ? HEAD_DIM / 2 : HEAD_DIM; }
+
+// what a call takes beside its tensors
+struct Options {
+    long window, fmt[3], block = 64, fp32;
+    bool read(PyObject* w, PyObject* fmts, PyObject* f32) {
+        if (!as_int(w, &window) || !as_int(f32, &fp32) || !PyTuple_CheckExact(fmts) || PyTuple_GET_SIZE(fmts) != 3) return false;
+        for (int i = 0; i < 3; ++i)
+            if (!as_int(PyTuple_GET_ITEM(fmts, i), &fmt[i])) return false;
+        return block == 32 || block == 64 || block == 128;
+    }
+};
+at::Tensor empty(at::IntArrayRef shape, at::ScalarType type, c10::Device dev) { return at::empty(shape, at::TensorOptions().dtype(type).device(dev)); }
+
+constexpr int REFUSED = -1;
+// the results of a call, allocated, and the call itself
+struct Prefill {
+    hyq_prefill_args a{};
+    std::vector<int32_t> lens, ks;
+    std::vector<const void*> q, k, v;
+    at::Tensor idx, codes[3], scales[3], out, status;
+
+    int run(int64_t B, int64_t Hq, int64_t Hkv, const Options& o, c10::Device dev) {
+        a.struct_size = sizeof(a);
+        a.n_seq = (int)lens.size(); a.B = (int)B; a.Hq = (int)Hq; a.Hkv = (int)Hkv; a.D = HEAD_DIM;
+        a.window = (int)o.window; a.block_tokens = (int)o.block;
+        a.q_format = (int)o.fmt[0]; a.k_format = (int)o.fmt[1]; a.v_format = (int)o.fmt[2];
+        a.out_dtype = o.fp32 ? 1 : 0;
+        a.lengths = lens.data(); a.k_per_seq = ks.data();
+        a.q = q.data(); a.k_ = k.data(); a.v = v.data();
+        a.idx = static_cast<int32_t*>(idx.data_ptr());
+        a.q_codes = codes[0].data_ptr(); a.k_codes = codes[1].data_ptr(); a.v_codes = codes[2].data_ptr();
+        a.q_scales = static_cast<float*>(scales[0].data_ptr()); a.k_scales = static_cast<float*>(scales[1].data_ptr());
+        a.v_scales = static_cast<float*>(scales[2].data_ptr());
+        a.out = out.data_ptr();
+        a.status_word = status.defined() ? static_cast<int32_t*>(status.data_ptr()) : nullptr;
+        size_t need = 0;
+        if (hyq_hybrid_prefill_workspace(&a, &need) != HYQ_OK) return REFUSED;       // (the caller's general path says why)
+        need = std::max<size_t>(need, 16);
+        const at::Tensor ws = empty({(int64_t)need}, at::kByte, dev);
+        a.workspace = ws.data_ptr(); a.workspace_bytes = need;
+        void* st = current_stream();
+        int rc;
+        Py_BEGIN_ALLOW_THREADS
+        rc = hyq_hybrid_prefill(&a, st);
+        Py_END_ALLOW_THREADS
+        return rc;
+    }
+};
+PyObject* as_dict(const at::Tensor& idx, const at::Tensor* codes, const at::Tensor* scales, const at::Tensor& out) {
+    static const char* const names[8] = {"idx", "q_codes", "k_codes", "v_codes", "q_scales", "k_scales", "v_scales", "out"};
+    const at::Tensor* const ts[8] = {&idx, codes, codes + 1, codes + 2, scales, scales + 1, scales + 2, &out};
+    THPObjectPtr d(PyDict_New());
+    for (int i = 0; d && i < 8; ++i) {
+        THPObjectPtr t(THPVariable_Wrap(*ts[i]));
+        if (!t || PyDict_SetItemString(d.get(), names[i], t.get())) return nullptr;
+    }
+    return d.release();
+}
+
+// prefill(q, k, v, window, k_sel, fmts, fp32): api.hybrid_prefill on plain [B, H, L, 128] tensors that belong together.  Returns the
+// dict of results, a status code, or None for a call that the caller has to look at.
+PyObject* prefill(PyObject*, PyObject* const* x, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (n != 7) return PyErr_Format(PyExc_TypeError, "prefill takes 7 arguments");
+    const at::Tensor* t[3];
+    Options o;
+    long k_sel;
+    if (!o.read(x[3], x[5], x[6]) || !as_int(x[4], &k_sel)) Py_RETURN_NONE;
+    for (int i = 0; i < 3; ++i)
+        if (!plain(x[i], &t[i]) || t[i]->scalar_type() != at::kBFloat16 || t[i]->dim() != 4) Py_RETURN_NONE;
+    const at::Tensor &q = *t[0], &k = *t[1], &v = *t[2];
+    const int64_t B = q.size(0), Hq = q.size(1), Hkv = k.size(1), L = q.size(2), nb = (L + 63) / 64;
+    if (q.size(3) != HEAD_DIM || k.size(0) != B || k.size(2) != L || k.size(3) != HEAD_DIM || v.sizes() != k.sizes() || L > 0x7fffffffL) Py_RETURN_NONE;
+    const int64_t kk = L > o.window ? k_sel : 0;
+    const c10::Device dev = q.device();
+    Prefill p;
+    p.lens = {(int32_t)L}; p.ks = {(int32_t)kk};
+    p.q = {q.const_data_ptr()}; p.k = {k.const_data_ptr()}; p.v = {v.const_data_ptr()};
+    p.idx = empty({B, Hq, kk}, at::kInt, dev);
+    for (int i = 0; i < 3; ++i) {
+        const int64_t H = i ? Hkv : Hq;
+        p.codes[i] = empty({B, H, L, code_row_bytes(o.fmt[i])}, at::kByte, dev);
+        p.scales[i] = empty({B, H, nb}, at::kFloat, dev);
+    }
+    p.out = empty({B, Hq, L, HEAD_DIM}, o.fp32 ? at::kFloat : at::kBFloat16, dev);
+    const int rc = p.run(B, Hq, Hkv, o, dev);
+    if (rc == REFUSED) Py_RETURN_NONE;
+    return rc == HYQ_OK ? as_dict(p.idx, p.codes, p.scales, p.out) : PyLong_FromLong(rc);
+    END_HANDLE_TH_ERRORS
+}
+
+// prefill_varlen(qs, ks, vs, window, k_per_seq, fmts, block_tokens, fp32): api.hybrid_prefill_varlen on lists of plain
+// [H, L_s, 128] tensors that belong together, each on a 16-byte boundary.  Returns (list of dicts, status word), a status code, or
+// None for a call that the caller has to look at.
+PyObject* prefill_varlen(PyObject*, PyObject* const* x, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (n != 8) return PyErr_Format(PyExc_TypeError, "prefill_varlen takes 8 arguments");
+    Options o;
+    if (!as_int(x[6], &o.block) || !o.read(x[3], x[5], x[7])) Py_RETURN_NONE;
+    for (int i : {0, 1, 2, 4})
+        if (!PyList_CheckExact(x[i]) || PyList_GET_SIZE(x[i]) != PyList_GET_SIZE(x[0])) Py_RETURN_NONE;
+    const Py_ssize_t N = PyList_GET_SIZE(x[0]);
+    if (N == 0) Py_RETURN_NONE;
+    Prefill p;
+    int64_t H[3] = {}, total = 0, blocks = 0, ks = 0;
+    for (Py_ssize_t s = 0; s < N; ++s) {
+        const at::Tensor* t[3];
+        long k_sel;
+        for (int i = 0; i < 3; ++i)
+            if (!plain(PyList_GET_ITEM(x[i], s), &t[i]) || t[i]->scalar_type() != at::kBFloat16 || t[i]->dim() != 3 ||
+                (reinterpret_cast<uintptr_t>(t[i]->const_data_ptr()) & 15u)) Py_RETURN_NONE;
+        if (!as_int(PyList_GET_ITEM(x[4], s), &k_sel)) Py_RETURN_NONE;
+        const int64_t L = t[0]->size(1);
+        for (int i = 0; i < 3; ++i) {
+            if (s == 0) H[i] = t[i]->size(0);
+            if (t[i]->size(0) != H[i] || t[i]->size(1) != L || t[i]->size(2) != HEAD_DIM) Py_RETURN_NONE;
+        }
+        if (H[1] != H[2] || L > 0x7fffffffL) Py_RETURN_NONE;
+        p.lens.push_back((int32_t)L); p.ks.push_back(L > o.window ? (int32_t)k_sel : 0);
+        p.q.push_back(t[0]->const_data_ptr()); p.k.push_back(t[1]->const_data_ptr()); p.v.push_back(t[2]->const_data_ptr());
+        total += L; blocks += (L + o.block - 1) / o.block; ks += p.ks.back();
+    }
+    const c10::Device dev = THPVariable_Unpack(PyList_GET_ITEM(x[0], 0)).device();
+    p.status = at::zeros({1}, at::TensorOptions().dtype(at::kInt).device(dev));
+    p.idx = empty({H[0] * ks}, at::kInt, dev);
+    for (int i = 0; i < 3; ++i) {
+        p.codes[i] = empty({H[i] * total * code_row_bytes(o.fmt[i])}, at::kByte, dev);
+        p.scales[i] = empty({H[i] * blocks}, at::kFloat, dev);
+    }
+    p.out = empty({H[0] * total * HEAD_DIM}, o.fp32 ? at::kFloat : at::kBFloat16, dev);
+    const int rc = p.run(1, H[0], H[1], o, dev);
+    if (rc == REFUSED) Py_RETURN_NONE;
+    if (rc != HYQ_OK) return PyLong_FromLong(rc);
+    THPObjectPtr list(PyList_New(N));
+    int64_t t0 = 0, k0 = 0, b0 = 0;
+    for (Py_ssize_t s = 0; list && s < N; ++s) {
+        const int64_t L = p.lens[s], kk = p.ks[s], nb = (L + o.block - 1) / o.block;
+        auto part = [](const at::Tensor& all, int64_t at, at::IntArrayRef shape) {
+            int64_t len = 1;
+            for (int64_t d : shape) len *= d;
+            return all.narrow(0, at, len).view(shape);
+        };
+        at::Tensor c[3], sc[3];
+        for (int i = 0; i < 3; ++i) {
+            const int64_t row = code_row_bytes(o.fmt[i]);
+            c[i] = part(p.codes[i], H[i] * row * t0, {H[i], L, row});
+            sc[i] = part(p.scales[i], H[i] * b0, {H[i], nb});
+        }
+        PyObject* d = as_dict(part(p.idx, H[0] * k0, {H[0], kk}), c, sc, part(p.out, H[0] * HEAD_DIM * t0, {H[0], L, HEAD_DIM}));
+        if (!d) return nullptr;
+        PyList_SET_ITEM(list.get(), s, d);
+        t0 += L; k0 += kk; b0 += nb;
+    }
+    THPObjectPtr status(list ? THPVariable_Wrap(p.status) : nullptr);
+    return status ? PyTuple_Pack(2, list.get(), status.get()) : nullptr;
+    END_HANDLE_TH_ERRORS
+}
+
+PyMethodDef methods[] = {{"append", (PyCFunction)(void (*)())append, METH_FASTCALL, nullptr},
+                         {"append_ragged", (PyCFunction)(void (*)())append_ragged, METH_FASTCALL, nullptr},
+                         {"decode", (PyCFunction)(void (*)())decode, METH_FASTCALL, nullptr},
+                         {"prefill", (PyCFunction)(void (*)())prefill, METH_FASTCALL, nullptr},
+                         {"prefill_varlen", (PyCFunction)(void (*)())prefill_varlen, METH_FASTCALL, nullptr},
+                         {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__binding() { return PyModule_Create(&module); }

@@ -33,11 +33,10 @@ class KvCacheSizes(ctypes.Structure):
 
 
 _bound = False
-_append_ragged = None          # the library's function, once bound (a step of a batch calls it for every sequence)
 
 
 def _lib():
-    global _bound, _append_ragged
+    global _bound
     L = api.lib()
     if not _bound:
         L.hyq_kv_cache_query_sizes.argtypes = [ctypes.POINTER(KvCacheDesc), ctypes.POINTER(KvCacheSizes)]
@@ -52,7 +51,6 @@ def _lib():
         L.hyq_hybrid_attention_decode_ragged.argtypes = [ctypes.c_void_p, ctypes.POINTER(KvCacheDesc), ctypes.c_void_p,
                                                          ctypes.c_float, ctypes.c_int, ctypes.c_int, ctypes.c_void_p,
                                                          ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]
-        _append_ragged = L.hyq_kv_cache_append_ragged
         _bound = True
     return L
 
@@ -86,10 +84,14 @@ class HybridKvCache:
 
     def append(self, k_new: torch.Tensor, v_new: torch.Tensor) -> None:
         """Places one token's rows ([B,Hkv,D] bf16, contiguous) in the staging buffer (hyq_kv_cache_append)."""
-        api._dev(k_new, torch.bfloat16, "k_new"), api._dev(v_new, torch.bfloat16, "v_new")
-        api._check(_lib().hyq_kv_cache_append(k_new.data_ptr(), v_new.data_ptr(), ctypes.byref(self.desc), api._stream()),
-                   "hyq_kv_cache_append")
-        self.desc.n_staging = self.n_staging + 1
+        rc = api._native.append(self.desc, k_new, v_new) if api._native else -1
+        if rc < 0:
+            api._dev(k_new, torch.bfloat16, "k_new"), api._dev(v_new, torch.bfloat16, "v_new")
+            rc = _lib().hyq_kv_cache_append(k_new.data_ptr(), v_new.data_ptr(), ctypes.byref(self.desc), api._stream())
+            if rc == 0:
+                self.desc.n_staging = self.n_staging + 1
+        if rc:
+            api._check(rc, "hyq_kv_cache_append")
 
     def bytes_read_per_token(self) -> int:
         """Bytes of cache one attention call reads: codes, scales and the valid bf16 rows."""
@@ -148,17 +150,24 @@ def hyq_hybrid_attention_decode(q: torch.Tensor, cache: HybridKvCache, softmax_s
                                 out_dtype=torch.bfloat16, out: torch.Tensor | None = None,
                                 lse: torch.Tensor | None = None, workspace: torch.Tensor | None = None) -> torch.Tensor:
     """Algorithm 3.  q [B,Hq,D] bf16 CUDA -> out [B,Hq,D]."""
-    api._dev(q, torch.bfloat16, "q")
-    B, Hq, D = q.shape
-    if out is None:
-        out = torch.empty(B, Hq, D, dtype=out_dtype, device=q.device)
-    if workspace is None:
-        workspace = torch.empty(max(hyq_hybrid_attention_decode_workspace(cache, splits), 16), dtype=torch.uint8,
-                                device=q.device)
-    api._check(_lib().hyq_hybrid_attention_decode(q.data_ptr(), ctypes.byref(cache.desc), softmax_scale, splits,
+    if out is None or workspace is None:
+        api._dev(q, torch.bfloat16, "q")
+        B, Hq, D = q.shape
+        if out is None:
+            out = torch.empty(B, Hq, D, dtype=out_dtype, device=q.device)
+        if workspace is None:
+            workspace = torch.empty(max(hyq_hybrid_attention_decode_workspace(cache, splits), 16), dtype=torch.uint8,
+                                    device=q.device)
+    rc = api._native.decode(cache.desc, q, out, workspace, lse, None, softmax_scale, splits) if api._native else -1
+    if rc < 0:
+        api._dev(q, torch.bfloat16, "q")
+        B, Hq, D = q.shape
+        rc = _lib().hyq_hybrid_attention_decode(q.data_ptr(), ctypes.byref(cache.desc), softmax_scale, splits,
                                                   1 if out.dtype == torch.float32 else 0, out.data_ptr(),
                                                   lse.data_ptr() if lse is not None else None, workspace.data_ptr(),
-                                                  workspace.numel(), api._stream()), "hyq_hybrid_attention_decode")
+                                                  workspace.numel(), api._stream())
+    if rc:
+        api._check(rc, "hyq_hybrid_attention_decode")
     return out
 
 
@@ -196,16 +205,16 @@ class RaggedKvCache:
 
     def append(self, b: int, k_new: torch.Tensor, v_new: torch.Tensor) -> None:
         """One token's rows ([Hkv,D] bf16) of sequence b into its staging buffer."""
-        for t, n in ((k_new, "k_new"), (v_new, "v_new")):
-            if not (t.is_cuda and t.dtype is torch.bfloat16 and t.is_contiguous()):
-                api._dev(t, torch.bfloat16, n)
         desc = self.batch.desc
         B = desc.B
-        if not -B <= b < B:
-            raise IndexError(f"sequence {b} of a batch of {B}")
-        rc = (_append_ragged or _lib().hyq_kv_cache_append_ragged)(
-            k_new.data_ptr(), v_new.data_ptr(), ctypes.byref(desc), b % B, self.lengths_host.data_ptr(), self.lengths.data_ptr(),
-            api._stream())
+        inside = -B <= b < B
+        rc = api._native.append_ragged(desc, k_new, v_new, b % B, self.lengths_host, self.lengths) if api._native and inside else -1
+        if rc < 0:
+            api._dev(k_new, torch.bfloat16, "k_new"), api._dev(v_new, torch.bfloat16, "v_new")
+            if not inside:
+                raise IndexError(f"sequence {b} of a batch of {B}")
+            rc = _lib().hyq_kv_cache_append_ragged(k_new.data_ptr(), v_new.data_ptr(), ctypes.byref(desc), b % B,
+                                                   self.lengths_host.data_ptr(), self.lengths.data_ptr(), api._stream())
         if rc:
             api._check(rc, "hyq_kv_cache_append_ragged")
 
@@ -214,16 +223,22 @@ def hyq_hybrid_attention_decode_ragged(q: torch.Tensor, cache: RaggedKvCache, so
                                        out_dtype=torch.bfloat16, out: torch.Tensor | None = None,
                                        lse: torch.Tensor | None = None, workspace: torch.Tensor | None = None) -> torch.Tensor:
     """Algorithm 3 for a batch of sequences of different lengths.  q [B,Hq,D] bf16 CUDA -> out [B,Hq,D]."""
-    api._dev(q, torch.bfloat16, "q")
-    B, Hq, D = q.shape
-    if out is None:
-        out = torch.empty(B, Hq, D, dtype=out_dtype, device=q.device)
-    if workspace is None:
-        workspace = torch.empty(max(hyq_hybrid_attention_decode_workspace(cache.batch, splits), 16), dtype=torch.uint8,
-                                device=q.device)
-    api._check(_lib().hyq_hybrid_attention_decode_ragged(q.data_ptr(), ctypes.byref(cache.batch.desc), cache.lengths.data_ptr(),
+    if out is None or workspace is None:
+        api._dev(q, torch.bfloat16, "q")
+        B, Hq, D = q.shape
+        if out is None:
+            out = torch.empty(B, Hq, D, dtype=out_dtype, device=q.device)
+        if workspace is None:
+            workspace = torch.empty(max(hyq_hybrid_attention_decode_workspace(cache.batch, splits), 16), dtype=torch.uint8,
+                                    device=q.device)
+    rc = api._native.decode(cache.batch.desc, q, out, workspace, lse, cache.lengths, softmax_scale, splits) if api._native else -1
+    if rc < 0:
+        api._dev(q, torch.bfloat16, "q")
+        B, Hq, D = q.shape
+        rc = _lib().hyq_hybrid_attention_decode_ragged(q.data_ptr(), ctypes.byref(cache.batch.desc), cache.lengths.data_ptr(),
                                                          softmax_scale, splits, 1 if out.dtype == torch.float32 else 0,
                                                          out.data_ptr(), lse.data_ptr() if lse is not None else None,
-                                                         workspace.data_ptr(), workspace.numel(), api._stream()),
-               "hyq_hybrid_attention_decode_ragged")
+                                                         workspace.data_ptr(), workspace.numel(), api._stream())
+    if rc:
+        api._check(rc, "hyq_hybrid_attention_decode_ragged")
     return out

@@ -1,0 +1,100 @@
+"""The native marshalling of calls (csrc/binding.cpp) against the general path of the same calls: the same results, and what it
+does not take is taken or refused there as before."""
+import pytest
+import torch
+
+from gpu_util import ensure_built, rand_bf16
+from paper_2608_27875_b200 import api, decode_api as dapi, workloads as wl
+
+pytestmark = pytest.mark.gpu
+INT8 = (wl.FMT_INT8,) * 3
+INT4FP8 = (wl.FMT_INT4, wl.FMT_INT4, wl.FMT_FP8_E4M3)
+
+
+def _both(monkeypatch, call):
+    """Results of the native and of the general path."""
+    ensure_built()
+    assert api._native is not None, "the binding is not built"
+    native = call()
+    with monkeypatch.context() as m:
+        m.setattr(api, "_native", None)
+        general = call()
+    torch.cuda.synchronize()
+    return native, general
+
+
+def _same(a, b):
+    assert a.keys() == b.keys()
+    for n in a:
+        assert a[n].shape == b[n].shape and a[n].dtype == b[n].dtype, n
+        assert torch.equal(a[n].reshape(-1).view(torch.uint8), b[n].reshape(-1).view(torch.uint8)), n
+
+
+@pytest.mark.parametrize("fmts", [INT8, INT4FP8])
+@pytest.mark.parametrize("out", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B,Hq,Hkv,L,W,k", [(1, 2, 2, 300, 64, 7), (2, 4, 1, 130, 128, 2), (1, 2, 1, 100, 200, 5)])
+def test_prefill(monkeypatch, fmts, out, B, Hq, Hkv, L, W, k):
+    q, k_, v = (rand_bf16((B, h, L, 128), seed=n).cuda() for n, h in enumerate((Hq, Hkv, Hkv)))
+    _same(*_both(monkeypatch, lambda: api.hybrid_prefill(q, k_, v, W, k, fmts, out_dtype=out)))
+
+
+@pytest.mark.parametrize("bt", [32, 64])
+@pytest.mark.parametrize("fmts", [INT8, INT4FP8])
+def test_prefill_varlen(monkeypatch, fmts, bt):
+    lens, ks = [257, 40, 600], [9, 0, 11]
+    qs, ks_, vs = ([rand_bf16((h, n, 128), seed=n + h).cuda() for n in lens] for h in (4, 2, 2))
+    for view in (False, True):               # (a strided prompt is copied on the general path)
+        if view:
+            ks_[1] = torch.cat([ks_[1], ks_[1]], 2)[:, :, :128]
+        for r in zip(*_both(monkeypatch, lambda: api.hybrid_prefill_varlen(qs, ks_, vs, 64, ks, fmts, bt))):
+            _same(*r)
+
+
+@pytest.mark.parametrize("bad", ["dtype", "strided", "shape", "window", "vertical", "formats"])
+def test_refused_prefills_stay_refused(monkeypatch, bad):
+    q, k, v = (rand_bf16((1, 2, 200, 128), seed=n).cuda() for n in range(3))
+    W, n, fmts = 64, 5, INT8
+    if bad == "dtype": q = q.half()                                      # noqa: E701
+    if bad == "strided": k = k.transpose(1, 2).contiguous().transpose(1, 2)   # noqa: E701
+    if bad == "shape": v = v[:, :1]                                      # noqa: E701
+    if bad == "window": W = -1                                           # noqa: E701
+    if bad == "vertical": n = 137                                        # noqa: E701
+    if bad == "formats": fmts = (wl.FMT_INT4,) * 3                       # noqa: E701
+    seen = []
+
+    def call():
+        try:
+            api.hybrid_prefill(q, k, v, W, n, fmts)
+        except Exception as e:               # noqa: BLE001
+            seen.append((type(e), str(e)))
+    _both(monkeypatch, call)
+    assert len(seen) == 2 and seen[0] == seen[1]
+
+
+@pytest.mark.parametrize("ragged", [False, True])
+def test_decode_step(monkeypatch, ragged):
+    B, Hq, Hkv, N, W = 2, 4, 2, 300, 64
+    new_k, new_v = (rand_bf16((B, Hkv, 128), seed=n).cuda() for n in (1, 2))
+    q = rand_bf16((B, Hq, 128), seed=3).cuda()
+    k, v = (rand_bf16((B, Hkv, N, 128), seed=n).cuda() for n in (4, 5))
+
+    def call():
+        lse = torch.empty(B, Hq, device="cuda")
+        if ragged:
+            c = dapi.RaggedKvCache(B, Hq, Hkv, N, W, 1)
+            for b in range(B):
+                c.freeze_sequence(b, k[b:b + 1], v[b:b + 1], None)
+                c.append(b - B, new_k[b], new_v[b])
+            with pytest.raises(IndexError):
+                c.append(B, new_k[0], new_v[0])
+            out = dapi.hyq_hybrid_attention_decode_ragged(q, c, lse=lse)
+            staged, count = c.batch.buffers["k_s"], c.lengths.clone()
+        else:
+            c = dapi.hyq_freeze(k, v, None, W, Hq)
+            c.append(new_k, new_v)
+            with pytest.raises(ValueError):
+                c.append(new_k.float(), new_v)
+            out = dapi.hyq_hybrid_attention_decode(q, c, lse=lse)
+            staged, count = c.buffers["k_s"], torch.tensor([c.n_staging])
+        return dict(out=out, lse=lse, staged=staged[:, :, :1].contiguous(), count=count)
+    _same(*_both(monkeypatch, call))
