@@ -246,6 +246,7 @@ int hyq_select_vertical_varlen(const void* q_, const void* k_, int n_seq, const 
     size_t k_before = 0;
     for (int s = 0; s < n_seq && rc == HYQ_OK;) {
         SelTable tab;
+        tab.early = 0;
         tab.n_seq = 0; tab.heads = Hq; tab.g = Hq / Hkv;
         for (; s < n_seq && tab.n_seq < SEL_MAX_SEQ; ++s) {
             const int L = cu[s + 1] - cu[s];
@@ -276,6 +277,7 @@ int hyq_quantize_blocks_varlen(const void* x, int n_seq, const int32_t* cu, int 
     size_t nb_before = 0;
     for (int s = 0; s < n_seq && rc == HYQ_OK;) {
         QuantJobs jobs;
+        jobs.beside = 0;
         for (jobs.n = 0; s < n_seq && jobs.n < QUANT_MAX_JOBS; ++s) {
             const int L = cu[s + 1] - cu[s];
             QuantJob& j = jobs.job[jobs.n++] = QuantJob{};
@@ -502,6 +504,7 @@ int hyq_hybrid_prefill_workspace(const hyq_prefill_args* args, size_t* bytes) {
     return HYQ_OK;
 }
 
+constexpr size_t BESIDE_BYTES = (size_t)256 << 20;
 int hyq_hybrid_prefill(const hyq_prefill_args* args, void* stream) {
     int rc = check_prefill(args, true);
     if (rc != HYQ_OK) return rc;
@@ -522,6 +525,7 @@ int hyq_hybrid_prefill(const hyq_prefill_args* args, void* stream) {
         QuantJobs jobs;
         TcSources src;
         jobs.n = 3 * n;
+        bool selects = false;
         size_t tt = 0, nb = 0;
         for (int i = 0; i < n; ++i) {
             const int L = a.lengths[s + i];
@@ -546,9 +550,16 @@ int hyq_hybrid_prefill(const hyq_prefill_args* args, void* stream) {
             jk.kv_fac = jv.kv_fac = reinterpret_cast<float4*>(base + g.plan.w.kv_fac) + a.Hkv * nb;
             tt += (size_t)L; nb += (size_t)((L + a.block_tokens - 1) / a.block_tokens);
             k0 += (size_t)a.k_per_seq[s + i];
+            selects |= g.sel.seq[i].P > 0 && g.sel.seq[i].k_sel > 0;          // (the selection launches something)
         }
-        rc = launch_quantize_jobs(jobs, a.block_tokens, st);
+        // Neither needs the other: the quantizer, which moves memory, runs beside the selection's three kernels, which wait for
+        // latencies and the fp64 pipe (2 heads x 2048 tokens 45.5 -> 42.8 us a call, eight prompts with 0.2 GB of Q, K and V 624 -> 616).
+        // Where both fill the GPU for long they only get in each other's way: 0.4 GB 6861 -> 6863 us, 0.9 GB 9924 -> 9977.
+        const bool beside = selects && 2 * (size_t)a.B * (a.Hq + 2 * a.Hkv) * tt * HYQ_D <= BESIDE_BYTES;
+        jobs.beside = g.sel.early = beside;
+        if (!beside) rc = launch_quantize_jobs(jobs, a.block_tokens, st);
         if (rc == HYQ_OK) rc = launch_select_table(g.sel, const_cast<int32_t*>(x.vl_idx), base + g.sel_at, st);
+        if (rc == HYQ_OK && beside) rc = launch_quantize_jobs(jobs, a.block_tokens, st);
         if (rc == HYQ_OK) rc = launch_planned(x, g.plan, &src, alpha, st);
         if (rc != HYQ_OK) return rc;
         t0 += tt; nb0 += nb;

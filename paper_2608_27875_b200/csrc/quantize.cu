@@ -126,13 +126,16 @@ __device__ __forceinline__ void quantize_tile(const QuantJob& job, int tile) {  
 template <int FMT, int BT, bool EXTRAS, int MAX>
 __global__ void __launch_bounds__(2 * BT)
 quantize_kernel(const __grid_constant__ QuantList<MAX> jobs) {
-    pdl_wait();
+    if (jobs.beside) pdl_launch_dependents();             // (a second launch, for the other format)
+    else pdl_wait();
     int lo = 0, hi = jobs.n - 1;                          // the job whose tiles this one is among
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (jobs.job[mid].tile0 <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
     }
     quantize_tile<FMT, BT, EXTRAS>(jobs.job[lo], blockIdx.x - jobs.job[lo].tile0);
+    // one block's wait is enough: the kernel behind this one waits for all its blocks, and so for the kernels before it
+    if (jobs.beside && blockIdx.x == 0) pdl_wait();
 }
 
 template <int FMT, int BT, bool EXTRAS>
@@ -140,7 +143,7 @@ static int launch_quantize_bt(const QuantJobs& jobs, long tiles, cudaStream_t st
     if (jobs.n > QUANT_FEW_JOBS)
         return launch_pdl(quantize_kernel<FMT, BT, EXTRAS, QUANT_MAX_JOBS>, dim3((unsigned)tiles), dim3(2 * BT), 0, st, jobs);
     QuantList<QUANT_FEW_JOBS> few;
-    few.n = jobs.n;
+    few.n = jobs.n; few.beside = jobs.beside;
     for (int j = 0; j < jobs.n; ++j) few.job[j] = jobs.job[j];
     return launch_pdl(quantize_kernel<FMT, BT, EXTRAS, QUANT_FEW_JOBS>, dim3((unsigned)tiles), dim3(2 * BT), 0, st, few);
 }
@@ -149,7 +152,7 @@ static int launch_quantize_bt(const QuantJobs& jobs, long tiles, cudaStream_t st
 template <int FMT>
 static int launch_quantize_fmt(const QuantJobs& all, int block_tokens, cudaStream_t st) {
     QuantJobs jobs;
-    jobs.n = 0;
+    jobs.n = 0; jobs.beside = all.beside;
     long tiles = 0;
     bool extras = false;
     for (int j = 0; j < all.n; ++j) {
@@ -176,7 +179,7 @@ int launch_quantize_jobs(const QuantJobs& jobs, int block_tokens, cudaStream_t s
 int launch_quantize(const void* x, long n_heads, int L, int block_tokens, int format, void* codes, float* scales, cudaStream_t st) {
     if (n_heads > 0x7fffffffL) return HYQ_ERR_INVALID_ARG;
     QuantJobs jobs;
-    jobs.n = 1;
+    jobs.n = 1; jobs.beside = 0;
     QuantJob& j = jobs.job[0] = QuantJob{};
     j.x = static_cast<const uint4*>(x); j.codes = static_cast<uint8_t*>(codes); j.scales = scales;
     j.L = L; j.heads = (int)n_heads; j.format = format;

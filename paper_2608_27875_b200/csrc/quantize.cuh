@@ -23,6 +23,7 @@ struct QuantJob {
 };
 template <int MAX> struct QuantList {
     int n;
+    int beside;                              // launched behind launch_select_table's kernels: runs beside them, is complete after them
     QuantJob job[MAX];
 };
 typedef QuantList<QUANT_MAX_JOBS> QuantJobs;

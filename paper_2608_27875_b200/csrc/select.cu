@@ -31,6 +31,7 @@ constexpr int MEAN_THREADS = 256, MEAN_CH = 32, MEAN_GROUPS = MEAN_THREADS / (ME
 __global__ void __launch_bounds__(MEAN_THREADS)
 tail_mean_kernel(const __grid_constant__ SelTable tab, double* __restrict__ qbar) {
     pdl_wait();
+    if (tab.early) pdl_launch_dependents();                      // (see launch_select_table)
     __shared__ double part[MEAN_GROUPS][MEAN_CH];
     __shared__ uint32_t red_max[MEAN_THREADS / 32], red_min[MEAN_THREADS / 32];
     const SelSeq& sq = tab.seq[blockIdx.y];
@@ -120,7 +121,7 @@ vscore_kernel(const __grid_constant__ SelTable tab, const double* __restrict__ q
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint4* ktile = reinterpret_cast<uint4*>(smem_raw);                              // [KEYS][SCORE_PITCH]
     double* qs = reinterpret_cast<double*>(smem_raw + KEYS * SCORE_PITCH * 16);     // [GC][D]
-    pdl_wait();
+    if (tab.early) pdl_launch_dependents();
     int n_s = 0;
     while (n_s + 1 < tab.n_seq && tab.seq[n_s + 1].block0 <= (int)blockIdx.x) ++n_s;
     const SelSeq& sq = tab.seq[n_s];
@@ -138,6 +139,7 @@ vscore_kernel(const __grid_constant__ SelTable tab, const double* __restrict__ q
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
+    pdl_wait();                                                      // (for the means; the keys are an input)
 
     for (int r0 = 0; r0 < tab.g; r0 += GC) {
         const long h0 = (long)n_s * tab.heads + (long)kvh * tab.g + r0;
@@ -225,6 +227,7 @@ topk_kernel(const __grid_constant__ SelTable tab, const double* __restrict__ sco
     __shared__ int wsum[NW], warp_gt[NW], warp_eq[NW], tot_gt, tot_eq, n_cand, sh_bin, sh_above, sh_cnt, sh_krem;
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    if (tab.early) pdl_launch_dependents();
     pdl_wait();
     const int row_no = blockIdx.x / C, s_no = row_no / tab.heads, head = row_no - s_no * tab.heads;
     const SelSeq& sq = tab.seq[s_no];
@@ -419,6 +422,10 @@ static int launch_vscore(const SelTable& tab, long blocks, const double* qbar, d
     return launch_pdl(vscore_kernel<GC, KPT>, dim3((unsigned)blocks), dim3(SCORE_THREADS), smem, st, tab, qbar, scores);
 }
 
+// tab.early: every kernel lets the next one be launched early, the mean's blocks behind their wait for what came before on the stream, the others'
+// at once, each waiting for the kernel before it where it reads its results.  All blocks of a kernel have started before a block of
+// the next one does, so that none waits for one without a place.  A kernel behind the three that needs none of their results may so
+// run beside them (the quantizer of the whole-path call): what came before the mean is complete when it starts.
 int launch_select_table(SelTable& tab, int32_t* idx_out, void* ws, cudaStream_t st) {
     double* qbar = static_cast<double*>(ws);
     double* scores = reinterpret_cast<double*>(static_cast<char*>(ws) + qbar_bytes(tab));

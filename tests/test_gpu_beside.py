@@ -1,0 +1,37 @@
+"""The whole-path call runs the quantizer beside the selection's kernels up to a size of its inputs and before them beyond it: on
+both sides of that line, and back to back on one workspace, its results are those of the stages called one by one."""
+import pytest
+import torch
+
+from gpu_util import ensure_built
+from paper_2608_27875_b200 import api, workloads as wl
+
+pytestmark = pytest.mark.gpu
+INT8 = (wl.FMT_INT8,) * 3
+INT4FP8 = (wl.FMT_INT4, wl.FMT_INT4, wl.FMT_FP8_E4M3)
+
+
+@pytest.mark.parametrize("fmts", [INT8, INT4FP8])                # (one launch of the quantizer, two)
+@pytest.mark.parametrize("B,Hq,Hkv,L,W,k", [
+    (1, 2, 2, 300, 64, 7),            # a few blocks
+    (1, 4, 1, 9000, 512, 180),        # clusters in the top-k
+    (1, 2, 1, 100, 200, 5),           # nothing to select: the quantizer waits by itself
+    (2, 32, 8, 10912, 256, 30),       # 255.75 MiB of Q, K and V (2 * 48 * 10912 * 256 bytes): beside
+    (2, 32, 8, 10944, 256, 30),       # 256.5 MiB: before
+])
+def test_stages_beside_each_other(fmts, B, Hq, Hkv, L, W, k):
+    ensure_built()
+    g = torch.Generator(device="cuda").manual_seed(L)
+    for _ in range(2):                # new inputs in the same memory: nothing of the call before may be in use any more
+        q, k_, v = (torch.randn(B, h, L, 128, device="cuda", generator=g).bfloat16() for h in (Hq, Hkv, Hkv))
+        res = [api.hybrid_prefill(q, k_, v, W, k, fmts) for _ in range(2)][1]
+        idx = api.hyq_select_vertical(q, k_, W, k if L > W else 0)
+        assert torch.equal(res["idx"], idx)
+        for n, x, f in zip("qkv", (q, k_, v), fmts):
+            c, s = api.hyq_quantize_blocks(x, f)
+            assert torch.equal(res[n + "_codes"], c) and torch.equal(res[n + "_scales"], s), n
+        if L < 1000:
+            out = api.hyq_hybrid_attention_prefill(q, k_, v, *(res[n + "_codes"] for n in "qkv"), *(res[n + "_scales"] for n in "qkv"), fmts,
+                                                   idx if idx.shape[2] else None, W)
+            assert torch.equal(res["out"], out)
+        del q, k_, v, res
